@@ -112,7 +112,13 @@ struct Elem<kSimFp8> {                       // FP8 E4M3
 // of the tile's columns into registers (16 candidate slots per thread) and
 // releasing the accumulators before it compares or stores: the next tile's
 // main products wait only for the TMEM loads.  FP8 tiles get eight warps too.
-template <int MODE, int BN_, int CM_, bool PAIR_ = false, bool EMIT_ = false>
+// WIDE_ (BF16, 256-object tiles, short rows): sixteen epilogue warps, four per
+// TMEM lane quarter.  A tile of a K-element row takes 8 K cycles of MMAs while
+// one warp per quarter needs some 6,800 cycles to drain and compare it (one
+// warp per scheduler: 85% of the cycles have no warp to issue), so below about
+// 800 elements the epilogue sets the pace; with four warps per scheduler its
+// TMEM loads and compares overlap one another (kWideMaxDim states the rule).
+template <int MODE, int BN_, int CM_, bool PAIR_ = false, bool EMIT_ = false, bool WIDE_ = false>
 struct Cfg {
     using E = Elem<MODE>;
     static constexpr int BN = BN_;
@@ -130,9 +136,9 @@ struct Cfg {
     // tiles whose epilogue bounds the tile (FP32-accurate tiles, which hold
     // TMEM alone; FP8, whose MMAs are few); BF16 tiles overlap four warps'
     // epilogue with the next tile's MMAs
-    static constexpr int EPI_WARPS = BN_ == 256 && (FOLD || MODE == kSimFp8) ? 8 : 4;
+    static constexpr int EPI_WARPS = WIDE_ ? 16 : (BN_ == 256 && (FOLD || MODE == kSimFp8) ? 8 : 4);
     static constexpr int THREADS = 64 + 32 * EPI_WARPS;         // + the producer and MMA warps
-    static constexpr int EMIT_SLOTS = 32 * 4 / EPI_WARPS;       // candidate words per epilogue thread
+    static constexpr int EMIT_SLOTS = WIDE_ ? 4 : 32 * 4 / EPI_WARPS;   // candidate words per epilogue thread
     static constexpr int EMIT_BYTES = EMIT_ ? EPI_WARPS * 32 * EMIT_SLOTS * 8 : 0;
     static constexpr int STAGING_BYTES = EPI_WARPS * 32 * 32 * 4;      // epilogue: one 32 x 32 FP32 block per warp
     static constexpr int SCALE_BYTES = MODE == kSimFp8 ? EPI_WARPS * BN_ * 4 : 0;   // FP8: a tile's column scales per warp
@@ -140,6 +146,7 @@ struct Cfg {
     static constexpr int BUDGET = STAGE_BUDGET < 227 * 1024 - FIXED_BYTES ? STAGE_BUDGET : 227 * 1024 - FIXED_BYTES;
     static constexpr int STAGES = BUDGET / STAGE_BYTES < 8 ? BUDGET / STAGE_BYTES : 8;
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + FIXED_BYTES;
+    static_assert(!WIDE_ || (MODE == kSimBf16 && BN_ == 256), "wide epilogues: BF16, 256-object tiles");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory per CTA");
     static_assert(BN_ % 128 == 0 && BN_ <= 256, "tile width");
     static_assert(STAGES >= 3, "pipeline depth");
@@ -476,15 +483,15 @@ __device__ __forceinline__ void store_rows_staged(float4 *blk, const float4 (&va
     __syncwarp();
 }
 
-template <int MODE, int BN_, int CM_, bool GROUPED, bool PAIR, bool EMIT = false>
-__global__ void __launch_bounds__((Cfg<MODE, BN_, CM_, PAIR, EMIT>::THREADS), 1)
+template <int MODE, int BN_, int CM_, bool GROUPED, bool PAIR, bool EMIT = false, bool WIDE = false>
+__global__ void __launch_bounds__((Cfg<MODE, BN_, CM_, PAIR, EMIT, WIDE>::THREADS), 1)
 sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant__ CUtensorMap map_q1,
               const __grid_constant__ CUtensorMap map_d0, const __grid_constant__ CUtensorMap map_d1,
               const GemmPiece *__restrict__ pieces, int32_t n_pieces, const GemmPiece single,
               float *__restrict__ S, float *__restrict__ tops, int32_t k_slices, int32_t total,
               const float *__restrict__ scale_q, int32_t *err, const FuseEmit emit)
 {
-    using C = Cfg<MODE, BN_, CM_, PAIR, EMIT>;
+    using C = Cfg<MODE, BN_, CM_, PAIR, EMIT, WIDE>;
     using M = Elem<MODE>;
     constexpr bool TWO_OPERAND_TILES = !M::SPLIT;
     constexpr int B_SMEM = C::B_SMEM;
@@ -737,14 +744,17 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
         uint32_t tc = 0;
         for (int tile = cluster_id; tile < total; tile += n_clusters, ++tc) {
             const uint32_t buf = tc % NACC, use = tc / NACC;
-            // EMIT: the row's threshold is read before the accumulator is waited for
+            // EMIT: the row's threshold is read before the accumulator is waited for;
+            // tiles without a fold keep their piece from then on too (a fold's
+            // registers leave no room for it: there it is looked up again)
             uint32_t tk = 0xffffffffu;
-            if constexpr (EMIT) {
-                const GemmPiece pt = piece_of<GROUPED>(tile, pieces, n_pieces, single);
-                int tm0, tn0, tc0;
-                piece_tile<BN_, CM_>(pt, tile, rank, tm0, tn0, tc0);
-                const int64_t tr = (int64_t)tm0 + quad * 32 + lane;
-                if (tr < pt.rows) tk = __ldg(emit.tau_key + pt.q_row0 + tr);
+            GemmPiece pc;
+            int m0 = 0, n0 = 0, c0 = 0;
+            if constexpr (EMIT || !FOLD) {
+                pc = piece_of<GROUPED>(tile, pieces, n_pieces, single);
+                piece_tile<BN_, CM_>(pc, tile, rank, m0, n0, c0);
+                const int64_t tr = (int64_t)m0 + quad * 32 + lane;
+                if (EMIT && tr < pc.rows) tk = __ldg(emit.tau_key + pc.q_row0 + tr);
             }
             if (!mbar_wait(&acc_full[buf], use & 1u) || *abort_flag) {
                 *abort_flag = 1;
@@ -794,9 +804,10 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
                     }
                 }
             }
-            const GemmPiece pc = piece_of<GROUPED>(tile, pieces, n_pieces, single);
-            int m0, n0, c0;
-            piece_tile<BN_, CM_>(pc, tile, rank, m0, n0, c0);
+            if constexpr (FOLD) {
+                pc = piece_of<GROUPED>(tile, pieces, n_pieces, single);
+                piece_tile<BN_, CM_>(pc, tile, rank, m0, n0, c0);
+            }
             const int64_t r = (int64_t)m0 + quad * 32 + lane;    // row within the piece
             const int64_t rows = pc.rows, n = pc.n;
             const bool live = r < rows;
@@ -1016,6 +1027,16 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
                     for (int j = 0; j < NCH; ++j)
                         t4[j] = make_float4(gmax[4 * j], gmax[4 * j + 1], gmax[4 * j + 2], gmax[4 * j + 3]);
                     store_rows_staged<NCH>(blk, t4, lane, tblk + c0 / 8 + 4 * cbase, gs, rows - r_blk);
+                } else if constexpr (NCH < 4) {
+                    // (two groups of 32 per row and warp: one 8-byte store per row)
+                    static_assert(NCH == 2 || NCH >= 4, "groups per warp");
+                    float g2[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        g2[u] = fmaxf(fmaxf(gmax[4 * u], gmax[4 * u + 1]), fmaxf(gmax[4 * u + 2], gmax[4 * u + 3]));
+                    if (live)
+                        *reinterpret_cast<float2 *>(tblk + (int64_t)lane * gs + c0 / 32 + cbase) =
+                            make_float2(g2[0], g2[1]);
                 } else {
                     float4 t4[NCH / 4];
 #pragma unroll
@@ -1088,16 +1109,16 @@ bool make_map(CUtensorMap *m, const void *base, int64_t inner, int64_t outer, in
 // as can be resident at once (a GPC with an odd number of free SMs cannot
 // hold a whole cluster on its last SM); the count is cached per device and
 // kernel (concurrent first calls compute the same value).
-template <int MODE, int BN_, int CM_, bool GROUPED, bool PAIR = false, bool EMIT = false>
+template <int MODE, int BN_, int CM_, bool GROUPED, bool PAIR = false, bool EMIT = false, bool WIDE = false>
 cudaError_t launch_impl(const CUtensorMap &mq0, const CUtensorMap &mq1, const CUtensorMap &md0,
                         const CUtensorMap &md1, const GemmPiece *pieces, int32_t n_pieces, const GemmPiece &single,
                         float *S, float *tops, int32_t k_slices, int64_t total_tiles, const float *scale_q,
                         int num_sms, int32_t *err, cudaStream_t s, const FuseEmit &emit = FuseEmit{})
 {
-    using C = Cfg<MODE, BN_, CM_, PAIR, EMIT>;
+    using C = Cfg<MODE, BN_, CM_, PAIR, EMIT, WIDE>;
     if (total_tiles <= 0) return cudaSuccess;
     if (total_tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    auto kernel = sim_tc_kernel<MODE, BN_, CM_, GROUPED, PAIR, EMIT>;
+    auto kernel = sim_tc_kernel<MODE, BN_, CM_, GROUPED, PAIR, EMIT, WIDE>;
     const int smem_bytes = C::SMEM_BYTES;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
     if (e != cudaSuccess) return e;
@@ -1132,6 +1153,14 @@ cudaError_t launch_impl(const CUtensorMap &mq0, const CUtensorMap &mq1, const CU
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
+
+// Grouped BF16 launches over rows of at most this many elements take the wide
+// (sixteen-warp) epilogue: at 128 elements (6,001 queries with 15,105
+// landmark rows over 100,000 objects) the launch that stores the group maxima
+// took 574 us against 1,332 with four warps and the emitting one 902 against
+// 1,530; at 1,152 elements the MMAs set the pace and eight warps measured no
+// faster than four (0.459 against 0.453 ms, 14,200 rows x 20,000 objects).
+constexpr int kWideMaxDim = 512;
 
 // Rows are padded to kDimAlign (64) elements; the FP8 K slice (128 bytes) may
 // run past the row end, where the tensor map's bounds fill zeros.
@@ -1211,12 +1240,22 @@ cudaError_t launch_grouped(const void *q0, const void *q1, int64_t rows_total, i
     if (emit) {
         if constexpr (BN_ == 256) {
             if (!emit->tau_key || !emit->cnt || !emit->cand || emit->cap < 1) return cudaErrorInvalidValue;
+            if constexpr (MODE == kSimBf16)
+                if (dim_pad <= kWideMaxDim)
+                    return launch_impl<MODE, BN_, CM_, true, PAIR, true, true>(
+                        mq0, mq1, mq0, mq1, pieces, n_pieces, unused, S, tops, k_slices_of<MODE>(dim_pad), total_tiles,
+                        scale_q, num_sms, err, s, *emit);
             return launch_impl<MODE, BN_, CM_, true, PAIR, true>(mq0, mq1, mq0, mq1, pieces, n_pieces, unused, S,
                                                            tops, k_slices_of<MODE>(dim_pad), total_tiles, scale_q,
                                                            num_sms, err, s, *emit);
         }
         return cudaErrorInvalidValue;     // the fused selection samples tiles of 256 objects
     }
+    if constexpr (MODE == kSimBf16 && BN_ == 256)
+        if (dim_pad <= kWideMaxDim)
+            return launch_impl<MODE, BN_, CM_, true, PAIR, false, true>(
+                mq0, mq1, mq0, mq1, pieces, n_pieces, unused, S, tops, k_slices_of<MODE>(dim_pad), total_tiles, scale_q,
+                num_sms, err, s);
     return launch_impl<MODE, BN_, CM_, true, PAIR>(mq0, mq1, mq0, mq1, pieces, n_pieces, unused, S, tops,
                                              k_slices_of<MODE>(dim_pad), total_tiles, scale_q, num_sms, err, s);
 }
