@@ -1034,6 +1034,7 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
             Batch &bt = batches.back();
             farm::Piece pc{};
             pc.d32 = s.desc32;
+            pc.cls = s.cls;
             pc.s_off = bt.s_floats;
             pc.row_begin = bt.rows;
             pc.block_begin = bt.blocks;
@@ -1121,6 +1122,12 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
     }
     int32_t *d_rowlist;
     CK(ws_get(ctx, farm::B_SELLIST, (size_t)tblocks_max + 1, &d_rowlist));
+    int32_t *d_resc = nullptr;
+    if (reduced) {
+        size_t ints = 0;
+        for (const auto &bt : batches) ints = std::max(ints, farm::rescore_scratch_ints(bt.rows - bt.exact_rows));
+        if (ints > 0) CK(ws_get(ctx, farm::B_RESCORE, ints, &d_resc));
+    }
     if (any_chunked) {
         CK(ws_get(ctx, farm::B_CHUNK_IDX, (size_t)tmp_need, &tmp_idx));
         CK(ws_get(ctx, farm::B_CHUNK_VAL, (size_t)tmp_need, &tmp_val));
@@ -1431,7 +1438,7 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
                                                     precision == FARM_PREC_LEARNED ? nullptr : bsel_tv, cstride_t,
                                                     bsel_l, precision == FARM_PREC_LEARNED ? nullptr : bsel_lv,
                                                     cstride_l, band, tsel_idx, tsel_cos, stride_t, lsel_idx, stride_l,
-                                                    c.d_err, c.stream));
+                                                    d_resc, c.stream));
             }
             mark_end(ctx, bt.fused_rows > 0 ? m2c : m2);
         }

@@ -115,6 +115,7 @@ enum Buf {
     B_FUSE_CAND,    // uint64 [rows, cap] its candidate words
     B_FUSE_OVF,     // int32 [2 + 2 rows] overflow count, long-row count, overflowed launch rows, long launch rows
     B_FUSE_SLAB,    // float [blocks, n] the exact fallback's similarity rows
+    B_RESCORE,      // int32 the rescore's processing order (bucket counts, places, order)
     B_RAW_PIPE,     // farm_query_batch's host rows: two slots, each [n_q + n_c, dim] (copy stream)
     B_COUNT
 };
@@ -428,6 +429,7 @@ cudaError_t launch_select_rows_ex(const float *S, int64_t ld_s, int64_t n, int64
 // afterwards.  Pieces of a launch are ordered by every *_begin field.
 struct Piece {
     const float *d32;       // the scene's unit FP32 descriptors (rescore)
+    const int32_t *cls;     // its objects' classes (the rescore's processing order)
     int64_t s_off;          // offset of the block's first row in S (floats)
     int64_t row_begin;      // first launch row of the block
     int64_t block_begin;    // first shared-memory-select block (th0 x chunks blocks)
@@ -541,13 +543,14 @@ cudaError_t launch_copy_lists(const Piece *pieces, int32_t n_pieces, int64_t row
 // exact FP32 dot products of the unit rows Q32 and the descriptors d32, and
 // the R / klm best in rank order go to tsel_idx / tsel_cos and lsel_idx (-1 /
 // 0 past the list).  With values, a candidate more than `band` below the
-// list's R-th value is skipped.  A bulk copy that does not arrive within the
-// bounded wait sets kErrTimeout in *err and leaves that row's list empty.
+// list's R-th value is skipped.  scratch: rescore_scratch_ints(total_rows)
+// int32 of device memory (the processing order of large launches).
+size_t rescore_scratch_ints(int64_t rows);
 cudaError_t launch_rescore_grouped(const Piece *pieces, int32_t n_pieces, int64_t total_rows, const float *Q32,
                                    int32_t dim_pad, const int32_t *bsel_t, const float *bsel_tv, int32_t cstride_t,
                                    const int32_t *bsel_l, const float *bsel_lv, int32_t cstride_l, float band,
                                    int32_t *tsel_idx, float *tsel_cos, int32_t stride_t, int32_t *lsel_idx,
-                                   int32_t stride_l, int32_t *err, cudaStream_t s);
+                                   int32_t stride_l, int32_t *scratch, cudaStream_t s);
 constexpr int kSelectRowMax = 24576;    // longest row the shared-memory select stages
 
 #ifdef __CUDACC__

@@ -16,16 +16,15 @@
 // (Piece::exact) already hold their final lists: copy_lists_kernel copies
 // them, a warp per row.
 //
-// One CTA per row.  The work is a gather of whole descriptor rows (4.6 KB at
-// D = 1152), mostly from L2, so what bounds it is the bytes in flight per SM.
-// Rows of up to kTmaDimMax floats: each warp keeps SPW candidate rows in
-// flight as bulk asynchronous copies (cp.async.bulk, completion counted on one
-// mbarrier per slot) into its own shared-memory slots, and refills a slot as
-// soon as its lanes have read it; the dot product is taken from shared memory.
-// Longer rows: each warp loads two candidates at a time with four float4 loads
-// of each in flight per lane.  The in-band candidates' keys (cosine key, index;
-// all distinct) are then ranked: by counting up to 256 of them, else by a
-// bitonic sort.
+// The work is a gather of whole descriptor rows (4.6 KB at D = 1152): the rows
+// of one class of objects list mostly the same candidates, so a block takes
+// four rows that are neighbours in an order by class and loads each candidate
+// of their union once (rescore_group_kernel; launches of few rows take a row
+// per block).  At 100,000 objects, D = 1152: 1.35 ms against 1.98 with a row
+// per block (lists of 512 / 128, 6,001 target and 15,105 landmark rows, then
+// bound by DRAM at 74% of its peak), 1.41 against 2.20 (lists of 256 / 64,
+// 16,384 and 40,900 rows).  Rows longer than kGroupDimMax floats: a row per block, two
+// candidates per warp step.
 #include "farm_internal.h"
 
 namespace farm {
@@ -46,221 +45,393 @@ __device__ __forceinline__ float key_value(uint32_t k)
     return __uint_as_float(u);
 }
 
-constexpr uint32_t WAIT_LIMIT = 1u << 22;   // try_wait polls before giving up (a fraction of a second)
 constexpr int kWarps = TH / 32;
-constexpr int kTmaDimMax = 2048;            // longest rows (floats) staged through shared-memory slots
+constexpr int kGroupDimMax = 2048;          // longest rows (floats) the grouped kernel stages
+// Rows a block takes together, and the launch size from which it does: below
+// it a row per block keeps more SMs busy (2,048 rows are 512 blocks of four).
+constexpr int kGroupRows = 4;
+constexpr int64_t kGroupFrom = 2048;
+constexpr int kBuckets = 4096;              // of the processing order's counting sort
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-// Bounded wait for the phase with the given parity; false on expiry.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity)
-{
-    const uint32_t a = smem_u32(bar);
-    for (uint32_t i = 0; i < WAIT_LIMIT; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
-// bytes (a multiple of 16) from global src (16-byte aligned) into shared dst
-// (16-byte aligned), completion counted on bar, which expects them.
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-
-// Dynamic shared memory of the slot routine: the query row, the warps' slots,
-// the in-band candidates, their keys, the slots' mbarriers.
-struct RescoreSmem {
-    size_t q, slots, cand, key, bar, bytes;
-    __host__ __device__ RescoreSmem(int dim_pad, int spw, int cmax)
+// Dynamic shared memory of a block of G rows with lists of at most cmax:
+// the unit rows; the union's hash table (object, a byte of row bits), whose
+// place the rows' keys take once the union is listed; the union's list.
+struct GroupSmem {
+    size_t q, hkey, hmask, key, obj, mask, bytes;
+    int H;
+    __host__ __device__ GroupSmem(int dim_pad, int G, int cmax)
     {
-        const size_t row = (size_t)dim_pad * 4;
+        auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
+        const int E = G * cmax;
+        H = 64;
+        while (G > 1 && H < E + (E >> 1)) H <<= 1;
         q = 0;
-        slots = q + row;
-        cand = slots + (size_t)kWarps * spw * row;
-        int p2 = 1;
-        while (p2 < cmax) p2 <<= 1;          // the keys' sort pads to a power of two
-        key = cand + (((size_t)cmax * 4 + 7) / 8) * 8;
-        bar = key + (size_t)p2 * 8;
-        bytes = bar + (size_t)kWarps * spw * 8;
+        hkey = up(q + (size_t)G * dim_pad * 4);
+        hmask = hkey + (size_t)H * 4;
+        key = hkey;
+        const size_t a = up(hmask + H), k = up(key + (size_t)E * 8);
+        obj = a > k ? a : k;
+        mask = up(obj + (size_t)E * 4);
+        bytes = up(mask + E);
     }
 };
 
-// The R best of the n in-band keys (all distinct) into oi / oc in rank
-// order, -1 / 0 past them.  Up to 256 keys: each one's rank counted against
-// the others (a count stops once it reaches R: that key is not kept); more: a
-// bitonic sort of the keys padded with zeros to a power of two (key holds
-// that many slots).
-__device__ __forceinline__ void rank_out(uint64_t *key, int n, int R, int32_t *__restrict__ oi,
-                                         float *__restrict__ oc, int32_t out_stride)
+// What a block needs of one of its rows.
+struct GroupRow {
+    const float *d32;
+    int64_t co;              // its list's offset
+    int64_t oo;              // its output list's offset
+    int64_t q_row;
+    float thr;               // candidates valued below it are out of the band
+    int32_t C, R, n_obj, tgt;
+};
+
+__device__ __forceinline__ int find_row_piece(const Piece *__restrict__ pieces, int n_pieces, int64_t r)
 {
-    const int tid = threadIdx.x;
-    if (n <= 256) {
-        for (int i = tid; i < n; i += TH) {
-            const uint64_t k = key[i];
-            int c = 0;
-            for (int j = 0; j < n && c < R; ++j) c += key[j] > k ? 1 : 0;
-            if (c < R && c < out_stride) {
-                oi[c] = (int32_t)(0xffffffffu - (uint32_t)(k & 0xffffffffu));
-                if (oc) oc[c] = key_value((uint32_t)(k >> 32));
-            }
-        }
-    } else {
-        int P = 1;
-        while (P < n) P <<= 1;
-        for (int i = n + tid; i < P; i += TH) key[i] = 0ull;
-        __syncthreads();
-        for (int k = 2; k <= P; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = tid; i < P; i += TH) {
-                    const int ixj = i ^ j;
-                    if (ixj > i) {
-                        const uint64_t a = key[i], b = key[ixj];
-                        const bool desc = (i & k) == 0;
-                        if (desc ? (a < b) : (a > b)) { key[i] = b; key[ixj] = a; }
-                    }
-                }
-                __syncthreads();
-            }
-        }
-        for (int i = tid; i < R && i < n && i < out_stride; i += TH) {
-            oi[i] = (int32_t)(0xffffffffu - (uint32_t)(key[i] & 0xffffffffu));
-            if (oc) oc[i] = key_value((uint32_t)(key[i] >> 32));
+    int lo = 0, hi = n_pieces - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (pieces[mid].row_begin <= r) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// The R best of the n distinct keys of one row (shared memory, n <= 32 REG),
+// by one warp, into oi / oc in rank order, -1 / 0 past them.  The R-th largest
+// 32-bit value key T by a bitwise search below the leading bits that the
+// smallest and largest share (stopped once exactly R keys reach the
+// candidate); the words reaching T gathered in place; those ranked by counting.
+template <int REG>
+__device__ __forceinline__ void warp_rank_out(uint64_t *key, int n, int R, int32_t *__restrict__ oi,
+                                              float *__restrict__ oc, int out_stride, int lane)
+{
+    const unsigned FULL = 0xffffffffu;
+    uint64_t w[REG];
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll
+    for (int k = 0; k < REG; ++k) {
+        const int t = lane + 32 * k;
+        w[k] = t < n ? key[t] : 0ull;          // (no real word is 0: its key would encode a NaN)
+        if (t < n) {
+            kmin = min(kmin, (uint32_t)(w[k] >> 32));
+            kmax = max(kmax, (uint32_t)(w[k] >> 32));
         }
     }
-    for (int i = min(n, R) + tid; i < out_stride; i += TH) {
-        oi[i] = -1;
-        if (oc) oc[i] = 0.f;
+    kmin = __reduce_min_sync(FULL, kmin);
+    kmax = __reduce_max_sync(FULL, kmax);
+    const int keep = min(n, min(R, out_stride));
+    uint32_t T = 0u;
+    if (n > keep) {
+        const uint32_t diff = kmin ^ kmax;
+        const int top = diff ? 31 - __clz(diff) : -1;
+        T = top < 0 ? kmin : (top == 31 ? 0u : kmin & ~((2u << top) - 1u));
+#pragma unroll 1
+        for (int bit = top; bit >= 0; --bit) {
+            const uint32_t c = T | (1u << bit);
+            int cnt = 0;
+#pragma unroll
+            for (int k = 0; k < REG; ++k) cnt += (uint32_t)(w[k] >> 32) >= c ? 1 : 0;
+            cnt = (int)__reduce_add_sync(FULL, (unsigned)cnt);
+            if (cnt >= keep) {
+                T = c;
+                if (cnt == keep) break;        // no lower bit changes which words reach T
+            }
+        }
+    }
+    __syncwarp();                              // every lane holds its words before they are overwritten
+    int nc = 0;
+#pragma unroll
+    for (int k = 0; k < REG; ++k) {
+        const bool take = w[k] != 0ull && (uint32_t)(w[k] >> 32) >= T;
+        const unsigned bal = __ballot_sync(FULL, take);
+        if (take) key[nc + __popc(bal & ((1u << lane) - 1u))] = w[k];
+        nc += __popc(bal);
+    }
+    __syncwarp();
+    for (int j = lane; j < nc; j += 32) {
+        const uint64_t x = key[j];
+        int c = 0;
+        for (int t = 0; t < nc; ++t) c += key[t] > x ? 1 : 0;
+        if (c < keep) {
+            oi[c] = (int32_t)(0xffffffffu - (uint32_t)(x & 0xffffffffu));
+            if (oc) oc[c] = key_value((uint32_t)(x >> 32));
+        }
+    }
+    for (int k = keep + lane; k < out_stride; k += 32) {
+        oi[k] = -1;
+        if (oc) oc[k] = 0.f;
     }
 }
 
-// One row through shared-memory slots: the C candidates cr (values cv,
-// nullable) against the unit row q (global, dim_pad floats) -> the R best in
-// rank order into oi / oc.  SPW slots per warp.
-__device__ void rescore_row_slots(const float *__restrict__ q, int32_t dim_pad, const float *__restrict__ D32,
-                                  const int32_t *__restrict__ cr, const float *__restrict__ cv, float band, int32_t C,
-                                  int32_t R, int32_t *__restrict__ oi, float *__restrict__ oc, int32_t out_stride,
-                                  int32_t n_obj, int spw, int cmax, int32_t *__restrict__ err)
+// One step of the warp's sums of NV values at once: each half of the lanes
+// keeps half of the values (the sums pair the same lanes as a butterfly per
+// value would, so they are bitwise those).
+template <int NV>
+__device__ __forceinline__ void fold_sums(float *v, int lane, int o)
 {
-    extern __shared__ __align__(128) uint8_t sm[];
-    const RescoreSmem L(dim_pad, spw, cmax);
-    float4 *q4 = reinterpret_cast<float4 *>(sm + L.q);
-    float *slots = reinterpret_cast<float *>(sm + L.slots);
-    int32_t *cand = reinterpret_cast<int32_t *>(sm + L.cand);
-    uint64_t *key = reinterpret_cast<uint64_t *>(sm + L.key);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + L.bar);
-    __shared__ int s_n;
-    __shared__ int s_fail;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nv = dim_pad / 4;
-    const uint32_t row_bytes = (uint32_t)dim_pad * 4u;
-    if (tid == 0) {
-        s_n = 0;
-        s_fail = 0;
-        for (int i = 0; i < kWarps * spw; ++i) mbar_init(&bar[i], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    const float4 *src = reinterpret_cast<const float4 *>(q);
-    for (int i = tid; i < nv; i += TH) q4[i] = src[i];
-    __syncthreads();
-    // the in-band candidates, compacted (their order is free: keys are ranked by counting)
-    const float thr = cv ? cv[R - 1] - band : 0.f;
-    for (int c0 = warp * 32; c0 < C; c0 += TH) {
-        const int c = c0 + lane;
-        // (an index outside the scene is never copied: such a candidate is dropped)
-        const bool in = c < C && !(cv && cv[c] < thr) && cr[c] >= 0 && cr[c] < n_obj;
-        const uint32_t m = __ballot_sync(0xffffffffu, in);
-        int base = 0;
-        if (lane == 0 && m) base = atomicAdd(&s_n, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (in) cand[base + __popc(m & ((1u << lane) - 1u))] = cr[c];
-    }
-    __syncthreads();
-    const int n = s_n;
-    // warp w takes candidates w, w + W, ...; its i-th goes to its slot i % spw
-    float *mine = slots + (size_t)warp * spw * dim_pad;
-    uint64_t *mbar = bar + warp * spw;
-    if (lane == 0)
-        for (int k = 0; k < spw; ++k) {
-            const int j = warp + kWarps * k;
-            if (j < n) bulk_load(mine + (size_t)k * dim_pad, D32 + (int64_t)cand[j] * dim_pad, row_bytes, &mbar[k]);
-        }
-    bool ok = true;
-    int issued = min(spw, (n - warp + kWarps - 1) / kWarps), done = 0;
-    for (int i = 0;; ++i) {
-        const int j = warp + kWarps * i;
-        if (j >= n) break;
-        const int k = i % spw;
-        // (the lanes agree: a lane that gave up makes the whole warp give up)
-        if (!__all_sync(0xffffffffu, mbar_wait(&mbar[k], (uint32_t)(i / spw) & 1u))) {
-            ok = false;
-            break;
-        }
-        const float4 *d4 = reinterpret_cast<const float4 *>(mine + (size_t)k * dim_pad);
-        float a = 0.f;
-        for (int v = lane; v < nv; v += 32) {
-            const float4 x = d4[v], y = q4[v];
-            a = fmaf(y.x, x.x, a);
-            a = fmaf(y.y, x.y, a);
-            a = fmaf(y.z, x.z, a);
-            a = fmaf(y.w, x.w, a);
-        }
+    if constexpr (NV == 1) {
+        for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    } else {
+        const bool up = (lane & o) != 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        ++done;
-        __syncwarp();     // every lane has read the slot
-        if (lane == 0) {
-            const int jn = j + kWarps * spw;
-            if (jn < n) {
-                bulk_load(mine + (size_t)k * dim_pad, D32 + (int64_t)cand[jn] * dim_pad, row_bytes, &mbar[k]);
-                ++issued;
-            }
-            const int32_t e = cand[j];
-            key[j] = ((uint64_t)order_key(a) << 32) | (uint64_t)(0xffffffffu - (uint32_t)e);
+        for (int k = 0; k < NV / 2; ++k) {
+            const float keep = up ? v[k + NV / 2] : v[k];
+            const float send = up ? v[k] : v[k + NV / 2];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
-        issued = __shfl_sync(0xffffffffu, issued, 0);
+        fold_sums<NV / 2>(v, lane, o >> 1);
     }
-    if (!ok) {
-        // a copy did not arrive: record it, wait (bounded) for this warp's
-        // copies still in flight, which target its slots, and give up the row
-        if (lane == 0) {
-            atomicOr(err, kErrTimeout);
-            s_fail = 1;
-            for (int i = done; i < issued; ++i) mbar_wait(&mbar[i % spw], (uint32_t)(i / spw) & 1u);
+}
+
+// G rows of the processing order per block (rows of up to kGroupDimMax
+// floats).  Rows of one class of objects list mostly the same candidates, and
+// what bounds the work is the bytes of their descriptor rows: the block takes
+// the union of its rows' in-band candidates, loads each one once (two per
+// warp in flight, straight into registers) and multiplies it with every row
+// that lists it.  Each dot product has the order of a row on its own: lane l
+// adds the products of float4 l, l + 32, ..., then the lanes' sums are added
+// in a butterfly.
+template <int G>
+__global__ void __launch_bounds__(TH, 4)
+rescore_group_kernel(const Piece *__restrict__ pieces, int32_t n_pieces, int64_t total_rows,
+                     const int32_t *__restrict__ order, const float *__restrict__ Q32, int32_t dim_pad,
+                     const int32_t *__restrict__ bsel_t, const float *__restrict__ bsel_tv, int32_t cstride_t,
+                     const int32_t *__restrict__ bsel_l, const float *__restrict__ bsel_lv, int32_t cstride_l,
+                     float band, int32_t *__restrict__ tsel_idx, float *__restrict__ tsel_cos, int32_t stride_t,
+                     int32_t *__restrict__ lsel_idx, int32_t stride_l, int cmax)
+{
+    extern __shared__ __align__(16) uint8_t sm[];
+    const GroupSmem L(dim_pad, G, cmax);
+    float4 *q4 = reinterpret_cast<float4 *>(sm + L.q);
+    int32_t *hkey = reinterpret_cast<int32_t *>(sm + L.hkey);
+    uint32_t *hmask = reinterpret_cast<uint32_t *>(sm + L.hmask);     // four byte masks per word
+    uint64_t *key = reinterpret_cast<uint64_t *>(sm + L.key);         // [G][cmax], after the union is listed
+    int32_t *uobj = reinterpret_cast<int32_t *>(sm + L.obj);
+    uint8_t *umask = sm + L.mask;
+    __shared__ GroupRow rows[G];
+    __shared__ int s_n, s_cnt[G];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nv = dim_pad >> 2;
+    const int64_t p0 = (int64_t)blockIdx.x * G;
+    if (tid < G) {
+        GroupRow w{};
+        if (p0 + tid < total_rows) {
+            const int64_t r = order ? order[p0 + tid] : p0 + tid;
+            const Piece &pc = pieces[find_row_piece(pieces, n_pieces, r)];
+            const int i = (int)(r - pc.row_begin);
+            const bool tgt = i < pc.ntr;
+            const int64_t l = pc.l_row0 + (i - pc.ntr);
+            w.d32 = pc.d32;
+            w.co = tgt ? (pc.t_row0 + i) * (int64_t)cstride_t : l * (int64_t)cstride_l;
+            w.oo = tgt ? (pc.t_row0 + i) * (int64_t)stride_t : l * (int64_t)stride_l;
+            w.q_row = pc.q_row0 + i;
+            w.C = tgt ? pc.fkeep_t : pc.fkeep_l;
+            w.R = tgt ? pc.R : pc.klm;
+            w.n_obj = pc.n_obj;
+            w.tgt = tgt;
+            const float *vals = tgt ? bsel_tv : bsel_lv;
+            w.thr = vals ? vals[w.co + w.R - 1] - band : -__int_as_float(0x7f800000);
         }
+        rows[tid] = w;
     }
     __syncthreads();
-    if (s_fail) {
-        for (int i = tid; i < out_stride; i += TH) {
-            oi[i] = -1;
-            if (oc) oc[i] = 0.f;
-        }
-        return;
+    for (int g = 0; g < G; ++g) {
+        if (!rows[g].d32) continue;
+        const float4 *src = reinterpret_cast<const float4 *>(Q32 + rows[g].q_row * (int64_t)dim_pad);
+        for (int i = tid; i < nv; i += TH) q4[g * nv + i] = src[i];
     }
-    rank_out(key, n, R, oi, oc, out_stride);
+    // the rows of one scene at a time (as a rule all of them)
+    uint32_t todo = 0u;
+    for (int g = 0; g < G; ++g) todo |= rows[g].d32 ? 1u << g : 0u;
+    while (todo) {
+        const float *D32 = rows[__ffs(todo) - 1].d32;
+        uint32_t sub = 0u;
+        for (int g = 0; g < G; ++g) sub |= ((todo >> g) & 1u) && rows[g].d32 == D32 ? 1u << g : 0u;
+        todo &= ~sub;
+        if (G > 1) {
+            for (int s = tid; s < L.H; s += TH) hkey[s] = -1;
+            for (int s = tid; s < L.H / 4; s += TH) hmask[s] = 0u;
+        }
+        if (tid == 0) s_n = 0;
+        if (tid < G) s_cnt[tid] = 0;
+        __syncthreads();
+        // the union of the rows' in-band candidates (an index outside the scene is dropped)
+        for (int g = 0; g < G; ++g) {
+            if (!((sub >> g) & 1u)) continue;
+            const int32_t *cr = (rows[g].tgt ? bsel_t : bsel_l) + rows[g].co;
+            const float *vals = rows[g].tgt ? bsel_tv : bsel_lv;
+            const float *cv = vals ? vals + rows[g].co : nullptr;
+            const float thr = rows[g].thr;
+            const int C = rows[g].C, n_obj = rows[g].n_obj;
+            for (int c0 = warp * 32; c0 < C; c0 += TH) {
+                const int c = c0 + lane;
+                const int32_t e = c < C ? cr[c] : -1;
+                const bool in = c < C && !(cv && cv[c] < thr) && e >= 0 && e < n_obj;
+                if (G == 1) {
+                    const uint32_t m = __ballot_sync(0xffffffffu, in);
+                    int base = 0;
+                    if (lane == 0 && m) base = atomicAdd(&s_n, __popc(m));
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    if (in) {
+                        const int at = base + __popc(m & ((1u << lane) - 1u));
+                        uobj[at] = e;
+                        umask[at] = 1;
+                    }
+                } else if (in) {
+                    // (at most G cmax distinct objects in a table of at least half as many more slots)
+                    uint32_t s = ((uint32_t)e * 2654435761u) & (uint32_t)(L.H - 1);
+                    for (int t = 0; t < L.H; ++t) {
+                        const int32_t old = atomicCAS(&hkey[s], -1, e);
+                        if (old == -1 || old == e) {
+                            atomicOr(&hmask[s >> 2], 1u << (8 * (s & 3u) + g));
+                            break;
+                        }
+                        s = (s + 1) & (uint32_t)(L.H - 1);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (G > 1) {
+            for (int s = tid; s < L.H; s += TH) {       // (H is a multiple of the warp)
+                const int32_t e = hkey[s];
+                const uint32_t m = __ballot_sync(0xffffffffu, e >= 0);
+                int base = 0;
+                if (lane == 0 && m) base = atomicAdd(&s_n, __popc(m));
+                base = __shfl_sync(0xffffffffu, base, 0);
+                if (e >= 0) {
+                    const int at = base + __popc(m & ((1u << lane) - 1u));
+                    uobj[at] = e;
+                    umask[at] = (uint8_t)(hmask[s >> 2] >> (8 * (s & 3)));
+                }
+            }
+            __syncthreads();
+        }
+        const int n = s_n;
+        constexpr int U = 3;                // float4 of each candidate in flight per lane
+        for (int p = 2 * warp; p < n; p += 2 * kWarps) {
+            const bool two = p + 1 < n;
+            const int32_t e0 = uobj[p], e1 = uobj[two ? p + 1 : p];
+            const uint32_t m0 = umask[p], m1 = two ? umask[p + 1] : 0u, mm = m0 | m1;
+            const float4 *x0 = reinterpret_cast<const float4 *>(D32 + (int64_t)e0 * dim_pad);
+            const float4 *x1 = reinterpret_cast<const float4 *>(D32 + (int64_t)e1 * dim_pad);
+            float acc[2 * G];
+#pragma unroll
+            for (int k = 0; k < 2 * G; ++k) acc[k] = 0.f;
+            for (int base = 0; base < nv; base += 32 * U) {
+                float4 a[U], b[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int i = base + u * 32 + lane;
+                    a[u] = i < nv ? __ldg(x0 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    b[u] = i < nv ? __ldg(x1 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int i = base + u * 32 + lane;
+                    if (i >= nv) continue;
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        if (G > 1 && !((mm >> g) & 1u)) continue;       // (warp-uniform)
+                        const float4 y = q4[g * nv + i];
+                        acc[g] = fmaf(y.x, a[u].x, acc[g]);
+                        acc[g] = fmaf(y.y, a[u].y, acc[g]);
+                        acc[g] = fmaf(y.z, a[u].z, acc[g]);
+                        acc[g] = fmaf(y.w, a[u].w, acc[g]);
+                        acc[G + g] = fmaf(y.x, b[u].x, acc[G + g]);
+                        acc[G + g] = fmaf(y.y, b[u].y, acc[G + g]);
+                        acc[G + g] = fmaf(y.z, b[u].z, acc[G + g]);
+                        acc[G + g] = fmaf(y.w, b[u].w, acc[G + g]);
+                    }
+                }
+            }
+            fold_sums<2 * G>(acc, lane, 16);
+            // the lane's value is that of candidate (lane bit 4) and row (the bits
+            // below it), held by 32 / 2G lanes
+            constexpr int REP = 32 / (2 * G);
+            const int which = lane / REP;
+            const int c = which / G, g = which % G;
+            if ((lane % REP) == 0 && (((c ? m1 : m0) >> g) & 1u)) {
+                const int32_t e = c ? e1 : e0;
+                key[g * cmax + atomicAdd(&s_cnt[g], 1)] =
+                    ((uint64_t)order_key(acc[0]) << 32) | (uint64_t)(0xffffffffu - (uint32_t)e);
+            }
+        }
+        __syncthreads();
+        // the rows' lists, a warp per row
+        for (int g = warp; g < G; g += kWarps) {
+            if (!((sub >> g) & 1u)) continue;
+            const bool tgt = rows[g].tgt != 0;
+            int32_t *oi = (tgt ? tsel_idx : lsel_idx) + rows[g].oo;
+            float *oc = tgt && tsel_cos ? tsel_cos + rows[g].oo : nullptr;
+            const int stride = tgt ? stride_t : stride_l;
+            const int m = s_cnt[g], R = rows[g].R;
+            uint64_t *kg = key + g * cmax;
+            if (m <= 128) warp_rank_out<4>(kg, m, R, oi, oc, stride, lane);
+            else if (m <= 256) warp_rank_out<8>(kg, m, R, oi, oc, stride, lane);
+            else warp_rank_out<kMaxTargetCands / 32>(kg, m, R, oi, oc, stride, lane);
+        }
+        if (todo) __syncthreads();       // the next scene's rows reuse the table
+    }
+}
+
+// The processing order of a grouped launch: its rows by the class of their
+// best candidate (a counting sort by a hash of class and piece; the order
+// within a bucket is free, and so is the whole order as far as results go), so
+// that a block's rows and its neighbours' list mostly the same objects.
+__global__ void __launch_bounds__(256)
+rescore_bucket_kernel(const Piece *__restrict__ pieces, int32_t n_pieces, int32_t rows,
+                      const int32_t *__restrict__ bsel_t, int32_t cstride_t, const int32_t *__restrict__ bsel_l,
+                      int32_t cstride_l, int32_t *__restrict__ hist, int2 *__restrict__ place)
+{
+    const int r = blockIdx.x * 256 + threadIdx.x;
+    if (r >= rows) return;
+    const int k = find_row_piece(pieces, n_pieces, r);
+    const Piece &pc = pieces[k];
+    const int i = (int)(r - pc.row_begin);
+    const int32_t e = i < pc.ntr ? bsel_t[(pc.t_row0 + i) * (int64_t)cstride_t]
+                                 : bsel_l[(pc.l_row0 + (i - pc.ntr)) * (int64_t)cstride_l];
+    const int32_t c = e >= 0 && e < pc.n_obj ? pc.cls[e] : -1;
+    const int b = (int)(((uint32_t)c + (uint32_t)k * 7919u) & (uint32_t)(kBuckets - 1));
+    place[r] = make_int2(b, atomicAdd(&hist[b], 1));
+}
+
+__global__ void __launch_bounds__(256)
+rescore_order_kernel(int32_t rows, const int32_t *__restrict__ hist, const int2 *__restrict__ place,
+                     int32_t *__restrict__ order)
+{
+    __shared__ int32_t base[kBuckets];
+    __shared__ int32_t wsum[8];
+    constexpr int PER = kBuckets / 256;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int32_t v[PER], sum = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        v[k] = hist[tid * PER + k];
+        sum += v[k];
+    }
+    int32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int32_t at = incl - sum;
+    for (int w = 0; w < warp; ++w) at += wsum[w];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        base[tid * PER + k] = at;
+        at += v[k];
+    }
+    __syncthreads();
+    const int r = blockIdx.x * 256 + tid;
+    if (r < rows) {
+        const int2 p = place[r];
+        order[base[p.x] + p.y] = r;
+    }
 }
 
 // One row, loads from global memory: the C candidates cr (values cv, nullable) against the unit row q
@@ -357,16 +528,13 @@ __device__ __forceinline__ void rescore_row_ldg(const float *__restrict__ q, int
     }
 }
 
-// Grouped rescore: block -> (piece, row) through the piece table; SLOTS:
-// the rows go through spw shared-memory slots per warp, else global loads.
-template <bool SLOTS>
+// Rows longer than kGroupDimMax: a row per block, found through the piece table.
 __global__ void __launch_bounds__(TH)
 rescore_grouped_kernel(const Piece *__restrict__ pieces, int32_t n_pieces, const float *__restrict__ Q32,
                        int32_t dim_pad, const int32_t *__restrict__ bsel_t, const float *__restrict__ bsel_tv,
                        int32_t cstride_t, const int32_t *__restrict__ bsel_l, const float *__restrict__ bsel_lv,
                        int32_t cstride_l, float band, int32_t *__restrict__ tsel_idx, float *__restrict__ tsel_cos,
-                       int32_t stride_t, int32_t *__restrict__ lsel_idx, int32_t stride_l, int spw, int cmax,
-                       int32_t *__restrict__ err)
+                       int32_t stride_t, int32_t *__restrict__ lsel_idx, int32_t stride_l)
 {
     const int64_t r = blockIdx.x;
     const Piece pc = pieces[find_piece(pieces, n_pieces, r, [](const Piece &x) { return x.row_begin; })];
@@ -382,10 +550,7 @@ rescore_grouped_kernel(const Piece *__restrict__ pieces, int32_t n_pieces, const
     int32_t *oi = tgt ? tsel_idx + (pc.t_row0 + i) * (int64_t)stride_t : lsel_idx + l * (int64_t)stride_l;
     float *oc = tgt && tsel_cos ? tsel_cos + (pc.t_row0 + i) * (int64_t)stride_t : nullptr;
     const int32_t out = tgt ? stride_t : stride_l;
-    if constexpr (SLOTS)
-        rescore_row_slots(q, dim_pad, pc.d32, cr, cv, band, C, R, oi, oc, out, pc.n_obj, spw, cmax, err);
-    else
-        rescore_row_ldg(q, dim_pad, pc.d32, cr, cv, band, C, R, oi, oc, out);
+    rescore_row_ldg(q, dim_pad, pc.d32, cr, cv, band, C, R, oi, oc, out);
 }
 
 // The final lists of launch rows [row0, row0 + rows) -- rows of FP32-accurate
@@ -441,50 +606,59 @@ cudaError_t launch_copy_lists(const Piece *pieces, int32_t n_pieces, int64_t row
     return cudaGetLastError();
 }
 
+size_t rescore_scratch_ints(int64_t rows)
+{
+    return rows >= kGroupFrom ? (size_t)kBuckets + 3 * (size_t)rows : 0;
+}
+
 cudaError_t launch_rescore_grouped(const Piece *pieces, int32_t n_pieces, int64_t total_rows, const float *Q32,
                                    int32_t dim_pad, const int32_t *bsel_t, const float *bsel_tv, int32_t cstride_t,
                                    const int32_t *bsel_l, const float *bsel_lv, int32_t cstride_l, float band,
                                    int32_t *tsel_idx, float *tsel_cos, int32_t stride_t, int32_t *lsel_idx,
-                                   int32_t stride_l, int32_t *err, cudaStream_t s)
+                                   int32_t stride_l, int32_t *scratch, cudaStream_t s)
 {
     if (total_rows <= 0) return cudaSuccess;
-    if (n_pieces < 1 || total_rows > 0x7fffffff || dim_pad % 4 != 0 || cstride_t > SORT_MAX || cstride_l > SORT_MAX ||
-        !err)
+    if (n_pieces < 1 || total_rows > 0x7fffffff || dim_pad % 4 != 0 || cstride_t > kMaxTargetCands ||
+        cstride_l > kMaxTargetCands)
         return cudaErrorInvalidValue;
-    // slots per warp: the count that keeps the most row copies in flight per
-    // SM (resident CTAs x warps x slots; 228 KB of shared memory per SM, 1 KB
-    // of it reserved per CTA); rows longer than kTmaDimMax floats take the
-    // global-load routine
     const int cmax = cstride_t > cstride_l ? cstride_t : cstride_l;
-    int spw = 0;
-    if (dim_pad <= kTmaDimMax) {
-        static const int regs = [] {
-            cudaFuncAttributes a{};
-            return cudaFuncGetAttributes(&a, rescore_grouped_kernel<true>) == cudaSuccess ? a.numRegs : 64;
-        }();
-        const int by_regs = 65536 / (((regs + 7) / 8 * 8) * TH), by_threads = 2048 / TH;
-        int best = 0;
-        for (int k = 1; k <= 4; ++k) {
-            const size_t b = RescoreSmem(dim_pad, k, cmax).bytes + 256;
-            if (b > 227 * 1024) break;
-            int ctas = (int)((228 * 1024) / (b + 1024));
-            ctas = ctas < by_regs ? ctas : by_regs;
-            ctas = ctas < by_threads ? ctas : by_threads;
-            if (ctas * kWarps * k > best) {
-                best = ctas * kWarps * k;
-                spw = k;
-            }
-        }
+    const bool group = total_rows >= kGroupFrom;
+    cudaError_t e;
+    if (dim_pad > kGroupDimMax) {
+        const size_t smem = (size_t)dim_pad * sizeof(float);
+        if (smem > 48 * 1024 &&
+            (e = cudaFuncSetAttribute(rescore_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)smem)) != cudaSuccess)
+            return e;
+        rescore_grouped_kernel<<<(unsigned)total_rows, TH, smem, s>>>(pieces, n_pieces, Q32, dim_pad, bsel_t, bsel_tv,
+                                                                      cstride_t, bsel_l, bsel_lv, cstride_l, band,
+                                                                      tsel_idx, tsel_cos, stride_t, lsel_idx, stride_l);
+        return cudaGetLastError();
     }
-    const size_t smem = spw > 0 ? RescoreSmem(dim_pad, spw, cmax).bytes : (size_t)dim_pad * sizeof(float);
-    auto kern = spw > 0 ? rescore_grouped_kernel<true> : rescore_grouped_kernel<false>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
+    int32_t *order = nullptr;
+    if (group) {
+        if (!scratch) return cudaErrorInvalidValue;
+        int32_t *hist = scratch;
+        int2 *place = reinterpret_cast<int2 *>(scratch + kBuckets);
+        order = scratch + kBuckets + 2 * total_rows;
+        if ((e = cudaMemsetAsync(hist, 0, kBuckets * sizeof(int32_t), s)) != cudaSuccess) return e;
+        const unsigned nb = (unsigned)((total_rows + 255) / 256);
+        rescore_bucket_kernel<<<nb, 256, 0, s>>>(pieces, n_pieces, (int32_t)total_rows, bsel_t, cstride_t, bsel_l,
+                                                 cstride_l, hist, place);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        rescore_order_kernel<<<nb, 256, 0, s>>>((int32_t)total_rows, hist, place, order);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    kern<<<(unsigned)total_rows, TH, smem, s>>>(pieces, n_pieces, Q32, dim_pad, bsel_t, bsel_tv, cstride_t, bsel_l,
-                                                bsel_lv, cstride_l, band, tsel_idx, tsel_cos, stride_t, lsel_idx,
-                                                stride_l, spw, cmax, err);
+    const int G = group ? kGroupRows : 1;
+    const size_t smem = GroupSmem(dim_pad, G, cmax).bytes;
+    auto kern = group ? rescore_group_kernel<kGroupRows> : rescore_group_kernel<1>;
+    if (smem + 1024 > 48 * 1024 && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+                                cudaSuccess)
+        return e;
+    kern<<<(unsigned)((total_rows + G - 1) / G), TH, smem, s>>>(pieces, n_pieces, total_rows, order, Q32, dim_pad,
+                                                                bsel_t, bsel_tv, cstride_t, bsel_l, bsel_lv, cstride_l,
+                                                                band, tsel_idx, tsel_cos, stride_t, lsel_idx, stride_l,
+                                                                cmax);
     return cudaGetLastError();
 }
 
