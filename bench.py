@@ -241,9 +241,9 @@ def cpu_baseline_mc(scene, spaces, qb, cq, k, n_sample, seed=0, budget_s=15.0):
 # (code_digest: the source without its comments):
 # (workload, precision, tile variant, fused) -> bytes
 SIM_TRAFFIC = {
-    ("site_n20k_d1152", "fp32", 2, True): (88.905216e6 + 123.177472e6) + (667.047680e6 + 20.749312e6),
+    ("site_n20k_d1152", "fp32", 2, True): (88.919808e6 + 123.629568e6) + (666.217216e6 + 20.915712e6),
 }
-SIM_TRAFFIC_SOURCE = "33338d4039976e64"
+SIM_TRAFFIC_SOURCE = "cd0fbf40425fef7a"
 
 
 def code_digest(text):

@@ -93,10 +93,8 @@ enum Buf {
     B_QSCALE,       // float [rows] their scales
     B_QCOMP,        // bf16 [rows, P] learned embeddings of the rows
     B_MLP_H,        // float [chunk, H] pre-activations (inference)
-    B_MLP_A,        // float [chunk, H] activations
     B_MLP_AB,       // bf16 [chunk, H]
     B_MLP_Z,        // float [chunk, P]
-    B_MLP_E,        // float [chunk, P]
     B_PIECES,       // Piece tables of the batch's grouped launches
     B_CHUNK_IDX,    // int32 chunk lists of long rows (select, then merge)
     B_CHUNK_VAL,    // float their values
@@ -181,15 +179,30 @@ struct Ctx {
 // ---- learned prefilter (k_mlp.cu) ----
 cudaError_t mlp_gemm(bool ta, bool tb, int M, int N, int K, float alpha, const float *A, int lda, const float *B,
                      int ldb, float beta, float *C, int ldc, cudaStream_t s);
-cudaError_t mlp_bias_gelu(float *h, const float *b, float *a, int64_t rows, int cols, cudaStream_t s,
-                          uint16_t *ab = nullptr);
-// BF16 rows gathered from several tables: dst[r] = base[sel[r]] + idx[r] * lds
-// (sel null: base[0]); cols, lds, ldd multiples of 8, dst 16-byte aligned.
-cudaError_t mlp_gather_rows_bf16(const uint16_t *const *base, const int32_t *sel, const int32_t *idx, int64_t lds,
-                                 int64_t rows, int cols, uint16_t *dst, int64_t ldd, cudaStream_t s);
-// dst[c * ldd + col0 + r] = bf16(src[r * lds + c]) (src FP32 src32, or BF16 src16).
-cudaError_t mlp_transpose_bf16(const float *src32, const uint16_t *src16, int64_t lds, int64_t rows, int cols,
-                               uint16_t *dst, int64_t ldd, int64_t col0, cudaStream_t s);
+cudaError_t mlp_bias_gelu(float *h, const float *b, float *a, int64_t rows, int cols, cudaStream_t s);
+// The network's shape and its weights' BF16 copies (Mlp::w1b, w2b, w2t).
+struct MlpShape {
+    int32_t D, H, P, D_pad;
+    uint16_t *w1b, *w2b, *w2t;
+};
+// The training step's kernels (k_mlp.cu): its stacked rows and their transpose,
+// clearing the bias-gradient sums gb1 [H], gb2 [P]; GELU's BF16 output and
+// transpose (aT nullable); the pairs' loss and the gradient down to the second
+// contraction's output; GELU's backward.  K: the padded length of the
+// transposed operands (a multiple of 64, zero from the last row on).
+cudaError_t mlp_train_rows(const uint16_t *const *base, int32_t n_scenes, const int32_t *idx, int64_t n_pairs, int64_t b,
+                           int D, int D_pad, uint16_t *x, uint16_t *xT, int64_t K, float *gb1, int H, float *gb2, int P,
+                           cudaStream_t s);
+cudaError_t mlp_gelu_bf16(const float *h, const float *b, int64_t rows, int cols, uint16_t *ab, uint16_t *aT, int64_t K,
+                          cudaStream_t s);
+cudaError_t mlp_gelu_backward_t(const float *h, const float *b, const float *da, int64_t rows, int cols, uint16_t *dhT,
+                                int64_t K, float *gb, cudaStream_t s);
+cudaError_t mlp_pair_step(const float *z, const float *b2, const float *y, const float *w, float wsum, int64_t b, int P,
+                          uint16_t *dzb, uint16_t *dzT, int64_t K, float *gb2, float *loss, cudaStream_t s);
+// e = bf16((z + b) / |z + b|) per row.
+cudaError_t mlp_normalize_bf16(const float *z, const float *b, int64_t rows, int cols, uint16_t *e, cudaStream_t s);
+// All BF16 copies of the parameters p (count of them).
+cudaError_t mlp_weights_bf16(const float *p, int64_t count, const MlpShape &m, cudaStream_t s);
 // BF16 copy of a row-major FP32 [rows, cols] matrix with rows zero-padded to ldd.
 cudaError_t mlp_to_bf16_padded(const float *src, int64_t rows, int cols, uint16_t *dst, int ldd, cudaStream_t s);
 cudaError_t mlp_bias_normalize(float *z, const float *b, float *e, float *norm, int64_t rows, int cols,
@@ -200,10 +213,8 @@ cudaError_t mlp_normalize_backward(const float *e, const float *norm, float *de,
                                    cudaStream_t s);
 cudaError_t mlp_gelu_backward(const float *h, float *da, int64_t count, cudaStream_t s);
 cudaError_t mlp_colsum(const float *x, int64_t rows, int cols, float *out, bool accumulate, cudaStream_t s);
-cudaError_t mlp_gather_rows(const float *src, int lds, const int32_t *idx, int64_t rows, int cols, float *dst,
-                            cudaStream_t s);
-cudaError_t mlp_adam(float *p, const float *g, float *m, float *v, int64_t count, float lr, int t, cudaStream_t s);
-cudaError_t mlp_to_bf16(const float *x, int64_t count, uint16_t *y, cudaStream_t s);
+cudaError_t mlp_adam(float *p, const float *g, float *m, float *v, int64_t count, float lr, int t, const MlpShape &shape,
+                     cudaStream_t s);
 
 // Grow-only workspace buffer of the context (synchronises before a regrow).
 cudaError_t ws_alloc(farm_ctx *ctx, Buf b, size_t bytes, void **out);
@@ -267,9 +278,13 @@ cudaError_t launch_sim_simt(const float *q, const float *d, float *S, int64_t ro
 // Every variant computes each output with the same K order, so they give
 // bitwise identical results; the planner's autotuner picks the fastest.
 constexpr int kSimTileM = 128;
+// Internal to the library (farm_sim_variant_pin does not name it): 3, 128 x 64
+// tiles on one CTA each, for BF16 contractions whose output is too small for
+// the wider tiles to occupy the chip (the training step's weight gradients).
 constexpr int kSimVariants = 3;
+constexpr int kSimNarrowVariant = 3;
 constexpr int kSimPairVariant = 2;      // the single-problem launches use the CTA pairs
-inline int sim_variant_bn(int v) { return v == 1 ? 128 : 256; }
+inline int sim_variant_bn(int v) { return v == kSimNarrowVariant ? 64 : v == 1 ? 128 : 256; }
 inline int sim_variant_cluster(int v) { return v == 2 ? 2 : 1; }
 enum SimMode { kSimF16x3 = 0, kSimBf16 = 1, kSimFp8 = 2 };
 

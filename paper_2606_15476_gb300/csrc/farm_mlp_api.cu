@@ -115,122 +115,183 @@ cudaError_t backward(const Mlp &M, const float *X, int64_t b, float *h, const fl
     return farm::mlp_colsum(da, b, (int)H, gb1, beta != 0.f, s);
 }
 
+farm::MlpShape shape_of(const Mlp &M) { return {M.D, M.H, M.P, M.D_pad, M.w1b, M.w2b, M.w2t}; }
+
 // BF16 copies of the weights for the tensor-core products: W1 padded to D_pad
 // columns, W2, and W2 transposed ([H, P], the operand of the backward pass).
 cudaError_t refresh_bf16_weights(Ctx &c)
 {
     Mlp &M = c.mlp;
-    cudaError_t e = farm::mlp_to_bf16_padded(M.W1(), M.H, M.D, M.w1b, M.D_pad, c.stream);
-    if (e == cudaSuccess) e = farm::mlp_to_bf16(M.W2(), (int64_t)M.P * M.H, M.w2b, c.stream);
-    if (e == cudaSuccess) e = farm::mlp_transpose_bf16(M.W2(), nullptr, M.H, M.P, M.H, M.w2t, M.P, 0, c.stream);
-    c.launches += 3;
+    c.launches += 1;
     M.version += 1;
-    return e;
+    return farm::mlp_weights_bf16(M.params, M.count(), shape_of(M), c.stream);
 }
 
 // Device buffers of one tensor-core training step over up to B pairs: the
 // two towers' rows are stacked (query rows 0..b-1, descriptor rows b..2b-1),
-// so each contraction is one launch over 2b rows; the weight gradients
-// contract over those 2b rows (K), padded with zero columns to a multiple of 64.
+// so each contraction is one launch over them; the weight gradients contract
+// over those rows (K), padded with zero columns to a multiple of 64.  dT
+// holds dz^T (P rows), then dh^T (H rows): the operand rows of both weight
+// gradients, computed by one launch.
 struct TcBufs {
     void *base = nullptr;
     int64_t B = 0, K_pad = 0;
-    uint16_t *x, *ab, *dzb, *xT, *aT, *dzT, *dhT;
-    float *h, *a, *z, *e, *nrm, *dz, *da, *grad, *m, *v, *loss, *y, *w;
+    uint16_t *x, *ab, *dzb, *xT, *aT, *dT;
+    float *h, *z, *da, *grad, *m, *v, *loss, *y, *w;
+    uint8_t *blob;               // the contractions' pieces, then their B tensor maps
 };
 
 int64_t round64(int64_t x) { return (x + 63) / 64 * 64; }
 
-cudaError_t tc_alloc(TcBufs &t, const Mlp &M, int64_t B, int64_t loss_slots)
+// The step's contractions: H = x W1^T, Z = a W2^T, dA = dz W2, and the two
+// weight gradients.
+enum { G_H = 0, G_Z, G_DA, G_DW, G_COUNT };
+constexpr int kGemmPieces = 5;   // the weight gradients are two pieces
+constexpr size_t kBlobMaps = 512;
+static_assert(kGemmPieces * sizeof(farm::GemmPiece) <= kBlobMaps && kBlobMaps % 128 == 0, "piece table");
+constexpr size_t kBlobBytes = kBlobMaps + kGemmPieces * 2 * farm::kTensorMapBytes;
+
+// CTA pairs where their tiles occupy most of the chip, else 128 x 64 tiles: at
+// 8,192 rows, D = 1152 the weight gradients (128 x 512 and 512 x 1152,
+// contracting over the 8,192 rows) are 12 pair tiles and 80 narrow ones, and a
+// step's contractions took 143 us with the pairs alone, 82 us with this rule.
+// Every variant sums each output's products in the same order.
+int gemm_variant(int64_t rows, int64_t n, int num_sms)
 {
-    const int64_t R = 2 * B, K = round64(2 * B), D = M.D, Dp = M.D_pad, H = M.H, P = M.P, cnt = M.count();
+    return farm::sim_cluster_tiles(rows, n, farm::kSimPairVariant) * 8 >= (int64_t)num_sms * 3 ? farm::kSimPairVariant
+                                                                                               : farm::kSimNarrowVariant;
+}
+
+struct GemmShape { int64_t rows, n; const uint16_t *b; int32_t k; float *out; int piece0, pieces; };
+
+void gemm_shapes(const TcBufs &t, const Mlp &M, GemmShape (&g)[kGemmPieces])
+{
+    const int64_t R = 2 * t.B;
+    float *gW1 = t.grad, *gW2 = t.grad + (int64_t)M.H * M.D + M.H;
+    g[0] = {R, M.H, M.w1b, M.D_pad, t.h, 0, 1};
+    g[1] = {R, M.P, M.w2b, M.H, t.z, 1, 1};
+    g[2] = {R, M.H, M.w2t, M.P, t.da, 2, 1};
+    g[3] = {M.P, M.H, t.aT, (int32_t)t.K_pad, gW2, 3, 2};
+    g[4] = {M.H, M.D, t.xT, (int32_t)t.K_pad, gW1, 3, 2};
+}
+
+cudaError_t tc_alloc(Ctx &c, TcBufs &t, int64_t B, int64_t loss_slots)
+{
+    const Mlp &M = c.mlp;
+    const int64_t R = 2 * B, K = round64(2 * B), Dp = M.D_pad, H = M.H, P = M.P, cnt = M.count();
     t.B = B;
     t.K_pad = K;
     // (element count, element bytes) of each array, 256-byte aligned in one allocation
-    const int64_t n16[] = {R * Dp, R * H, R * P, Dp * K, H * K, P * K, H * K};
-    uint16_t **d16[] = {&t.x, &t.ab, &t.dzb, &t.xT, &t.aT, &t.dzT, &t.dhT};
-    const int64_t n32[] = {R * H, R * H, R * P, R * P, R, R * P, R * H, cnt, cnt, cnt, loss_slots, B, B};
-    float **d32[] = {&t.h, &t.a, &t.z, &t.e, &t.nrm, &t.dz, &t.da, &t.grad, &t.m, &t.v, &t.loss, &t.y, &t.w};
-    (void)D;
+    const int64_t n16[] = {R * Dp, R * H, R * P, Dp * K, H * K, (P + H) * K};
+    uint16_t **d16[] = {&t.x, &t.ab, &t.dzb, &t.xT, &t.aT, &t.dT};
+    const int64_t n32[] = {R * H, R * P, R * H, cnt, cnt, cnt, loss_slots, B, B};
+    float **d32[] = {&t.h, &t.z, &t.da, &t.grad, &t.m, &t.v, &t.loss, &t.y, &t.w};
     auto al = [](int64_t bytes) { return (bytes + 255) / 256 * 256; };
     int64_t total = 0;
     for (int64_t n : n16) total += al(n * 2);
     for (int64_t n : n32) total += al(n * 4);
+    total += (int64_t)kBlobBytes;
     cudaError_t e = cudaMalloc(&t.base, (size_t)total);
     if (e != cudaSuccess) return e;
     char *p = static_cast<char *>(t.base);
     for (size_t i = 0; i < sizeof(n16) / sizeof(n16[0]); ++i) { *d16[i] = reinterpret_cast<uint16_t *>(p); p += al(n16[i] * 2); }
     for (size_t i = 0; i < sizeof(n32) / sizeof(n32[0]); ++i) { *d32[i] = reinterpret_cast<float *>(p); p += al(n32[i] * 4); }
-    // the padding columns of the transposed operands stay zero unless a step writes them
-    return cudaMemsetAsync(t.base, 0, (size_t)total);
+    t.blob = reinterpret_cast<uint8_t *>(p);
+    // (rows past a partial batch hold the last batch's, or zeros: every
+    // contraction over them is finite and read by nothing)
+    if ((e = cudaMemsetAsync(t.base, 0, (size_t)total, c.stream))) return e;
+    GemmShape g[kGemmPieces];
+    gemm_shapes(t, M, g);
+    alignas(128) uint8_t host[kBlobBytes] = {};
+    for (int k = 0; k < kGemmPieces; ++k) {
+        const GemmShape &s = g[k];
+        const int v = k >= G_DW ? farm::kSimNarrowVariant : gemm_variant(s.rows, s.n, c.num_sms);
+        farm::GemmPiece gp{};
+        gp.q_row0 = k == 4 ? P : 0;
+        gp.s_off = k >= G_DW ? s.out - t.grad : 0;
+        gp.tops_off = -1;
+        gp.bmap = t.blob + kBlobMaps + (size_t)k * 2 * farm::kTensorMapBytes;
+        gp.rows = (int32_t)s.rows;
+        gp.n = gp.n_store = (int32_t)s.n;
+        gp.ld = (int32_t)s.n;
+        gp.tile_begin = k == 4 ? (int32_t)farm::sim_cluster_tiles(g[3].rows, g[3].n, farm::kSimNarrowVariant) : 0;
+        gp.gshift = farm::kGroupShift;
+        gp.col_mode = farm::kColAll;
+        std::memcpy(host + k * sizeof(gp), &gp, sizeof(gp));
+        if (!farm::sim_tc_encode_b(farm::kSimBf16, v,
+                                   host + kBlobMaps + (size_t)k * 2 * farm::kTensorMapBytes, s.b, nullptr, s.n, s.k))
+            return cudaErrorInvalidValue;
+    }
+    // (pageable source: staged when the call returns)
+    return cudaMemcpyAsync(t.blob, host, kBlobBytes, cudaMemcpyHostToDevice, c.stream);
 }
 
-// Loss and gradient of b pairs whose stacked BF16 input rows (query rows,
-// then descriptor rows, D_pad long) are in t.x; targets / weights t.y, t.w
-// (device, b each; w null: 1), wsum their sum.  The loss is added to *lslot,
-// the gradient [W1 | b1 | W2 | b2] written to t.grad.
-cudaError_t tc_loss_grad(Ctx &c, TcBufs &t, int64_t b, bool weighted, float wsum, float *lslot, int64_t &launches)
+cudaError_t tc_gemm(Ctx &c, const TcBufs &t, int which)
+{
+    GemmShape g[kGemmPieces];
+    gemm_shapes(t, c.mlp, g);
+    const GemmShape &s = g[which];
+    const bool dw = which == G_DW;
+    const int v = dw ? farm::kSimNarrowVariant : gemm_variant(s.rows, s.n, c.num_sms);
+    const uint16_t *a[] = {t.x, t.ab, t.dzb, t.dT};
+    const int64_t rows = dw ? (int64_t)c.mlp.P + c.mlp.H : s.rows;
+    int64_t tiles = 0;
+    for (int k = s.piece0; k < s.piece0 + s.pieces; ++k) tiles += farm::sim_cluster_tiles(g[k].rows, g[k].n, v);
+    return farm::launch_sim_tc_grouped(farm::kSimBf16, v, a[which], nullptr, rows, s.k,
+                                       reinterpret_cast<const farm::GemmPiece *>(t.blob) + s.piece0, s.pieces, tiles,
+                                       dw ? t.grad : s.out, nullptr, nullptr, c.num_sms, c.d_err, c.stream);
+}
+
+// Loss and gradient of b pairs: their stacked BF16 input rows gathered by idx
+// (train_rows_kernel; base and the index arrays of the epoch, at the batch's
+// first pair), or already in t.x (idx null); targets / weights y, w (device, b
+// each; w null: 1), wsum their sum.  The loss is added to *lslot, the gradient
+// [W1 | b1 | W2 | b2] written to t.grad.
+cudaError_t tc_loss_grad(Ctx &c, TcBufs &t, int64_t b, const uint16_t *const *base, int32_t n_scenes,
+                         const int32_t *idx, int64_t n_pairs, const float *y, const float *w, float wsum, float *lslot,
+                         int64_t &launches)
 {
     const Mlp &M = c.mlp;
     const int64_t R = 2 * b, K = t.K_pad, H = M.H, P = M.P, D = M.D;
-    float *gW1 = t.grad, *gb1 = gW1 + H * D, *gW2 = gb1 + H, *gb2 = gW2 + P * H;
+    float *gb1 = t.grad + H * D, *gb2 = gb1 + H + P * H;
     cudaStream_t st = c.stream;
     cudaError_t r;
-    // zero the padding columns [R, K) of the transposed operands (rows of K entries)
-    if (R < K) {
-        uint16_t *tr[] = {t.xT, t.aT, t.dzT, t.dhT};
-        const int64_t nr[] = {M.D_pad, H, P, H};
-        for (int i = 0; i < 4; ++i)
-            if ((r = cudaMemset2DAsync(tr[i] + R, (size_t)K * 2, 0, (size_t)(K - R) * 2, (size_t)nr[i], st)))
-                return r;
-    }
-    launches += 17;
-    // forward: h = x W1^T + b1, a = gelu(h), z = a W2^T + b2, e = z / |z|
-    if ((r = farm::mlp_transpose_bf16(nullptr, t.x, M.D_pad, R, (int)D, t.xT, K, 0, st))) return r;
-    if ((r = farm::launch_sim_tc_bf16(t.x, M.w1b, t.h, R, H, M.D_pad, H, nullptr, c.num_sms, c.d_err, st))) return r;
-    if ((r = farm::mlp_bias_gelu(t.h, M.b1(), t.a, R, (int)H, st, t.ab))) return r;
-    if ((r = farm::mlp_transpose_bf16(t.a, nullptr, H, R, (int)H, t.aT, K, 0, st))) return r;
-    if ((r = farm::launch_sim_tc_bf16(t.ab, M.w2b, t.z, R, P, H, P, nullptr, c.num_sms, c.d_err, st))) return r;
-    if ((r = farm::mlp_bias_normalize(t.z, M.b2(), t.e, t.nrm, R, (int)P, st))) return r;
-    // loss; de of both towers
-    if ((r = farm::mlp_pair_loss(t.e, t.e + b * P, t.y, weighted ? t.w : nullptr, wsum, b, (int)P, t.dz,
-                                 t.dz + b * P, lslot, st)))
+    launches += 8;
+    if ((r = farm::mlp_train_rows(base, n_scenes, idx, n_pairs, b, (int)D, M.D_pad, t.x, t.xT, K, gb1, (int)H, gb2,
+                                  (int)P, st)))
         return r;
-    // backward: dz, gb2, dW2 = dz^T a, da = dz W2, dh = gelu'(h) da, gb1, dW1 = dh^T x
-    if ((r = farm::mlp_normalize_backward(t.e, t.nrm, t.dz, R, (int)P, st))) return r;
-    if ((r = farm::mlp_colsum(t.dz, R, (int)P, gb2, false, st))) return r;
-    if ((r = farm::mlp_to_bf16(t.dz, R * P, t.dzb, st))) return r;
-    if ((r = farm::mlp_transpose_bf16(t.dz, nullptr, P, R, (int)P, t.dzT, K, 0, st))) return r;
-    if ((r = farm::launch_sim_tc_bf16(t.dzT, t.aT, gW2, P, H, K, H, nullptr, c.num_sms, c.d_err, st))) return r;
-    if ((r = farm::launch_sim_tc_bf16(t.dzb, M.w2t, t.da, R, H, P, H, nullptr, c.num_sms, c.d_err, st))) return r;
-    if ((r = farm::mlp_gelu_backward(t.h, t.da, R * H, st))) return r;
-    if ((r = farm::mlp_colsum(t.da, R, (int)H, gb1, false, st))) return r;
-    if ((r = farm::mlp_transpose_bf16(t.da, nullptr, H, R, (int)H, t.dhT, K, 0, st))) return r;
-    return farm::launch_sim_tc_bf16(t.dhT, t.xT, gW1, H, D, K, D, nullptr, c.num_sms, c.d_err, st);
+    // forward: h = x W1^T, a = gelu(h + b1), z = a W2^T
+    if ((r = tc_gemm(c, t, G_H))) return r;
+    if ((r = farm::mlp_gelu_bf16(t.h, M.b1(), R, (int)H, t.ab, t.aT, K, st))) return r;
+    if ((r = tc_gemm(c, t, G_Z))) return r;
+    // e = (z + b2) / |z + b2|, the loss, dz and its column sums
+    if ((r = farm::mlp_pair_step(t.z, M.b2(), y, w, wsum, b, (int)P, t.dzb, t.dT, K, gb2, lslot, st))) return r;
+    // backward: da = dz W2, dh = gelu'(h + b1) da, then dW2 = dz^T a and dW1 = dh^T x together
+    if ((r = tc_gemm(c, t, G_DA))) return r;
+    if ((r = farm::mlp_gelu_backward_t(t.h, M.b1(), t.da, R, (int)H, t.dT + P * K, K, gb1, st))) return r;
+    return tc_gemm(c, t, G_DW);
 }
 
 }  // namespace
 
 namespace {
 
-cudaError_t embed_buffers(farm_ctx *ctx, int64_t rows, void **h, void **a, void **ab, void **z, void **e)
+cudaError_t embed_buffers(farm_ctx *ctx, int64_t rows, void **h, void **ab, void **z)
 {
     const Mlp &M = farm::ctx_of(ctx)->mlp;
     const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(rows, kEmbedChunk));
     cudaError_t r;
     if ((r = farm::ws_alloc(ctx, farm::B_MLP_H, (size_t)chunk * M.H * 4, h))) return r;
-    if ((r = farm::ws_alloc(ctx, farm::B_MLP_A, (size_t)chunk * M.H * 4, a))) return r;
     if ((r = farm::ws_alloc(ctx, farm::B_MLP_AB, (size_t)chunk * M.H * 2, ab))) return r;
-    if ((r = farm::ws_alloc(ctx, farm::B_MLP_Z, (size_t)chunk * M.P * 4, z))) return r;
-    return farm::ws_alloc(ctx, farm::B_MLP_E, (size_t)chunk * M.P * 4, e);
+    return farm::ws_alloc(ctx, farm::B_MLP_Z, (size_t)chunk * M.P * 4, z);
 }
 
 }  // namespace
 
 cudaError_t farm::learned_reserve(farm_ctx *ctx, int64_t rows)
 {
-    void *h, *a, *ab, *z, *e;
-    return embed_buffers(ctx, rows, &h, &a, &ab, &z, &e);
+    void *h, *ab, *z;
+    return embed_buffers(ctx, rows, &h, &ab, &z);
 }
 
 cudaError_t farm::learned_embed_rows(farm_ctx *ctx, const uint16_t *xb, int64_t rows, uint16_t *out)
@@ -238,22 +299,20 @@ cudaError_t farm::learned_embed_rows(farm_ctx *ctx, const uint16_t *xb, int64_t 
     Ctx &c = *ctx_of(ctx);
     const Mlp &M = c.mlp;
     const int64_t chunk = std::min<int64_t>(rows, kEmbedChunk);
-    void *h, *a, *ab, *z, *e;
+    void *h, *ab, *z;
     cudaError_t r;
-    if ((r = embed_buffers(ctx, rows, &h, &a, &ab, &z, &e))) return r;
+    if ((r = embed_buffers(ctx, rows, &h, &ab, &z))) return r;
     for (int64_t r0 = 0; r0 < rows; r0 += chunk) {
         const int64_t b = std::min(chunk, rows - r0);
-        c.launches += 6;
+        c.launches += 4;
         if ((r = launch_sim_tc_bf16(xb + r0 * M.D_pad, M.w1b, (float *)h, b, M.H, M.D_pad, M.H, nullptr, c.num_sms, c.d_err,
                                     c.stream)))
             return r;
-        if ((r = mlp_bias_gelu((float *)h, M.b1(), (float *)a, b, M.H, c.stream))) return r;
-        if ((r = mlp_to_bf16((float *)a, b * M.H, (uint16_t *)ab, c.stream))) return r;
+        if ((r = mlp_gelu_bf16((float *)h, M.b1(), b, M.H, (uint16_t *)ab, nullptr, 0, c.stream))) return r;
         if ((r = launch_sim_tc_bf16((uint16_t *)ab, M.w2b, (float *)z, b, M.P, M.H, M.P, nullptr, c.num_sms, c.d_err,
                                     c.stream)))
             return r;
-        if ((r = mlp_bias_normalize((float *)z, M.b2(), (float *)e, nullptr, b, M.P, c.stream))) return r;
-        if ((r = mlp_to_bf16((float *)e, b * M.P, out + r0 * M.P, c.stream))) return r;
+        if ((r = mlp_normalize_bf16((float *)z, M.b2(), b, M.P, out + r0 * M.P, c.stream))) return r;
     }
     return cudaSuccess;
 }
@@ -359,8 +418,10 @@ farm_status farm_mlp_loss_grad(farm_ctx *ctx, int64_t n_pairs, const float *xq, 
         // the training step's arithmetic: stacked rows in BF16, tensor-core contractions
         TcBufs t;
         float *raw = nullptr;
-        MCK(tc_alloc(t, M, n_pairs, 1));
         auto done = [&](farm_status st) { cudaStreamSynchronize(c.stream); cudaFree(t.base); cudaFree(raw); return st; };
+        e = tc_alloc(c, t, n_pairs, 1);
+        if (e) return done(fail(c, e == cudaErrorMemoryAllocation ? FARM_ENOMEM : FARM_ECUDA,
+                                std::string("farm_mlp_loss_grad: ") + cudaGetErrorString(e)));
         if (!e) e = cudaMalloc(&raw, 2 * xb);
         if (!e) e = cudaMemcpyAsync(raw, xq, xb, cudaMemcpyHostToDevice, c.stream);
         if (!e) e = cudaMemcpyAsync(raw + (size_t)n_pairs * M.D, xd, xb, cudaMemcpyHostToDevice, c.stream);
@@ -368,7 +429,7 @@ farm_status farm_mlp_loss_grad(farm_ctx *ctx, int64_t n_pairs, const float *xq, 
         if (!e && w) e = cudaMemcpyAsync(t.w, w, (size_t)n_pairs * 4, cudaMemcpyHostToDevice, c.stream);
         if (!e) e = cudaMemsetAsync(t.loss, 0, 4, c.stream);
         if (!e) e = farm::mlp_to_bf16_padded(raw, 2 * n_pairs, M.D, t.x, M.D_pad, c.stream);
-        if (!e) e = tc_loss_grad(c, t, n_pairs, w != nullptr, (float)wsum, t.loss, L);
+        if (!e) e = tc_loss_grad(c, t, n_pairs, nullptr, 0, nullptr, 0, t.y, w ? t.w : nullptr, (float)wsum, t.loss, L);
         if (!e) e = cudaMemcpyAsync(loss, t.loss, 4, cudaMemcpyDeviceToHost, c.stream);
         if (!e && grad) e = cudaMemcpyAsync(grad, t.grad, (size_t)M.count() * 4, cudaMemcpyDeviceToHost, c.stream);
         if (!e) e = cudaStreamSynchronize(c.stream);
@@ -434,7 +495,6 @@ farm_status farm_mlp_train(farm_ctx *ctx, int32_t n_scenes, const int32_t *scene
     const int64_t B = std::min<int64_t>(batch, n_pairs);
     const int64_t steps = (n_pairs + B - 1) / B;
     TcBufs t;
-    MCK(tc_alloc(t, M, B, steps * (int64_t)epochs));
     uint16_t *qnb = nullptr;   // normalised training rows, BF16 [n_rows, D_pad]
     float *raw = nullptr;
     int32_t *d_idx = nullptr;  // per epoch: query rows [n_pairs] | object indices [n_pairs] | scenes [n_pairs]
@@ -445,7 +505,9 @@ farm_status farm_mlp_train(farm_ctx *ctx, int32_t n_scenes, const int32_t *scene
         cudaFree(t.base); cudaFree(qnb); cudaFree(raw); cudaFree(d_idx); cudaFree(d_yw); cudaFree(d_bases);
         return st;
     };
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = tc_alloc(c, t, B, steps * (int64_t)epochs);
+    if (e) return done(fail(c, e == cudaErrorMemoryAllocation ? FARM_ENOMEM : FARM_ECUDA,
+                            std::string("farm_mlp_train: ") + cudaGetErrorString(e)));
     if (!e) e = cudaMalloc(&qnb, (size_t)n_rows * M.D_pad * 2);
     if (!e) e = cudaMalloc(&raw, (size_t)n_rows * M.D * 4);
     if (!e) e = cudaMalloc(&d_idx, (size_t)n_pairs * 3 * 4);
@@ -457,9 +519,7 @@ farm_status farm_mlp_train(farm_ctx *ctx, int32_t n_scenes, const int32_t *scene
     if (!e) e = cudaMemcpyAsync(raw, rows, (size_t)n_rows * M.D * 4, cudaMemcpyHostToDevice, c.stream);
     if (!e) e = farm::launch_normalize_rows(raw, nullptr, n_rows, M.D, M.D_pad, nullptr, nullptr, nullptr, qnb,
                                             c.d_err, farm::kErrBadRow, c.stream);
-    if (!e) e = cudaMemsetAsync(t.m, 0, (size_t)M.count() * 4, c.stream);
-    if (!e) e = cudaMemsetAsync(t.v, 0, (size_t)M.count() * 4, c.stream);
-    if (!e) e = cudaMemsetAsync(t.loss, 0, (size_t)steps * epochs * 4, c.stream);
+    // (the moments and the losses start at zero: tc_alloc clears them)
     if (e) return done(fail(c, FARM_ECUDA, std::string("farm_mlp_train: ") + cudaGetErrorString(e)));
     std::vector<int32_t> perm((size_t)n_pairs), hidx((size_t)n_pairs * 3);
     std::vector<float> hyw((size_t)n_pairs * 2);
@@ -490,17 +550,10 @@ farm_status farm_mlp_train(farm_ctx *ctx, int32_t n_scenes, const int32_t *scene
             for (int64_t i = 0; i < b; ++i) wsum += hyw[n_pairs + off + i];
             if (!(wsum > 0.0)) continue;
             float *lslot = t.loss + (int64_t)ep * steps + sidx;
-            // stacked input rows: the pairs' query rows, then their descriptors
-            L += 2;
-            e = farm::mlp_gather_rows_bf16(d_bases + n_scenes, nullptr, d_idx + off, M.D_pad, b, M.D_pad, t.x,
-                                           M.D_pad, c.stream);
-            if (!e) e = farm::mlp_gather_rows_bf16(d_bases, d_idx + 2 * n_pairs + off, d_idx + n_pairs + off, M.D_pad,
-                                                   b, M.D_pad, t.x + b * M.D_pad, M.D_pad, c.stream);
-            if (!e) e = cudaMemcpyAsync(t.y, d_yw + off, (size_t)b * 4, cudaMemcpyDeviceToDevice, c.stream);
-            if (!e) e = cudaMemcpyAsync(t.w, d_yw + n_pairs + off, (size_t)b * 4, cudaMemcpyDeviceToDevice, c.stream);
-            if (!e) e = tc_loss_grad(c, t, b, true, (float)wsum, lslot, L);
-            if (!e) e = farm::mlp_adam(M.params, t.grad, t.m, t.v, M.count(), lr, ++t_adam, c.stream);
-            if (!e) e = refresh_bf16_weights(c);
+            e = tc_loss_grad(c, t, b, d_bases, n_scenes, d_idx + off, n_pairs, d_yw + off, d_yw + n_pairs + off,
+                             (float)wsum, lslot, L);
+            if (!e) e = farm::mlp_adam(M.params, t.grad, t.m, t.v, M.count(), lr, ++t_adam, shape_of(M), c.stream);
+            M.version += 1;
             L += 1;
         }
     }

@@ -95,17 +95,15 @@ __device__ __forceinline__ uint16_t bf16_bits(float x)
     return *reinterpret_cast<uint16_t *>(&b);
 }
 
-// h[r, j] += b[j] (pre-activation kept), a[r, j] = gelu(h[r, j]) (and its BF16 copy ab, nullable).
+// h[r, j] += b[j] (pre-activation kept), a[r, j] = gelu(h[r, j]).
 __global__ void bias_gelu_kernel(float *__restrict__ h, const float *__restrict__ b, float *__restrict__ a,
-                                 uint16_t *__restrict__ ab, int64_t rows, int cols)
+                                 int64_t rows, int cols)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * cols) return;
     const float v = h[i] + b[i % cols];
     h[i] = v;
-    const float g = gelu(v);
-    a[i] = g;
-    if (ab) ab[i] = bf16_bits(g);
+    a[i] = gelu(v);
 }
 
 // z[r, :] += b, then e = z / |z| (norm kept); one warp per row.
@@ -197,68 +195,6 @@ __global__ void colsum_kernel(const float *__restrict__ x, int64_t rows, int col
     }
 }
 
-__global__ void to_bf16_kernel(const float *__restrict__ x, int64_t count, uint16_t *__restrict__ y)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    __nv_bfloat16 b = __float2bfloat16_rn(x[i]);
-    y[i] = *reinterpret_cast<uint16_t *>(&b);
-}
-
-// dst[r, :] = src[idx[r], :] (rows of `cols` floats, source leading dimension lds).
-__global__ void gather_rows_kernel(const float *__restrict__ src, int lds, const int32_t *__restrict__ idx,
-                                   int64_t rows, int cols, float *__restrict__ dst)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * cols) return;
-    const int64_t r = i / cols;
-    const int c = (int)(i - r * cols);
-    dst[i] = src[(int64_t)idx[r] * lds + c];
-}
-
-// dst[r, 0:cols] = src_r[0:cols] with src_r = base[sel[r]] + idx[r] * lds (BF16 rows;
-// sel null: table entry 0), 16 bytes per thread (cols and the strides multiples of 8).
-__global__ void gather_rows_bf16_kernel(const uint16_t *const *__restrict__ base, const int32_t *__restrict__ sel,
-                                        const int32_t *__restrict__ idx, int64_t lds, int64_t rows, int cols,
-                                        uint16_t *__restrict__ dst, int64_t ldd)
-{
-    const int per_row = cols >> 3;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * per_row) return;
-    const int64_t r = i / per_row;
-    const int c = (int)(i - r * per_row);
-    const uint16_t *src = base[sel ? sel[r] : 0] + (int64_t)idx[r] * lds;
-    reinterpret_cast<uint4 *>(dst + r * ldd)[c] = reinterpret_cast<const uint4 *>(src)[c];
-}
-
-// dst[c, col0 + r] = bf16(src[r, c]) for r < rows, c < cols (32 x 32 tiles
-// through shared memory: reads along rows of src, writes along rows of dst).
-template <class T>
-__global__ void transpose_bf16_kernel(const T *__restrict__ src, int64_t lds, int64_t rows, int cols,
-                                      uint16_t *__restrict__ dst, int64_t ldd, int64_t col0)
-{
-    __shared__ uint16_t tile[32][33];
-    const int64_t r0 = (int64_t)blockIdx.y * 32;
-    const int c0 = blockIdx.x * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;    // 32 x 8 threads
-    for (int k = ty; k < 32; k += 8) {
-        const int64_t r = r0 + k;
-        const int c = c0 + tx;
-        uint16_t v = 0;
-        if (r < rows && c < cols) {
-            if constexpr (sizeof(T) == 4) v = bf16_bits(src[r * lds + c]);
-            else v = src[r * lds + c];
-        }
-        tile[k][tx] = v;
-    }
-    __syncthreads();
-    for (int k = ty; k < 32; k += 8) {
-        const int c = c0 + k;
-        const int64_t r = r0 + tx;
-        if (c < cols && r < rows) dst[(int64_t)c * ldd + col0 + r] = tile[tx][k];
-    }
-}
-
 // dst[r, c] = bf16(src[r, c]) for c < cols, 0 for cols <= c < ldd.
 __global__ void to_bf16_padded_kernel(const float *__restrict__ src, int64_t rows, int cols, uint16_t *__restrict__ dst,
                                       int ldd)
@@ -270,10 +206,318 @@ __global__ void to_bf16_padded_kernel(const float *__restrict__ src, int64_t row
     dst[i] = c < cols ? bf16_bits(src[r * cols + c]) : (uint16_t)0;
 }
 
-// Adam with bias correction (step t >= 1).
-__global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                            float *__restrict__ v, int64_t count, float lr, float b1, float b2, float eps, int t)
+// ---------------------------------------------------------------------------
+// The tensor-core training step's elementwise kernels.  The step is bound by
+// the passes over its activations (8,192 stacked rows x 512), so each kernel
+// reads its input once and writes every form the contractions need -- the row-
+// major BF16 operand and the transposed one (rows as K, zero past the last row
+// up to the contraction's padded length) -- from one 32 x 64 tile staged in
+// shared memory.
+// ---------------------------------------------------------------------------
+
+constexpr int TR = 32, TC = 64;         // rows and columns of a tile
+constexpr int TSTRIDE = TC + 2;         // (transposed reads of a column pair stay conflict-free)
+
+// Eight consecutive BF16 values of the tile's row tid / 8 into the tile.
+__device__ __forceinline__ void tile_put(uint16_t (*tile)[TSTRIDE], int tid, const uint16_t v[8])
 {
+    uint32_t *w = reinterpret_cast<uint32_t *>(&tile[tid >> 3][(tid & 7) * 8]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w[u] = (uint32_t)v[2 * u] | (uint32_t)v[2 * u + 1] << 16;
+}
+
+// The tile transposed: dst[c0 + c][r0 .. r0 + 31] (16 bytes per thread; ldd a
+// multiple of 8, r0 of 32) for c0 + c < cols.
+__device__ __forceinline__ void tile_write_t(const uint16_t (*tile)[TSTRIDE], int tid, uint16_t *__restrict__ dst,
+                                             int64_t ldd, int c0, int cols, int64_t r0)
+{
+    const int c = tid >> 2, k = (tid & 3) * 8;
+    if (c0 + c >= cols) return;
+    uint32_t w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w[u] = (uint32_t)tile[k + 2 * u][c] | (uint32_t)tile[k + 2 * u + 1][c] << 16;
+    *reinterpret_cast<uint4 *>(dst + (int64_t)(c0 + c) * ldd + r0 + k) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// The step's stacked input rows (query rows 0 .. b - 1, descriptor rows b ..
+// 2b - 1; D_pad long) and their transpose [D, K].  idx non-null: gathered (row
+// r < b: base[n_scenes] row idx[r]; else base[scene] row idx[n_pairs + r - b],
+// scene idx[2 n_pairs + r - b]) and written to x; null: read from x.  The
+// block of the origin also clears the step's bias-gradient sums.
+__global__ void __launch_bounds__(256)
+train_rows_kernel(const uint16_t *const *__restrict__ base, int32_t n_scenes, const int32_t *__restrict__ idx,
+                  int64_t n_pairs, int64_t b, int D, int D_pad, uint16_t *__restrict__ x, uint16_t *__restrict__ xT,
+                  int64_t K, float *__restrict__ gb1, int H, float *__restrict__ gb2, int P)
+{
+    __shared__ __align__(4) uint16_t tile[TR][TSTRIDE];
+    const int tid = threadIdx.x;
+    const int c0 = blockIdx.x * TC;
+    const int64_t r0 = (int64_t)blockIdx.y * TR;
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
+        for (int j = tid; j < H; j += 256) gb1[j] = 0.f;
+        for (int j = tid; j < P; j += 256) gb2[j] = 0.f;
+    }
+    const int64_t r = r0 + (tid >> 3);
+    const int c = c0 + (tid & 7) * 8;           // (D_pad is a multiple of 64: the tile's columns exist)
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (r < 2 * b) {
+        const uint16_t *src;
+        if (idx) {
+            src = r < b ? base[n_scenes] + (int64_t)idx[r] * D_pad
+                        : base[idx[2 * n_pairs + r - b]] + (int64_t)idx[n_pairs + r - b] * D_pad;
+        } else {
+            src = x + r * D_pad;
+        }
+        v = *reinterpret_cast<const uint4 *>(src + c);
+        if (idx) *reinterpret_cast<uint4 *>(x + r * D_pad + c) = v;
+    }
+    const uint16_t h[8] = {(uint16_t)v.x, (uint16_t)(v.x >> 16), (uint16_t)v.y, (uint16_t)(v.y >> 16),
+                           (uint16_t)v.z, (uint16_t)(v.z >> 16), (uint16_t)v.w, (uint16_t)(v.w >> 16)};
+    tile_put(tile, tid, h);
+    __syncthreads();
+    tile_write_t(tile, tid, xT, K, c0, D, r0);
+}
+
+// ab = bf16(gelu(h + b)) [rows, cols], and its transpose aT [cols, K]
+// (nullable); h is left as the contraction wrote it (the backward pass adds b
+// again).  cols a multiple of 64.
+__global__ void __launch_bounds__(256)
+gelu_bf16_kernel(const float *__restrict__ h, const float *__restrict__ b, int64_t rows, int cols,
+                 uint16_t *__restrict__ ab, uint16_t *__restrict__ aT, int64_t K)
+{
+    __shared__ __align__(4) uint16_t tile[TR][TSTRIDE];
+    const int tid = threadIdx.x;
+    const int c0 = blockIdx.x * TC;
+    const int64_t r0 = (int64_t)blockIdx.y * TR;
+    const int64_t r = r0 + (tid >> 3);
+    const int c = c0 + (tid & 7) * 8;
+    uint16_t g[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (r < rows) {
+        const float4 *hp = reinterpret_cast<const float4 *>(h + r * cols + c);
+        const float4 *bp = reinterpret_cast<const float4 *>(b + c);
+        const float4 h0 = hp[0], h1 = hp[1], b0 = __ldg(bp), b1 = __ldg(bp + 1);
+        const float v[8] = {h0.x + b0.x, h0.y + b0.y, h0.z + b0.z, h0.w + b0.w,
+                            h1.x + b1.x, h1.y + b1.y, h1.z + b1.z, h1.w + b1.w};
+#pragma unroll
+        for (int u = 0; u < 8; ++u) g[u] = bf16_bits(gelu(v[u]));
+        *reinterpret_cast<uint4 *>(ab + r * cols + c) =
+            make_uint4((uint32_t)g[0] | (uint32_t)g[1] << 16, (uint32_t)g[2] | (uint32_t)g[3] << 16,
+                       (uint32_t)g[4] | (uint32_t)g[5] << 16, (uint32_t)g[6] | (uint32_t)g[7] << 16);
+    }
+    if (!aT) return;
+    tile_put(tile, tid, g);
+    __syncthreads();
+    tile_write_t(tile, tid, aT, K, c0, cols, r0);
+}
+
+// dh = da gelu'(h + b) as its BF16 transpose dhT [cols, K], and its column
+// sums added to gb (one atomic per column and block of GB_TILES tiles).
+constexpr int GB_TILES = 4;
+__global__ void __launch_bounds__(256)
+gelu_backward_t_kernel(const float *__restrict__ h, const float *__restrict__ b, const float *__restrict__ da,
+                       int64_t rows, int cols, uint16_t *__restrict__ dhT, int64_t K, float *__restrict__ gb)
+{
+    __shared__ __align__(4) uint16_t tile[TR][TSTRIDE];
+    __shared__ float sums[TR][TC + 1];
+    const int tid = threadIdx.x;
+    const int c0 = blockIdx.x * TC;
+    const int c = c0 + (tid & 7) * 8;
+    float part[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const float4 *bp = reinterpret_cast<const float4 *>(b + c);
+    const float4 b0 = __ldg(bp), b1 = __ldg(bp + 1);
+    for (int t = 0; t < GB_TILES; ++t) {
+        const int64_t r0 = ((int64_t)blockIdx.y * GB_TILES + t) * TR;
+        if (r0 >= K) break;
+        const int64_t r = r0 + (tid >> 3);
+        uint16_t g[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (r < rows) {
+            const float4 *hp = reinterpret_cast<const float4 *>(h + r * cols + c);
+            const float4 *dp = reinterpret_cast<const float4 *>(da + r * cols + c);
+            const float4 h0 = hp[0], h1 = hp[1], d0 = dp[0], d1 = dp[1];
+            const float v[8] = {h0.x + b0.x, h0.y + b0.y, h0.z + b0.z, h0.w + b0.w,
+                                h1.x + b1.x, h1.y + b1.y, h1.z + b1.z, h1.w + b1.w};
+            const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float x = d[u] * gelu_grad(v[u]);
+                part[u] += x;
+                g[u] = bf16_bits(x);
+            }
+        }
+        tile_put(tile, tid, g);
+        __syncthreads();
+        tile_write_t(tile, tid, dhT, K, c0, cols, r0);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) sums[tid >> 3][(tid & 7) * 8 + u] = part[u];
+    __syncthreads();
+    if (tid < TC) {
+        float t = 0.f;
+        for (int i = 0; i < TR; ++i) t += sums[i][tid];
+        atomicAdd(gb + c0 + tid, t);
+    }
+}
+
+// One warp per pair (LP_PAIRS pairs per block): both rows' bias and
+// normalisation, the pair's loss, and the gradient back through the
+// normalisation, held in registers (NPL values of each row per lane) and
+// written as dz BF16 [2b, P] and its transpose dzT [P, K] (zero from 2b), with
+// its column sums added to gb2 and the loss to *loss.
+constexpr int LP_PAIRS = 32;
+template <int NPL>
+__global__ void __launch_bounds__(256)
+pair_step_kernel(const float *__restrict__ z, const float *__restrict__ b2, const float *__restrict__ y,
+                 const float *__restrict__ w, float wsum, int64_t b, int P, uint16_t *__restrict__ dzb,
+                 uint16_t *__restrict__ dzT, int64_t K, float *__restrict__ gb2, float *__restrict__ loss)
+{
+    extern __shared__ __align__(16) uint16_t lp_tile[];     // [2][LP_PAIRS][P + 2]
+    __shared__ float s_loss[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t i0 = (int64_t)blockIdx.x * LP_PAIRS;
+    const int ldt = P + 2;
+    const unsigned FULL = 0xffffffffu;
+    float colsum[NPL];
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) colsum[k] = 0.f;
+    float lsum = 0.f;
+    for (int t = warp; t < LP_PAIRS; t += 8) {
+        const int64_t i = i0 + t;
+        if (i >= b) break;
+        const float *zr[2] = {z + i * P, z + (b + i) * P};
+        float e[2][NPL], nrm[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            float ss = 0.f;
+#pragma unroll
+            for (int k = 0; k < NPL; ++k) {
+                const int j = lane + 32 * k;
+                const float v = j < P ? zr[q][j] + __ldg(b2 + j) : 0.f;
+                e[q][k] = v;
+                ss = fmaf(v, v, ss);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(FULL, ss, o);
+            nrm[q] = fmaxf(sqrtf(ss), 1e-20f);
+#pragma unroll
+            for (int k = 0; k < NPL; ++k) e[q][k] = e[q][k] / nrm[q];
+        }
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < NPL; ++k) s = fmaf(e[0][k], e[1][k], s);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+        const float wi = w ? w[i] : 1.f;
+        const float r = s - y[i];
+        const float g = 2.f * wi * r / wsum;
+        lsum += wi * r * r / wsum;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            float dot = 0.f;
+#pragma unroll
+            for (int k = 0; k < NPL; ++k) dot = fmaf(e[q][k], g * e[1 - q][k], dot);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(FULL, dot, o);
+            const float inv = 1.f / nrm[q];
+#pragma unroll
+            for (int k = 0; k < NPL; ++k) {
+                const int j = lane + 32 * k;
+                if (j >= P) continue;
+                const float dz = (g * e[1 - q][k] - e[q][k] * dot) * inv;
+                colsum[k] += dz;
+                const uint16_t h = bf16_bits(dz);
+                dzb[(q * b + i) * P + j] = h;
+                lp_tile[(q * LP_PAIRS + t) * ldt + j] = h;
+            }
+        }
+    }
+    if (lane == 0) s_loss[warp] = lsum;
+    __syncthreads();
+    // the transposes: a warp per column, its lanes the block's pairs
+    const int np = (int)min((int64_t)LP_PAIRS, b - i0);
+    for (int p = warp; p < P; p += 8) {
+        if (lane < np) {
+            dzT[(int64_t)p * K + i0 + lane] = lp_tile[lane * ldt + p];
+            dzT[(int64_t)p * K + b + i0 + lane] = lp_tile[(LP_PAIRS + lane) * ldt + p];
+        }
+    }
+    // this block's share of the columns past the last row
+    const int64_t pad = K - 2 * b, share = (pad + gridDim.x - 1) / gridDim.x;
+    const int64_t z0 = 2 * b + blockIdx.x * share, z1 = min(K, z0 + share);
+    for (int p = warp; p < P; p += 8)
+        for (int64_t k = z0 + lane; k < z1; k += 32) dzT[(int64_t)p * K + k] = 0;
+    __syncthreads();
+    // column sums and the loss over the block's warps
+    float *red = reinterpret_cast<float *>(lp_tile);        // [8][P], inside the tile's bytes
+#pragma unroll
+    for (int k = 0; k < NPL; ++k)
+        if (lane + 32 * k < P) red[warp * P + lane + 32 * k] = colsum[k];
+    __syncthreads();
+    for (int j = tid; j < P; j += 256) {
+        float t = 0.f;
+        for (int v = 0; v < 8; ++v) t += red[v * P + j];
+        atomicAdd(gb2 + j, t);
+    }
+    if (tid == 0) {
+        float t = 0.f;
+        for (int v = 0; v < 8; ++v) t += s_loss[v];
+        atomicAdd(loss, t);
+    }
+}
+
+// e = bf16((z + b) / |z + b|), one warp per row (the inference path).
+__global__ void normalize_bf16_kernel(const float *__restrict__ z, const float *__restrict__ b, int64_t rows, int cols,
+                                      uint16_t *__restrict__ e)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (r >= rows) return;
+    const float *zr = z + r * cols;
+    float ss = 0.f;
+    for (int j = lane; j < cols; j += 32) {
+        const float v = zr[j] + b[j];
+        ss = fmaf(v, v, ss);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    const float nrm = fmaxf(sqrtf(ss), 1e-20f);
+    for (int j = lane; j < cols; j += 32) e[r * cols + j] = bf16_bits((zr[j] + b[j]) / nrm);
+}
+
+// The BF16 operand copies of parameter i of [W1 | b1 | W2 | b2]: W1 in w1b
+// [H, D_pad] (whose padding stays zero), W2 in w2b [P, H] and transposed in
+// w2t [H, P].
+__device__ __forceinline__ void store_weight(int64_t i, float v, const MlpShape &m)
+{
+    const int64_t n1 = (int64_t)m.H * m.D;
+    if (i < n1) {
+        const int64_t h = i / m.D;
+        m.w1b[h * m.D_pad + (i - h * m.D)] = bf16_bits(v);
+        return;
+    }
+    const int64_t j = i - n1 - m.H;
+    if (j >= 0 && j < (int64_t)m.P * m.H) {
+        const int64_t p = j / m.H;
+        const uint16_t x = bf16_bits(v);
+        m.w2b[j] = x;
+        m.w2t[(j - p * m.H) * m.P + p] = x;
+    }
+}
+
+__global__ void weights_bf16_kernel(const float *__restrict__ p, int64_t count, MlpShape m)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < count) store_weight(i, p[i], m);
+}
+
+// Adam with bias correction (step t >= 1), then the updated weights' BF16 copies.
+__global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
+                            float *__restrict__ v, int64_t count, float lr, float b1, float b2, float eps, int t,
+                            MlpShape shape)
+{
+    __shared__ float s_c[2];
+    if (threadIdx.x < 2) s_c[threadIdx.x] = 1.f - powf(threadIdx.x ? b2 : b1, (float)t);
+    __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     const float gi = g[i];
@@ -281,9 +525,11 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, 
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    const float mh = mi / (1.f - powf(b1, (float)t));
-    const float vh = vi / (1.f - powf(b2, (float)t));
-    p[i] -= lr * mh / (sqrtf(vh) + eps);
+    const float mh = mi / s_c[0];
+    const float vh = vi / s_c[1];
+    const float x = p[i] - lr * mh / (sqrtf(vh) + eps);
+    p[i] = x;
+    store_weight(i, x, shape);
 }
 
 unsigned blocks_for(int64_t n, int th) { return (unsigned)((n + th - 1) / th); }
@@ -302,31 +548,10 @@ cudaError_t mlp_gemm(bool ta, bool tb, int M, int N, int K, float alpha, const f
     return cudaGetLastError();
 }
 
-cudaError_t mlp_bias_gelu(float *h, const float *b, float *a, int64_t rows, int cols, cudaStream_t s,
-                          uint16_t *ab)
+cudaError_t mlp_bias_gelu(float *h, const float *b, float *a, int64_t rows, int cols, cudaStream_t s)
 {
     if (rows * cols <= 0) return cudaSuccess;
-    bias_gelu_kernel<<<blocks_for(rows * cols, 256), 256, 0, s>>>(h, b, a, ab, rows, cols);
-    return cudaGetLastError();
-}
-
-cudaError_t mlp_gather_rows_bf16(const uint16_t *const *base, const int32_t *sel, const int32_t *idx, int64_t lds,
-                                 int64_t rows, int cols, uint16_t *dst, int64_t ldd, cudaStream_t s)
-{
-    if (rows * cols <= 0) return cudaSuccess;
-    if ((cols & 7) || (lds & 7) || (ldd & 7) || (reinterpret_cast<uintptr_t>(dst) & 15)) return cudaErrorInvalidValue;
-    gather_rows_bf16_kernel<<<blocks_for(rows * (cols >> 3), 256), 256, 0, s>>>(base, sel, idx, lds, rows, cols, dst,
-                                                                                ldd);
-    return cudaGetLastError();
-}
-
-cudaError_t mlp_transpose_bf16(const float *src32, const uint16_t *src16, int64_t lds, int64_t rows, int cols,
-                               uint16_t *dst, int64_t ldd, int64_t col0, cudaStream_t s)
-{
-    if (rows <= 0 || cols <= 0) return cudaSuccess;
-    dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
-    if (src32) transpose_bf16_kernel<float><<<grid, 256, 0, s>>>(src32, lds, rows, cols, dst, ldd, col0);
-    else transpose_bf16_kernel<uint16_t><<<grid, 256, 0, s>>>(src16, lds, rows, cols, dst, ldd, col0);
+    bias_gelu_kernel<<<blocks_for(rows * cols, 256), 256, 0, s>>>(h, b, a, rows, cols);
     return cudaGetLastError();
 }
 
@@ -382,25 +607,71 @@ cudaError_t mlp_colsum(const float *x, int64_t rows, int cols, float *out, bool 
     return cudaGetLastError();
 }
 
-cudaError_t mlp_to_bf16(const float *x, int64_t count, uint16_t *y, cudaStream_t s)
+cudaError_t mlp_train_rows(const uint16_t *const *base, int32_t n_scenes, const int32_t *idx, int64_t n_pairs, int64_t b,
+                           int D, int D_pad, uint16_t *x, uint16_t *xT, int64_t K, float *gb1, int H, float *gb2, int P,
+                           cudaStream_t s)
 {
-    if (count <= 0) return cudaSuccess;
-    to_bf16_kernel<<<blocks_for(count, 256), 256, 0, s>>>(x, count, y);
+    if (b < 1 || D_pad % TC != 0 || K % 64 != 0 || K < 2 * b) return cudaErrorInvalidValue;
+    dim3 grid((unsigned)(D_pad / TC), (unsigned)(K / TR));
+    train_rows_kernel<<<grid, 256, 0, s>>>(base, n_scenes, idx, n_pairs, b, D, D_pad, x, xT, K, gb1, H, gb2, P);
     return cudaGetLastError();
 }
 
-cudaError_t mlp_gather_rows(const float *src, int lds, const int32_t *idx, int64_t rows, int cols, float *dst,
-                            cudaStream_t s)
+cudaError_t mlp_gelu_bf16(const float *h, const float *b, int64_t rows, int cols, uint16_t *ab, uint16_t *aT, int64_t K,
+                          cudaStream_t s)
 {
-    if (rows * cols <= 0) return cudaSuccess;
-    gather_rows_kernel<<<blocks_for(rows * cols, 256), 256, 0, s>>>(src, lds, idx, rows, cols, dst);
+    if (rows < 1 || cols % TC != 0 || (aT && (K % 64 != 0 || K < rows))) return cudaErrorInvalidValue;
+    dim3 grid((unsigned)(cols / TC), (unsigned)(((aT ? K : rows) + TR - 1) / TR));
+    gelu_bf16_kernel<<<grid, 256, 0, s>>>(h, b, rows, cols, ab, aT, K);
     return cudaGetLastError();
 }
 
-cudaError_t mlp_adam(float *p, const float *g, float *m, float *v, int64_t count, float lr, int t, cudaStream_t s)
+cudaError_t mlp_gelu_backward_t(const float *h, const float *b, const float *da, int64_t rows, int cols, uint16_t *dhT,
+                                int64_t K, float *gb, cudaStream_t s)
+{
+    if (rows < 1 || cols % TC != 0 || K % 64 != 0 || K < rows) return cudaErrorInvalidValue;
+    dim3 grid((unsigned)(cols / TC), (unsigned)((K / TR + GB_TILES - 1) / GB_TILES));
+    gelu_backward_t_kernel<<<grid, 256, 0, s>>>(h, b, da, rows, cols, dhT, K, gb);
+    return cudaGetLastError();
+}
+
+cudaError_t mlp_pair_step(const float *z, const float *b2, const float *y, const float *w, float wsum, int64_t b, int P,
+                          uint16_t *dzb, uint16_t *dzT, int64_t K, float *gb2, float *loss, cudaStream_t s)
+{
+    if (b < 1 || P < 32 || P > 1024 || K < 2 * b) return cudaErrorInvalidValue;
+    // the tile, 64 rows of P + 2 values (more than the 8 P floats of the column sums)
+    const size_t smem = (size_t)2 * LP_PAIRS * (P + 2) * sizeof(uint16_t);
+    auto kern = P <= 64 ? pair_step_kernel<2> : P <= 128 ? pair_step_kernel<4> : P <= 256 ? pair_step_kernel<8>
+                : P <= 512 ? pair_step_kernel<16> : pair_step_kernel<32>;
+    if (smem + 1024 > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    kern<<<(unsigned)((b + LP_PAIRS - 1) / LP_PAIRS), 256, smem, s>>>(z, b2, y, w, wsum, b, P, dzb, dzT, K, gb2, loss);
+    return cudaGetLastError();
+}
+
+cudaError_t mlp_normalize_bf16(const float *z, const float *b, int64_t rows, int cols, uint16_t *e, cudaStream_t s)
+{
+    if (rows <= 0) return cudaSuccess;
+    normalize_bf16_kernel<<<blocks_for(rows, 8), 256, 0, s>>>(z, b, rows, cols, e);
+    return cudaGetLastError();
+}
+
+cudaError_t mlp_weights_bf16(const float *p, int64_t count, const MlpShape &m, cudaStream_t s)
 {
     if (count <= 0) return cudaSuccess;
-    adam_kernel<<<blocks_for(count, 256), 256, 0, s>>>(p, g, m, v, count, lr, 0.9f, 0.999f, 1e-8f, t);
+    cudaError_t e = cudaMemsetAsync(m.w1b, 0, (size_t)m.H * m.D_pad * sizeof(uint16_t), s);
+    if (e != cudaSuccess) return e;
+    weights_bf16_kernel<<<blocks_for(count, 256), 256, 0, s>>>(p, count, m);
+    return cudaGetLastError();
+}
+
+cudaError_t mlp_adam(float *p, const float *g, float *m, float *v, int64_t count, float lr, int t, const MlpShape &shape,
+                     cudaStream_t s)
+{
+    if (count <= 0) return cudaSuccess;
+    adam_kernel<<<blocks_for(count, 256), 256, 0, s>>>(p, g, m, v, count, lr, 0.9f, 0.999f, 1e-8f, t, shape);
     return cudaGetLastError();
 }
 

@@ -148,7 +148,7 @@ struct Cfg {
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + FIXED_BYTES;
     static_assert(!WIDE_ || (MODE == kSimBf16 && BN_ == 256), "wide epilogues: BF16, 256-object tiles");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory per CTA");
-    static_assert(BN_ % 128 == 0 && BN_ <= 256, "tile width");
+    static_assert((BN_ % 128 == 0 || BN_ == 64) && BN_ <= 256, "tile width");
     static_assert(STAGES >= 3, "pipeline depth");
     static_assert(BN_ / CM_ >= 8 && (B_PART % 1024) == 0, "B share must keep the swizzle atoms whole");
     static_assert(!PAIR_ || (CM_ == 2 && BN_ == 256), "CTA pairs: clusters of two, 256-object tiles");
@@ -1276,6 +1276,11 @@ cudaError_t launch_grouped_variant(int variant, const void *q0, const void *q1, 
     case 2:
         return launch_grouped<MODE, 256, 2, true>(q0, q1, rows_total, dim_pad, pieces, n_pieces, total_tiles, S,
                                                   tops, scale_q, num_sms, err, s, emit);
+    case kSimNarrowVariant:
+        if constexpr (MODE == kSimBf16)
+            return launch_grouped<MODE, 64, 1>(q0, q1, rows_total, dim_pad, pieces, n_pieces, total_tiles, S, tops,
+                                               scale_q, num_sms, err, s, emit);
+        return cudaErrorInvalidValue;
     default:
         return cudaErrorInvalidValue;
     }
@@ -1296,7 +1301,8 @@ bool sim_tc_available() { return get_encoder(); }
 bool sim_tc_encode_b(int mode, int variant, void *out, const void *d0, const void *d1, int64_t n, int32_t dim_pad)
 {
     static_assert(sizeof(CUtensorMap) == kTensorMapBytes, "tensor map size");
-    if (!get_encoder() || n < 1 || variant < 0 || variant >= kSimVariants || (reinterpret_cast<uintptr_t>(out) & 63u))
+    if (!get_encoder() || n < 1 || variant < 0 || variant > kSimNarrowVariant ||
+        (variant == kSimNarrowVariant && mode != kSimBf16) || (reinterpret_cast<uintptr_t>(out) & 63u))
         return false;
     switch (mode) {
     case kSimF16x3: return encode_b_variant<kSimF16x3>(out, d0, d1, n, dim_pad, variant);
