@@ -241,9 +241,9 @@ def cpu_baseline_mc(scene, spaces, qb, cq, k, n_sample, seed=0, budget_s=15.0):
 # (code_digest: the source without its comments):
 # (workload, precision, tile variant, fused) -> bytes
 SIM_TRAFFIC = {
-    ("site_n20k_d1152", "fp32", 2, True): (88.919808e6 + 123.629568e6) + (666.217216e6 + 20.915712e6),
+    ("site_n20k_d1152", "fp32", 2, True): (87.526656e6 + 122.278144e6) + (668.671232e6 + 20.659200e6),
 }
-SIM_TRAFFIC_SOURCE = "cd0fbf40425fef7a"
+SIM_TRAFFIC_SOURCE = "5dc1101cc8af4cd0"
 
 
 def code_digest(text):

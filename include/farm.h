@@ -227,7 +227,8 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
  *              fuses every scene of a FARM_PREC_FP32 or FARM_PREC_BF16
  *              batch, FARM_UNFUSED none; by default FARM_PREC_FP32 fuses
  *              the scenes whose sample holds at least 16 times the target
- *              list (about 12,000 objects and more) and FARM_PREC_BF16
+ *              list (about 12,000 objects and more) in batches of at least
+ *              two 128-row x 256-object tiles per SM, and FARM_PREC_BF16
  *              none, the faster choices measured.  All give the same ranks.
  *   batch_handle  receives the handle that farm_topk takes
  * Only target candidates whose rank r can still place them in the top k_max
@@ -388,8 +389,10 @@ farm_status farm_select_fallbacks(farm_ctx *ctx, int64_t *rows_out, int32_t rese
  * ("variants": 0 = 128 query rows x 256 objects per CTA; 1 = 128 x 128 per
  * CTA; 2 = 256 x 256 tiles computed by a pair of CTAs with two-SM MMAs).
  * All compute each cosine with the same sequence of products, so they give
- * bitwise identical results.  The first farm_query_batch of each class of
- * batch (similarity mode, and the powers of two of its total rows and of its
+ * bitwise identical results.  A FARM_PREC_FP32 batch of at most 128 rows
+ * (targets and constraints) takes a kernel for few rows with the same results
+ * instead, unless a variant is pinned or FARM_FUSED given.  The first other
+ * farm_query_batch of each class of batch (similarity mode, and the powers of two of its total rows and of its
  * mean objects per row) times every variant on its first similarity block and
  * keeps the fastest for the context.
  *

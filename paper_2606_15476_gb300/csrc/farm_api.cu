@@ -928,7 +928,7 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
     //      reduced-precision paths
     struct Batch { size_t p0 = 0, np = 0; int64_t s_floats = 0, rows = 0, blocks = 0, tblocks = 0, tmp = 0,
                    tops = 0, fused_rows = 0, twopass_rows = 0, exact_rows = 0; int32_t smem_sel = 1, smem_merge = 0,
-                   max_union = 1, gmax_twopass = 1; bool chunked = false; };
+                   max_union = 1, gmax_twopass = 1, sel_kinds = 0; bool chunked = false; };
     std::vector<farm::Piece> pieces;
     std::vector<int32_t> piece_sid;
     std::vector<Batch> batches;
@@ -975,11 +975,23 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
     };
     const int32_t keep_max = reduced ? std::max(cstride_t, cstride_l) : std::max(stride_t, stride_l);
     const int32_t fs = keep_max <= 128 ? 8 : (keep_max <= 256 ? 4 : 2);
+    // A FP32 batch of at most kSimFewRows rows takes the few-row similarity
+    // (k_sim_few.cu) and selects from its stored rows: for so few rows the
+    // fused selection's two launches and its merge cost more than the stores.
+    // So they do for a batch of fewer tiles (128 rows x 256 objects) than two
+    // per SM, whose sample and other tiles each fill a part of one wave (64
+    // queries, 224 rows, 20,000 objects, cold caches: similarity and selection
+    // 90 us stored, 99 us fused).
+    const bool few = precision == FARM_PREC_FP32 && c.pinned_variant < 0 && !(flags & FARM_FUSED) &&
+                     rows_total <= farm::kSimFewRows;
+    int64_t tiles_all = 0;
+    for (const auto &g : groups) tiles_all += farm::sim_cluster_tiles(g.nq + g.nc, c.scenes[g.sid].n, 0);
+    const bool fill = tiles_all >= 2 * (int64_t)c.num_sms;
     auto fuse_scene = [&](const Scene &s) {
         if (twopass_scene(s)) return true;
-        if (!fusable) return false;
+        if (!fusable || few) return false;
         if (flags & FARM_FUSED) return true;
-        if (precision != FARM_PREC_FP32) return false;
+        if (precision != FARM_PREC_FP32 || !fill) return false;
         const int64_t Rs = std::min<int64_t>(Rb, s.n);
         return farm::sample_width(s.n, fs) >= 16 * Rs;
     };
@@ -1081,6 +1093,8 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
                 if (pc.th0 < pc.rows) {
                     bt.tblocks += pc.rows - pc.th0;
                     bt.max_union = std::max(bt.max_union, uni);
+                    if (pc.th0 < pc.ntr) bt.sel_kinds |= farm::select_kind(nsel, gshift, pc.keep_t);
+                    if (pc.ntr < pc.rows) bt.sel_kinds |= farm::select_kind(nsel, gshift, pc.keep_l);
                 }
             }
             pc.chunks = fz ? 1 : (global_select ? 0 : chunks);
@@ -1181,7 +1195,9 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
                    log2i(rows_total) * 100 +
                    log2i((int64_t)(wn / (double)rows_total));
         auto it = c.tuned.find(tune_key);
-        if (c.pinned_variant >= 0) {
+        if (few) {
+            vlist = {farm::kSimFewVariant};
+        } else if (c.pinned_variant >= 0) {
             vlist = {c.pinned_variant};
         } else if (it != c.tuned.end()) {
             vlist = {it->second};
@@ -1295,11 +1311,8 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
         // (with FP32-accurate scenes in a reduced-precision batch, their rows
         // -- the last ones -- get the FP16 split only, the others no split)
         const int64_t split = any_exact ? exact_row0 : -1;
-        LAUNCH(farm::launch_normalize_rows(src_t, d_rowmap, n_q, dim, dim_pad, ops.q32, ops.qhi, ops.qlo, ops.qbf,
-                                           c.d_err, farm::kErrBadRow, c.stream, split));
-        if (n_c > 0)
-            LAUNCH(farm::launch_normalize_rows(src_c, d_rowmap + n_q, n_c, dim, dim_pad, ops.q32, ops.qhi, ops.qlo,
-                                               ops.qbf, c.d_err, farm::kErrBadRow, c.stream, split));
+        LAUNCH(farm::launch_normalize_rows2(src_t, n_q, src_c, n_c, d_rowmap, dim, dim_pad, ops.q32, ops.qhi, ops.qlo,
+                                            ops.qbf, c.d_err, farm::kErrBadRow, c.stream, split));
         if (precision == FARM_PREC_FP8)
             LAUNCH(farm::launch_quantize_fp8_rows(ops.q32, exact_row0, dim_pad, ops.qf8, ops.qscale, c.stream));
         if (precision == FARM_PREC_LEARNED) CK(farm::learned_embed_rows(ctx, ops.qbf, rows_total, ops.qcomp));
@@ -1399,7 +1412,7 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
             if (bt.tblocks > 0)
                 LAUNCH(farm::launch_select_thresh(d_sim, d_tops, dp, (int32_t)bt.np, bt.tblocks, bt.max_union, sel_ti,
                                                   sel_tc, sel_st, sel_li, sel_lc, sel_sl, c.d_fallback, d_rowlist,
-                                                  c.stream));
+                                                  bt.sel_kinds, c.stream));
             for (size_t k = bt.p0; k < bt.p0 + bt.np; ++k) {
                 const farm::Piece &pc = pieces[k];
                 if (pc.fs != 0 || pc.chunks != 0 || pc.th0 == 0) continue;
@@ -1805,12 +1818,8 @@ farm_status farm_query_batch_rrf(farm_ctx *ctx, int32_t scene_id, int64_t n_q, i
     int64_t off_t = 0, off_c = 0;
     for (int32_t k = 0; k < n_ch; ++k) {
         const int m0 = mark_begin(ctx, 0);
-        LAUNCH(farm::launch_normalize_rows(src_t + off_t, nullptr, n_q, dims[k], dpad[k], nullptr, qhi, qlo, nullptr,
-                                           c.d_err, farm::kErrBadRow, c.stream));
-        if (n_c > 0)
-            LAUNCH(farm::launch_normalize_rows(src_c + off_c, nullptr, n_c, dims[k], dpad[k], nullptr,
-                                               qhi + (size_t)n_q * dpad[k], qlo + (size_t)n_q * dpad[k], nullptr,
-                                               c.d_err, farm::kErrBadRow, c.stream));
+        LAUNCH(farm::launch_normalize_rows2(src_t + off_t, n_q, src_c + off_c, n_c, nullptr, dims[k], dpad[k], nullptr,
+                                            qhi, qlo, nullptr, c.d_err, farm::kErrBadRow, c.stream));
         mark_end(ctx, m0);
         off_t += n_q * dims[k];
         off_c += n_c * dims[k];
@@ -1826,7 +1835,10 @@ farm_status farm_query_batch_rrf(farm_ctx *ctx, int32_t scene_id, int64_t n_q, i
         if (th0 < rows)
             LAUNCH(farm::launch_select_thresh(d_sim, d_tops, reinterpret_cast<farm::Piece *>(d_pieces) + k, 1,
                                               rows - th0, uni, tl, nullptr, Rt, ll, nullptr, Rl, c.d_fallback,
-                                              d_rowlist, c.stream));
+                                              d_rowlist,
+                                              farm::select_kind(n, gshift, Rl) |
+                                                  (th0 < n_q ? farm::select_kind(n, gshift, Rt) : 0),
+                                              c.stream));
         mark_end(ctx, m2);
     }
 

@@ -255,6 +255,13 @@ cudaError_t launch_normalize_rows(const float *src, const int32_t *dst_rows, int
                                   uint16_t *dst_lo, uint16_t *dst_bf16, int32_t *err, int err_bit,
                                   cudaStream_t s, int64_t split = -1);
 
+// The same for the rows of two sources end to end: rows [0, rows) from src,
+// rows [rows, rows + rows2) from src2 (dst_rows covers both).
+cudaError_t launch_normalize_rows2(const float *src, int64_t rows, const float *src2, int64_t rows2,
+                                   const int32_t *dst_rows, int32_t dim, int32_t dim_pad, float *dst32,
+                                   uint16_t *dst_hi, uint16_t *dst_lo, uint16_t *dst_bf16, int32_t *err, int err_bit,
+                                   cudaStream_t s, int64_t split = -1);
+
 // E4M3 copy of unit rows with a per-row scale (max|x| / 448).
 cudaError_t launch_quantize_fp8_rows(const float *src, int64_t rows, int32_t dim_pad, uint8_t *dst, float *scale,
                                      cudaStream_t s);
@@ -281,10 +288,14 @@ constexpr int kSimTileM = 128;
 // Internal to the library (farm_sim_variant_pin does not name it): 3, 128 x 64
 // tiles on one CTA each, for BF16 contractions whose output is too small for
 // the wider tiles to occupy the chip (the training step's weight gradients).
+// 4, at most kSimFewRows query rows per block and 128 objects per CTA
+// (k_sim_few.cu), FP32-accurate.
 constexpr int kSimVariants = 3;
 constexpr int kSimNarrowVariant = 3;
+constexpr int kSimFewVariant = 4;
+constexpr int kSimFewRows = 128;
 constexpr int kSimPairVariant = 2;      // the single-problem launches use the CTA pairs
-inline int sim_variant_bn(int v) { return v == kSimNarrowVariant ? 64 : v == 1 ? 128 : 256; }
+inline int sim_variant_bn(int v) { return v == kSimNarrowVariant ? 64 : v == 1 || v == kSimFewVariant ? 128 : 256; }
 inline int sim_variant_cluster(int v) { return v == 2 ? 2 : 1; }
 enum SimMode { kSimF16x3 = 0, kSimBf16 = 1, kSimFp8 = 2 };
 
@@ -396,6 +407,18 @@ cudaError_t launch_sim_tc_grouped(int mode, int variant, const void *q0, const v
                                   float *S, float *tops, const float *scale_q, int num_sms, int32_t *err,
                                   cudaStream_t s, const FuseEmit *emit = nullptr);
 
+// The FP32-accurate similarity of blocks of at most kSimFewRows query rows
+// (k_sim_few.cu): one problem, or the pieces of a device table numbered with
+// kSimFewVariant's tiles, whose tensor maps are that variant's.  Cosines and
+// group maxima as the other variants', bit for bit.
+cudaError_t launch_sim_few(const uint16_t *q_hi, const uint16_t *q_lo, const uint16_t *d_hi, const uint16_t *d_lo,
+                           float *S, int64_t rows, int64_t n, int32_t dim_pad, int64_t ld_s, float *tops, int32_t *err,
+                           cudaStream_t s);
+cudaError_t launch_sim_few_grouped(const uint16_t *q_hi, const uint16_t *q_lo, int64_t rows_total, int32_t dim_pad,
+                                   const GemmPiece *pieces, int32_t n_pieces, int64_t total_tiles, float *S,
+                                   float *tops, int32_t *err, cudaStream_t s);
+cudaError_t preload_sim_few();
+
 // One problem (rows x n, S leading dimension ld_s, group maxima at tops with
 // group_stride(n) floats per row, nullable) on the tensor cores, variant 2 (CTA pairs).
 // Three FP16 terms, hi*hi + 2^-11 (hi*lo + lo*hi), from the split the
@@ -492,14 +515,17 @@ cudaError_t launch_merge_chunks(const Piece *pieces, int32_t n_pieces, int64_t t
 // max_union: the largest group count of the launch (at most 8,192 are used).  Rows
 // whose candidates overflow fall back to an exact global-memory select and
 // are counted in *n_fallback (device).  Outputs as launch_select_grouped.
-// With row_list (device, total_blocks + 1 int32 of scratch) a warp-level
-// select takes every row of a list of at most 256 entries and at most 1,024
-// group maxima first (one warp per row, no block barriers) and hands the
-// rest to the block-level select; both give the same lists.
+// With row_list (device, total_blocks + 1 int32 of scratch) the warp-level
+// selects take their rows first (one warp per row, no block barriers) and
+// hand the rest to the block-level select; all give the same lists.  kinds:
+// the select_kind bits of the launch's rows (a kernel that none of them needs
+// is not launched).
+enum { kSelectSmallRows = 1, kSelectOtherRows = 2 };
+int select_kind(int64_t n, int gshift, int32_t keep);
 cudaError_t launch_select_thresh(const float *S, const float *tops, const Piece *pieces, int32_t n_pieces,
                                  int64_t total_blocks, int32_t max_union, int32_t *tsel_idx, float *tsel_cos,
                                  int32_t stride_t, int32_t *lsel_idx, float *lsel_cos, int32_t stride_l,
-                                 int32_t *n_fallback, int32_t *row_list, cudaStream_t s);
+                                 int32_t *n_fallback, int32_t *row_list, int kinds, cudaStream_t s);
 // The fused rank selection (k_fuse_select.cu) over the launch rows of the
 // fused pieces (fs > 0; the other pieces' rows are skipped), whose sample
 // rows (sampling stride fs) the similarity kernel

@@ -24,9 +24,10 @@ __device__ __forceinline__ uint16_t half_bits(__half h) { return *reinterpret_ca
 // lane), then the unit row written to each requested copy.  split >= 0: a
 // destination row below split gets the FP32 and BF16 copies only, one at or
 // above it the FP16 split only (a batch whose last rows run the FP32-accurate
-// similarity); split < 0: every requested copy of every row.
-__global__ void normalize_rows_kernel(const float *__restrict__ src, const int32_t *__restrict__ dst_rows,
-                                      int64_t rows, int32_t dim, int32_t dim_pad,
+// similarity); split < 0: every requested copy of every row.  Rows from rows1
+// on come from src2.
+__global__ void normalize_rows_kernel(const float *__restrict__ src, int64_t rows1, const float *__restrict__ src2,
+                                      const int32_t *__restrict__ dst_rows, int64_t rows, int32_t dim, int32_t dim_pad,
                                       float *__restrict__ dst32, uint16_t *__restrict__ dst_hi,
                                       uint16_t *__restrict__ dst_lo, uint16_t *__restrict__ dst_bf16,
                                       int64_t split, int32_t *err, int err_bit)
@@ -34,11 +35,11 @@ __global__ void normalize_rows_kernel(const float *__restrict__ src, const int32
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
-    const float *x = src + row * (int64_t)dim;
+    const float *x = row < rows1 ? src + row * (int64_t)dim : src2 + (row - rows1) * (int64_t)dim;
     // float4 loads and stores where every row starts on a 16-byte boundary
     // (8 bytes for the 16-bit copies)
     auto al = [](const void *q, uintptr_t a) { return q == nullptr || (reinterpret_cast<uintptr_t>(q) & (a - 1)) == 0; };
-    const bool vec = ((dim | dim_pad) & 3) == 0 && al(src, 16) && al(dst32, 16) && al(dst_hi, 8) && al(dst_lo, 8) &&
+    const bool vec = ((dim | dim_pad) & 3) == 0 && al(x, 16) && al(dst32, 16) && al(dst_hi, 8) && al(dst_lo, 8) &&
                      al(dst_bf16, 8);
     float ss = 0.f;
     if (vec) {
@@ -198,18 +199,28 @@ cudaError_t launch_quantize_fp8_rows(const float *src, int64_t rows, int32_t dim
     return cudaGetLastError();
 }
 
+cudaError_t launch_normalize_rows2(const float *src, int64_t rows1, const float *src2, int64_t rows2,
+                                   const int32_t *dst_rows, int32_t dim, int32_t dim_pad, float *dst32,
+                                   uint16_t *dst_hi, uint16_t *dst_lo, uint16_t *dst_bf16, int32_t *err, int err_bit,
+                                   cudaStream_t s, int64_t split)
+{
+    const int64_t rows = rows1 + rows2;
+    if (rows <= 0) return cudaSuccess;
+    const int warps = 8;
+    const int64_t blocks = (rows + warps - 1) / warps;
+    normalize_rows_kernel<<<(unsigned)blocks, warps * 32, 0, s>>>(src, rows1, src2, dst_rows, rows, dim, dim_pad,
+                                                                   dst32, dst_hi, dst_lo, dst_bf16,
+                                                                   split, err, err_bit);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_normalize_rows(const float *src, const int32_t *dst_rows, int64_t rows,
                                   int32_t dim, int32_t dim_pad, float *dst32, uint16_t *dst_hi,
                                   uint16_t *dst_lo, uint16_t *dst_bf16, int32_t *err, int err_bit,
                                   cudaStream_t s, int64_t split)
 {
-    if (rows <= 0) return cudaSuccess;
-    const int warps = 8;
-    const int64_t blocks = (rows + warps - 1) / warps;
-    normalize_rows_kernel<<<(unsigned)blocks, warps * 32, 0, s>>>(src, dst_rows, rows, dim, dim_pad,
-                                                                   dst32, dst_hi, dst_lo, dst_bf16,
-                                                                   split, err, err_bit);
-    return cudaGetLastError();
+    return launch_normalize_rows2(src, rows, nullptr, 0, dst_rows, dim, dim_pad, dst32, dst_hi, dst_lo, dst_bf16, err,
+                                  err_bit, s, split);
 }
 
 cudaError_t launch_prepare_views(const float *views_soa, const float *pos, int64_t n, int32_t n_views, float *out,

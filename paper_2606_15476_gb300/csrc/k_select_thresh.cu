@@ -704,10 +704,18 @@ select_warp_kernel(const float *__restrict__ S, const float *__restrict__ tops, 
 
 }  // namespace
 
+// (the rule by which the warp-level kernels above part the rows)
+int select_kind(int64_t n, int gshift, int32_t keep)
+{
+    const int64_t g = group_count(n, gshift);
+    return gshift == kGroupShiftSmall && keep <= NARROW_R && (g < keep ? n : g) <= 32 * WS_KPL ? kSelectSmallRows
+                                                                                               : kSelectOtherRows;
+}
+
 cudaError_t launch_select_thresh(const float *S, const float *tops, const Piece *pieces, int32_t n_pieces,
                                  int64_t total_blocks, int32_t max_union, int32_t *tsel_idx, float *tsel_cos,
                                  int32_t stride_t, int32_t *lsel_idx, float *lsel_cos, int32_t stride_l,
-                                 int32_t *n_fallback, int32_t *row_list, cudaStream_t s)
+                                 int32_t *n_fallback, int32_t *row_list, int kinds, cudaStream_t s)
 {
     if (total_blocks <= 0) return cudaSuccess;
     if (n_pieces < 1 || total_blocks > 0x7fffffff || max_union < 1 || ((uintptr_t)S & 15u) != 0 ||
@@ -729,12 +737,18 @@ cudaError_t launch_select_thresh(const float *S, const float *tops, const Piece 
     // the warp-level selects first (each takes its own rows); the rows they
     // hand on go to the block-level one
     if ((e = cudaMemsetAsync(row_list, 0, sizeof(int32_t), s)) != cudaSuccess) return e;
-    select_warp_small_kernel<<<(unsigned)((total_blocks + WW - 1) / WW), WW * 32, 0, s>>>(
-        S, tops, pieces, n_pieces, total_blocks, tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos, stride_l, row_list);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    select_warp_kernel<<<(unsigned)((total_blocks + WW - 1) / WW), WW * 32, 0, s>>>(
-        S, tops, pieces, n_pieces, total_blocks, tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos, stride_l, row_list);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (kinds & kSelectSmallRows) {
+        select_warp_small_kernel<<<(unsigned)((total_blocks + WW - 1) / WW), WW * 32, 0, s>>>(
+            S, tops, pieces, n_pieces, total_blocks, tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos, stride_l,
+            row_list);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (kinds & kSelectOtherRows) {
+        select_warp_kernel<<<(unsigned)((total_blocks + WW - 1) / WW), WW * 32, 0, s>>>(
+            S, tops, pieces, n_pieces, total_blocks, tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos, stride_l,
+            row_list);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     e = cudaFuncSetAttribute(select_thresh_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t grid = total_blocks < 2048 ? total_blocks : 2048;

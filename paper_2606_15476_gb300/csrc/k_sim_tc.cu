@@ -57,50 +57,16 @@
 // frees its TMEM and returns.
 #include <algorithm>
 
-#include <cuda.h>
-#include <cudaTypedefs.h>
-
-#include "farm_internal.h"
+#include "tc_common.cuh"
 
 namespace farm {
 namespace {
 
+using namespace tc;
+
 constexpr int BM = kSimTileM;
 constexpr int STAGE_BUDGET = 192 * 1024;     // shared memory for the operand pipeline
-constexpr uint32_t WAIT_LIMIT = 1u << 24;    // try_wait polls before giving up (about a second)
 constexpr int GROUP_M = 8;                   // tile raster: 8 cluster rows share each column tile
-constexpr float RESID_SCALE_INV = 1.f / 2048.f;   // the residual operands carry a factor 2^11
-
-// Per-mode element layout of the operand rows of a K slice.
-template <int MODE>
-struct Elem;
-template <>
-struct Elem<kSimF16x3> {                     // three-term FP16 with scaled residuals
-    static constexpr int BK = 32;            // FP16 elements per K slice (64-byte rows)
-    static constexpr int ROW_BYTES = 64;
-    static constexpr int KSTEPS = 2;         // 16 FP16 values (32 bytes) per MMA
-    static constexpr bool SPLIT = true;      // hi and lo tiles of each operand
-    static constexpr uint64_t LAYOUT = 4;    // 64-byte swizzle
-    static constexpr uint32_t SBO = 512;     // 8 rows x 64 bytes
-};
-template <>
-struct Elem<kSimBf16> {                      // BF16
-    static constexpr int BK = 64;            // BF16 elements per K slice (128-byte rows)
-    static constexpr int ROW_BYTES = 128;
-    static constexpr int KSTEPS = 4;         // 16 BF16 values (32 bytes) per MMA
-    static constexpr bool SPLIT = false;
-    static constexpr uint64_t LAYOUT = 2;    // 128-byte swizzle
-    static constexpr uint32_t SBO = 1024;    // 8 rows x 128 bytes
-};
-template <>
-struct Elem<kSimFp8> {                       // FP8 E4M3
-    static constexpr int BK = 128;           // FP8 elements per K slice (128-byte rows)
-    static constexpr int ROW_BYTES = 128;
-    static constexpr int KSTEPS = 4;         // 32 FP8 values (32 bytes) per MMA
-    static constexpr bool SPLIT = false;
-    static constexpr uint64_t LAYOUT = 2;    // 128-byte swizzle
-    static constexpr uint32_t SBO = 1024;    // 8 rows x 128 bytes
-};
 
 // A tile configuration: BN objects per tile, CM CTAs per cluster (1, or 2
 // for a pair); PAIR: the two CTAs of a cluster compute one 256 x BN tile with
@@ -155,62 +121,6 @@ struct Cfg {
     static_assert(PAIR_ || CM_ == 1, "clusters of two only as CTA pairs");
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-// Bounded wait for the phase with the given parity; false on expiry.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity)
-{
-    const uint32_t a = smem_u32(bar);
-    for (uint32_t i = 0; i < WAIT_LIMIT; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
-// One non-blocking test of the phase with the given parity.
-__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
-        : "memory");
-}
-
 __device__ __forceinline__ uint32_t cluster_rank()
 {
     uint32_t r;
@@ -222,32 +132,6 @@ __device__ __forceinline__ uint32_t cluster_rank()
 __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// Shared-memory matrix descriptor of a K-major operand tile with rows of
-// ROW_BYTES swizzled in 8-row core groups SBO bytes apart; version 1.  The
-// leading byte offset is unused for swizzled K-major layouts.
-template <int MODE>
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);              // start address
-    d |= (uint64_t)(Elem<MODE>::SBO >> 4) << 32;            // stride byte offset
-    d |= (uint64_t)1 << 46;                                 // descriptor version
-    d |= Elem<MODE>::LAYOUT << 61;                          // swizzle mode
-    return d;
-}
-
-// Instruction descriptors: D = F32, A and B K-major, M = m (128, or 256 for
-// a CTA pair), N = n; operand format FP16 (0, kind::f16), BF16 (1,
-// kind::f16) or E4M3 (0, kind::f8f6f4).
-__host__ __device__ constexpr uint32_t idesc(uint32_t ab_format, int n, int m)
-{
-    return (1u << 4)                      // D format F32
-           | (ab_format << 7)             // A format
-           | (ab_format << 10)            // B format
-           | ((uint32_t)(n >> 3) << 17)   // N / 8
-           | ((uint32_t)(m >> 4) << 24);  // M / 16
 }
 
 // One MMA of the mode's kind (FP16 and BF16 operands: kind::f16; E4M3:
@@ -282,12 +166,6 @@ __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b
             "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
             ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(id), "r"(accumulate));
     }
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t *bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
 }
 
 // 32 columns of the warp's 32 TMEM lanes (lane = row), without the wait.
@@ -384,11 +262,6 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32])
         : "memory");
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 // Cluster tile id -> this CTA's (first row, first column).  A cluster tile is
 // CM vertically adjacent row tiles (CTA rank r takes the r-th) of one column
 // tile; under the grouped raster GROUP_M cluster rows share each column tile
@@ -425,20 +298,6 @@ __device__ __forceinline__ void tile_origin(int tile, int m_super, int n_tiles, 
 // Maps (FP16x3 mode): q_hi, q_lo, d_hi, d_lo.  (BF16, FP8 modes): q, d, and
 // the second of each pair is unused.  scale_q: per-row scales of the query
 // rows, pieces' scale_d: per-object scales (FP8 mode only).
-template <bool GROUPED>
-__device__ __forceinline__ GemmPiece piece_of(int tile, const GemmPiece *pieces, int n_pieces,
-                                              const GemmPiece &single)
-{
-    if (!GROUPED) return single;
-    int lo = 0, hi = n_pieces - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pieces[mid].tile_begin <= tile) lo = mid;
-        else hi = mid - 1;
-    }
-    return pieces[lo];
-}
-
 // This CTA's tile of cluster tile `tile` within piece pc: first row (local
 // to the piece), first object column n0 and first stored column c0 (they
 // differ for the compacted sample tiles).
@@ -449,18 +308,6 @@ __device__ __forceinline__ void piece_tile(const GemmPiece &pc, int tile, uint32
     const int n_tiles = (int)col_tiles(pc.n, BN_, pc.col_mode, pc.col_stride);
     tile_origin<BN_, CM_>(tile - pc.tile_begin, (m_tiles + CM_ - 1) / CM_, n_tiles, rank, m0, c0);
     n0 = (int)col_tile_of(c0 / BN_, pc.col_mode, pc.col_stride) * BN_;
-}
-
-__device__ __forceinline__ uint32_t order_key(float f)
-{
-    const uint32_t u = __float_as_uint(f + 0.0f);   // -0 -> +0
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-__device__ __forceinline__ float key_value(uint32_t k)
-{
-    const uint32_t u = (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k;
-    return __uint_as_float(u);
 }
 
 // Store SL float4 values per row of the warp's 32 rows (lane = row) to
@@ -1071,40 +918,6 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
     }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-
-bool get_encoder()
-{
-    if (g_encode) return true;
-    void *fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess || !fn)
-        return false;
-    g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    return true;
-}
-
-// 2D tensor [outer, inner] row-major (FP16, BF16 or FP8 bytes), box
-// [box_outer, BK], swizzle matching the mode's row width.
-template <int MODE>
-bool make_map(CUtensorMap *m, const void *base, int64_t inner, int64_t outer, int box_outer)
-{
-    using M = Elem<MODE>;
-    const int esize = MODE == kSimFp8 ? 1 : 2;
-    const CUtensorMapDataType dt = MODE == kSimF16x3 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                   : (MODE == kSimBf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8);
-    cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
-    cuuint64_t strides[1] = {(cuuint64_t)inner * esize};
-    cuuint32_t box[2] = {(cuuint32_t)M::BK, (cuuint32_t)box_outer};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = g_encode(m, dt, 2, const_cast<void *>(base), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          MODE == kSimF16x3 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
-}
-
 // Launch with the cluster attribute and a persistent grid of as many clusters
 // as can be resident at once (a GPC with an odd number of free SMs cannot
 // hold a whole cluster on its last SM); the count is cached per device and
@@ -1301,8 +1114,9 @@ bool sim_tc_available() { return get_encoder(); }
 bool sim_tc_encode_b(int mode, int variant, void *out, const void *d0, const void *d1, int64_t n, int32_t dim_pad)
 {
     static_assert(sizeof(CUtensorMap) == kTensorMapBytes, "tensor map size");
-    if (!get_encoder() || n < 1 || variant < 0 || variant > kSimNarrowVariant ||
-        (variant == kSimNarrowVariant && mode != kSimBf16) || (reinterpret_cast<uintptr_t>(out) & 63u))
+    if (!get_encoder() || n < 1 || variant < 0 || variant > kSimFewVariant ||
+        (variant == kSimNarrowVariant && mode != kSimBf16) || (variant == kSimFewVariant && mode != kSimF16x3) ||
+        (reinterpret_cast<uintptr_t>(out) & 63u))
         return false;
     switch (mode) {
     case kSimF16x3: return encode_b_variant<kSimF16x3>(out, d0, d1, n, dim_pad, variant);
@@ -1317,6 +1131,11 @@ cudaError_t launch_sim_tc_grouped(int mode, int variant, const void *q0, const v
                                   float *S, float *tops, const float *scale_q, int num_sms, int32_t *err,
                                   cudaStream_t s, const FuseEmit *emit)
 {
+    if (variant == kSimFewVariant) {
+        if (mode != kSimF16x3 || emit) return cudaErrorInvalidValue;
+        return launch_sim_few_grouped(static_cast<const uint16_t *>(q0), static_cast<const uint16_t *>(q1), rows_total,
+                                      dim_pad, pieces, n_pieces, total_tiles, S, tops, err, s);
+    }
     switch (mode) {
     case kSimF16x3:
         return launch_grouped_variant<kSimF16x3>(variant, q0, q1, rows_total, dim_pad, pieces, n_pieces, total_tiles,
@@ -1336,6 +1155,8 @@ cudaError_t launch_sim_tc_f16x3(const uint16_t *q_hi, const uint16_t *q_lo, cons
                                 const uint16_t *d_lo, float *S, int64_t rows, int64_t n, int32_t dim_pad, int64_t ld_s,
                                 float *tops, int num_sms, int32_t *err, cudaStream_t s)
 {
+    if (rows <= kSimFewRows)
+        return launch_sim_few(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, tops, err, s);
     return launch_tc<kSimF16x3>(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, nullptr, nullptr, tops, num_sms,
                                 err, s);
 }
@@ -1355,12 +1176,13 @@ cudaError_t launch_sim_tc_fp8(const uint8_t *q, const float *scale_q, const uint
                               err, s);
 }
 
-// Loads the single-problem FP32-accurate kernel (CTA pairs; modules and
-// functions load lazily on first use).
+// Loads the single-problem FP32-accurate kernels (modules and functions load
+// lazily on first use).
 cudaError_t preload_sim_tc_f16x3()
 {
     cudaFuncAttributes a;
-    return cudaFuncGetAttributes(&a, sim_tc_kernel<kSimF16x3, 256, 2, false, true>);
+    const cudaError_t e = cudaFuncGetAttributes(&a, sim_tc_kernel<kSimF16x3, 256, 2, false, true>);
+    return e == cudaSuccess ? preload_sim_few() : e;
 }
 
 }  // namespace farm
