@@ -928,7 +928,8 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
     //      reduced-precision paths
     struct Batch { size_t p0 = 0, np = 0; int64_t s_floats = 0, rows = 0, blocks = 0, tblocks = 0, tmp = 0,
                    tops = 0, fused_rows = 0, twopass_rows = 0, exact_rows = 0; int32_t smem_sel = 1, smem_merge = 0,
-                   max_union = 1, gmax_twopass = 1, sel_kinds = 0; bool chunked = false; };
+                   max_union = 1, gmax_twopass = 1; int64_t general = 0;
+                   bool chunked = false, small = false; };
     std::vector<farm::Piece> pieces;
     std::vector<int32_t> piece_sid;
     std::vector<Batch> batches;
@@ -1093,8 +1094,6 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
                 if (pc.th0 < pc.rows) {
                     bt.tblocks += pc.rows - pc.th0;
                     bt.max_union = std::max(bt.max_union, uni);
-                    if (pc.th0 < pc.ntr) bt.sel_kinds |= farm::select_kind(nsel, gshift, pc.keep_t);
-                    if (pc.ntr < pc.rows) bt.sel_kinds |= farm::select_kind(nsel, gshift, pc.keep_l);
                 }
             }
             pc.chunks = fz ? 1 : (global_select ? 0 : chunks);
@@ -1119,7 +1118,8 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
         }
     }
     int64_t s_need = 1, tmp_need = 4, tops_need = 4;
-    for (const auto &bt : batches) {
+    for (auto &bt : batches) {
+        farm::select_general_rows(pieces.data() + bt.p0, bt.np, bt.tblocks, &bt.general, &bt.small);
         s_need = std::max(s_need, bt.s_floats);
         tmp_need = std::max(tmp_need, bt.tmp);
         tops_need = std::max(tops_need, bt.tops);
@@ -1410,9 +1410,9 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
                 LAUNCH(farm::launch_merge_chunks(dp, (int32_t)bt.np, bt.rows, bt.smem_merge, tmp_idx, tmp_val, tmp_stride,
                                                  sel_ti, sel_tc, sel_st, sel_li, sel_lc, sel_sl, c.stream));
             if (bt.tblocks > 0)
-                LAUNCH(farm::launch_select_thresh(d_sim, d_tops, dp, (int32_t)bt.np, bt.tblocks, bt.max_union, sel_ti,
-                                                  sel_tc, sel_st, sel_li, sel_lc, sel_sl, c.d_fallback, d_rowlist,
-                                                  bt.sel_kinds, c.stream));
+                LAUNCH(farm::launch_select_thresh(d_sim, d_tops, dp, (int32_t)bt.np, bt.tblocks, bt.general, bt.small,
+                                                  bt.max_union, sel_ti, sel_tc, sel_st, sel_li, sel_lc, sel_sl,
+                                                  c.d_fallback, d_rowlist, c.stream));
             for (size_t k = bt.p0; k < bt.p0 + bt.np; ++k) {
                 const farm::Piece &pc = pieces[k];
                 if (pc.fs != 0 || pc.chunks != 0 || pc.th0 == 0) continue;
@@ -1774,6 +1774,8 @@ farm_status farm_query_batch_rrf(farm_ctx *ctx, int32_t scene_id, int64_t n_q, i
     const int64_t th0 = t_thresh ? (l_thresh ? 0 : -1) : (l_thresh ? n_q : rows);
     if (th0 < 0) return fail(ctx, FARM_EINVAL, "unsupported scene size for a fused batch");
     std::vector<farm::Piece> pcs((size_t)n_ch);
+    int64_t general = 0;             // (the same for every channel)
+    bool small_rows = false;
     for (int32_t k = 0; k < n_ch; ++k) {
         farm::Piece pc{};
         pc.d32 = nullptr;
@@ -1801,6 +1803,7 @@ farm_status farm_query_batch_rrf(farm_ctx *ctx, int32_t scene_id, int64_t n_q, i
         pc.chunk_len = (int32_t)n;
         pc.th0 = (int32_t)th0;
         pc.gshift = gshift;
+        farm::select_general_rows(&pc, 1, rows - th0, &general, &small_rows);
         pcs[k] = pc;
     }
     // (pageable sources: each copy has been staged when the call returns)
@@ -1834,11 +1837,8 @@ farm_status farm_query_batch_rrf(farm_ctx *ctx, int32_t scene_id, int64_t n_q, i
                                                nullptr, 0, Rl, c.stream));
         if (th0 < rows)
             LAUNCH(farm::launch_select_thresh(d_sim, d_tops, reinterpret_cast<farm::Piece *>(d_pieces) + k, 1,
-                                              rows - th0, uni, tl, nullptr, Rt, ll, nullptr, Rl, c.d_fallback,
-                                              d_rowlist,
-                                              farm::select_kind(n, gshift, Rl) |
-                                                  (th0 < n_q ? farm::select_kind(n, gshift, Rt) : 0),
-                                              c.stream));
+                                              rows - th0, general, small_rows, uni, tl, nullptr, Rt, ll, nullptr, Rl,
+                                              c.d_fallback, d_rowlist, c.stream));
         mark_end(ctx, m2);
     }
 

@@ -471,7 +471,8 @@ struct Piece {
     int64_t s_off;          // offset of the block's first row in S (floats)
     int64_t row_begin;      // first launch row of the block
     int64_t block_begin;    // first shared-memory-select block (th0 x chunks blocks)
-    int64_t tblock_begin;   // first thresholded-select block (rows - th0 blocks)
+    int64_t tblock_begin;   // first row of the thresholded select (rows - th0 of them)
+    int64_t gblock_begin;   // first of them that takes a CTA (select_general_rows)
     int64_t q_row0;         // row of the block's first row in the normalised operand rows
     int64_t t_row0;         // list row of the first target row
     int64_t l_row0;         // list row of the first landmark row
@@ -482,6 +483,7 @@ struct Piece {
     int32_t R, klm;         // list lengths after a rescore
     int32_t chunks, chunk_len;
     int32_t th0;
+    int32_t g0;             // the first row of those (row g0 of the piece on)
     int32_t gshift;         // group maxima over 2^gshift objects (thresholded select)
     int32_t fkeep_t, fkeep_l; // fused selection: list lengths over the whole row (keep_t / keep_l: over its sample)
     int32_t n_obj;          // objects of the scene (n: the selected row length, its sample's when fused)
@@ -508,24 +510,22 @@ cudaError_t launch_merge_chunks(const Piece *pieces, int32_t n_pieces, int64_t t
                                 const int32_t *tmp_idx, const float *tmp_val, int32_t tmp_stride,
                                 int32_t *tsel_idx, float *tsel_cos, int32_t stride_t, int32_t *lsel_idx,
                                 float *lsel_cos, int32_t stride_l, cudaStream_t s);
-// Thresholded select of rows [th0, rows) of every piece (one block per row,
-// total_blocks of them), from the group maxima `tops` the tensor-core
-// similarity kernel wrote; each row needs group_count(n, gshift) >= its list
-// length, or n <= kSelectSortAll (then every entry is a candidate).
-// max_union: the largest group count of the launch (at most 8,192 are used).  Rows
-// whose candidates overflow fall back to an exact global-memory select and
-// are counted in *n_fallback (device).  Outputs as launch_select_grouped.
-// With row_list (device, total_blocks + 1 int32 of scratch) the warp-level
-// selects take their rows first (one warp per row, no block barriers) and
-// hand the rest to the block-level select; all give the same lists.  kinds:
-// the select_kind bits of the launch's rows (a kernel that none of them needs
-// is not launched).
-enum { kSelectSmallRows = 1, kSelectOtherRows = 2 };
-int select_kind(int64_t n, int gshift, int32_t keep);
+// Thresholded select of rows [th0, rows) of every piece (total_rows of them),
+// from the group maxima `tops` the tensor-core similarity kernel wrote; each
+// row needs group_count(n, gshift) >= its list length, or n <= kSelectSortAll
+// (then every entry is a candidate).  select_general_rows parts the rows (it
+// fills g0 and gblock_begin of the pieces, on the host): `general` of them take
+// a CTA each, the others, when `small`, a warp each (row_list: total_rows + 1
+// int32 of scratch).  max_union: the largest group count of the launch (at
+// most 8,192 are used).  Rows whose candidates overflow fall back to an exact
+// global-memory select and are counted in *n_fallback (device).  Outputs as
+// launch_select_grouped.
+void select_general_rows(Piece *pieces, size_t n, int64_t total_rows, int64_t *general, bool *small);
 cudaError_t launch_select_thresh(const float *S, const float *tops, const Piece *pieces, int32_t n_pieces,
-                                 int64_t total_blocks, int32_t max_union, int32_t *tsel_idx, float *tsel_cos,
-                                 int32_t stride_t, int32_t *lsel_idx, float *lsel_cos, int32_t stride_l,
-                                 int32_t *n_fallback, int32_t *row_list, int kinds, cudaStream_t s);
+                                 int64_t total_rows, int64_t general, bool small, int32_t max_union,
+                                 int32_t *tsel_idx, float *tsel_cos, int32_t stride_t, int32_t *lsel_idx,
+                                 float *lsel_cos, int32_t stride_l, int32_t *n_fallback, int32_t *row_list,
+                                 cudaStream_t s);
 // The fused rank selection (k_fuse_select.cu) over the launch rows of the
 // fused pieces (fs > 0; the other pieces' rows are skipped), whose sample
 // rows (sampling stride fs) the similarity kernel

@@ -19,8 +19,13 @@
 // are taken from the staged keys.
 //
 // One CTA of 256 threads per row: the group maxima (at most 8,192 values) are
-// staged in shared memory and their R-th largest key found by three radix
-// passes.
+// staged in shared memory and the bound tau found by counting them into value
+// bins; the candidates are ranked by value bins too (rank_words), so a row is a
+// dozen barriers and no sort.  What bounds it is that chain and the gather of
+// the groups: 100,000 objects, lists of 256: 263 us for 10,737 rows (24 ns a
+// row, 1.3 TB/s of groups; the warp-per-row select it replaced took 360),
+// lists of 64: 157 us (196); 20,000 objects, 1,024 lists of 321 and 2,546 of
+// 65: 56 us (110).
 #include "select_common.cuh"
 
 namespace farm {
@@ -33,6 +38,8 @@ constexpr int CAP = 2048;          // candidate words per row before the exact f
 constexpr int UNION_MAX = 8192;    // union values staged (a prefix of a longer union is still a subset)
 constexpr int GLIST = 2048;        // qualifying groups gathered before the row is streamed whole
 constexpr int UNROLL = 4;          // float4 loads in flight per thread
+constexpr int COUNT_MAX = 96;      // candidates ranked by counting each against all
+constexpr int RANK_MAX = 768;      // candidates ranked by value bins; more are sorted
 
 __device__ __forceinline__ void push_cand(uint64_t *cand, int *s_cnt, float x, int32_t j)
 {
@@ -71,6 +78,129 @@ __device__ __forceinline__ void stream_tail(const float *__restrict__ row, int j
     }
 }
 
+// A lower bound of the R-th largest of n keys in shared memory (n >= R >= 1;
+// the caller has just written them) that at most `slack` more than R keys
+// reach, or the R-th largest itself.  The keys between the smallest and the
+// largest are counted in up to 2,048 equal bins (the group maxima of a row
+// share their leading bits, so digits of the key itself would crowd a few
+// bins), the bin of the R-th largest found, and refined while too many keys
+// reach its lower edge: one pass as a rule.  s_mm: 2 TT / 32 words; top: the
+// largest key.
+__device__ __forceinline__ uint32_t kth_lower(const uint32_t *keys, int n, int R, int slack, uint32_t *hist,
+                                              uint32_t *wsum, uint32_t *s3, uint32_t *s_mm, uint32_t &top)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    for (int j = tid; j < n; j += TT) {       // (the thread's own keys: no barrier yet)
+        lo = min(lo, keys[j]);
+        hi = max(hi, keys[j]);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+        s_mm[2 * warp] = lo;
+        s_mm[2 * warp + 1] = hi;
+    }
+    for (int i = tid; i < 2048; i += TT) hist[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < TT / 32; ++w) {
+        lo = min(lo, s_mm[2 * w]);
+        hi = max(hi, s_mm[2 * w + 1]);
+    }
+    uint32_t base = lo, span = hi - lo, remaining = (uint32_t)R;
+    top = hi;
+#pragma unroll 1
+    for (;;) {
+        const int bits = span ? 32 - __clz(span) : 0, shift = bits > 11 ? bits - 11 : 0;
+        for (int j = tid; j < n; j += TT) {
+            const uint32_t d = keys[j] - base;
+            if (keys[j] >= base && d <= span) atomicAdd(&hist[d >> shift], 1u);
+        }
+        __syncthreads();
+        find_bucket<2048, TT>(hist, remaining, wsum, &s3[0], &s3[1], &s3[2]);
+        const uint32_t bin = s3[0], rem = s3[1], cnt = s3[2];
+        base += bin << shift;
+        // R - rem keys lie above the bin, cnt in it
+        if (shift == 0 || cnt - rem <= (uint32_t)slack) break;
+        span = min(span - (bin << shift), (1u << shift) - 1u);
+        remaining = rem;
+        for (int i = tid; i < 2048; i += TT) hist[i] = 0;
+        __syncthreads();
+    }
+    return base;
+}
+
+// The R best of the cnt distinct candidate words (cnt <= RANK_MAX, their keys in
+// [T, top]) written in rank order.  Few: each one's rank counted against the
+// others.  More: counted into 2,048 equal value bins, laid out bin by bin from
+// the top, and ranked within their bin, which holds one or two as a rule.
+__device__ __forceinline__ void rank_words(const uint64_t *cand, int cnt, int R, uint32_t T, uint32_t top,
+                                           uint32_t *hist, uint32_t *wsum, uint64_t *sorted, int32_t *__restrict__ oi,
+                                           float *__restrict__ oc)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    auto put = [&](uint64_t w, int r) {
+        if (r >= R) return;
+        oi[r] = (int32_t)(0xffffffffu - (uint32_t)(w & 0xffffffffu));
+        if (oc) oc[r] = key_value((uint32_t)(w >> 32));
+    };
+    if (cnt <= COUNT_MAX) {
+        for (int c = tid; c < cnt; c += TT) {
+            const uint64_t w = cand[c];
+            int r = 0;
+#pragma unroll 4
+            for (int j = 0; j < cnt; ++j) r += cand[j] > w ? 1 : 0;
+            put(w, r);
+        }
+        return;
+    }
+    const uint32_t span = top - T;
+    const int bits = span ? 32 - __clz(span) : 0, shift = bits > 11 ? bits - 11 : 0;
+    for (int i = tid; i < 2048; i += TT) hist[i] = 0;
+    __syncthreads();
+    for (int c = tid; c < cnt; c += TT) atomicAdd(&hist[((uint32_t)(cand[c] >> 32) - T) >> shift], 1u);
+    __syncthreads();
+    // each bin's first place: the entries of the higher bins
+    constexpr int BPT = 2048 / TT;
+    uint32_t loc[BPT], sum = 0;
+#pragma unroll
+    for (int i = 0; i < BPT; ++i) {
+        loc[i] = hist[2047 - (tid * BPT + i)];
+        sum += loc[i];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    uint32_t at = incl - sum;
+    for (int w = 0; w < warp; ++w) at += wsum[w];
+#pragma unroll
+    for (int i = 0; i < BPT; ++i) {
+        hist[2047 - (tid * BPT + i)] = at;
+        at += loc[i];
+    }
+    __syncthreads();
+    for (int c = tid; c < cnt; c += TT) {
+        const uint64_t w = cand[c];
+        sorted[atomicAdd(&hist[((uint32_t)(w >> 32) - T) >> shift], 1u)] = w;
+    }
+    __syncthreads();
+    // (a bin's places now end at its counter and start at the next higher bin's)
+    for (int c = tid; c < cnt; c += TT) {
+        const uint64_t w = sorted[c];
+        const uint32_t b = ((uint32_t)(w >> 32) - T) >> shift;
+        const uint32_t e0 = b == 2047u ? 0u : hist[b + 1], e1 = hist[b];
+        int r = (int)e0;
+        for (uint32_t k = e0; k < e1; ++k) r += sorted[k] > w ? 1 : 0;
+        put(w, r);
+    }
+}
+
 // Shared memory of one CTA of the block-level select.
 struct ThreshSmem {
     uint32_t *ukeys;        // staged group maxima or a short row (dynamic)
@@ -78,13 +208,14 @@ struct ThreshSmem {
     uint32_t *hist;         // radix histogram, then the list of qualifying groups (2048 words)
     uint32_t *wsum, *s3;
     int *s_cnt, *s_ng, *s_misc;
+    uint32_t *s_mm;
+    uint64_t *sorted;       // RANK_MAX words
 };
 
-// The block-level select of thresholded row b (ends with the row written;
-// the caller separates rows by a barrier).
+// The block-level select of row i of piece pc (ends with the row written; the
+// caller separates rows by a barrier).
 __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const float *__restrict__ tops,
-                                           const Piece *__restrict__ pieces, int32_t n_pieces, int64_t b,
-                                           int32_t *__restrict__ tsel_idx, float *__restrict__ tsel_cos,
+                                           const Piece &pc, int i, int32_t *__restrict__ tsel_idx, float *__restrict__ tsel_cos,
                                            int32_t stride_t, int32_t *__restrict__ lsel_idx,
                                            float *__restrict__ lsel_cos, int32_t stride_l,
                                            int32_t *__restrict__ n_fallback, const ThreshSmem &sm)
@@ -96,8 +227,6 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     static_assert(GLIST <= 2048, "the group list reuses the histogram");
 
     const int tid = threadIdx.x;
-    const Piece pc = pieces[find_piece(pieces, n_pieces, b, [](const Piece &x) { return x.tblock_begin; })];
-    const int i = pc.th0 + (int)(b - pc.tblock_begin);
     const bool is_tgt = i < pc.ntr;
     const int R = is_tgt ? pc.keep_t : pc.keep_l;
     int32_t *oi;
@@ -120,17 +249,20 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     const int64_t n_groups = group_count(n, gshift);
     const int U = (int)min(n_groups, (int64_t)UNION_MAX);
     if (tid == 0) { s_cnt = 0; s_ng = 0; }
+    uint32_t T = 0u, top = 0xffffffffu;    // the candidates' keys lie in [T, top]
 
-    // tau = key_value(T) is an entry of the row (never -0), and for non-NaN x,
+    // For tau = key_value(T) and non-NaN x,
     // x >= tau holds exactly when order_key(x) >= T, so the passes below
-    // compare floats and build keys only for the entries they keep.
+    // compare floats and build keys only for the entries they keep.  (T lies
+    // between two keys of the row, so tau is a number, and -0 only for a T
+    // that both zeros' key reaches.)
     if (U >= R) {
-        // tau: the R-th largest of the group maxima; then the groups whose
+        // (tau at most the R-th largest of the group maxima: a few groups more
+        // cost less than the last bits of the search); then the groups whose
         // maximum reaches it, in any order
         const float *tp = tops + pc.tops_off + (int64_t)i * group_stride(n, gshift);
         for (int j = tid; j < U; j += TT) ukeys[j] = order_key(__ldg(tp + j));
-        __syncthreads();
-        const uint32_t T = kth_key<TT>(ukeys, U, R, hist, wsum, s3);
+        T = kth_lower(ukeys, U, R, R / 8 + 8, hist, wsum, s3, sm.s_mm, top);
         const float tau = key_value(T);
         for (int j = tid; j < U; j += TT) {
             if (ukeys[j] >= T) {
@@ -174,8 +306,7 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     } else if (n <= kSelectSortAll) {
         // a short row: every entry staged, its R-th largest key found in shared memory
         for (int j = tid; j < n; j += TT) ukeys[j] = order_key(__ldcs(row + j));
-        __syncthreads();
-        const uint32_t T = kth_key<TT>(ukeys, n, R, hist, wsum, s3);
+        T = kth_lower(ukeys, n, R, R / 8 + 8, hist, wsum, s3, sm.s_mm, top);
         for (int j = tid; j < n; j += TT) {
             const uint32_t k = ukeys[j];
             if (k >= T) {
@@ -193,7 +324,13 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     const int cnt = s_cnt;
     // (fewer than R candidates cannot happen with group maxima of this row;
     // the exact select then stands in rather than list unfilled entries)
-    if (cnt >= R && cnt <= CAP) {
+    if (cnt >= R && cnt <= RANK_MAX) {
+        rank_words(cand, cnt, R, T, top, hist, wsum, sm.sorted, oi, oc);
+        for (int c = R + tid; c < stride; c += TT) {
+            oi[c] = -1;
+            if (oc) oc[c] = 0.f;
+        }
+    } else if (cnt >= R && cnt <= CAP) {
         int P = 1;
         while (P < cnt) P <<= 1;
         for (int j = cnt + tid; j < P; j += TT) cand[j] = 0ull;
@@ -214,9 +351,11 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     __shared__ uint32_t s3[3];                        \
     __shared__ int s_cnt, s_ng;                       \
     __shared__ int s_misc[TT / 32 + 3];               \
-    const ThreshSmem sm{ukeys, cand, hist, wsum, s3, &s_cnt, &s_ng, s_misc};
+    __shared__ uint32_t s_mm[TT / 16];                \
+    __shared__ uint64_t sorted[RANK_MAX];             \
+    const ThreshSmem sm{ukeys, cand, hist, wsum, s3, &s_cnt, &s_ng, s_misc, s_mm, sorted};
 
-// One CTA per thresholded row.
+// One CTA per row of the pieces' general rows.
 __global__ void __launch_bounds__(TT)
 select_thresh_kernel(const float *__restrict__ S, const float *__restrict__ tops, const Piece *__restrict__ pieces,
                      int32_t n_pieces, int32_t *__restrict__ tsel_idx, float *__restrict__ tsel_cos, int32_t stride_t,
@@ -224,8 +363,9 @@ select_thresh_kernel(const float *__restrict__ S, const float *__restrict__ tops
                      int32_t *__restrict__ n_fallback)
 {
     THRESH_SMEM
-    thresh_row(S, tops, pieces, n_pieces, blockIdx.x, tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos, stride_l,
-               n_fallback, sm);
+    const Piece pc = pieces[find_piece(pieces, n_pieces, blockIdx.x, [](const Piece &x) { return x.gblock_begin; })];
+    thresh_row(S, tops, pc, pc.g0 + (int)(blockIdx.x - pc.gblock_begin), tsel_idx, tsel_cos, stride_t, lsel_idx,
+               lsel_cos, stride_l, n_fallback, sm);
 }
 
 // The rows the warp-level select handed on (row_list[0] of them, listed
@@ -240,40 +380,33 @@ select_thresh_list_kernel(const float *__restrict__ S, const float *__restrict__
     THRESH_SMEM
     const int count = row_list[0];
     for (int k = blockIdx.x; k < count; k += gridDim.x) {
-        thresh_row(S, tops, pieces, n_pieces, row_list[1 + k], tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos,
+        const int64_t b = row_list[1 + k];
+        const Piece pc = pieces[find_piece(pieces, n_pieces, b, [](const Piece &x) { return x.tblock_begin; })];
+        thresh_row(S, tops, pc, pc.th0 + (int)(b - pc.tblock_begin), tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos,
                    stride_l, n_fallback, sm);
         __syncthreads();            // the next row reuses the shared arrays
     }
 }
 
 // ---------------------------------------------------------------------------
-// Warp-level select: one warp per row for the common case -- a list of at
-// most WS_R entries, at most 4,096 group maxima keyed as at most 1,024 keys
-// (maxima of 1, 2 or 4 consecutive groups; or, for a row with fewer group
-// maxima than its list length, at most 1,024 entries, ranked directly) --
-// with no block barriers.
+// Warp-level select of the rows of small scenes (groups of 8 objects) with
+// lists of at most NARROW_R entries, in launches of many rows: one warp per
+// row, no block barriers, the group maxima as keys (at most 1,024; or, for a
+// row with fewer group maxima than its list length, at most 1,024 entries,
+// ranked directly).
 // The R-th largest key T is found by a bitwise search (the largest T with
 // #{keys >= T} >= R), the groups whose maximum reaches it are gathered, and
-// the candidates are ranked by counting (at most 32) or sorted by a warp
-// bitonic sort (their words are all distinct).  A row outside these limits,
-// or whose groups or candidates overflow the warp's buffers, is appended to
+// the candidates are ranked by counting (their words are all distinct).  A row
+// whose groups or candidates overflow the warp's buffers is appended to
 // row_list for the block-level select.
-constexpr int WS_R = 256;       // longest list a warp selects (the BF16 path's 256 candidates)
+// (On the 67-scene batch, whose many small scenes' lists of 95 and 16 entries
+// these are: 0.68 ms, against 1.02 ms with a CTA per row.)
 constexpr int WS_KPL = 32;      // keys per lane (1,024 per row)
-constexpr int WS_GL = 448;      // qualifying groups per warp
 constexpr int WS_CAP = 512;     // candidate words per warp
 constexpr int WW = 8;           // warps (rows) per CTA
-constexpr int WS_GU = 8;        // float4 loads in flight per lane while gathering the groups
 constexpr int WS_GL_NARROW = 320;   // qualifying groups per warp (the small-scene kernel)
 constexpr int NARROW_R = 128;       // longest list of the small-scene kernel
 
-// The warp-level select of the rows of small scenes (groups of 8 objects)
-// with lists of at most NARROW_R entries: the group maxima themselves as
-// keys, the qualifying groups gathered with scalar loads, the candidates
-// ranked by counting.  (Measured on the 67-scene batch, whose many small
-// scenes' lists of 95 and 16 entries these are: 0.95 ms for the select stage
-// against 1.05 ms with the general kernel below taking every row.)  Every
-// other row is the general kernel's.
 __global__ void __launch_bounds__(WW * 32, 4)
 select_warp_small_kernel(const float *__restrict__ S, const float *__restrict__ tops, const Piece *__restrict__ pieces,
                    int32_t n_pieces, int64_t total_rows, int32_t *__restrict__ tsel_idx,
@@ -310,7 +443,7 @@ select_warp_small_kernel(const float *__restrict__ S, const float *__restrict__ 
     // themselves: their R-th largest key, then every entry reaching it
     const bool entries = n_groups < R;
     if (gshift != kGroupShiftSmall || R > NARROW_R || (entries ? (int64_t)n : n_groups) > 32 * WS_KPL)
-        return;    // the general kernel's row
+        return;    // the block-level select's row
     const int U = entries ? n : (int)n_groups;
     const int kpl = (U + 31) >> 5;
     const float *row = S + pc.s_off + (int64_t)i * pc.ld;
@@ -450,308 +583,67 @@ select_warp_small_kernel(const float *__restrict__ S, const float *__restrict__ 
     }
 }
 
-
-// Descending bitonic sort of P words (a power of two, at least 2) by one
-// warp, each lane taking compare-exchange pairs (a, a + j) of every stage.
-__device__ __forceinline__ void warp_bitonic_desc(uint64_t *w, int P, int lane)
-{
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int p = lane; p < (P >> 1); p += 32) {
-                const int a = ((p & ~(j - 1)) << 1) | (p & (j - 1));
-                const uint64_t x = w[a], y = w[a + j];
-                const bool desc = (a & k) == 0;
-                if (desc ? (x < y) : (x > y)) {
-                    w[a] = y;
-                    w[a + j] = x;
-                }
-            }
-            __syncwarp();
-        }
-    }
-}
-
-__global__ void __launch_bounds__(WW * 32, 4)
-select_warp_kernel(const float *__restrict__ S, const float *__restrict__ tops, const Piece *__restrict__ pieces,
-                   int32_t n_pieces, int64_t total_rows, int32_t *__restrict__ tsel_idx,
-                   float *__restrict__ tsel_cos, int32_t stride_t, int32_t *__restrict__ lsel_idx,
-                   float *__restrict__ lsel_cos, int32_t stride_l, int32_t *__restrict__ row_list)
-{
-    __shared__ uint32_t glist_all[WW][WS_GL];
-    __shared__ uint64_t cand_all[WW][WS_CAP];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t t = (int64_t)blockIdx.x * WW + warp;
-    if (t >= total_rows) return;            // (warp-uniform)
-    uint32_t *glist = glist_all[warp];
-    uint64_t *cand = cand_all[warp];
-    const unsigned FULL = 0xffffffffu;
-    const unsigned lt = (1u << lane) - 1u;
-    auto hand_on = [&]() {
-        if (lane == 0) row_list[1 + atomicAdd(&row_list[0], 1)] = (int32_t)t;
-    };
-    // the piece of thresholded row t (the last whose tblock_begin <= t)
-    int lo = 0, hi = n_pieces - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pieces[mid].tblock_begin <= t) lo = mid;
-        else hi = mid - 1;
-    }
-    const Piece &pc = pieces[lo];
-    const int i = pc.th0 + (int)(t - pc.tblock_begin);
-    const bool is_tgt = i < pc.ntr;
-    const int R = is_tgt ? pc.keep_t : pc.keep_l;
-    const int n = pc.n;
-    const int gshift = pc.gshift;
-    const int64_t n_groups = group_count(n, gshift);
-    // a row with fewer group maxima than R (a short row) ranks its entries
-    // themselves: their R-th largest key, then every entry reaching it
-    const bool entries = n_groups < R;
-    if (gshift == kGroupShiftSmall && R <= NARROW_R && (entries ? (int64_t)n : n_groups) <= 32 * WS_KPL)
-        return;    // the small-scene kernel's row
-    // a row of more than 1,024 group maxima keys the maxima of 2 or 4
-    // consecutive groups instead (super-groups: entries of the row too, one
-    // per super-group, so their R-th largest still bounds the row's from below)
-    int sgs = 0;
-    if (!entries)
-        while (sgs < 2 && ((n_groups + (1 << sgs) - 1) >> sgs) > 32 * WS_KPL) ++sgs;
-    const int64_t n_keys = entries ? (int64_t)n : (n_groups + (1 << sgs) - 1) >> sgs;
-    if (R > WS_R || n_keys > 32 * WS_KPL || n_keys < R) { hand_on(); return; }
-    const int U = (int)n_keys;
-    const int kpl = (U + 31) >> 5;
-    const float *row = S + pc.s_off + (int64_t)i * pc.ld;
-    // (a row of maxima is 16-byte aligned and holds whole tiles' groups, -inf
-    // past the row end, so the 2- and 4-wide loads stay inside it)
-    const float *tp = tops + pc.tops_off + (int64_t)i * group_stride(n, gshift);
-    uint32_t key[WS_KPL];
-#pragma unroll
-    for (int k = 0; k < WS_KPL; ++k) {
-        const int g = lane + 32 * k;
-        uint32_t kk = 0u;   // 0: no value
-        if (k < kpl && g < U) {
-            if (entries) {
-                kk = order_key(__ldcs(row + g));
-            } else if (sgs == 0) {
-                kk = order_key(__ldg(tp + g));
-            } else if (sgs == 1) {
-                const float2 v = __ldg(reinterpret_cast<const float2 *>(tp) + g);
-                kk = order_key(fmaxf(v.x, v.y));
-            } else {
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(tp) + g);
-                kk = order_key(fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
-            }
-        }
-        key[k] = kk;
-    }
-    // T: the R-th largest key.  It lies between the smallest and the largest
-    // key, so it shares their common leading bits; the search sets the bits
-    // below them one at a time (keeping a bit while at least R keys reach
-    // it), and stops early once exactly R keys reach the candidate: T is
-    // then the smallest of those R.
-    uint32_t kmax = 0u, kmin = 0xffffffffu;
-#pragma unroll
-    for (int k = 0; k < WS_KPL; ++k) {
-        if (k < kpl && lane + 32 * k < U) {
-            kmax = max(kmax, key[k]);
-            kmin = min(kmin, key[k]);
-        }
-    }
-    kmax = __reduce_max_sync(FULL, kmax);
-    kmin = __reduce_min_sync(FULL, kmin);
-    uint32_t T;
-    if (kmax == kmin) {
-        T = kmax;
-    } else {
-        const int hb = 31 - __clz(kmax ^ kmin);
-        T = hb == 31 ? 0u : (kmax >> (hb + 1)) << (hb + 1);
-        for (int bit = hb; bit >= 0; --bit) {
-            const uint32_t c = T | (1u << bit);
-            int cnt = 0;
-#pragma unroll
-            for (int k = 0; k < WS_KPL; ++k) cnt += (k < kpl && key[k] >= c) ? 1 : 0;
-            const unsigned tot = __reduce_add_sync(FULL, (unsigned)cnt);
-            if (tot == (unsigned)R) {
-                uint32_t mn = 0xffffffffu;
-#pragma unroll
-                for (int k = 0; k < WS_KPL; ++k)
-                    if (k < kpl && key[k] >= c) mn = min(mn, key[k]);
-                T = __reduce_min_sync(FULL, mn);
-                break;
-            }
-            if (tot > (unsigned)R) T = c;
-        }
-    }
-    int cnt = 0;
-    if (entries) {
-        // the entries reaching T (the top R and their ties) are the candidates
-#pragma unroll
-        for (int k = 0; k < WS_KPL; ++k) {
-            if (k >= kpl) break;
-            const bool q = key[k] >= T;
-            const unsigned bal = __ballot_sync(FULL, q);
-            if (q) {
-                const int pos = cnt + __popc(bal & lt);
-                if (pos < WS_CAP) cand[pos] = cand_word(key[k], lane + 32 * k);
-            }
-            cnt += __popc(bal);
-        }
-    } else {
-        // the groups whose maximum reaches T (those of the super-groups whose
-        // maximum does)
-        const float tau = key_value(T);
-        int ng = 0;
-#pragma unroll
-        for (int k = 0; k < WS_KPL; ++k) {
-            if (k >= kpl) break;
-            const bool qs = key[k] >= T;
-            if (sgs == 0) {
-                const unsigned bal = __ballot_sync(FULL, qs);
-                if (qs) {
-                    const int pos = ng + __popc(bal & lt);
-                    if (pos < WS_GL) glist[pos] = (uint32_t)(lane + 32 * k);
-                }
-                ng += __popc(bal);
-            } else if (__any_sync(FULL, qs)) {
-                for (int c = 0; c < (1 << sgs); ++c) {
-                    const int g = ((lane + 32 * k) << sgs) + c;
-                    const bool q = qs && g < n_groups && __ldg(tp + g) >= tau;
-                    const unsigned bal = __ballot_sync(FULL, q);
-                    if (q) {
-                        const int pos = ng + __popc(bal & lt);
-                        if (pos < WS_GL) glist[pos] = (uint32_t)g;
-                    }
-                    ng += __popc(bal);
-                }
-            }
-        }
-        if (ng > WS_GL) { hand_on(); return; }
-        __syncwarp();
-        // their entries >= tau, read as float4 slots (a group of 32 is eight
-        // slots, of 8 two; group starts are 32-byte aligned and a row holds
-        // round_up(n, 32) floats, so a slot never leaves it), WS_GU slots in
-        // flight per lane
-        const int sshift = gshift - 2;
-        const int smask = (1 << sshift) - 1;
-        const int slots = ng << sshift;
-        for (int s0 = 0; s0 < slots; s0 += 32 * WS_GU) {
-            float4 v[WS_GU];
-            int j4[WS_GU];
-#pragma unroll
-            for (int u = 0; u < WS_GU; ++u) {
-                const int sl = s0 + 32 * u + lane;
-                j4[u] = sl < slots ? (int)((glist[sl >> sshift] << gshift) + ((sl & smask) << 2)) : n;
-                v[u] = j4[u] < n ? __ldcs(reinterpret_cast<const float4 *>(row + j4[u])) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int u = 0; u < WS_GU; ++u) {
-                if (s0 + 32 * u >= slots) break;     // (warp-uniform: short lists take few ballots)
-                const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const bool q = j4[u] + c < n && x[c] >= tau;
-                    const unsigned bal = __ballot_sync(FULL, q);
-                    if (q) {
-                        const int pos = cnt + __popc(bal & lt);
-                        if (pos < WS_CAP) cand[pos] = cand_word(order_key(x[c]), j4[u] + c);
-                    }
-                    cnt += __popc(bal);
-                }
-            }
-        }
-    }
-    if (cnt > WS_CAP || cnt < R) { hand_on(); return; }
-    // order the candidate words (distinct: distinct positions): at most 32
-    // are ranked by counting, more sorted by a bitonic sort (padded with zero
-    // words to a power of two), in descending order
-    __syncwarp();
-    if (cnt <= 32) {
-        const uint64_t w = lane < cnt ? cand[lane] : 0ull;
-        int r = 0;
-        for (int k = 0; k < cnt; ++k) r += cand[k] > w ? 1 : 0;
-        __syncwarp();
-        if (lane < cnt) cand[r] = w;
-        __syncwarp();
-    } else {
-        int P = 64;
-        while (P < cnt) P <<= 1;
-        for (int k = cnt + lane; k < P; k += 32) cand[k] = 0ull;
-        __syncwarp();
-        warp_bitonic_desc(cand, P, lane);
-    }
-    int32_t *oi;
-    float *oc;
-    int stride;
-    if (is_tgt) {
-        const int64_t o = (pc.t_row0 + i) * (int64_t)stride_t;
-        oi = tsel_idx + o;
-        oc = tsel_cos ? tsel_cos + o : nullptr;
-        stride = stride_t;
-    } else {
-        const int64_t o = (pc.l_row0 + (i - pc.ntr)) * (int64_t)stride_l;
-        oi = lsel_idx + o;
-        oc = lsel_cos ? lsel_cos + o : nullptr;
-        stride = stride_l;
-    }
-    for (int r = lane; r < R; r += 32) {
-        const uint64_t w = cand[r];
-        oi[r] = (int32_t)(0xffffffffu - (uint32_t)(w & 0xffffffffu));
-        if (oc) oc[r] = key_value((uint32_t)(w >> 32));
-    }
-    for (int k = R + lane; k < stride; k += 32) {
-        oi[k] = -1;
-        if (oc) oc[k] = 0.f;
-    }
-}
-
 }  // namespace
 
-// (the rule by which the warp-level kernels above part the rows)
-int select_kind(int64_t n, int gshift, int32_t keep)
+// Rows of launches of at most this many take a CTA per row whatever their
+// kind: the warps of the small-row kernel would leave most of the chip idle
+// and each run its whole chain of searches and loads alone (one query in a
+// 200-object scene: 6.5 us against 15 for the small-row kernel and its list).
+constexpr int64_t kBlockRows = 1216;
+
+void select_general_rows(Piece *pieces, size_t n, int64_t total_rows, int64_t *general, bool *small)
 {
-    const int64_t g = group_count(n, gshift);
-    return gshift == kGroupShiftSmall && keep <= NARROW_R && (g < keep ? n : g) <= 32 * WS_KPL ? kSelectSmallRows
-                                                                                               : kSelectOtherRows;
+    auto small_kind = [](const Piece &p, int32_t keep) {
+        const int64_t g = group_count(p.n, p.gshift);
+        return p.gshift == kGroupShiftSmall && keep <= NARROW_R && (g < keep ? (int64_t)p.n : g) <= 32 * WS_KPL;
+    };
+    *general = 0;
+    *small = false;
+    for (size_t k = 0; k < n; ++k) {
+        Piece &p = pieces[k];
+        // target rows [th0, ntr), landmark rows [max(th0, ntr), rows)
+        const int32_t t1 = p.th0 < p.ntr ? p.ntr : p.th0;
+        const bool st = total_rows > kBlockRows && small_kind(p, p.keep_t);
+        const bool sl = total_rows > kBlockRows && small_kind(p, p.keep_l);
+        *small |= (st && p.th0 < t1) || (sl && t1 < p.rows);
+        p.g0 = st ? t1 : p.th0;
+        const int32_t g1 = sl ? t1 : p.rows;
+        p.gblock_begin = *general;
+        *general += g1 > p.g0 ? g1 - p.g0 : 0;
+    }
 }
 
 cudaError_t launch_select_thresh(const float *S, const float *tops, const Piece *pieces, int32_t n_pieces,
-                                 int64_t total_blocks, int32_t max_union, int32_t *tsel_idx, float *tsel_cos,
-                                 int32_t stride_t, int32_t *lsel_idx, float *lsel_cos, int32_t stride_l,
-                                 int32_t *n_fallback, int32_t *row_list, int kinds, cudaStream_t s)
+                                 int64_t total_rows, int64_t general, bool small, int32_t max_union,
+                                 int32_t *tsel_idx, float *tsel_cos, int32_t stride_t, int32_t *lsel_idx,
+                                 float *lsel_cos, int32_t stride_l, int32_t *n_fallback, int32_t *row_list,
+                                 cudaStream_t s)
 {
-    if (total_blocks <= 0) return cudaSuccess;
-    if (n_pieces < 1 || total_blocks > 0x7fffffff || max_union < 1 || ((uintptr_t)S & 15u) != 0 ||
-        ((uintptr_t)tops & 15u) != 0 || !n_fallback)
+    if (total_rows <= 0) return cudaSuccess;
+    if (n_pieces < 1 || total_rows > 0x7fffffff || max_union < 1 || ((uintptr_t)S & 15u) != 0 ||
+        ((uintptr_t)tops & 15u) != 0 || !n_fallback || (small && !row_list))
         return cudaErrorInvalidValue;
     // the staged group maxima, or a whole short row
     const int32_t staged = max_union < UNION_MAX ? (max_union > kSelectSortAll ? max_union : kSelectSortAll) : UNION_MAX;
     const size_t smem = (size_t)staged * sizeof(uint32_t);
     static_assert(CAP >= kSelectSortAll, "rows that take every entry fit the candidate buffer");
     cudaError_t e;
-    if (!row_list) {
+    if (general > 0) {
         e = cudaFuncSetAttribute(select_thresh_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        select_thresh_kernel<<<(unsigned)total_blocks, TT, smem, s>>>(S, tops, pieces, n_pieces, tsel_idx, tsel_cos,
-                                                                      stride_t, lsel_idx, lsel_cos, stride_l,
-                                                                      n_fallback);
-        return cudaGetLastError();
+        select_thresh_kernel<<<(unsigned)general, TT, smem, s>>>(S, tops, pieces, n_pieces, tsel_idx, tsel_cos,
+                                                                 stride_t, lsel_idx, lsel_cos, stride_l, n_fallback);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    // the warp-level selects first (each takes its own rows); the rows they
-    // hand on go to the block-level one
+    if (!small) return cudaSuccess;
+    // the small rows, then those they hand on
     if ((e = cudaMemsetAsync(row_list, 0, sizeof(int32_t), s)) != cudaSuccess) return e;
-    if (kinds & kSelectSmallRows) {
-        select_warp_small_kernel<<<(unsigned)((total_blocks + WW - 1) / WW), WW * 32, 0, s>>>(
-            S, tops, pieces, n_pieces, total_blocks, tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos, stride_l,
-            row_list);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (kinds & kSelectOtherRows) {
-        select_warp_kernel<<<(unsigned)((total_blocks + WW - 1) / WW), WW * 32, 0, s>>>(
-            S, tops, pieces, n_pieces, total_blocks, tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos, stride_l,
-            row_list);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+    select_warp_small_kernel<<<(unsigned)((total_rows + WW - 1) / WW), WW * 32, 0, s>>>(
+        S, tops, pieces, n_pieces, total_rows, tsel_idx, tsel_cos, stride_t, lsel_idx, lsel_cos, stride_l, row_list);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     e = cudaFuncSetAttribute(select_thresh_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int64_t grid = total_blocks < 2048 ? total_blocks : 2048;
+    const int64_t grid = total_rows < 304 ? total_rows : 304;
     select_thresh_list_kernel<<<(unsigned)grid, TT, smem, s>>>(S, tops, pieces, n_pieces, tsel_idx, tsel_cos,
                                                                stride_t, lsel_idx, lsel_cos, stride_l, n_fallback,
                                                                row_list);
