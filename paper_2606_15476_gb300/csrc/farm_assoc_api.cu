@@ -82,6 +82,11 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
     float *h_emu = nullptr, *h_ecov = nullptr, *h_efeat = nullptr, *h_ew = nullptr, *h_dmu = nullptr,
           *h_dcov = nullptr, *h_dfeat = nullptr;
     int32_t *h_eact = nullptr;
+    // more detections than the few-row similarity takes: only the cosines
+    // reaching tau_f are kept, up to `cap` per detection (about as many as a
+    // fused selection's row; more of them: the stored rows)
+    const bool emitting = B > farm::kSimFewRows;
+    const int32_t cap = farm::fuse_merge_capacity(1);
     // the layout of the call's device memory: sized with a null base, then
     // carved from the context's grow-only buffer
     auto layout = [&](Carve &cv) {
@@ -96,7 +101,15 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
         S = cv.take<float>((size_t)B * ld);
         a.label = cv.take<int32_t>((size_t)T);
         a.win = cv.take<unsigned long long>((size_t)T);
-        a.acc = cv.take<float>((size_t)T * (10 + F));
+        a.mcnt = cv.take<int32_t>((size_t)T); a.off = cv.take<int32_t>((size_t)T);
+        a.pos = cv.take<int32_t>((size_t)T); a.members = cv.take<int32_t>((size_t)T);
+        a.counters = cv.take<int32_t>(2);
+        if (emitting) {
+            a.over = cv.take<int32_t>((size_t)B);
+            a.emit.tau_key = cv.take<uint32_t>((size_t)B); a.emit.cnt = cv.take<int32_t>((size_t)B);
+            a.emit.cand = cv.take<uint64_t>((size_t)B * cap);
+            a.emit.cap = cap;
+        }
         if (dev) {
             a.match_cnt = match_cnt; a.match_idx = match_idx; a.match_h = match_h; a.parent = parent;
             a.out_w = out_w; a.out_mu = out_mu; a.out_cov = out_cov; a.out_feat = out_feat;
@@ -130,14 +143,12 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
         d_dmu = h_dmu; d_dcov = h_dcov; d_dfeat = h_dfeat;
     }
     // feature cosines: unit rows in the FP16 split, the FP32-accurate similarity kernel
-    c.launches += 3;
+    c.launches += 2;
     ACK(farm::launch_normalize_rows(d_dfeat, nullptr, B, F, F_pad, nullptr, dhi, dlo, nullptr, c.d_err,
                                     farm::kErrBadRow, c.stream), "normalise detections");
     ACK(farm::launch_normalize_rows(d_efeat, nullptr, N, F, F_pad, nullptr, ehi, elo, nullptr, c.d_err,
                                     farm::kErrBadDesc, c.stream), "normalise entities");
     if (!farm::sim_tc_available()) return afail(c, FARM_EINVAL, "the tensor-core similarity path is not built");
-    ACK(farm::launch_sim_tc_f16x3(dhi, dlo, ehi, elo, S, B, N, F_pad, ld, nullptr, c.num_sms, c.d_err, c.stream),
-        "feature cosines");
     // search, components, fusion
     a.N = N;
     a.B = B;
@@ -156,7 +167,15 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
     a.h_max = h_max;
     a.max_m = max_m;
     a.err = c.d_err;
-    c.launches += 9;
+    c.launches += emitting ? 10 : 8;
+    ACK(farm::launch_assoc_init(a, c.stream), "association kernels");
+    if (emitting) {
+        ACK(farm::launch_sim_tc_f16x3(dhi, dlo, ehi, elo, nullptr, B, N, F_pad, ld, nullptr, c.num_sms, c.d_err,
+                                      c.stream, &a.emit), "feature cosines");
+        ACK(farm::launch_assoc_match(a, c.stream), "association kernels");
+    }
+    ACK(farm::launch_sim_tc_f16x3(dhi, dlo, ehi, elo, S, B, N, F_pad, ld, nullptr, c.num_sms, c.d_err, c.stream,
+                                  nullptr, emitting ? a.counters + 1 : nullptr), "feature cosines");
     ACK(farm::launch_assoc(a, c.stream), "association kernels");
     if (!dev) {
         const cudaMemcpyKind k = cudaMemcpyDeviceToHost;

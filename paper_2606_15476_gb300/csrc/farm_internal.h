@@ -380,11 +380,13 @@ inline int64_t sim_cluster_tiles(int64_t rows, int64_t n, int variant, int mode 
 // row: each row's threshold (order-preserving key of its sample's R-th
 // value), candidate count and buffer of `cap` candidate words
 // (key << 32 | (2^32 - 1 - object index)).
+// gate (nullable, any launch): the kernel returns at once when *gate is 0.
 struct FuseEmit {
     uint32_t *tau_key;
     int32_t *cnt;
     uint64_t *cand;
     int32_t cap;
+    const int32_t *gate;
 };
 
 // The two B tensor maps (hi / lo, or the one operand twice) of a scene's
@@ -423,9 +425,13 @@ cudaError_t preload_sim_few();
 // group_stride(n) floats per row, nullable) on the tensor cores, variant 2 (CTA pairs).
 // Three FP16 terms, hi*hi + 2^-11 (hi*lo + lo*hi), from the split the
 // normalisation writes.
+// With `emit` (more than kSimFewRows rows) nothing is stored: every entry
+// reaching its row's threshold is appended to the row's buffer; with a gate the
+// launch does its work only when *gate is not 0.
 cudaError_t launch_sim_tc_f16x3(const uint16_t *q_hi, const uint16_t *q_lo, const uint16_t *d_hi,
                                 const uint16_t *d_lo, float *S, int64_t rows, int64_t n, int32_t dim_pad,
-                                int64_t ld_s, float *tops, int num_sms, int32_t *err, cudaStream_t s);
+                                int64_t ld_s, float *tops, int num_sms, int32_t *err, cudaStream_t s,
+                                const FuseEmit *emit = nullptr, const int32_t *gate = nullptr);
 // BF16 operands, FP32 accumulation (first stage of the reduced-precision path).
 cudaError_t launch_sim_tc_bf16(const uint16_t *q, const uint16_t *d, float *S, int64_t rows, int64_t n,
                                int32_t dim_pad, int64_t ld_s, float *tops, int num_sms, int32_t *err,
@@ -685,13 +691,21 @@ struct AssocArgs {
     int32_t max_m;
     int32_t *match_cnt, *match_idx;     // [B], [B, max_m]
     float *match_h;                     // [B, max_m]
-    int32_t *label;                     // [N + B] scratch
-    unsigned long long *win;            // [N + B] scratch
-    float *acc;                         // [(N + B) * (10 + F)] scratch
+    int32_t *label;                     // [N + B] scratch: component labels
+    unsigned long long *win;            // [N + B] scratch: winners
+    int32_t *mcnt, *off, *pos, *members;    // [N + B] scratch: each winner's members
+    int32_t *counters;                  // [2] scratch: members' array in use; detections whose list overflowed
+    int32_t *over;                      // [B] scratch: those detections
+    FuseEmit emit;                      // the emitting similarity's lists (cnt null: stored rows)
     int32_t *parent;                    // [N + B]
     float *out_w, *out_mu, *out_cov, *out_feat;         // [T], [3, T], [6, T], [T, F]
     int32_t *err;
 };
+// In stream order: init; the similarity (emitting, then launch_assoc_match and
+// the storing form behind the gate counters + 1; or storing every row); the
+// rest.
+cudaError_t launch_assoc_init(const AssocArgs &a, cudaStream_t s);
+cudaError_t launch_assoc_match(const AssocArgs &a, cudaStream_t s);
 cudaError_t launch_assoc(const AssocArgs &a, cudaStream_t s);
 
 // out[q * k + j] = src[perm[q] * ld + j] (and the 4-wide breakdown): the TopK

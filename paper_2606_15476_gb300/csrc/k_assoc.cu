@@ -8,19 +8,32 @@
 //      H = sqrt(1 - BC),  ln BC = (ln det S_d + ln det S_e) / 4 - ln det S / 2
 //                                 - dmu' S^-1 dmu / 8,  S = (S_d + S_e) / 2,
 //    (1 - BC evaluated as -expm1(ln BC)); those with H <= h_max are sorted by
-//    (H, index) and the first max_m kept (one CTA per detection);
+//    (H, index) and the first max_m kept (one CTA per detection).  For more
+//    than kSimFewRows detections the similarity kernel keeps only the cosines
+//    reaching tau_f (the emitting form of the fused rank selection, its
+//    threshold tau_f for every row), so the detection-by-entity block is
+//    neither written nor read; a detection with more of them than its buffer
+//    holds is searched over its stored row, which is then computed;
 //  * correspondence: the connected components of the graph joining each
-//    detection (node N + d) to its matches, by min-label hooking and pointer
-//    jumping (one CTA: the graph has at most B x max_m edges); the winner of a
-//    component is its entity of largest weight (lower index on ties), a
-//    component without an entity is a lone detection that starts a new
-//    entity;
-//  * fusion: every slot adds w (mu - c) and w f into its winner (c the
-//    winner's own mean: a shift that keeps FP32 digits at site coordinates),
-//    then w (S + (mu - mu_g)(mu - mu_g)') -- the sufficient-statistics merge
-//    M1 = w mu, M2 = w (S + mu mu') in a form free of the cancellation of
-//    M2 / w - mu mu'.  Sums use atomics, so their order (and the last bits)
-//    may vary from run to run.
+//    detection (node N + d) to its matches: a union-find over smallest nodes
+//    (roots hooked by compare-and-swap: every step moves a label to a smaller
+//    node, so it ends whatever the order), each detection's matches united as
+//    soon as they are found; the winner of a component is its entity of
+//    largest weight (lower index on ties), a component without an entity is a
+//    lone detection that starts a new entity;
+//  * fusion: a warp per slot; a winner sums w (mu - c) and w f over the slots
+//    merged into it (listed per winner; c the winner's own mean: a shift that
+//    keeps FP32 digits at site coordinates), then w (S + (mu - mu_g)(mu -
+//    mu_g)') -- the sufficient-statistics merge M1 = w mu, M2 = w (S + mu mu')
+//    in a form free of the cancellation of M2 / w - mu mu'.  The members'
+//    order (and the last bits) may vary from run to run.
+//
+// 4,096 detections x 20,000 entities, F = 256: 183 us a call against 300 when
+// the similarity stored the 328 MB block and a scan read it back, the
+// components took one CTA's rounds and the fusion four passes of atomics
+// (search 106 -> 25 us, components 57 -> the match kernel's tail, fusion and its
+// clearing 106 -> 39; the similarity 124 -> 111, 60% of the tensor rate: 17
+// tiles of eight K slices per CTA pair, each waiting for its fold).
 #include "farm_internal.h"
 
 namespace farm {
@@ -75,74 +88,47 @@ __device__ __noinline__ float entity_distance(int e, int32_t N, const float *__r
     return hellinger_f(md, cd, me, ce);
 }
 
-__global__ void __launch_bounds__(TA)
-assoc_search_kernel(const float *__restrict__ S, int64_t ld, int32_t N, int32_t B, const float *__restrict__ ent_mu,
-                    const float *__restrict__ ent_cov, const int32_t *__restrict__ ent_active,
-                    const float *__restrict__ det_mu, const float *__restrict__ det_cov, float tau_f, float h_max,
-                    int32_t max_m, int32_t *__restrict__ match_cnt, int32_t *__restrict__ match_idx,
-                    float *__restrict__ match_h, int32_t *err)
+// The union-find over node labels (label[x] <= x, a root labels itself).  Nodes
+// on a walk are pointed at their grandparents; labels are read past L1.
+__device__ __forceinline__ int find_root(int32_t *label, int x)
 {
-    __shared__ uint64_t cand[CAPA];
-    __shared__ int32_t pre[CAPP];
-    __shared__ int s_cnt, s_np;
-    const int d = blockIdx.x, tid = threadIdx.x;
-    if (tid == 0) {
-        s_cnt = 0;
-        s_np = 0;
-    }
-    __syncthreads();
-    float md[3], cd[6];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) md[k] = det_mu[(int64_t)k * B + d];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) cd[k] = det_cov[(int64_t)k * B + d];
-    // the row is streamed in float4 loads, four in flight per thread (its
-    // leading dimension is a multiple of 32 floats, so the row is 16-byte
-    // aligned and a load never leaves it); the entities past the cosine
-    // prefilter are listed in shared memory and evaluated by all threads
-    // together (one entity per thread), whenever the list could overflow in
-    // the next pass and at the end: evaluated where they are found, they
-    // would each run on one lane of a warp
-    const float *row = S + (int64_t)d * ld;
-    const float4 *row4 = reinterpret_cast<const float4 *>(row);
-    const int n4 = (N + 3) >> 2;
-    auto evaluate = [&](int np) {
-        for (int i = tid; i < np; i += TA) {
-            const int e = pre[i];
-            const float h = entity_distance(e, N, ent_mu, ent_cov, ent_active, md, cd);
-            if (h >= 0.f && h <= h_max) {
-                const int pos = atomicAdd(&s_cnt, 1);
-                if (pos < CAPA) cand[pos] = ((uint64_t)__float_as_uint(h) << 32) | (uint32_t)e;   // H >= 0: bits order like H
-            }
-        }
-    };
-    for (int g0 = 0; g0 < n4; g0 += TA * 4) {
-        float4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int g = g0 + u * TA + tid;
-            v[u] = g < n4 ? __ldcs(row4 + g) : make_float4(-2.f, -2.f, -2.f, -2.f);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int e0 = 4 * (g0 + u * TA + tid);
-            const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (x[c] >= tau_f && e0 + c < N) pre[atomicAdd(&s_np, 1)] = e0 + c;
-        }
-        __syncthreads();
-        const int np = s_np;
-        if (np > CAPP - PER_PASS) {      // (uniform) at most PER_PASS more could come in the next pass
-            evaluate(np);
-            __syncthreads();
-            if (tid == 0) s_np = 0;
-            __syncthreads();
+    volatile int32_t *l = label;
+    int cur = l[x];
+    if (cur != x) {
+        int prev = x, next;
+        while (cur > (next = l[cur])) {
+            l[prev] = next;
+            prev = cur;
+            cur = next;
         }
     }
-    evaluate(s_np);
-    __syncthreads();
-    const int cnt = s_cnt;
+    return cur;
+}
+
+__device__ __forceinline__ void unite(int32_t *label, int u, int v)
+{
+    int a = find_root(label, u), b = find_root(label, v);
+    while (a != b) {
+        if (a < b) {
+            const int t = a;
+            a = b;
+            b = t;
+        }
+        // a, the larger root, takes b's label, unless it has been hooked meanwhile
+        const int old = atomicCAS(&label[a], a, b);
+        if (old == a) break;
+        a = find_root(label, old);
+    }
+}
+
+// The matches of detection d: cnt candidates (H bits, entity) in cand (the
+// first CAPA of them), ordered by (H, index), the first max_m written and
+// united with the detection's node.  Every thread of the block calls it.
+__device__ __forceinline__ void finish_matches(uint64_t *cand, int cnt, int d, int32_t N, int32_t max_m,
+                                               int32_t *__restrict__ match_cnt, int32_t *__restrict__ match_idx,
+                                               float *__restrict__ match_h, int32_t *label, int32_t *err)
+{
+    const int tid = threadIdx.x;
     if (cnt > CAPA) {
         if (tid == 0) atomicOr(err, kErrAssocOverflow);
     }
@@ -167,80 +153,196 @@ assoc_search_kernel(const float *__restrict__ S, int64_t ld, int32_t N, int32_t 
     if (tid == 0) match_cnt[d] = cnt;
     for (int j = tid; j < max_m; j += TA) {
         const bool has = j < nc;
-        match_idx[(int64_t)d * max_m + j] = has ? (int32_t)(cand[j] & 0xffffffffu) : -1;
+        const int e = has ? (int)(cand[j] & 0xffffffffu) : -1;
+        match_idx[(int64_t)d * max_m + j] = e;
         match_h[(int64_t)d * max_m + j] = has ? __uint_as_float((uint32_t)(cand[j] >> 32)) : -1.f;
+        if (has) unite(label, N + d, e);
     }
 }
 
-// Connected components of the match graph: label[t] ends as the smallest
-// node of t's component.  One CTA; hooking rounds until nothing changes (at
-// most max_rounds, else the error bit).  With in_smem the labels live in
-// shared memory (T * 4 bytes of dynamic shared memory) and are written to
-// `label` at the end; otherwise they are worked on in `label` directly.
-__global__ void __launch_bounds__(1024)
-assoc_components_kernel(int32_t N, int32_t B, int32_t max_m, const int32_t *__restrict__ match_idx,
-                        int32_t *label_out, int32_t max_rounds, int32_t *err, int32_t in_smem)
+// Before the search: labels, winners and member counts cleared; with the
+// emitting similarity, every detection's threshold and an empty buffer.
+__global__ void __launch_bounds__(256)
+assoc_init_kernel(int32_t T, int32_t B, float tau_f, int32_t *__restrict__ label, unsigned long long *__restrict__ win,
+                  int32_t *__restrict__ mcnt, int32_t *__restrict__ counters, uint32_t *__restrict__ tau_key,
+                  int32_t *__restrict__ cnt)
 {
-    extern __shared__ int32_t s_label[];
-    __shared__ int s_changed;
-    const int T = N + B, tid = threadIdx.x;
-    int32_t *label = in_smem ? s_label : label_out;
-    for (int t = tid; t < T; t += blockDim.x) label[t] = t;
+    const int t = blockIdx.x * 256 + threadIdx.x;
+    if (t < 2) counters[t] = 0;
+    if (t < T) {
+        label[t] = t;
+        win[t] = 0ull;
+        mcnt[t] = 0;
+    }
+    if (tau_key && t < B) {
+        const uint32_t u = __float_as_uint(tau_f + 0.0f);      // the order key of the similarity kernels
+        tau_key[t] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+        cnt[t] = 0;
+    }
+}
+
+// One CTA per detection over the entities its cosine row reached tau_f for
+// (buffered by the similarity kernel, in any order); a detection whose buffer
+// overflowed is listed for assoc_search_kernel.
+__global__ void __launch_bounds__(TA)
+assoc_match_kernel(FuseEmit emit, int32_t N, int32_t B, const float *__restrict__ ent_mu,
+                   const float *__restrict__ ent_cov, const int32_t *__restrict__ ent_active,
+                   const float *__restrict__ det_mu, const float *__restrict__ det_cov, float h_max, int32_t max_m,
+                   int32_t *__restrict__ match_cnt, int32_t *__restrict__ match_idx, float *__restrict__ match_h,
+                   int32_t *label, int32_t *n_over, int32_t *__restrict__ over, int32_t *err)
+{
+    __shared__ uint64_t cand[CAPA];
+    __shared__ int s_cnt;
+    const int d = blockIdx.x, tid = threadIdx.x;
+    const int np = emit.cnt[d];
+    if (np > emit.cap) {
+        if (tid == 0) over[atomicAdd(n_over, 1)] = d;
+        return;
+    }
+    if (tid == 0) s_cnt = 0;
+    float md[3], cd[6];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) md[k] = det_mu[(int64_t)k * B + d];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) cd[k] = det_cov[(int64_t)k * B + d];
     __syncthreads();
-    const int E = B * max_m;
-    int round = 0;
-    for (; round < max_rounds; ++round) {
-        if (tid == 0) s_changed = 0;
-        __syncthreads();
-        // hooking: the parent of the larger label takes the smaller one
-        for (int k = tid; k < E; k += blockDim.x) {
-            const int e = match_idx[k];
-            if (e < 0) continue;
-            const int u = N + k / max_m;
-            const int pu = ((volatile int32_t *)label)[u], pv = ((volatile int32_t *)label)[e];
-            if (pu != pv) {
-                atomicMin(&label[max(pu, pv)], min(pu, pv));
-                s_changed = 1;
-            }
+    const uint64_t *words = emit.cand + (int64_t)d * emit.cap;
+    for (int i = tid; i < np; i += TA) {
+        const int e = (int)(0xffffffffu - (uint32_t)(words[i] & 0xffffffffu));
+        const float h = entity_distance(e, N, ent_mu, ent_cov, ent_active, md, cd);
+        if (h >= 0.f && h <= h_max) {
+            const int pos = atomicAdd(&s_cnt, 1);
+            if (pos < CAPA) cand[pos] = ((uint64_t)__float_as_uint(h) << 32) | (uint32_t)e;   // H >= 0: bits order like H
         }
-        __syncthreads();
-        // pointer jumping until every node points at a root
-        for (int t = tid; t < T; t += blockDim.x) {
-            int l = label[t];
-            for (int it = 0; it < 4096; ++it) {
-                const int ll = ((volatile int32_t *)label)[l];
-                if (ll == l) break;
-                l = ll;
-            }
-            label[t] = l;
-        }
-        __syncthreads();
-        if (!s_changed) break;
-        __syncthreads();
     }
-    if (tid == 0 && round >= max_rounds) atomicOr(err, kErrTimeout);
-    if (in_smem)
-        for (int t = tid; t < T; t += blockDim.x) label_out[t] = s_label[t];
+    __syncthreads();
+    finish_matches(cand, s_cnt, d, N, max_m, match_cnt, match_idx, match_h, label, err);
 }
 
-// win[r]: the heaviest entity of component r as (w bits, ~index).
-__global__ void assoc_winner_kernel(int32_t N, const float *__restrict__ ent_w, const int32_t *__restrict__ label,
-                                    unsigned long long *win)
+// Detections over their stored cosine rows: all B of them, or (over non-null)
+// the *n_over listed ones.
+__global__ void __launch_bounds__(TA)
+assoc_search_kernel(const float *__restrict__ S, int64_t ld, int32_t N, int32_t B, const float *__restrict__ ent_mu,
+                    const float *__restrict__ ent_cov, const int32_t *__restrict__ ent_active,
+                    const float *__restrict__ det_mu, const float *__restrict__ det_cov, float tau_f, float h_max,
+                    int32_t max_m, int32_t *__restrict__ match_cnt, int32_t *__restrict__ match_idx,
+                    float *__restrict__ match_h, int32_t *label, const int32_t *n_over,
+                    const int32_t *__restrict__ over, int32_t *err)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= N) return;
-    const unsigned long long k = ((unsigned long long)__float_as_uint(fmaxf(ent_w[e], 0.f)) << 32) |
-                                 (unsigned long long)(0xffffffffu - (uint32_t)e);
-    atomicMax(&win[label[e]], k);
+    __shared__ uint64_t cand[CAPA];
+    __shared__ int32_t pre[CAPP];
+    __shared__ int s_cnt, s_np;
+    const int tid = threadIdx.x;
+    const int count = over ? *n_over : B;
+    for (int at = blockIdx.x; at < count; at += gridDim.x) {
+        const int d = over ? over[at] : at;
+        if (tid == 0) {
+            s_cnt = 0;
+            s_np = 0;
+        }
+        __syncthreads();
+        float md[3], cd[6];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) md[k] = det_mu[(int64_t)k * B + d];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) cd[k] = det_cov[(int64_t)k * B + d];
+        // the row is streamed in float4 loads, four in flight per thread (its
+        // leading dimension is a multiple of 32 floats, so the row is 16-byte
+        // aligned and a load never leaves it); the entities past the cosine
+        // prefilter are listed in shared memory and evaluated by all threads
+        // together (one entity per thread), whenever the list could overflow in
+        // the next pass and at the end: evaluated where they are found, they
+        // would each run on one lane of a warp
+        const float *row = S + (int64_t)d * ld;
+        const float4 *row4 = reinterpret_cast<const float4 *>(row);
+        const int n4 = (N + 3) >> 2;
+        auto evaluate = [&](int np) {
+            for (int i = tid; i < np; i += TA) {
+                const int e = pre[i];
+                const float h = entity_distance(e, N, ent_mu, ent_cov, ent_active, md, cd);
+                if (h >= 0.f && h <= h_max) {
+                    const int pos = atomicAdd(&s_cnt, 1);
+                    if (pos < CAPA) cand[pos] = ((uint64_t)__float_as_uint(h) << 32) | (uint32_t)e;   // H >= 0: bits order like H
+                }
+            }
+        };
+        for (int g0 = 0; g0 < n4; g0 += TA * 4) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int g = g0 + u * TA + tid;
+                v[u] = g < n4 ? __ldcs(row4 + g) : make_float4(-2.f, -2.f, -2.f, -2.f);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int e0 = 4 * (g0 + u * TA + tid);
+                const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (x[c] >= tau_f && e0 + c < N) pre[atomicAdd(&s_np, 1)] = e0 + c;
+            }
+            __syncthreads();
+            const int np = s_np;
+            if (np > CAPP - PER_PASS) {      // (uniform) at most PER_PASS more could come in the next pass
+                evaluate(np);
+                __syncthreads();
+                if (tid == 0) s_np = 0;
+                __syncthreads();
+            }
+        }
+        evaluate(s_np);
+        __syncthreads();
+        finish_matches(cand, s_cnt, d, N, max_m, match_cnt, match_idx, match_h, label, err);
+        __syncthreads();          // the next detection reuses the shared arrays
+    }
 }
 
-__global__ void assoc_parent_kernel(int32_t T, const int32_t *__restrict__ label,
-                                    const unsigned long long *__restrict__ win, int32_t *parent)
+// root[t]: its component's smallest node; win[r]: the heaviest entity of
+// component r as (w bits, ~index).  (Every union is done: the labels are only
+// read.)
+__global__ void assoc_winner_kernel(int32_t N, int32_t T, const float *__restrict__ ent_w,
+                                    const int32_t *__restrict__ label, int32_t *__restrict__ root,
+                                    unsigned long long *win)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
-    const unsigned long long k = win[label[t]];
-    parent[t] = k ? (int32_t)(0xffffffffu - (uint32_t)(k & 0xffffffffu)) : t;
+    int r = label[t];
+    for (int up = label[r]; up != r; up = label[r]) r = up;
+    root[t] = r;
+    if (t >= N) return;
+    const unsigned long long k = ((unsigned long long)__float_as_uint(fmaxf(ent_w[t], 0.f)) << 32) |
+                                 (unsigned long long)(0xffffffffu - (uint32_t)t);
+    atomicMax(&win[r], k);
+}
+
+// The winner each slot merges into, and the slot's place among its members.
+__global__ void assoc_parent_kernel(int32_t T, const int32_t *__restrict__ root,
+                                    const unsigned long long *__restrict__ win, int32_t *__restrict__ parent,
+                                    int32_t *__restrict__ mcnt, int32_t *__restrict__ pos)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= T) return;
+    const unsigned long long k = win[root[t]];
+    const int p = k ? (int)(0xffffffffu - (uint32_t)(k & 0xffffffffu)) : t;
+    parent[t] = p;
+    if (p != t) pos[t] = atomicAdd(&mcnt[p], 1);
+}
+
+// Each winner's stretch of the members' array (their order is free).
+__global__ void assoc_offset_kernel(int32_t T, const int32_t *__restrict__ mcnt, int32_t *__restrict__ off,
+                                    int32_t *bump)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < T && mcnt[t] > 0) off[t] = atomicAdd(bump, mcnt[t]);
+}
+
+__global__ void assoc_members_kernel(int32_t T, const int32_t *__restrict__ parent, const int32_t *__restrict__ off,
+                                     const int32_t *__restrict__ pos, int32_t *__restrict__ members)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= T) return;
+    const int p = parent[t];
+    if (p != t) members[off[p] + pos[t]] = t;
 }
 
 struct Slots {
@@ -248,109 +350,228 @@ struct Slots {
     const float *ent_mu, *ent_cov, *ent_feat, *ent_w, *det_mu, *det_cov, *det_feat;
     __device__ float mu(int t, int k) const { return t < N ? ent_mu[(int64_t)k * N + t] : det_mu[(int64_t)k * B + (t - N)]; }
     __device__ float cv(int t, int k) const { return t < N ? ent_cov[(int64_t)k * N + t] : det_cov[(int64_t)k * B + (t - N)]; }
-    __device__ float ft(int t, int k) const
+    __device__ const float *feat(int t) const
     {
-        return t < N ? ent_feat[(int64_t)t * F + k] : det_feat[(int64_t)(t - N) * F + k];
+        return t < N ? ent_feat + (int64_t)t * F : det_feat + (int64_t)(t - N) * F;
     }
     __device__ float w(int t) const { return t < N ? ent_w[t] : 1.f; }
 };
 
-// pass 1: w, w (mu - c_g), w f into the winner g (acc arrays zeroed)
-__global__ void assoc_sum1_kernel(Slots sl, const int32_t *__restrict__ parent, float *acc_w, float *acc_m,
-                                  float *acc_f)
-{
-    const int T = sl.N + sl.B;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)T * (4 + sl.F)) return;
-    const int t = (int)(i / (4 + sl.F)), k = (int)(i - (int64_t)t * (4 + sl.F));
-    const int g = parent[t];
-    const float w = sl.w(t);
-    if (k == 0) atomicAdd(&acc_w[g], w);
-    else if (k < 4) atomicAdd(&acc_m[(int64_t)(k - 1) * T + g], w * (sl.mu(t, k - 1) - sl.mu(g, k - 1)));
-    else atomicAdd(&acc_f[(int64_t)g * sl.F + (k - 4)], w * sl.ft(t, k - 4));
-}
+constexpr int FW = 8;              // slots (warps) per block of the fusion
+constexpr int BIG_MEMBERS = 64;    // a winner of more is fused by its whole block
+constexpr int FCHUNK = 512;        // features of a big winner at a time
 
-// finalise the means and features of the winners
-__global__ void assoc_fin1_kernel(Slots sl, const int32_t *__restrict__ parent, const float *__restrict__ acc_w,
-                                  const float *__restrict__ acc_m, const float *__restrict__ acc_f, float *out_w,
-                                  float *out_mu, float *out_feat)
+// out_w, out_mu, out_cov and out_feat of every slot: zeros for a merged one,
+// the slot's own values for a winner without members, sums over the members
+// (listed at members + off) otherwise.
+__global__ void __launch_bounds__(FW * 32)
+assoc_fuse_kernel(Slots sl, const int32_t *__restrict__ parent, const int32_t *__restrict__ mcnt,
+                  const int32_t *__restrict__ off, const int32_t *__restrict__ members, float *__restrict__ out_w,
+                  float *__restrict__ out_mu, float *__restrict__ out_cov, float *__restrict__ out_feat, int vec)
 {
-    const int T = sl.N + sl.B;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)T * (4 + sl.F)) return;
-    const int t = (int)(i / (4 + sl.F)), k = (int)(i - (int64_t)t * (4 + sl.F));
-    const bool own = parent[t] == t && acc_w[t] > 0.f;
-    if (k == 0) out_w[t] = own ? acc_w[t] : 0.f;
-    else if (k < 4) out_mu[(int64_t)(k - 1) * T + t] = own ? sl.mu(t, k - 1) + acc_m[(int64_t)(k - 1) * T + t] / acc_w[t] : 0.f;
-    else out_feat[(int64_t)t * sl.F + (k - 4)] = own ? acc_f[(int64_t)t * sl.F + (k - 4)] / acc_w[t] : 0.f;
-}
-
-// pass 2: w (S + (mu - mu_g)(mu - mu_g)') into the winner
-__global__ void assoc_sum2_kernel(Slots sl, const int32_t *__restrict__ parent, const float *__restrict__ out_mu,
-                                  float *acc_c)
-{
-    const int T = sl.N + sl.B;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const int g = parent[t];
-    const float w = sl.w(t);
-    float dm[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) dm[k] = sl.mu(t, k) - out_mu[(int64_t)k * T + g];
+    __shared__ float s_part[FW][FCHUNK];
+    __shared__ float s_sum[FW][4], s_cov[FW][6], s_mean[4];
+    const int T = sl.N + sl.B, F = sl.F;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
+    const int t0 = blockIdx.x * FW, t = t0 + warp;
+    const unsigned FULL = 0xffffffffu;
+    if (t < T) {
+        // (the slot's first features are in flight while the rest is looked up)
+        const float4 *ft4 = reinterpret_cast<const float4 *>(sl.feat(t));
+        const int nf4 = vec ? F / 4 : 0;
+        float4 pre[2];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) atomicAdd(&acc_c[(int64_t)k * T + g], w * (sl.cv(t, k) + dm[ia[k]] * dm[ib[k]]));
-}
-
-__global__ void assoc_fin2_kernel(int32_t T, const int32_t *__restrict__ parent, const float *__restrict__ acc_w,
-                                  const float *__restrict__ acc_c, float *out_cov)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)T * 6) return;
-    const int t = (int)(i / 6), k = (int)(i - (int64_t)t * 6);
-    const bool own = parent[t] == t && acc_w[t] > 0.f;
-    out_cov[(int64_t)k * T + t] = own ? acc_c[(int64_t)k * T + t] / acc_w[t] : 0.f;
+        for (int u = 0; u < 2; ++u)
+            pre[u] = lane + 32 * u < nf4 ? __ldg(ft4 + lane + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const int m = parent[t] == t ? mcnt[t] : -1;      // -1: merged away
+        float *of = out_feat + (int64_t)t * F;
+        if (m >= 0 && m <= BIG_MEMBERS) {
+            const int32_t *mem = members + (m > 0 ? off[t] : 0);
+            // weight, and mean relative to the winner's own (lanes 0-2)
+            float W = sl.w(t), dm = 0.f;
+            const float mt = lane < 3 ? sl.mu(t, lane) : 0.f;
+            for (int k = 0; k < m; ++k) {
+                const int s = mem[k];
+                const float w = sl.w(s);
+                W += w;
+                if (lane < 3) dm += w * (sl.mu(s, lane) - mt);
+            }
+            const bool own = W > 0.f;
+            const float mean = own ? mt + dm / W : 0.f;
+            if (lane == 0) out_w[t] = own ? W : 0.f;
+            if (lane < 3) out_mu[(int64_t)lane * T + t] = mean;
+            // covariance about the fused mean (lanes 0-5)
+            const int c = lane < 6 ? lane : 0, a = ia[c], b = ib[c];
+            const float ma = __shfl_sync(FULL, mean, a), mb = __shfl_sync(FULL, mean, b);
+            if (lane < 6) {
+                float acc = sl.w(t) * (sl.cv(t, c) + (sl.mu(t, a) - ma) * (sl.mu(t, b) - mb));
+                for (int k = 0; k < m; ++k) {
+                    const int s = mem[k];
+                    acc += sl.w(s) * (sl.cv(s, c) + (sl.mu(s, a) - ma) * (sl.mu(s, b) - mb));
+                }
+                out_cov[(int64_t)c * T + t] = own ? acc / W : 0.f;
+            }
+            // features
+            const float wt = sl.w(t);
+            if (vec) {
+                for (int j = lane; j < nf4; j += 32) {
+                    float4 x = j < 32 ? pre[0] : j < 64 ? pre[1] : __ldg(ft4 + j);
+                    x.x *= wt; x.y *= wt; x.z *= wt; x.w *= wt;
+                    for (int k = 0; k < m; ++k) {
+                        const int s = mem[k];
+                        const float w = sl.w(s);
+                        const float4 y = __ldg(reinterpret_cast<const float4 *>(sl.feat(s)) + j);
+                        x.x = fmaf(w, y.x, x.x); x.y = fmaf(w, y.y, x.y);
+                        x.z = fmaf(w, y.z, x.z); x.w = fmaf(w, y.w, x.w);
+                    }
+                    if (own) { x.x /= W; x.y /= W; x.z /= W; x.w /= W; }
+                    else x = make_float4(0.f, 0.f, 0.f, 0.f);
+                    reinterpret_cast<float4 *>(of)[j] = x;
+                }
+            } else {
+                const float *ft = sl.feat(t);
+                for (int j = lane; j < F; j += 32) {
+                    float x = wt * ft[j];
+                    for (int k = 0; k < m; ++k) {
+                        const int s = mem[k];
+                        x = fmaf(sl.w(s), sl.feat(s)[j], x);
+                    }
+                    of[j] = own ? x / W : 0.f;
+                }
+            }
+        } else if (m < 0) {
+            if (lane == 0) out_w[t] = 0.f;
+            if (lane < 3) out_mu[(int64_t)lane * T + t] = 0.f;
+            if (lane < 6) out_cov[(int64_t)lane * T + t] = 0.f;
+            if (vec) {
+                for (int j = lane; j < nf4; j += 32)
+                    reinterpret_cast<float4 *>(of)[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            } else {
+                for (int j = lane; j < F; j += 32) of[j] = 0.f;
+            }
+        }
+    }
+    // winners of many members: the block's warps take every FW-th of them
+    for (int q = 0; q < FW; ++q) {
+        const int g = t0 + q;
+        if (g >= T || parent[g] != g || mcnt[g] <= BIG_MEMBERS) continue;     // (uniform across the block)
+        const int m = mcnt[g];
+        const int32_t *mem = members + off[g];
+        float W = warp == 0 ? sl.w(g) : 0.f, dm = 0.f;
+        const float mt = lane < 3 ? sl.mu(g, lane) : 0.f;
+        for (int k = warp; k < m; k += FW) {
+            const int s = mem[k];
+            const float w = sl.w(s);
+            W += w;
+            if (lane < 3) dm += w * (sl.mu(s, lane) - mt);
+        }
+        if (lane < 3) s_sum[warp][lane] = dm;
+        if (lane == 3) s_sum[warp][3] = W;
+        __syncthreads();
+        if (warp == 0 && lane < 4) {
+            float x = 0.f;
+            for (int v = 0; v < FW; ++v) x += s_sum[v][lane];
+            s_mean[lane] = x;
+        }
+        __syncthreads();
+        W = s_mean[3];
+        const bool own = W > 0.f;
+        const int c = lane < 6 ? lane : 0, a = ia[c], b = ib[c];
+        const float ma = sl.mu(g, a) + s_mean[a] / W, mb = sl.mu(g, b) + s_mean[b] / W;
+        if (lane < 6) {
+            float acc = warp == 0 ? sl.w(g) * (sl.cv(g, c) + (sl.mu(g, a) - ma) * (sl.mu(g, b) - mb)) : 0.f;
+            for (int k = warp; k < m; k += FW) {
+                const int s = mem[k];
+                acc += sl.w(s) * (sl.cv(s, c) + (sl.mu(s, a) - ma) * (sl.mu(s, b) - mb));
+            }
+            s_cov[warp][c] = acc;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            if (lane == 0) out_w[g] = own ? W : 0.f;
+            if (lane < 3) out_mu[(int64_t)lane * T + g] = own ? mt + s_mean[lane] / W : 0.f;
+            if (lane < 6) {
+                float x = 0.f;
+                for (int v = 0; v < FW; ++v) x += s_cov[v][lane];
+                out_cov[(int64_t)lane * T + g] = own ? x / W : 0.f;
+            }
+        }
+        for (int f0 = 0; f0 < F; f0 += FCHUNK) {
+            const int fn = min(FCHUNK, F - f0);
+            float acc[FCHUNK / 32];
+#pragma unroll
+            for (int u = 0; u < FCHUNK / 32; ++u) {
+                const int j = lane + 32 * u;
+                acc[u] = warp == 0 && j < fn ? sl.w(g) * sl.feat(g)[f0 + j] : 0.f;
+            }
+            for (int k = warp; k < m; k += FW) {
+                const int s = mem[k];
+                const float w = sl.w(s);
+                const float *fs = sl.feat(s) + f0;
+#pragma unroll
+                for (int u = 0; u < FCHUNK / 32; ++u) {
+                    const int j = lane + 32 * u;
+                    if (j < fn) acc[u] = fmaf(w, __ldg(fs + j), acc[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < FCHUNK / 32; ++u) s_part[warp][lane + 32 * u] = acc[u];
+            __syncthreads();
+            for (int j = threadIdx.x; j < fn; j += FW * 32) {
+                float x = 0.f;
+                for (int v = 0; v < FW; ++v) x += s_part[v][j];
+                out_feat[(int64_t)g * F + f0 + j] = own ? x / W : 0.f;
+            }
+            __syncthreads();
+        }
+    }
 }
 
 }  // namespace
 
+cudaError_t launch_assoc_init(const AssocArgs &a, cudaStream_t s)
+{
+    const int32_t T = a.N + a.B;
+    assoc_init_kernel<<<(unsigned)((T + 255) / 256), 256, 0, s>>>(T, a.B, a.tau_f, a.label, a.win, a.mcnt, a.counters,
+                                                                   a.emit.tau_key, a.emit.cnt);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_assoc_match(const AssocArgs &a, cudaStream_t s)
+{
+    assoc_match_kernel<<<(unsigned)a.B, TA, 0, s>>>(a.emit, a.N, a.B, a.ent_mu, a.ent_cov, a.ent_active, a.det_mu,
+                                                    a.det_cov, a.h_max, a.max_m, a.match_cnt, a.match_idx, a.match_h,
+                                                    a.label, a.counters + 1, a.over, a.err);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_assoc(const AssocArgs &a, cudaStream_t s)
 {
-    const int32_t N = a.N, B = a.B, F = a.F, T = a.N + a.B;
-    if (B < 1 || N < 0 || F < 1 || a.max_m < 1 || (int64_t)B * a.max_m > 0x7fffffff) return cudaErrorInvalidValue;
+    const int32_t N = a.N, B = a.B, T = a.N + a.B;
+    if (B < 1 || N < 0 || a.F < 1 || a.max_m < 1 || (int64_t)B * a.max_m > 0x7fffffff) return cudaErrorInvalidValue;
     cudaError_t e;
-    assoc_search_kernel<<<B, TA, 0, s>>>(a.S, a.ld, N, B, a.ent_mu, a.ent_cov, a.ent_active, a.det_mu, a.det_cov,
-                                         a.tau_f, a.h_max, a.max_m, a.match_cnt, a.match_idx, a.match_h, a.err);
+    // the stored rows: all of them, or those the emitted lists overflowed for
+    const int32_t *over = a.emit.cnt ? a.over : nullptr;
+    const unsigned grid = over ? (unsigned)(B < 304 ? B : 304) : (unsigned)B;
+    assoc_search_kernel<<<grid, TA, 0, s>>>(a.S, a.ld, N, B, a.ent_mu, a.ent_cov, a.ent_active, a.det_mu, a.det_cov,
+                                            a.tau_f, a.h_max, a.max_m, a.match_cnt, a.match_idx, a.match_h, a.label,
+                                            a.counters + 1, over, a.err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // the labels in shared memory when they fit (up to 200 KB: 51,200 nodes)
-    const size_t lab_bytes = (size_t)T * sizeof(int32_t);
-    const int32_t in_smem = lab_bytes <= 200 * 1024 ? 1 : 0;
-    if (in_smem && lab_bytes > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(assoc_components_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  200 * 1024)) != cudaSuccess)
-        return e;
-    assoc_components_kernel<<<1, 1024, in_smem ? lab_bytes : 0, s>>>(N, B, a.max_m, a.match_idx, a.label, 256,
-                                                                     a.err, in_smem);
+    const unsigned nb = (unsigned)((T + 255) / 256);
+    assoc_winner_kernel<<<nb, 256, 0, s>>>(N, T, a.ent_w, a.label, a.members, a.win);    // (roots: before the members)
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a.win, 0, (size_t)T * sizeof(unsigned long long), s)) != cudaSuccess) return e;
-    if (N > 0) {
-        assoc_winner_kernel<<<(N + 255) / 256, 256, 0, s>>>(N, a.ent_w, a.label, a.win);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    assoc_parent_kernel<<<(T + 255) / 256, 256, 0, s>>>(T, a.label, a.win, a.parent);
+    assoc_parent_kernel<<<nb, 256, 0, s>>>(T, a.members, a.win, a.parent, a.mcnt, a.pos);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a.acc, 0, (size_t)T * (10 + F) * sizeof(float), s)) != cudaSuccess) return e;
-    float *acc_w = a.acc, *acc_m = a.acc + T, *acc_c = a.acc + 4 * (int64_t)T, *acc_f = a.acc + 10 * (int64_t)T;
-    const Slots sl{N, B, F, a.ent_mu, a.ent_cov, a.ent_feat, a.ent_w, a.det_mu, a.det_cov, a.det_feat};
-    const int64_t n1 = (int64_t)T * (4 + F);
-    assoc_sum1_kernel<<<(unsigned)((n1 + 255) / 256), 256, 0, s>>>(sl, a.parent, acc_w, acc_m, acc_f);
+    assoc_offset_kernel<<<nb, 256, 0, s>>>(T, a.mcnt, a.off, a.counters);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    assoc_fin1_kernel<<<(unsigned)((n1 + 255) / 256), 256, 0, s>>>(sl, a.parent, acc_w, acc_m, acc_f, a.out_w,
-                                                                   a.out_mu, a.out_feat);
+    assoc_members_kernel<<<nb, 256, 0, s>>>(T, a.parent, a.off, a.pos, a.members);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    assoc_sum2_kernel<<<(T + 255) / 256, 256, 0, s>>>(sl, a.parent, a.out_mu, acc_c);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    assoc_fin2_kernel<<<(unsigned)(((int64_t)T * 6 + 255) / 256), 256, 0, s>>>(T, a.parent, acc_w, acc_c, a.out_cov);
+    const Slots sl{N, B, a.F, a.ent_mu, a.ent_cov, a.ent_feat, a.ent_w, a.det_mu, a.det_cov, a.det_feat};
+    const uintptr_t al = (uintptr_t)a.ent_feat | (uintptr_t)a.det_feat | (uintptr_t)a.out_feat;
+    const int vec = a.F % 4 == 0 && (al & 15u) == 0 ? 1 : 0;
+    assoc_fuse_kernel<<<(unsigned)((T + FW - 1) / FW), FW * 32, 0, s>>>(sl, a.parent, a.mcnt, a.off, a.members, a.out_w,
+                                                                        a.out_mu, a.out_cov, a.out_feat, vec);
     return cudaGetLastError();
 }
 

@@ -353,7 +353,6 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
     // MMAs) run while the main accumulator is drained to S (EMIT: compared
     // with the rows' thresholds).
     constexpr bool FOLD = C::FOLD;
-    static_assert(!EMIT || GROUPED, "the fused selection runs grouped launches");
     constexpr uint32_t TMEM_ALLOC = 512;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -369,6 +368,7 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
     uint64_t *emit_slots = reinterpret_cast<uint64_t *>(reinterpret_cast<uint8_t *>(tile_scales) + C::SCALE_BYTES);
     uint64_t *corr_free = acc_empty + 1;      // FOLD: the correction columns are free (tile accumulators: one)
 
+    if (emit.gate && *emit.gate == 0) return;      // (every thread of the launch alike)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const int cluster_id = blockIdx.x / CM, n_clusters = gridDim.x / CM;
@@ -987,7 +987,8 @@ int32_t k_slices_of(int32_t dim_pad)
 template <int MODE>
 cudaError_t launch_tc(const void *q0, const void *q1, const void *d0, const void *d1, float *S, int64_t rows,
                       int64_t n, int32_t dim_pad, int64_t ld_s, const float *scale_q, const float *scale_d,
-                      float *tops, int num_sms, int32_t *err, cudaStream_t s)
+                      float *tops, int num_sms, int32_t *err, cudaStream_t s, const FuseEmit *emit = nullptr,
+                      const int32_t *gate = nullptr)
 {
     constexpr int BN_ = 256, CM_ = 2;
     static_assert(BN_ == 256 && CM_ == 2, "the tile count below is that of the pair variant");
@@ -1026,9 +1027,19 @@ cudaError_t launch_tc(const void *q0, const void *q1, const void *d0, const void
     single.col_mode = kColAll;
     single.col_stride = 0;
     single.n_store = (int32_t)n;
+    const int64_t tiles = sim_cluster_tiles(rows, n, kSimPairVariant);
+    if constexpr (MODE == kSimF16x3) {
+        if (emit) {
+            if (!emit->tau_key || !emit->cnt || !emit->cand || emit->cap < 1) return cudaErrorInvalidValue;
+            return launch_impl<MODE, BN_, CM_, false, true, true>(mq0, mq1, md0, md1, nullptr, 1, single, S, tops,
+                                                                  k_slices_of<MODE>(dim_pad), tiles, scale_q, num_sms,
+                                                                  err, s, *emit);
+        }
+    }
+    FuseEmit none{};
+    none.gate = gate;
     return launch_impl<MODE, BN_, CM_, false, true>(mq0, mq1, md0, md1, nullptr, 1, single, S, tops,
-                                              k_slices_of<MODE>(dim_pad), sim_cluster_tiles(rows, n, kSimPairVariant), scale_q,
-                                              num_sms, err, s);
+                                              k_slices_of<MODE>(dim_pad), tiles, scale_q, num_sms, err, s, none);
 }
 
 template <int MODE, int BN_, int CM_, bool PAIR = false>
@@ -1153,12 +1164,14 @@ cudaError_t launch_sim_tc_grouped(int mode, int variant, const void *q0, const v
 
 cudaError_t launch_sim_tc_f16x3(const uint16_t *q_hi, const uint16_t *q_lo, const uint16_t *d_hi,
                                 const uint16_t *d_lo, float *S, int64_t rows, int64_t n, int32_t dim_pad, int64_t ld_s,
-                                float *tops, int num_sms, int32_t *err, cudaStream_t s)
+                                float *tops, int num_sms, int32_t *err, cudaStream_t s, const FuseEmit *emit,
+                                const int32_t *gate)
 {
+    if (rows <= kSimFewRows && (emit || gate)) return cudaErrorInvalidValue;
     if (rows <= kSimFewRows)
         return launch_sim_few(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, tops, err, s);
     return launch_tc<kSimF16x3>(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, nullptr, nullptr, tops, num_sms,
-                                err, s);
+                                err, s, emit, gate);
 }
 
 cudaError_t launch_sim_tc_bf16(const uint16_t *q, const uint16_t *d, float *S, int64_t rows, int64_t n,
