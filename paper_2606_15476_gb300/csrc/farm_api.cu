@@ -25,12 +25,13 @@ struct farm_ctx {
     // host copies of the last batch's plan (for farm_candidates)
     std::vector<int32_t> h_perm;      // caller query -> planned query
     std::vector<int32_t> h_cplan;     // caller constraint -> planned constraint
-    // pinned staging for per-batch metadata
-    int32_t *h_stage = nullptr;
-    size_t h_stage_n = 0;
-    uint8_t *h_blob = nullptr;        // pinned staging of the batch's piece tables and tensor maps
-    size_t h_blob_n = 0;
-    cudaEvent_t stage_done = nullptr;
+    // pinned staging of a batch's metadata, piece tables and tensor maps, which
+    // travel to the device in one copy: two slots used in turn, so that the
+    // host fills one while the other's copy still waits behind a running batch
+    struct Stage { uint8_t *p = nullptr; size_t n = 0; cudaEvent_t done = nullptr; } stage[2];
+    int stage_at = 0;
+    int32_t *d_perm = nullptr;        // the batch's planned position of each caller query (device)
+    uint8_t *h_topk = nullptr;        // pinned, written by the TopK kernel itself: small host results and the error word
     // host embedding rows of farm_query_batch travel on their own stream into
     // one of two slots, so that a batch's copy overlaps the previous batch's
     // kernels: the copy waits until the batch before last is done with the
@@ -76,6 +77,8 @@ namespace {
 
 constexpr int kMaxScenes = 4096;
 constexpr size_t kSimCapBytes = size_t(4) << 30;   // similarity block per launch group
+constexpr size_t kTopkPinned = size_t(256) << 10;  // largest host result written to pinned memory by the TopK kernel
+constexpr size_t kDirectRows = size_t(4) << 20;    // largest host rows copied on an idle ctx stream itself
 
 farm_status fail(farm_ctx *ctx, farm_status st, const std::string &msg)
 {
@@ -366,11 +369,26 @@ float *raw_slot_ptr(farm_ctx *ctx, int slot)
 }
 
 // The host rows into d_raw on the copy stream once the slot is free again;
-// the ctx stream waits for the copy.
+// the ctx stream waits for the copy.  A few rows for an idle ctx stream (a
+// caller that waits for each result) are copied on that stream: there is no
+// batch to overlap, and no event to wait for.
 cudaError_t copy_host_rows(farm_ctx *ctx, int slot, float *d_raw, const float *tgt_emb, const float *c_emb,
                            int64_t n_q, int64_t n_c, int32_t dim)
 {
-    cudaError_t e = cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_slot_free[slot], 0);
+    cudaError_t e = cudaSuccess;
+    if ((size_t)(n_q + n_c) * dim * 4 <= kDirectRows) {
+        e = cudaStreamQuery(ctx->c.stream);
+        if (e == cudaSuccess) {
+            e = cudaMemcpyAsync(d_raw, tgt_emb, (size_t)n_q * dim * 4, cudaMemcpyHostToDevice, ctx->c.stream);
+            if (e == cudaSuccess && n_c > 0)
+                e = cudaMemcpyAsync(d_raw + (size_t)n_q * dim, c_emb, (size_t)n_c * dim * 4, cudaMemcpyHostToDevice,
+                                    ctx->c.stream);
+            return e;
+        }
+        if (e != cudaErrorNotReady) return e;
+        (void)cudaGetLastError();        // (busy: not an error)
+    }
+    e = cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_slot_free[slot], 0);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d_raw, tgt_emb, (size_t)n_q * dim * 4, cudaMemcpyHostToDevice, ctx->copy_stream);
     if (e == cudaSuccess && n_c > 0)
@@ -494,9 +512,11 @@ farm_status farm_destroy(farm_ctx *ctx)
     cudaFree(c.mlp.w2b);
     cudaFree(c.mlp.w2t);
     if (c.h_err) cudaFreeHost(c.h_err);
-    if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
-    if (ctx->h_blob) cudaFreeHost(ctx->h_blob);
-    if (ctx->stage_done) cudaEventDestroy(ctx->stage_done);
+    for (auto &st : ctx->stage) {
+        if (st.p) cudaFreeHost(st.p);
+        if (st.done) cudaEventDestroy(st.done);
+    }
+    if (ctx->h_topk) cudaFreeHost(ctx->h_topk);
     if (ctx->copy_stream) {
         cudaStreamSynchronize(ctx->copy_stream);
         cudaStreamDestroy(ctx->copy_stream);
@@ -547,7 +567,8 @@ farm_status farm_create(farm_ctx **out, int device, void *cuda_stream, const far
     if (cudaHostAlloc(&c.h_err, sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) return bail(FARM_ENOMEM);
     if (cudaMalloc(&ctx->d_scenes, kMaxScenes * sizeof(SceneDev)) != cudaSuccess) return bail(FARM_ENOMEM);
     if (cudaMemset(ctx->d_scenes, 0, kMaxScenes * sizeof(SceneDev)) != cudaSuccess) return bail(FARM_ECUDA);
-    if (cudaEventCreateWithFlags(&ctx->stage_done, cudaEventDisableTiming) != cudaSuccess) return bail(FARM_ECUDA);
+    for (auto &st : ctx->stage)
+        if (cudaEventCreateWithFlags(&st.done, cudaEventDisableTiming) != cudaSuccess) return bail(FARM_ECUDA);
     if (cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess) return bail(FARM_ECUDA);
     for (int k = 0; k < 2; ++k)
         if (cudaEventCreateWithFlags(&ctx->ev_copied[k], cudaEventDisableTiming) != cudaSuccess ||
@@ -589,33 +610,54 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
     }
     CK(cudaSetDevice(c.device));
     Scene &s = c.scenes[scene_id];
-    if (s.present) {
+    Scene ns;
+    // a scene of the same shape is replaced in place: the copies and kernels
+    // below follow the queued work that reads it on the same stream
+    const bool reuse = s.present && s.n == n && s.dim == dim && s.n_views == n_views;
+    if (reuse) {
+        bool spaces = false;
+        for (const auto &sp : s.spaces) spaces |= sp.hi != nullptr;
+        if (spaces) {
+            CK(cudaStreamSynchronize(c.stream));
+            for (auto &sp : s.spaces) {
+                cudaFree(sp.hi);
+                cudaFree(sp.lo);
+                sp = farm::SpaceDesc{};
+            }
+        }
+        ns = s;
+        ns.present = false;
+        ns.comp_version = 0;              // (its learned embeddings are stale; weight versions start at 1)
+        s = Scene{};                      // (a failure below leaves the id without a scene)
+    } else if (s.present) {
         CK(cudaStreamSynchronize(c.stream));
         free_scene(s);
     }
-    Scene ns;
     ns.n = n;
     ns.dim = dim;
     ns.dim_pad = (int32_t)round_up(dim, farm::kDimAlign);
     ns.n_views = n_views;
     const size_t nd = (size_t)n * ns.dim_pad;
     auto bailmem = [&](cudaError_t e) {
+        if (reuse) cudaStreamSynchronize(c.stream);      // (queued work may still read it)
         free_scene(ns);
         return fail(ctx, e == cudaErrorMemoryAllocation ? FARM_ENOMEM : FARM_ECUDA,
                     std::string("scene upload: ") + cudaGetErrorString(e));
     };
     cudaError_t e;
-    if ((e = cudaMalloc(&ns.desc32, nd * 4)) != cudaSuccess) return bailmem(e);
-    if ((e = cudaMalloc(&ns.desc_hi, nd * 2)) != cudaSuccess) return bailmem(e);
-    if ((e = cudaMalloc(&ns.desc_lo, nd * 2)) != cudaSuccess) return bailmem(e);
-    if ((e = cudaMalloc(&ns.desc_bf16, nd * 2)) != cudaSuccess) return bailmem(e);
-    if ((e = cudaMalloc(&ns.desc_fp8, nd)) != cudaSuccess) return bailmem(e);
-    if ((e = cudaMalloc(&ns.desc_scale, (size_t)n * 4)) != cudaSuccess) return bailmem(e);
-    if ((e = cudaMalloc(&ns.cls, (size_t)n * 4)) != cudaSuccess) return bailmem(e);
-    if ((e = cudaMalloc(&ns.pos, (size_t)n * 12)) != cudaSuccess) return bailmem(e);
-    if ((e = cudaMalloc(&ns.size, (size_t)n * 12)) != cudaSuccess) return bailmem(e);
-    if ((e = cudaMalloc(&ns.views, (size_t)n * std::max(n_views, 1) * farm::kViewStride * 4)) != cudaSuccess)
-        return bailmem(e);
+    if (!reuse) {
+        if ((e = cudaMalloc(&ns.desc32, nd * 4)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMalloc(&ns.desc_hi, nd * 2)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMalloc(&ns.desc_lo, nd * 2)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMalloc(&ns.desc_bf16, nd * 2)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMalloc(&ns.desc_fp8, nd)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMalloc(&ns.desc_scale, (size_t)n * 4)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMalloc(&ns.cls, (size_t)n * 4)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMalloc(&ns.pos, (size_t)n * 12)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMalloc(&ns.size, (size_t)n * 12)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMalloc(&ns.views, (size_t)n * std::max(n_views, 1) * farm::kViewStride * 4)) != cudaSuccess)
+            return bailmem(e);
+    }
     const cudaMemcpyKind kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const float *d_desc = desc;
     float *tmp_desc = nullptr, *tmp_views = nullptr;
@@ -829,16 +871,27 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
             break;
         }
     // staging layout (int32): rowmap[n_q + n_c] | perm[n_q] | qmeta[n_q * 8]
-    const size_t need = (size_t)(n_q + n_c) + (size_t)n_q + (size_t)n_q * 8;
-    CK(cudaEventSynchronize(ctx->stage_done));
-    if (ctx->h_stage_n < need) {
-        if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
-        ctx->h_stage = nullptr;
-        ctx->h_stage_n = 0;
-        CK(cudaHostAlloc(&ctx->h_stage, need * sizeof(int32_t) * 5 / 4, cudaHostAllocDefault));
-        ctx->h_stage_n = need * 5 / 4;
-    }
-    int32_t *h_rowmap = ctx->h_stage;
+    // (then, at meta_bytes, the blob of piece tables and tensor maps below)
+    const size_t meta_bytes =
+        (size_t)round_up((int64_t)((size_t)(n_q + n_c) + (size_t)n_q + (size_t)n_q * 8) * 4, 128);
+    ctx->stage_at ^= 1;
+    farm_ctx::Stage &stage = ctx->stage[ctx->stage_at];
+    CK(cudaEventSynchronize(stage.done));
+    // room for `bytes`, the first `keep` of them as they are
+    auto stage_room = [&](size_t bytes, size_t keep) -> cudaError_t {
+        if (stage.n >= bytes) return cudaSuccess;
+        uint8_t *p = nullptr;
+        const size_t grow = bytes * 5 / 4 + 4096;
+        const cudaError_t e = cudaHostAlloc(&p, grow, cudaHostAllocDefault);
+        if (e != cudaSuccess) return e;
+        if (keep) std::memcpy(p, stage.p, keep);
+        if (stage.p) cudaFreeHost(stage.p);
+        stage.p = p;
+        stage.n = grow;
+        return cudaSuccess;
+    };
+    CK(stage_room(meta_bytes + 4096, 0));
+    int32_t *h_rowmap = reinterpret_cast<int32_t *>(stage.p);
     int32_t *h_perm = h_rowmap + (n_q + n_c);
     int32_t *h_meta = h_perm + n_q;
     ctx->h_perm.assign((size_t)n_q, 0);
@@ -877,11 +930,8 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
     }
 
     // ---- device buffers
-    int32_t *d_rowmap, *d_perm, *d_meta, *tsel_idx, *lsel_idx, *o_idx, *o_anc;
+    int32_t *tsel_idx, *lsel_idx, *o_idx, *o_anc;
     float *tsel_cos, *o_score, *o_t, *d_raw = nullptr;
-    CK(ws_get(ctx, farm::B_ROWMAP, (size_t)(n_q + n_c), &d_rowmap));
-    CK(ws_get(ctx, farm::B_PERM, (size_t)n_q, &d_perm));
-    CK(ws_get(ctx, farm::B_QMETA, (size_t)n_q * 8, &d_meta));
     CK(ws_get(ctx, farm::B_TSEL_IDX, (size_t)n_q * stride_t, &tsel_idx));
     CK(ws_get(ctx, farm::B_TSEL_COS, (size_t)n_q * stride_t, &tsel_cos));
     CK(ws_get(ctx, farm::B_LSEL_IDX, (size_t)std::max<int64_t>(n_c, 1) * stride_l, &lsel_idx));
@@ -1215,24 +1265,21 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
     const int n_tables = fused || any_exact ? 2 : 1;
     const size_t off_maps = off_gp + nv * n_tables * gp_table;
     const size_t blob_bytes = off_maps + map_scenes.size() * nv * 2 * farm::kTensorMapBytes;
-    uint8_t *d_blob;
-    CK(ws_get(ctx, farm::B_PIECES, blob_bytes, &d_blob));
-    if (ctx->h_blob_n < blob_bytes) {
-        if (ctx->h_blob) cudaFreeHost(ctx->h_blob);
-        ctx->h_blob = nullptr;
-        ctx->h_blob_n = 0;
-        CK(cudaHostAlloc(&ctx->h_blob, blob_bytes * 5 / 4 + 256, cudaHostAllocDefault));
-        ctx->h_blob_n = blob_bytes * 5 / 4 + 256;
-    }
+    uint8_t *d_stage;
+    CK(ws_get(ctx, farm::B_PIECES, meta_bytes + blob_bytes, &d_stage));
+    CK(stage_room(meta_bytes + blob_bytes, meta_bytes));
+    int32_t *d_rowmap = reinterpret_cast<int32_t *>(d_stage);
+    int32_t *d_perm = d_rowmap + (n_q + n_c), *d_meta = d_perm + n_q;
+    uint8_t *d_blob = d_stage + meta_bytes, *h_blob = stage.p + meta_bytes;
     farm::Piece *d_pieces = reinterpret_cast<farm::Piece *>(d_blob);
-    std::memcpy(ctx->h_blob, pieces.data(), pieces.size() * sizeof(farm::Piece));
+    std::memcpy(h_blob, pieces.data(), pieces.size() * sizeof(farm::Piece));
     // tiles of batch b, variant vi, table t at batch_tiles[(b * nv + vi) * n_tables + t]
     std::vector<int64_t> batch_tiles(batches.size() * nv * n_tables, 0);
     auto gp_base = [&](int vi, int t) { return off_gp + (size_t)(vi * n_tables + t) * gp_table; };
     if (sim_mode >= 0) {
         for (int vi = 0; vi < nv; ++vi) {
             for (int t = 0; t < n_tables; ++t) {
-                farm::GemmPiece *hg = reinterpret_cast<farm::GemmPiece *>(ctx->h_blob + gp_base(vi, t));
+                farm::GemmPiece *hg = reinterpret_cast<farm::GemmPiece *>(h_blob + gp_base(vi, t));
                 for (size_t b = 0; b < batches.size(); ++b) {
                     int64_t tiles = 0;
                     for (size_t k = batches[b].p0; k < batches[b].p0 + batches[b].np; ++k) {
@@ -1273,7 +1320,7 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
         for (size_t m = 0; m < map_scenes.size(); ++m) {
             const Scene &sc = c.scenes[map_scenes[m]];
             for (int vi = 0; vi < nv; ++vi) {
-                void *out = ctx->h_blob + off_maps + (m * nv + vi) * 2 * farm::kTensorMapBytes;
+                void *out = h_blob + off_maps + (m * nv + vi) * 2 * farm::kTensorMapBytes;
                 bool ok;
                 if (precision == FARM_PREC_FP32 || (reduced && exact_scene(sc)))
                     ok = farm::sim_tc_encode_b(farm::kSimF16x3, vlist[vi], out, sc.desc_hi, sc.desc_lo, sc.n,
@@ -1295,17 +1342,15 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
     // staged into library buffers first.
     const float *src_t = dev ? tgt_emb : d_raw;
     const float *src_c = dev ? c_emb : d_raw + (size_t)n_q * dim;
-    // Staging copies, always issued directly on the stream (never inside a
-    // graph): the host refills the pinned buffers for its next batch once the
-    // stage_done event after them has completed.  (Stage marks are taken for
+    // The staging copy, always issued directly on the stream (never inside a
+    // graph): the host refills the slot for the batch after next once the
+    // event behind the copy has completed.  (Stage marks are taken for
     // batches run directly only.)
     const int m0 = graph ? -1 : mark_begin(ctx, 0);
-    CK(cudaMemcpyAsync(d_rowmap, h_rowmap, (size_t)(n_q + n_c) * 4, cudaMemcpyHostToDevice, c.stream));
-    CK(cudaMemcpyAsync(d_perm, h_perm, (size_t)n_q * 4, cudaMemcpyHostToDevice, c.stream));
-    CK(cudaMemcpyAsync(d_meta, h_meta, (size_t)n_q * 8 * 4, cudaMemcpyHostToDevice, c.stream));
-    CK(cudaMemcpyAsync(d_blob, ctx->h_blob, blob_bytes, cudaMemcpyHostToDevice, c.stream));
-    CK(cudaEventRecord(ctx->stage_done, c.stream));
     if (!dev) CK(copy_host_rows(ctx, raw_slot, d_raw, tgt_emb, c_emb, n_q, n_c, dim));
+    CK(cudaMemcpyAsync(d_stage, stage.p, meta_bytes + blob_bytes, cudaMemcpyHostToDevice, c.stream));
+    CK(cudaEventRecord(stage.done, c.stream));
+    ctx->d_perm = d_perm;
     auto enqueue = [&]() -> farm_status {
         // ---- stage 0: normalisation (the staging copies above are not part of it)
         // (with FP32-accurate scenes in a reduced-precision batch, their rows
@@ -1733,6 +1778,7 @@ farm_status farm_query_batch_rrf(farm_ctx *ctx, int32_t scene_id, int64_t n_q, i
     CK(ws_get(ctx, farm::B_MC_FUSED, (size_t)(n_q * RF), &d_fused));
     CK(ws_get(ctx, farm::B_QMETA, (size_t)n_q * 8, &d_meta));
     CK(ws_get(ctx, farm::B_PERM, (size_t)n_q, &d_perm));
+    ctx->d_perm = d_perm;
     CK(ws_get(ctx, farm::B_TSEL_IDX, (size_t)n_q * RF, &tsel_idx));
     CK(ws_get(ctx, farm::B_LSEL_IDX, (size_t)std::max<int64_t>(n_c, 1) * Ka, &lsel_idx));
     CK(ws_get(ctx, farm::B_OUT_IDX, (size_t)n_q * RF, &o_idx));
@@ -1915,7 +1961,7 @@ farm_status farm_topk(farm_ctx *ctx, uint64_t batch_handle, int32_t k, int32_t *
     CK(cudaSetDevice(c.device));
     const bool dev = (flags & FARM_PTR_DEVICE) != 0;
     const int64_t n_q = c.batch_nq;
-    int32_t *d_perm = static_cast<int32_t *>(c.ws.ptr[farm::B_PERM]);
+    const int32_t *d_perm = ctx->d_perm;
     const int32_t *i_idx = static_cast<int32_t *>(c.ws.ptr[farm::B_OUT_IDX]);
     const float *i_score = static_cast<float *>(c.ws.ptr[farm::B_OUT_SCORE]);
     const float *i_t = static_cast<float *>(c.ws.ptr[farm::B_OUT_T]);
@@ -1924,6 +1970,26 @@ farm_status farm_topk(farm_ctx *ctx, uint64_t batch_handle, int32_t k, int32_t *
         LAUNCH(farm::launch_gather_topk(n_q, k, c.batch_rtgt, d_perm, i_idx, i_score, i_t, i_anc, out_idx,
                                         out_score, out_pred, out_anchor, c.stream));
         return FARM_OK;
+    }
+    // a small result that the call waits for: the kernel writes it and the error
+    // word to pinned memory, without a copy of each array
+    const size_t entries = (size_t)n_q * k;
+    if (!(flags & FARM_ASYNC) && entries * 40 <= kTopkPinned) {
+        if (!ctx->h_topk) CK(cudaHostAlloc(&ctx->h_topk, kTopkPinned + 64, cudaHostAllocDefault));
+        int32_t *p_idx = reinterpret_cast<int32_t *>(ctx->h_topk);
+        float *p_score = reinterpret_cast<float *>(p_idx + entries);
+        float *p_t = reinterpret_cast<float *>(p_idx + entries * 2);
+        int32_t *p_anc = p_idx + entries * 6;
+        volatile int32_t *p_err = reinterpret_cast<int32_t *>(ctx->h_topk + kTopkPinned);
+        LAUNCH(farm::launch_gather_topk(n_q, k, c.batch_rtgt, d_perm, i_idx, i_score, i_t, i_anc, p_idx, p_score,
+                                        out_pred ? p_t : nullptr, out_anchor ? p_anc : nullptr, c.stream, c.d_err,
+                                        reinterpret_cast<int32_t *>(ctx->h_topk + kTopkPinned)));
+        CK(cudaStreamSynchronize(c.stream));
+        std::memcpy(out_idx, p_idx, entries * 4);
+        std::memcpy(out_score, p_score, entries * 4);
+        if (out_pred) std::memcpy(out_pred, p_t, entries * 16);
+        if (out_anchor) std::memcpy(out_anchor, p_anc, entries * 16);
+        return *p_err ? check_device_errors(ctx) : FARM_OK;
     }
     // device staging: idx | score | t[4] | anchor[4] per entry
     int32_t *s_idx;

@@ -74,12 +74,11 @@ enum Buf {
     B_QLO,          // FP16 scaled residual
     B_QBF,          // BF16 rows
     B_SIM,          // similarity block [rows_chunk, n]
-    B_ROWMAP,       // int32 [n_q + n_c] planned row of each source row
-    B_PERM,         // int32 [n_q] planned position of each caller query
+    B_PERM,         // int32 [n_q] planned position of each caller query (batches of several channels)
     B_TSEL_IDX,     // int32 [n_q, r_tgt] target candidates
     B_TSEL_COS,     // float [n_q, r_tgt]
     B_LSEL_IDX,     // int32 [n_c, k_lm] landmark candidates
-    B_QMETA,        // int32 [n_q, 8] per-query metadata
+    B_QMETA,        // int32 [n_q, 8] per-query metadata (batches of several channels)
     B_OUT_IDX,      // int32 [n_q, r_tgt] composed candidates, best first
     B_OUT_SCORE,    // float [n_q, r_tgt]
     B_OUT_T,        // float [n_q, r_tgt, 4]
@@ -95,7 +94,7 @@ enum Buf {
     B_MLP_H,        // float [chunk, H] pre-activations (inference)
     B_MLP_AB,       // bf16 [chunk, H]
     B_MLP_Z,        // float [chunk, P]
-    B_PIECES,       // Piece tables of the batch's grouped launches
+    B_PIECES,       // the batch's plan: row map, query positions and metadata, piece tables, tensor maps
     B_CHUNK_IDX,    // int32 chunk lists of long rows (select, then merge)
     B_CHUNK_VAL,    // float their values
     B_TOPS,         // float per-row group maxima of the tensor-core similarity (thresholded select)
@@ -113,6 +112,8 @@ enum Buf {
     B_FUSE_CAND,    // uint64 [rows, cap] its candidate words
     B_FUSE_OVF,     // int32 [2 + 2 rows] overflow count, long-row count, overflowed launch rows, long launch rows
     B_FUSE_SLAB,    // float [blocks, n] the exact fallback's similarity rows
+    B_TRAIN,        // farm_mlp_train's activations, gradients and moments
+    B_TRAIN_IN,     // its inputs
     B_RESCORE,      // int32 the rescore's processing order (bucket counts, places, order)
     B_RAW_PIPE,     // farm_query_batch's host rows: two slots, each [n_q + n_c, dim] (copy stream)
     B_COUNT
@@ -185,20 +186,30 @@ struct MlpShape {
     int32_t D, H, P, D_pad;
     uint16_t *w1b, *w2b, *w2t;
 };
+// A training call's pairs on the device: the scenes' BF16 rows and, last, the
+// training rows' (base, n_scenes + 1 tables); each pair's row, object and scene
+// (scene null: the one scene; row null: the rows are already gathered), target
+// and weight (w null: 1); the epoch's order of the pairs.
+struct TrainPairs {
+    const uint16_t *const *base;
+    int32_t n_scenes;
+    const int32_t *row, *obj, *scene;
+    const float *y, *w;
+    const int32_t *perm;
+};
 // The training step's kernels (k_mlp.cu): its stacked rows and their transpose,
 // clearing the bias-gradient sums gb1 [H], gb2 [P]; GELU's BF16 output and
 // transpose (aT nullable); the pairs' loss and the gradient down to the second
 // contraction's output; GELU's backward.  K: the padded length of the
 // transposed operands (a multiple of 64, zero from the last row on).
-cudaError_t mlp_train_rows(const uint16_t *const *base, int32_t n_scenes, const int32_t *idx, int64_t n_pairs, int64_t b,
-                           int D, int D_pad, uint16_t *x, uint16_t *xT, int64_t K, float *gb1, int H, float *gb2, int P,
-                           cudaStream_t s);
+cudaError_t mlp_train_rows(const TrainPairs &pairs, int64_t off, int64_t b, int D, int D_pad, uint16_t *x, uint16_t *xT,
+                           int64_t K, float *gb1, int H, float *gb2, int P, cudaStream_t s);
 cudaError_t mlp_gelu_bf16(const float *h, const float *b, int64_t rows, int cols, uint16_t *ab, uint16_t *aT, int64_t K,
                           cudaStream_t s);
 cudaError_t mlp_gelu_backward_t(const float *h, const float *b, const float *da, int64_t rows, int cols, uint16_t *dhT,
                                 int64_t K, float *gb, cudaStream_t s);
-cudaError_t mlp_pair_step(const float *z, const float *b2, const float *y, const float *w, float wsum, int64_t b, int P,
-                          uint16_t *dzb, uint16_t *dzT, int64_t K, float *gb2, float *loss, cudaStream_t s);
+cudaError_t mlp_pair_step(const float *z, const float *b2, const TrainPairs &pairs, int64_t off, float wsum, int64_t b,
+                          int P, uint16_t *dzb, uint16_t *dzT, int64_t K, float *gb2, float *loss, cudaStream_t s);
 // e = bf16((z + b) / |z + b|) per row.
 cudaError_t mlp_normalize_bf16(const float *z, const float *b, int64_t rows, int cols, uint16_t *e, cudaStream_t s);
 // All BF16 copies of the parameters p (count of them).
@@ -709,11 +720,12 @@ cudaError_t launch_assoc_match(const AssocArgs &a, cudaStream_t s);
 cudaError_t launch_assoc(const AssocArgs &a, cudaStream_t s);
 
 // out[q * k + j] = src[perm[q] * ld + j] (and the 4-wide breakdown): the TopK
-// prefix of each query's sorted candidates, back in the caller's query order.
+// prefix of each query's sorted candidates, back in the caller's query order;
+// *o_err = *err when given.
 cudaError_t launch_gather_topk(int64_t n_q, int32_t k, int32_t ld, const int32_t *perm,
                                const int32_t *idx,
                                const float *score, const float *t, const int32_t *anchor,
                                int32_t *o_idx, float *o_score, float *o_t, int32_t *o_anchor,
-                               cudaStream_t s);
+                               cudaStream_t s, const int32_t *err = nullptr, int32_t *o_err = nullptr);
 
 }  // namespace farm

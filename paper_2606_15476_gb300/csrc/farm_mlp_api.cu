@@ -175,8 +175,14 @@ void gemm_shapes(const TcBufs &t, const Mlp &M, GemmShape (&g)[kGemmPieces])
     g[4] = {M.H, M.D, t.xT, (int32_t)t.K_pad, gW1, 3, 2};
 }
 
-cudaError_t tc_alloc(Ctx &c, TcBufs &t, int64_t B, int64_t loss_slots)
+// Buffers of a training call up to this size stay with the context for its next
+// one (allocating and freeing them takes longer than a few steps).
+constexpr int64_t kTrainKept = int64_t(512) << 20;
+
+// keep: the buffers may be the context's kept ones (t.base then stays null).
+cudaError_t tc_alloc(farm_ctx *ctx, TcBufs &t, int64_t B, int64_t loss_slots, bool keep)
 {
+    Ctx &c = *farm::ctx_of(ctx);
     const Mlp &M = c.mlp;
     const int64_t R = 2 * B, K = round64(2 * B), Dp = M.D_pad, H = M.H, P = M.P, cnt = M.count();
     t.B = B;
@@ -191,15 +197,21 @@ cudaError_t tc_alloc(Ctx &c, TcBufs &t, int64_t B, int64_t loss_slots)
     for (int64_t n : n16) total += al(n * 2);
     for (int64_t n : n32) total += al(n * 4);
     total += (int64_t)kBlobBytes;
-    cudaError_t e = cudaMalloc(&t.base, (size_t)total);
-    if (e != cudaSuccess) return e;
-    char *p = static_cast<char *>(t.base);
+    void *at = nullptr;
+    cudaError_t e;
+    if (keep && total <= kTrainKept) {
+        if ((e = farm::ws_alloc(ctx, farm::B_TRAIN, (size_t)total, &at)) != cudaSuccess) return e;
+    } else {
+        if ((e = cudaMalloc(&t.base, (size_t)total)) != cudaSuccess) return e;
+        at = t.base;
+    }
+    char *p = static_cast<char *>(at);
     for (size_t i = 0; i < sizeof(n16) / sizeof(n16[0]); ++i) { *d16[i] = reinterpret_cast<uint16_t *>(p); p += al(n16[i] * 2); }
     for (size_t i = 0; i < sizeof(n32) / sizeof(n32[0]); ++i) { *d32[i] = reinterpret_cast<float *>(p); p += al(n32[i] * 4); }
     t.blob = reinterpret_cast<uint8_t *>(p);
     // (rows past a partial batch hold the last batch's, or zeros: every
     // contraction over them is finite and read by nothing)
-    if ((e = cudaMemsetAsync(t.base, 0, (size_t)total, c.stream))) return e;
+    if ((e = cudaMemsetAsync(at, 0, (size_t)total, c.stream))) return e;
     GemmShape g[kGemmPieces];
     gemm_shapes(t, M, g);
     alignas(128) uint8_t host[kBlobBytes] = {};
@@ -242,14 +254,13 @@ cudaError_t tc_gemm(Ctx &c, const TcBufs &t, int which)
                                        dw ? t.grad : s.out, nullptr, nullptr, c.num_sms, c.d_err, c.stream);
 }
 
-// Loss and gradient of b pairs: their stacked BF16 input rows gathered by idx
-// (train_rows_kernel; base and the index arrays of the epoch, at the batch's
-// first pair), or already in t.x (idx null); targets / weights y, w (device, b
-// each; w null: 1), wsum their sum.  The loss is added to *lslot, the gradient
-// [W1 | b1 | W2 | b2] written to t.grad.
-cudaError_t tc_loss_grad(Ctx &c, TcBufs &t, int64_t b, const uint16_t *const *base, int32_t n_scenes,
-                         const int32_t *idx, int64_t n_pairs, const float *y, const float *w, float wsum, float *lslot,
-                         int64_t &launches)
+// Loss and gradient of b pairs, those at places off .. of the epoch's order
+// (pairs.perm; null: pairs off .. themselves): their stacked BF16 input rows
+// gathered, or already in t.x (pairs.row null); wsum the sum of their weights.
+// The loss is added to *lslot, the gradient [W1 | b1 | W2 | b2] written to
+// t.grad.
+cudaError_t tc_loss_grad(Ctx &c, TcBufs &t, int64_t b, const farm::TrainPairs &pairs, int64_t off, float wsum,
+                         float *lslot, int64_t &launches)
 {
     const Mlp &M = c.mlp;
     const int64_t R = 2 * b, K = t.K_pad, H = M.H, P = M.P, D = M.D;
@@ -257,15 +268,14 @@ cudaError_t tc_loss_grad(Ctx &c, TcBufs &t, int64_t b, const uint16_t *const *ba
     cudaStream_t st = c.stream;
     cudaError_t r;
     launches += 8;
-    if ((r = farm::mlp_train_rows(base, n_scenes, idx, n_pairs, b, (int)D, M.D_pad, t.x, t.xT, K, gb1, (int)H, gb2,
-                                  (int)P, st)))
+    if ((r = farm::mlp_train_rows(pairs, off, b, (int)D, M.D_pad, t.x, t.xT, K, gb1, (int)H, gb2, (int)P, st)))
         return r;
     // forward: h = x W1^T, a = gelu(h + b1), z = a W2^T
     if ((r = tc_gemm(c, t, G_H))) return r;
     if ((r = farm::mlp_gelu_bf16(t.h, M.b1(), R, (int)H, t.ab, t.aT, K, st))) return r;
     if ((r = tc_gemm(c, t, G_Z))) return r;
     // e = (z + b2) / |z + b2|, the loss, dz and its column sums
-    if ((r = farm::mlp_pair_step(t.z, M.b2(), y, w, wsum, b, (int)P, t.dzb, t.dT, K, gb2, lslot, st))) return r;
+    if ((r = farm::mlp_pair_step(t.z, M.b2(), pairs, off, wsum, b, (int)P, t.dzb, t.dT, K, gb2, lslot, st))) return r;
     // backward: da = dz W2, dh = gelu'(h + b1) da, then dW2 = dz^T a and dW1 = dh^T x together
     if ((r = tc_gemm(c, t, G_DA))) return r;
     if ((r = farm::mlp_gelu_backward_t(t.h, M.b1(), t.da, R, (int)H, t.dT + P * K, K, gb1, st))) return r;
@@ -350,13 +360,17 @@ farm_status farm_mlp_set(farm_ctx *ctx, int32_t dim, int32_t hidden, int32_t out
     nm.D = dim; nm.H = hidden; nm.P = out_dim;
     nm.D_pad = (dim + farm::kDimAlign - 1) / farm::kDimAlign * farm::kDimAlign;
     const int64_t cnt = nm.count();
-    std::vector<float> host((size_t)cnt);
-    std::memcpy(host.data(), W1, (size_t)nm.H * nm.D * 4);
-    std::memcpy(host.data() + (size_t)nm.H * nm.D, b1, (size_t)nm.H * 4);
-    std::memcpy(host.data() + (size_t)nm.H * nm.D + nm.H, W2, (size_t)nm.P * nm.H * 4);
-    std::memcpy(host.data() + (size_t)nm.H * nm.D + nm.H + (size_t)nm.P * nm.H, b2, (size_t)nm.P * 4);
-    for (float x : host)
-        if (!std::isfinite(x)) return fail(c, FARM_EINVAL, "farm_mlp_set: non-finite weight");
+    const float *part[4] = {W1, b1, W2, b2};
+    const size_t len[4] = {(size_t)nm.H * nm.D, (size_t)nm.H, (size_t)nm.P * nm.H, (size_t)nm.P};
+    for (int k = 0; k < 4; ++k) {
+        uint32_t bad = 0;                 // (branch-free: the loop vectorises)
+        for (size_t i = 0; i < len[k]; ++i) {
+            uint32_t u;
+            std::memcpy(&u, part[k] + i, 4);
+            bad |= (u & 0x7f800000u) == 0x7f800000u ? 1u : 0u;
+        }
+        if (bad) return fail(c, FARM_EINVAL, "farm_mlp_set: non-finite weight");
+    }
     MCK(cudaStreamSynchronize(c.stream));
     if (M.set && (M.D != nm.D || M.H != nm.H || M.P != nm.P)) {
         cudaFree(M.params); cudaFree(M.w1b); cudaFree(M.w2b); cudaFree(M.w2t);
@@ -373,10 +387,14 @@ farm_status farm_mlp_set(farm_ctx *ctx, int32_t dim, int32_t hidden, int32_t out
         for (auto &s : c.scenes)
             if (s.comp) { cudaFree(s.comp); s.comp = nullptr; }
     }
-    MCK(cudaMemcpyAsync(M.params, host.data(), (size_t)cnt * 4, cudaMemcpyHostToDevice, c.stream));
+    float *to = M.params;
+    for (int k = 0; k < 4; ++k) {
+        MCK(cudaMemcpyAsync(to, part[k], len[k] * 4, cudaMemcpyHostToDevice, c.stream));
+        to += len[k];
+    }
     M.set = true;
     MCK(refresh_bf16_weights(c));
-    // the host copy above must have been read before `host` goes away
+    // the caller's arrays must have been read before the call returns
     MCK(cudaStreamSynchronize(c.stream));
     return FARM_OK;
 }
@@ -419,7 +437,7 @@ farm_status farm_mlp_loss_grad(farm_ctx *ctx, int64_t n_pairs, const float *xq, 
         TcBufs t;
         float *raw = nullptr;
         auto done = [&](farm_status st) { cudaStreamSynchronize(c.stream); cudaFree(t.base); cudaFree(raw); return st; };
-        e = tc_alloc(c, t, n_pairs, 1);
+        e = tc_alloc(ctx, t, n_pairs, 1, false);
         if (e) return done(fail(c, e == cudaErrorMemoryAllocation ? FARM_ENOMEM : FARM_ECUDA,
                                 std::string("farm_mlp_loss_grad: ") + cudaGetErrorString(e)));
         if (!e) e = cudaMalloc(&raw, 2 * xb);
@@ -429,7 +447,9 @@ farm_status farm_mlp_loss_grad(farm_ctx *ctx, int64_t n_pairs, const float *xq, 
         if (!e && w) e = cudaMemcpyAsync(t.w, w, (size_t)n_pairs * 4, cudaMemcpyHostToDevice, c.stream);
         if (!e) e = cudaMemsetAsync(t.loss, 0, 4, c.stream);
         if (!e) e = farm::mlp_to_bf16_padded(raw, 2 * n_pairs, M.D, t.x, M.D_pad, c.stream);
-        if (!e) e = tc_loss_grad(c, t, n_pairs, nullptr, 0, nullptr, 0, t.y, w ? t.w : nullptr, (float)wsum, t.loss, L);
+        if (!e) e = tc_loss_grad(c, t, n_pairs,
+                                 farm::TrainPairs{nullptr, 0, nullptr, nullptr, nullptr, t.y, w ? t.w : nullptr, nullptr},
+                                 0, (float)wsum, t.loss, L);
         if (!e) e = cudaMemcpyAsync(loss, t.loss, 4, cudaMemcpyDeviceToHost, c.stream);
         if (!e && grad) e = cudaMemcpyAsync(grad, t.grad, (size_t)M.count() * 4, cudaMemcpyDeviceToHost, c.stream);
         if (!e) e = cudaStreamSynchronize(c.stream);
@@ -495,25 +515,47 @@ farm_status farm_mlp_train(farm_ctx *ctx, int32_t n_scenes, const int32_t *scene
     const int64_t B = std::min<int64_t>(batch, n_pairs);
     const int64_t steps = (n_pairs + B - 1) / B;
     TcBufs t;
-    uint16_t *qnb = nullptr;   // normalised training rows, BF16 [n_rows, D_pad]
-    float *raw = nullptr;
-    int32_t *d_idx = nullptr;  // per epoch: query rows [n_pairs] | object indices [n_pairs] | scenes [n_pairs]
-    float *d_yw = nullptr;     // per epoch: targets [n_pairs] | weights [n_pairs]
+    // the call's inputs: normalised rows (BF16 [n_rows, D_pad]), the rows as
+    // given, the pairs' arrays as given, an epoch's order, the row tables
+    uint16_t *qnb = nullptr;
+    float *raw = nullptr, *d_y = nullptr, *d_w = nullptr;
+    int32_t *d_row = nullptr, *d_obj = nullptr, *d_scene = nullptr, *d_perm = nullptr;
     const uint16_t **d_bases = nullptr;
+    void *in_base = nullptr;       // the inputs' memory when it is this call's own
     auto done = [&](farm_status st) {
         cudaStreamSynchronize(c.stream);
-        cudaFree(t.base); cudaFree(qnb); cudaFree(raw); cudaFree(d_idx); cudaFree(d_yw); cudaFree(d_bases);
+        cudaFree(t.base); cudaFree(in_base);
         return st;
     };
-    cudaError_t e = tc_alloc(c, t, B, steps * (int64_t)epochs);
+    cudaError_t e = tc_alloc(ctx, t, B, steps * (int64_t)epochs, true);
     if (e) return done(fail(c, e == cudaErrorMemoryAllocation ? FARM_ENOMEM : FARM_ECUDA,
                             std::string("farm_mlp_train: ") + cudaGetErrorString(e)));
-    if (!e) e = cudaMalloc(&qnb, (size_t)n_rows * M.D_pad * 2);
-    if (!e) e = cudaMalloc(&raw, (size_t)n_rows * M.D * 4);
-    if (!e) e = cudaMalloc(&d_idx, (size_t)n_pairs * 3 * 4);
-    if (!e) e = cudaMalloc(&d_yw, (size_t)n_pairs * 2 * 4);
+    {
+        const size_t sizes[] = {(size_t)n_rows * M.D_pad * 2, (size_t)n_rows * M.D * 4, (size_t)n_pairs * 4,
+                                (size_t)n_pairs * 4, (size_t)n_pairs * 4, (size_t)n_pairs * 4, (size_t)n_pairs * 4,
+                                (size_t)n_pairs * 4, bases.size() * sizeof(void *)};
+        void **to[] = {(void **)&qnb, (void **)&raw, (void **)&d_y, (void **)&d_w, (void **)&d_row, (void **)&d_obj,
+                       (void **)&d_scene, (void **)&d_perm, (void **)&d_bases};
+        size_t total = 0;
+        for (size_t b : sizes) total += (b + 255) & ~size_t(255);
+        void *at = nullptr;
+        if ((int64_t)total <= kTrainKept) e = farm::ws_alloc(ctx, farm::B_TRAIN_IN, total, &at);
+        else if (!(e = cudaMalloc(&in_base, total))) at = in_base;
+        if (e) return done(fail(c, e == cudaErrorMemoryAllocation ? FARM_ENOMEM : FARM_ECUDA,
+                                std::string("farm_mlp_train: ") + cudaGetErrorString(e)));
+        uint8_t *p = static_cast<uint8_t *>(at);
+        for (size_t k = 0; k < sizeof(sizes) / sizeof(sizes[0]); ++k) {
+            *to[k] = p;
+            p += (sizes[k] + 255) & ~size_t(255);
+        }
+        const cudaMemcpyKind h2d = cudaMemcpyHostToDevice;
+        if (!e) e = cudaMemcpyAsync(d_y, y, (size_t)n_pairs * 4, h2d, c.stream);
+        if (!e && w) e = cudaMemcpyAsync(d_w, w, (size_t)n_pairs * 4, h2d, c.stream);
+        if (!e) e = cudaMemcpyAsync(d_row, pair_row, (size_t)n_pairs * 4, h2d, c.stream);
+        if (!e) e = cudaMemcpyAsync(d_obj, pair_obj, (size_t)n_pairs * 4, h2d, c.stream);
+        if (!e && pair_scene) e = cudaMemcpyAsync(d_scene, pair_scene, (size_t)n_pairs * 4, h2d, c.stream);
+    }
     bases[n_scenes] = qnb;
-    if (!e) e = cudaMalloc(&d_bases, bases.size() * sizeof(void *));
     if (!e) e = cudaMemcpyAsync(d_bases, bases.data(), bases.size() * sizeof(void *), cudaMemcpyHostToDevice,
                                 c.stream);
     if (!e) e = cudaMemcpyAsync(raw, rows, (size_t)n_rows * M.D * 4, cudaMemcpyHostToDevice, c.stream);
@@ -521,9 +563,10 @@ farm_status farm_mlp_train(farm_ctx *ctx, int32_t n_scenes, const int32_t *scene
                                             c.d_err, farm::kErrBadRow, c.stream);
     // (the moments and the losses start at zero: tc_alloc clears them)
     if (e) return done(fail(c, FARM_ECUDA, std::string("farm_mlp_train: ") + cudaGetErrorString(e)));
-    std::vector<int32_t> perm((size_t)n_pairs), hidx((size_t)n_pairs * 3);
-    std::vector<float> hyw((size_t)n_pairs * 2);
+    std::vector<int32_t> perm((size_t)n_pairs);
     for (int64_t i = 0; i < n_pairs; ++i) perm[i] = (int32_t)i;
+    const farm::TrainPairs pairs{d_bases, n_scenes, d_row, d_obj, pair_scene ? d_scene : nullptr, d_y,
+                                 w ? d_w : nullptr, d_perm};
     uint64_t st = seed;
     int64_t L = 2;
     int t_adam = 0;
@@ -532,26 +575,21 @@ farm_status farm_mlp_train(farm_ctx *ctx, int32_t n_scenes, const int32_t *scene
             const int64_t j = (int64_t)(splitmix64(st) % (uint64_t)(i + 1));
             std::swap(perm[i], perm[j]);
         }
-        for (int64_t i = 0; i < n_pairs; ++i) {
-            hidx[i] = pair_row[perm[i]];
-            hidx[n_pairs + i] = pair_obj[perm[i]];
-            hidx[2 * n_pairs + i] = pair_scene ? pair_scene[perm[i]] : 0;
-            hyw[i] = y[perm[i]];
-            hyw[n_pairs + i] = w ? w[perm[i]] : 1.f;
-        }
-        // the previous epoch's kernels may still read the device copies
+        // the previous epoch's kernels may still read the device copy
         e = cudaStreamSynchronize(c.stream);
-        if (!e) e = cudaMemcpyAsync(d_idx, hidx.data(), hidx.size() * 4, cudaMemcpyHostToDevice, c.stream);
-        if (!e) e = cudaMemcpyAsync(d_yw, hyw.data(), hyw.size() * 4, cudaMemcpyHostToDevice, c.stream);
+        if (!e) e = cudaMemcpyAsync(d_perm, perm.data(), (size_t)n_pairs * 4, cudaMemcpyHostToDevice, c.stream);
         for (int64_t sidx = 0; sidx < steps && !e; ++sidx) {
             const int64_t off = sidx * B;
             const int64_t b = std::min(B, n_pairs - off);
             double wsum = 0.0;
-            for (int64_t i = 0; i < b; ++i) wsum += hyw[n_pairs + off + i];
+            if (w) {
+                for (int64_t i = 0; i < b; ++i) wsum += w[perm[off + i]];
+            } else {
+                wsum = (double)b;
+            }
             if (!(wsum > 0.0)) continue;
             float *lslot = t.loss + (int64_t)ep * steps + sidx;
-            e = tc_loss_grad(c, t, b, d_bases, n_scenes, d_idx + off, n_pairs, d_yw + off, d_yw + n_pairs + off,
-                             (float)wsum, lslot, L);
+            e = tc_loss_grad(c, t, b, pairs, off, (float)wsum, lslot, L);
             if (!e) e = farm::mlp_adam(M.params, t.grad, t.m, t.v, M.count(), lr, ++t_adam, shape_of(M), c.stream);
             M.version += 1;
             L += 1;

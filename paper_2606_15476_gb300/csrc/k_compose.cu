@@ -566,9 +566,11 @@ compose_kernel(ComposeArgs a, int32_t KC)
 __global__ void gather_topk_kernel(int64_t n_q, int32_t k, int32_t ld, const int32_t *__restrict__ perm,
                                    const int32_t *__restrict__ idx, const float *__restrict__ score,
                                    const float *__restrict__ t, const int32_t *__restrict__ anchor,
-                                   int32_t *o_idx, float *o_score, float *o_t, int32_t *o_anchor)
+                                   int32_t *o_idx, float *o_score, float *o_t, int32_t *o_anchor,
+                                   const int32_t *err, int32_t *o_err)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (o_err && i == 0) *o_err = *err;
     if (i >= n_q * k) return;
     const int64_t qo = i / k;              // output (caller's) query
     const int32_t j = (int32_t)(i - qo * k);
@@ -604,13 +606,13 @@ cudaError_t launch_compose(const ComposeArgs &a, cudaStream_t s)
 cudaError_t launch_gather_topk(int64_t n_q, int32_t k, int32_t ld, const int32_t *perm,
                                const int32_t *idx, const float *score, const float *t,
                                const int32_t *anchor, int32_t *o_idx, float *o_score, float *o_t,
-                               int32_t *o_anchor, cudaStream_t s)
+                               int32_t *o_anchor, cudaStream_t s, const int32_t *err, int32_t *o_err)
 {
     const int64_t total = n_q * k;
     if (total <= 0) return cudaSuccess;
     const int th = 256;
     gather_topk_kernel<<<(unsigned)((total + th - 1) / th), th, 0, s>>>(
-        n_q, k, ld, perm, idx, score, t, anchor, o_idx, o_score, o_t, o_anchor);
+        n_q, k, ld, perm, idx, score, t, anchor, o_idx, o_score, o_t, o_anchor, err, o_err);
     return cudaGetLastError();
 }
 

@@ -240,14 +240,13 @@ __device__ __forceinline__ void tile_write_t(const uint16_t (*tile)[TSTRIDE], in
 }
 
 // The step's stacked input rows (query rows 0 .. b - 1, descriptor rows b ..
-// 2b - 1; D_pad long) and their transpose [D, K].  idx non-null: gathered (row
-// r < b: base[n_scenes] row idx[r]; else base[scene] row idx[n_pairs + r - b],
-// scene idx[2 n_pairs + r - b]) and written to x; null: read from x.  The
-// block of the origin also clears the step's bias-gradient sums.
+// 2b - 1; D_pad long) and their transpose [D, K].  With pairs.row gathered
+// (pair k of the order: base[n_scenes] row row[k], and base[scene[k]] row
+// obj[k]) and written to x; without read from x.  The block of the origin also
+// clears the step's bias-gradient sums.
 __global__ void __launch_bounds__(256)
-train_rows_kernel(const uint16_t *const *__restrict__ base, int32_t n_scenes, const int32_t *__restrict__ idx,
-                  int64_t n_pairs, int64_t b, int D, int D_pad, uint16_t *__restrict__ x, uint16_t *__restrict__ xT,
-                  int64_t K, float *__restrict__ gb1, int H, float *__restrict__ gb2, int P)
+train_rows_kernel(TrainPairs pairs, int64_t off, int64_t b, int D, int D_pad, uint16_t *__restrict__ x,
+                  uint16_t *__restrict__ xT, int64_t K, float *__restrict__ gb1, int H, float *__restrict__ gb2, int P)
 {
     __shared__ __align__(4) uint16_t tile[TR][TSTRIDE];
     const int tid = threadIdx.x;
@@ -262,14 +261,15 @@ train_rows_kernel(const uint16_t *const *__restrict__ base, int32_t n_scenes, co
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
     if (r < 2 * b) {
         const uint16_t *src;
-        if (idx) {
-            src = r < b ? base[n_scenes] + (int64_t)idx[r] * D_pad
-                        : base[idx[2 * n_pairs + r - b]] + (int64_t)idx[n_pairs + r - b] * D_pad;
+        if (pairs.row) {
+            const int k = pairs.perm[off + (r < b ? r : r - b)];
+            src = r < b ? pairs.base[pairs.n_scenes] + (int64_t)pairs.row[k] * D_pad
+                        : pairs.base[pairs.scene ? pairs.scene[k] : 0] + (int64_t)pairs.obj[k] * D_pad;
         } else {
             src = x + r * D_pad;
         }
         v = *reinterpret_cast<const uint4 *>(src + c);
-        if (idx) *reinterpret_cast<uint4 *>(x + r * D_pad + c) = v;
+        if (pairs.row) *reinterpret_cast<uint4 *>(x + r * D_pad + c) = v;
     }
     const uint16_t h[8] = {(uint16_t)v.x, (uint16_t)(v.x >> 16), (uint16_t)v.y, (uint16_t)(v.y >> 16),
                            (uint16_t)v.z, (uint16_t)(v.z >> 16), (uint16_t)v.w, (uint16_t)(v.w >> 16)};
@@ -367,8 +367,8 @@ gelu_backward_t_kernel(const float *__restrict__ h, const float *__restrict__ b,
 constexpr int LP_PAIRS = 32;
 template <int NPL>
 __global__ void __launch_bounds__(256)
-pair_step_kernel(const float *__restrict__ z, const float *__restrict__ b2, const float *__restrict__ y,
-                 const float *__restrict__ w, float wsum, int64_t b, int P, uint16_t *__restrict__ dzb,
+pair_step_kernel(const float *__restrict__ z, const float *__restrict__ b2, TrainPairs pairs, int64_t off, float wsum,
+                 int64_t b, int P, uint16_t *__restrict__ dzb,
                  uint16_t *__restrict__ dzT, int64_t K, float *__restrict__ gb2, float *__restrict__ loss)
 {
     extern __shared__ __align__(16) uint16_t lp_tile[];     // [2][LP_PAIRS][P + 2]
@@ -407,8 +407,9 @@ pair_step_kernel(const float *__restrict__ z, const float *__restrict__ b2, cons
         for (int k = 0; k < NPL; ++k) s = fmaf(e[0][k], e[1][k], s);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
-        const float wi = w ? w[i] : 1.f;
-        const float r = s - y[i];
+        const int64_t at = pairs.perm ? pairs.perm[off + i] : off + i;
+        const float wi = pairs.w ? pairs.w[at] : 1.f;
+        const float r = s - pairs.y[at];
         const float g = 2.f * wi * r / wsum;
         lsum += wi * r * r / wsum;
 #pragma unroll
@@ -607,13 +608,12 @@ cudaError_t mlp_colsum(const float *x, int64_t rows, int cols, float *out, bool 
     return cudaGetLastError();
 }
 
-cudaError_t mlp_train_rows(const uint16_t *const *base, int32_t n_scenes, const int32_t *idx, int64_t n_pairs, int64_t b,
-                           int D, int D_pad, uint16_t *x, uint16_t *xT, int64_t K, float *gb1, int H, float *gb2, int P,
-                           cudaStream_t s)
+cudaError_t mlp_train_rows(const TrainPairs &pairs, int64_t off, int64_t b, int D, int D_pad, uint16_t *x, uint16_t *xT,
+                           int64_t K, float *gb1, int H, float *gb2, int P, cudaStream_t s)
 {
-    if (b < 1 || D_pad % TC != 0 || K % 64 != 0 || K < 2 * b) return cudaErrorInvalidValue;
+    if (b < 1 || D_pad % TC != 0 || K % 64 != 0 || K < 2 * b || (pairs.row && !pairs.perm)) return cudaErrorInvalidValue;
     dim3 grid((unsigned)(D_pad / TC), (unsigned)(K / TR));
-    train_rows_kernel<<<grid, 256, 0, s>>>(base, n_scenes, idx, n_pairs, b, D, D_pad, x, xT, K, gb1, H, gb2, P);
+    train_rows_kernel<<<grid, 256, 0, s>>>(pairs, off, b, D, D_pad, x, xT, K, gb1, H, gb2, P);
     return cudaGetLastError();
 }
 
@@ -635,8 +635,8 @@ cudaError_t mlp_gelu_backward_t(const float *h, const float *b, const float *da,
     return cudaGetLastError();
 }
 
-cudaError_t mlp_pair_step(const float *z, const float *b2, const float *y, const float *w, float wsum, int64_t b, int P,
-                          uint16_t *dzb, uint16_t *dzT, int64_t K, float *gb2, float *loss, cudaStream_t s)
+cudaError_t mlp_pair_step(const float *z, const float *b2, const TrainPairs &pairs, int64_t off, float wsum, int64_t b,
+                          int P, uint16_t *dzb, uint16_t *dzT, int64_t K, float *gb2, float *loss, cudaStream_t s)
 {
     if (b < 1 || P < 32 || P > 1024 || K < 2 * b) return cudaErrorInvalidValue;
     // the tile, 64 rows of P + 2 values (more than the 8 P floats of the column sums)
@@ -647,7 +647,8 @@ cudaError_t mlp_pair_step(const float *z, const float *b2, const float *y, const
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    kern<<<(unsigned)((b + LP_PAIRS - 1) / LP_PAIRS), 256, smem, s>>>(z, b2, y, w, wsum, b, P, dzb, dzT, K, gb2, loss);
+    kern<<<(unsigned)((b + LP_PAIRS - 1) / LP_PAIRS), 256, smem, s>>>(z, b2, pairs, off, wsum, b, P, dzb, dzT, K, gb2,
+                                                                     loss);
     return cudaGetLastError();
 }
 
