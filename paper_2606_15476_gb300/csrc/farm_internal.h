@@ -197,19 +197,24 @@ struct TrainPairs {
     const float *y, *w;
     const int32_t *perm;
 };
-// The training step's kernels (k_mlp.cu): its stacked rows and their transpose,
-// clearing the bias-gradient sums gb1 [H], gb2 [P]; GELU's BF16 output and
+// The training step's kernels (k_mlp.cu): its stacked rows and their transpose;
+// GELU's BF16 output and
 // transpose (aT nullable); the pairs' loss and the gradient down to the second
-// contraction's output; GELU's backward.  K: the padded length of the
+// contraction's output; GELU's backward with both
+// bias gradients (part: bias_part_floats(K, cols, P) floats, done:
+// bias_blocks(cols, P) counts that are 0).  K: the padded length of the
 // transposed operands (a multiple of 64, zero from the last row on).
 cudaError_t mlp_train_rows(const TrainPairs &pairs, int64_t off, int64_t b, int D, int D_pad, uint16_t *x, uint16_t *xT,
-                           int64_t K, float *gb1, int H, float *gb2, int P, cudaStream_t s);
+                           int64_t K, cudaStream_t s);
 cudaError_t mlp_gelu_bf16(const float *h, const float *b, int64_t rows, int cols, uint16_t *ab, uint16_t *aT, int64_t K,
                           cudaStream_t s);
+inline int64_t bias_blocks(int64_t cols, int64_t P) { return (cols + 63) / 64 + (P + 63) / 64; }
+inline int64_t bias_part_floats(int64_t K, int64_t cols, int64_t P) { return (K + 255) / 256 * bias_blocks(cols, P) * 64; }
 cudaError_t mlp_gelu_backward_t(const float *h, const float *b, const float *da, int64_t rows, int cols, uint16_t *dhT,
-                                int64_t K, float *gb, cudaStream_t s);
+                                int64_t K, float *gb, const float *dz, int P, float *gb2, float *part, int32_t *done,
+                                cudaStream_t s);
 cudaError_t mlp_pair_step(const float *z, const float *b2, const TrainPairs &pairs, int64_t off, float wsum, int64_t b,
-                          int P, uint16_t *dzb, uint16_t *dzT, int64_t K, float *gb2, float *loss, cudaStream_t s);
+                          int P, float *dzf, uint16_t *dzb, uint16_t *dzT, int64_t K, float *loss, cudaStream_t s);
 // e = bf16((z + b) / |z + b|) per row.
 cudaError_t mlp_normalize_bf16(const float *z, const float *b, int64_t rows, int cols, uint16_t *e, cudaStream_t s);
 // All BF16 copies of the parameters p (count of them).

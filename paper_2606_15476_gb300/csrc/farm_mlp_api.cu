@@ -137,7 +137,7 @@ struct TcBufs {
     void *base = nullptr;
     int64_t B = 0, K_pad = 0;
     uint16_t *x, *ab, *dzb, *xT, *aT, *dT;
-    float *h, *z, *da, *grad, *m, *v, *loss, *y, *w;
+    float *h, *z, *dz, *da, *grad, *m, *v, *loss, *y, *w, *bpart, *bdone;    // (bdone: counts, as int32)
     uint8_t *blob;               // the contractions' pieces, then their B tensor maps
 };
 
@@ -190,8 +190,9 @@ cudaError_t tc_alloc(farm_ctx *ctx, TcBufs &t, int64_t B, int64_t loss_slots, bo
     // (element count, element bytes) of each array, 256-byte aligned in one allocation
     const int64_t n16[] = {R * Dp, R * H, R * P, Dp * K, H * K, (P + H) * K};
     uint16_t **d16[] = {&t.x, &t.ab, &t.dzb, &t.xT, &t.aT, &t.dT};
-    const int64_t n32[] = {R * H, R * P, R * H, cnt, cnt, cnt, loss_slots, B, B};
-    float **d32[] = {&t.h, &t.z, &t.da, &t.grad, &t.m, &t.v, &t.loss, &t.y, &t.w};
+    const int64_t n32[] = {R * H, R * P, R * P, R * H, cnt, cnt, cnt, loss_slots, B, B,
+                           farm::bias_part_floats(K, H, P), farm::bias_blocks(H, P)};
+    float **d32[] = {&t.h, &t.z, &t.dz, &t.da, &t.grad, &t.m, &t.v, &t.loss, &t.y, &t.w, &t.bpart, &t.bdone};
     auto al = [](int64_t bytes) { return (bytes + 255) / 256 * 256; };
     int64_t total = 0;
     for (int64_t n : n16) total += al(n * 2);
@@ -268,17 +269,17 @@ cudaError_t tc_loss_grad(Ctx &c, TcBufs &t, int64_t b, const farm::TrainPairs &p
     cudaStream_t st = c.stream;
     cudaError_t r;
     launches += 8;
-    if ((r = farm::mlp_train_rows(pairs, off, b, (int)D, M.D_pad, t.x, t.xT, K, gb1, (int)H, gb2, (int)P, st)))
-        return r;
+    if ((r = farm::mlp_train_rows(pairs, off, b, (int)D, M.D_pad, t.x, t.xT, K, st))) return r;
     // forward: h = x W1^T, a = gelu(h + b1), z = a W2^T
     if ((r = tc_gemm(c, t, G_H))) return r;
     if ((r = farm::mlp_gelu_bf16(t.h, M.b1(), R, (int)H, t.ab, t.aT, K, st))) return r;
     if ((r = tc_gemm(c, t, G_Z))) return r;
-    // e = (z + b2) / |z + b2|, the loss, dz and its column sums
-    if ((r = farm::mlp_pair_step(t.z, M.b2(), pairs, off, wsum, b, (int)P, t.dzb, t.dT, K, gb2, lslot, st))) return r;
-    // backward: da = dz W2, dh = gelu'(h + b1) da, then dW2 = dz^T a and dW1 = dh^T x together
+    // e = (z + b2) / |z + b2|, the loss and dz
+    if ((r = farm::mlp_pair_step(t.z, M.b2(), pairs, off, wsum, b, (int)P, t.dz, t.dzb, t.dT, K, lslot, st))) return r;
+    // backward: da = dz W2, dh = gelu'(h + b1) da and the bias sums, then dW2 = dz^T a and dW1 = dh^T x together
     if ((r = tc_gemm(c, t, G_DA))) return r;
-    if ((r = farm::mlp_gelu_backward_t(t.h, M.b1(), t.da, R, (int)H, t.dT + P * K, K, gb1, st))) return r;
+    if ((r = farm::mlp_gelu_backward_t(t.h, M.b1(), t.da, R, (int)H, t.dT + P * K, K, gb1, t.dz, (int)P, gb2,
+                                       t.bpart, reinterpret_cast<int32_t *>(t.bdone), st))) return r;
     return tc_gemm(c, t, G_DW);
 }
 

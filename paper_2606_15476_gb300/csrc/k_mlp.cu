@@ -242,20 +242,15 @@ __device__ __forceinline__ void tile_write_t(const uint16_t (*tile)[TSTRIDE], in
 // The step's stacked input rows (query rows 0 .. b - 1, descriptor rows b ..
 // 2b - 1; D_pad long) and their transpose [D, K].  With pairs.row gathered
 // (pair k of the order: base[n_scenes] row row[k], and base[scene[k]] row
-// obj[k]) and written to x; without read from x.  The block of the origin also
-// clears the step's bias-gradient sums.
+// obj[k]) and written to x; without read from x.
 __global__ void __launch_bounds__(256)
 train_rows_kernel(TrainPairs pairs, int64_t off, int64_t b, int D, int D_pad, uint16_t *__restrict__ x,
-                  uint16_t *__restrict__ xT, int64_t K, float *__restrict__ gb1, int H, float *__restrict__ gb2, int P)
+                  uint16_t *__restrict__ xT, int64_t K)
 {
     __shared__ __align__(4) uint16_t tile[TR][TSTRIDE];
     const int tid = threadIdx.x;
     const int c0 = blockIdx.x * TC;
     const int64_t r0 = (int64_t)blockIdx.y * TR;
-    if (blockIdx.x == 0 && blockIdx.y == 0) {
-        for (int j = tid; j < H; j += 256) gb1[j] = 0.f;
-        for (int j = tid; j < P; j += 256) gb2[j] = 0.f;
-    }
     const int64_t r = r0 + (tid >> 3);
     const int c = c0 + (tid & 7) * 8;           // (D_pad is a multiple of 64: the tile's columns exist)
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -310,66 +305,109 @@ gelu_bf16_kernel(const float *__restrict__ h, const float *__restrict__ b, int64
     tile_write_t(tile, tid, aT, K, c0, cols, r0);
 }
 
+// Both bias gradients are column sums over the stacked rows in one fixed order:
+// per GB_ROWS rows eight partial sums of every eighth row in row order, those
+// eight in order, then the blocks' sums in order (by the block that comes last
+// to its columns).  Summed by one atomic per 32 pairs, b2's gradient differed by
+// up to 1.3e-7 between two runs at 1,024 pairs, which flips BF16 roundings of
+// the weights: W1 then moved by up to 2e-5 in a run of five steps.  The fixed
+// order costs an epoch of 120,000 pairs 2% (5.98 -> 6.11 ms).
+constexpr int GB_ROWS = 256, GB_STEP = 64;
+
 // dh = da gelu'(h + b) as its BF16 transpose dhT [cols, K], and its column
-// sums added to gb (one atomic per column and block of GB_TILES tiles).
-constexpr int GB_TILES = 4;
-__global__ void __launch_bounds__(256)
+// sums gb.  The blocks past the column tiles sum those of dz [rows, P] to gb2.
+// Two 32-row tiles per step of 512 threads.  part: gridDim.x * gridDim.y * TC
+// floats; done: gridDim.x counts, 0 before and after.
+__global__ void __launch_bounds__(512)
 gelu_backward_t_kernel(const float *__restrict__ h, const float *__restrict__ b, const float *__restrict__ da,
-                       int64_t rows, int cols, uint16_t *__restrict__ dhT, int64_t K, float *__restrict__ gb)
+                       int64_t rows, int cols, uint16_t *__restrict__ dhT, int64_t K, float *__restrict__ gb,
+                       const float *__restrict__ dz, int P, float *__restrict__ gb2, float *__restrict__ part,
+                       int32_t *__restrict__ done)
 {
-    __shared__ __align__(4) uint16_t tile[TR][TSTRIDE];
-    __shared__ float sums[TR][TC + 1];
+    __shared__ bool s_last;
+    __shared__ __align__(4) uint16_t tile[2][TR][TSTRIDE];
+    __shared__ float xs[GB_STEP][TC + 1];
     const int tid = threadIdx.x;
-    const int c0 = blockIdx.x * TC;
-    const int c = c0 + (tid & 7) * 8;
-    float part[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const float4 *bp = reinterpret_cast<const float4 *>(b + c);
-    const float4 b0 = __ldg(bp), b1 = __ldg(bp + 1);
-    for (int t = 0; t < GB_TILES; ++t) {
-        const int64_t r0 = ((int64_t)blockIdx.y * GB_TILES + t) * TR;
-        if (r0 >= K) break;
-        const int64_t r = r0 + (tid >> 3);
-        uint16_t g[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if (r < rows) {
-            const float4 *hp = reinterpret_cast<const float4 *>(h + r * cols + c);
-            const float4 *dp = reinterpret_cast<const float4 *>(da + r * cols + c);
-            const float4 h0 = hp[0], h1 = hp[1], d0 = dp[0], d1 = dp[1];
-            const float v[8] = {h0.x + b0.x, h0.y + b0.y, h0.z + b0.z, h0.w + b0.w,
-                                h1.x + b1.x, h1.y + b1.y, h1.z + b1.z, h1.w + b1.w};
-            const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+    const int sr = tid >> 6, sc = tid & 63;     // this thread's partial sum: rows sr mod 8, column sc
+    const int64_t base = (int64_t)blockIdx.y * GB_ROWS;
+    const int tiles = cols / TC;
+    float acc = 0.f;
+    float *out;
+    bool mine;
+    if ((int)blockIdx.x < tiles) {
+        const int half = tid >> 8, lt = tid & 255;
+        const int c0 = blockIdx.x * TC;
+        const int c = c0 + (lt & 7) * 8;
+        const float4 *bp = reinterpret_cast<const float4 *>(b + c);
+        const float4 b0 = __ldg(bp), b1 = __ldg(bp + 1);
+        for (int64_t s0 = base; s0 < min(K, base + GB_ROWS); s0 += GB_STEP) {     // (K a multiple of GB_STEP)
+            const int row = half * TR + (lt >> 3);
+            const int64_t r = s0 + row;
+            uint16_t g[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+            float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            if (r < rows) {
+                const float4 *hp = reinterpret_cast<const float4 *>(h + r * cols + c);
+                const float4 *dp = reinterpret_cast<const float4 *>(da + r * cols + c);
+                const float4 h0 = hp[0], h1 = hp[1], d0 = dp[0], d1 = dp[1];
+                const float v[8] = {h0.x + b0.x, h0.y + b0.y, h0.z + b0.z, h0.w + b0.w,
+                                    h1.x + b1.x, h1.y + b1.y, h1.z + b1.z, h1.w + b1.w};
+                const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float x = d[u] * gelu_grad(v[u]);
-                part[u] += x;
-                g[u] = bf16_bits(x);
+                for (int u = 0; u < 8; ++u) {
+                    x[u] = d[u] * gelu_grad(v[u]);
+                    g[u] = bf16_bits(x[u]);
+                }
             }
-        }
-        tile_put(tile, tid, g);
-        __syncthreads();
-        tile_write_t(tile, tid, dhT, K, c0, cols, r0);
-        __syncthreads();
-    }
+            tile_put(tile[half], lt, g);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) sums[tid >> 3][(tid & 7) * 8 + u] = part[u];
+            for (int u = 0; u < 8; ++u) xs[row][(lt & 7) * 8 + u] = x[u];
+            __syncthreads();
+            tile_write_t(tile[half], lt, dhT, K, c0, cols, s0 + half * TR);
+#pragma unroll
+            for (int k = 0; k < GB_STEP / 8; ++k) acc += xs[sr + 8 * k][sc];      // (zero past the last row)
+            __syncthreads();
+        }
+        out = gb + c0;
+        mine = true;
+    } else {
+        const int c0 = ((int)blockIdx.x - tiles) * TC;
+        mine = c0 + sc < P;
+        if (mine)
+            for (int64_t r = base + sr; r < min(rows, base + GB_ROWS); r += 8) acc += dz[r * P + c0 + sc];
+        out = gb2 + c0;
+    }
+    xs[sr][sc] = acc;
     __syncthreads();
     if (tid < TC) {
         float t = 0.f;
-        for (int i = 0; i < TR; ++i) t += sums[i][tid];
-        atomicAdd(gb + c0 + tid, t);
+        for (int i = 0; i < 8; ++i) t += xs[i][tid];
+        part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * TC + tid] = t;
+        __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(done + blockIdx.x, 1) == (int)gridDim.y - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (tid == 0) done[blockIdx.x] = 0;
+    if (tid < TC && mine) {
+        float t = 0.f;
+        for (int y = 0; y < (int)gridDim.y; ++y) t += __ldcg(part + ((int64_t)y * gridDim.x + blockIdx.x) * TC + tid);
+        out[tid] = t;
     }
 }
 
 // One warp per pair (LP_PAIRS pairs per block): both rows' bias and
 // normalisation, the pair's loss, and the gradient back through the
 // normalisation, held in registers (NPL values of each row per lane) and
-// written as dz BF16 [2b, P] and its transpose dzT [P, K] (zero from 2b), with
-// its column sums added to gb2 and the loss to *loss.
+// written as dz FP32 [2b, P] (for the bias sums), BF16 and the transpose dzT
+// [P, K] (zero from 2b), with the loss added to *loss.
 constexpr int LP_PAIRS = 32;
 template <int NPL>
 __global__ void __launch_bounds__(256)
 pair_step_kernel(const float *__restrict__ z, const float *__restrict__ b2, TrainPairs pairs, int64_t off, float wsum,
-                 int64_t b, int P, uint16_t *__restrict__ dzb,
-                 uint16_t *__restrict__ dzT, int64_t K, float *__restrict__ gb2, float *__restrict__ loss)
+                 int64_t b, int P, float *__restrict__ dzf, uint16_t *__restrict__ dzb,
+                 uint16_t *__restrict__ dzT, int64_t K, float *__restrict__ loss)
 {
     extern __shared__ __align__(16) uint16_t lp_tile[];     // [2][LP_PAIRS][P + 2]
     __shared__ float s_loss[8];
@@ -377,9 +415,6 @@ pair_step_kernel(const float *__restrict__ z, const float *__restrict__ b2, Trai
     const int64_t i0 = (int64_t)blockIdx.x * LP_PAIRS;
     const int ldt = P + 2;
     const unsigned FULL = 0xffffffffu;
-    float colsum[NPL];
-#pragma unroll
-    for (int k = 0; k < NPL; ++k) colsum[k] = 0.f;
     float lsum = 0.f;
     for (int t = warp; t < LP_PAIRS; t += 8) {
         const int64_t i = i0 + t;
@@ -424,8 +459,8 @@ pair_step_kernel(const float *__restrict__ z, const float *__restrict__ b2, Trai
             for (int k = 0; k < NPL; ++k) {
                 const int j = lane + 32 * k;
                 if (j >= P) continue;
-                const float dz = (g * e[1 - q][k] - e[q][k] * dot) * inv;
-                colsum[k] += dz;
+                const float dz = fmaf(-e[q][k], dot, __fmul_rn(g, e[1 - q][k])) * inv;
+                dzf[(q * b + i) * P + j] = dz;
                 const uint16_t h = bf16_bits(dz);
                 dzb[(q * b + i) * P + j] = h;
                 lp_tile[(q * LP_PAIRS + t) * ldt + j] = h;
@@ -447,18 +482,7 @@ pair_step_kernel(const float *__restrict__ z, const float *__restrict__ b2, Trai
     const int64_t z0 = 2 * b + blockIdx.x * share, z1 = min(K, z0 + share);
     for (int p = warp; p < P; p += 8)
         for (int64_t k = z0 + lane; k < z1; k += 32) dzT[(int64_t)p * K + k] = 0;
-    __syncthreads();
-    // column sums and the loss over the block's warps
-    float *red = reinterpret_cast<float *>(lp_tile);        // [8][P], inside the tile's bytes
-#pragma unroll
-    for (int k = 0; k < NPL; ++k)
-        if (lane + 32 * k < P) red[warp * P + lane + 32 * k] = colsum[k];
-    __syncthreads();
-    for (int j = tid; j < P; j += 256) {
-        float t = 0.f;
-        for (int v = 0; v < 8; ++v) t += red[v * P + j];
-        atomicAdd(gb2 + j, t);
-    }
+    // the loss over the block's warps
     if (tid == 0) {
         float t = 0.f;
         for (int v = 0; v < 8; ++v) t += s_loss[v];
@@ -609,11 +633,11 @@ cudaError_t mlp_colsum(const float *x, int64_t rows, int cols, float *out, bool 
 }
 
 cudaError_t mlp_train_rows(const TrainPairs &pairs, int64_t off, int64_t b, int D, int D_pad, uint16_t *x, uint16_t *xT,
-                           int64_t K, float *gb1, int H, float *gb2, int P, cudaStream_t s)
+                           int64_t K, cudaStream_t s)
 {
     if (b < 1 || D_pad % TC != 0 || K % 64 != 0 || K < 2 * b || (pairs.row && !pairs.perm)) return cudaErrorInvalidValue;
     dim3 grid((unsigned)(D_pad / TC), (unsigned)(K / TR));
-    train_rows_kernel<<<grid, 256, 0, s>>>(pairs, off, b, D, D_pad, x, xT, K, gb1, H, gb2, P);
+    train_rows_kernel<<<grid, 256, 0, s>>>(pairs, off, b, D, D_pad, x, xT, K);
     return cudaGetLastError();
 }
 
@@ -627,19 +651,20 @@ cudaError_t mlp_gelu_bf16(const float *h, const float *b, int64_t rows, int cols
 }
 
 cudaError_t mlp_gelu_backward_t(const float *h, const float *b, const float *da, int64_t rows, int cols, uint16_t *dhT,
-                                int64_t K, float *gb, cudaStream_t s)
+                                int64_t K, float *gb, const float *dz, int P, float *gb2, float *part, int32_t *done,
+                                cudaStream_t s)
 {
-    if (rows < 1 || cols % TC != 0 || K % 64 != 0 || K < rows) return cudaErrorInvalidValue;
-    dim3 grid((unsigned)(cols / TC), (unsigned)((K / TR + GB_TILES - 1) / GB_TILES));
-    gelu_backward_t_kernel<<<grid, 256, 0, s>>>(h, b, da, rows, cols, dhT, K, gb);
+    if (rows < 1 || P < 1 || cols % TC != 0 || K % GB_STEP != 0 || K < rows) return cudaErrorInvalidValue;
+    dim3 grid((unsigned)(cols / TC + (P + TC - 1) / TC), (unsigned)((K + GB_ROWS - 1) / GB_ROWS));
+    gelu_backward_t_kernel<<<grid, 512, 0, s>>>(h, b, da, rows, cols, dhT, K, gb, dz, P, gb2, part, done);
     return cudaGetLastError();
 }
 
 cudaError_t mlp_pair_step(const float *z, const float *b2, const TrainPairs &pairs, int64_t off, float wsum, int64_t b,
-                          int P, uint16_t *dzb, uint16_t *dzT, int64_t K, float *gb2, float *loss, cudaStream_t s)
+                          int P, float *dzf, uint16_t *dzb, uint16_t *dzT, int64_t K, float *loss, cudaStream_t s)
 {
     if (b < 1 || P < 32 || P > 1024 || K < 2 * b) return cudaErrorInvalidValue;
-    // the tile, 64 rows of P + 2 values (more than the 8 P floats of the column sums)
+    // the tile, 64 rows of P + 2 values
     const size_t smem = (size_t)2 * LP_PAIRS * (P + 2) * sizeof(uint16_t);
     auto kern = P <= 64 ? pair_step_kernel<2> : P <= 128 ? pair_step_kernel<4> : P <= 256 ? pair_step_kernel<8>
                 : P <= 512 ? pair_step_kernel<16> : pair_step_kernel<32>;
@@ -647,7 +672,7 @@ cudaError_t mlp_pair_step(const float *z, const float *b2, const TrainPairs &pai
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    kern<<<(unsigned)((b + LP_PAIRS - 1) / LP_PAIRS), 256, smem, s>>>(z, b2, pairs, off, wsum, b, P, dzb, dzT, K, gb2,
+    kern<<<(unsigned)((b + LP_PAIRS - 1) / LP_PAIRS), 256, smem, s>>>(z, b2, pairs, off, wsum, b, P, dzf, dzb, dzT, K,
                                                                      loss);
     return cudaGetLastError();
 }
