@@ -310,6 +310,17 @@ constexpr int kSimVariants = 3;
 constexpr int kSimNarrowVariant = 3;
 constexpr int kSimFewVariant = 4;
 constexpr int kSimFewRows = 128;
+// A single problem of more than 96 of them takes the CTA pairs where the CTAs
+// of 128 objects fill less than a third of the SMs: there each CTA's own chain
+// of loads and MMAs is what takes the time, and it grows with the padded rows
+// (similarity and ranks of 128 rows, D = 1152: 2,000 objects 15.9 us with the
+// pairs, 16.6 so; 4,000: 16.5, 17.2; 8,000: 20.2, 19.3; 87 rows x 2,098
+// objects: 15.9, 15.8).
+constexpr int kSimFewRowsAlways = 96;
+inline bool sim_few_single(int64_t rows, int64_t n, int num_sms)
+{
+    return rows <= kSimFewRowsAlways || (rows <= kSimFewRows && (n + 127) / 128 * 3 >= num_sms);
+}
 constexpr int kSimPairVariant = 2;      // the single-problem launches use the CTA pairs
 inline int sim_variant_bn(int v) { return v == kSimNarrowVariant ? 64 : v == 1 || v == kSimFewVariant ? 128 : 256; }
 inline int sim_variant_cluster(int v) { return v == 2 ? 2 : 1; }

@@ -1168,7 +1168,7 @@ cudaError_t launch_sim_tc_f16x3(const uint16_t *q_hi, const uint16_t *q_lo, cons
                                 const int32_t *gate)
 {
     if (rows <= kSimFewRows && (emit || gate)) return cudaErrorInvalidValue;
-    if (rows <= kSimFewRows)
+    if (sim_few_single(rows, n, num_sms))
         return launch_sim_few(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, tops, err, s);
     return launch_tc<kSimF16x3>(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, nullptr, nullptr, tops, num_sms,
                                 err, s, emit, gate);
