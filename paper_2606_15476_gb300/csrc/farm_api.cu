@@ -670,11 +670,7 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
     ctx->c.launches += 1;
     if ((e = farm::launch_normalize_rows(d_desc, nullptr, n, dim, ns.dim_pad, ns.desc32, ns.desc_hi,
                                          ns.desc_lo, ns.desc_bf16, c.d_err, farm::kErrBadDesc,
-                                         c.stream)) != cudaSuccess)
-        return bailmem(e);
-    ctx->c.launches += 1;
-    if ((e = farm::launch_quantize_fp8_rows(ns.desc32, n, ns.dim_pad, ns.desc_fp8, ns.desc_scale, c.stream)) !=
-        cudaSuccess)
+                                         c.stream, -1, ns.desc_fp8, ns.desc_scale)) != cudaSuccess)
         return bailmem(e);
     if ((e = cudaMemcpyAsync(ns.cls, cls, (size_t)n * 4, kind, c.stream)) != cudaSuccess) return bailmem(e);
     if ((e = cudaMemcpyAsync(ns.pos, box, (size_t)n * 12, kind, c.stream)) != cudaSuccess) return bailmem(e);
@@ -1357,9 +1353,7 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
         // -- the last ones -- get the FP16 split only, the others no split)
         const int64_t split = any_exact ? exact_row0 : -1;
         LAUNCH(farm::launch_normalize_rows2(src_t, n_q, src_c, n_c, d_rowmap, dim, dim_pad, ops.q32, ops.qhi, ops.qlo,
-                                            ops.qbf, c.d_err, farm::kErrBadRow, c.stream, split));
-        if (precision == FARM_PREC_FP8)
-            LAUNCH(farm::launch_quantize_fp8_rows(ops.q32, exact_row0, dim_pad, ops.qf8, ops.qscale, c.stream));
+                                            ops.qbf, c.d_err, farm::kErrBadRow, c.stream, split, ops.qf8, ops.qscale));
         if (precision == FARM_PREC_LEARNED) CK(farm::learned_embed_rows(ctx, ops.qbf, rows_total, ops.qcomp));
         mark_end(ctx, m0);
 
@@ -2068,9 +2062,7 @@ farm_status farm_similarity(farm_ctx *ctx, int32_t scene_id, int64_t n_rows, con
     RowOps ops;
     CK(alloc_rows(ctx, precision, n_rows, s.dim_pad, ops));
     LAUNCH(farm::launch_normalize_rows(src, nullptr, n_rows, s.dim, s.dim_pad, ops.q32, ops.qhi, ops.qlo, ops.qbf,
-                                       c.d_err, farm::kErrBadRow, c.stream));
-    if (precision == FARM_PREC_FP8)
-        LAUNCH(farm::launch_quantize_fp8_rows(ops.q32, n_rows, s.dim_pad, ops.qf8, ops.qscale, c.stream));
+                                       c.d_err, farm::kErrBadRow, c.stream, -1, ops.qf8, ops.qscale));
     float *S = out;
     if (!dev) CK(ws_get(ctx, farm::B_SIM, (size_t)n_rows * s.n, &S));
     farm_status st = run_similarity(ctx, precision, ops, 0, n_rows, s, S, s.n);
@@ -2139,9 +2131,7 @@ farm_status farm_similarity_variant(farm_ctx *ctx, int32_t scene_id, int64_t n_r
     RowOps ops;
     CK(alloc_rows(ctx, precision, n_rows, s.dim_pad, ops));
     LAUNCH(farm::launch_normalize_rows(src, nullptr, n_rows, s.dim, s.dim_pad, ops.q32, ops.qhi, ops.qlo, ops.qbf,
-                                       c.d_err, farm::kErrBadRow, c.stream));
-    if (precision == FARM_PREC_FP8)
-        LAUNCH(farm::launch_quantize_fp8_rows(ops.q32, n_rows, s.dim_pad, ops.qf8, ops.qscale, c.stream));
+                                       c.d_err, farm::kErrBadRow, c.stream, -1, ops.qf8, ops.qscale));
     const int64_t ld = round_up(s.n, 32);
     float *S;
     CK(ws_get(ctx, farm::B_SIM, (size_t)n_rows * ld, &S));

@@ -266,21 +266,21 @@ cudaError_t preload_sim_tc_f16x3();
 // dst_rows: optional int32 [rows] scatter map (src row r goes to dst row dst_rows[r]).
 // split >= 0: dst rows below split get only dst32 / dst_bf16, the others only
 // the FP16 split (a reduced-precision batch whose last rows run FP32-accurate).
+// dst_fp8 (with scale, one per dst row): the rows that get dst32 also as E4M3,
+// scaled by their largest entry (max|x| / 448).
 cudaError_t launch_normalize_rows(const float *src, const int32_t *dst_rows, int64_t rows,
                                   int32_t dim, int32_t dim_pad, float *dst32, uint16_t *dst_hi,
                                   uint16_t *dst_lo, uint16_t *dst_bf16, int32_t *err, int err_bit,
-                                  cudaStream_t s, int64_t split = -1);
+                                  cudaStream_t s, int64_t split = -1, uint8_t *dst_fp8 = nullptr,
+                                  float *scale = nullptr);
 
 // The same for the rows of two sources end to end: rows [0, rows) from src,
 // rows [rows, rows + rows2) from src2 (dst_rows covers both).
 cudaError_t launch_normalize_rows2(const float *src, int64_t rows, const float *src2, int64_t rows2,
                                    const int32_t *dst_rows, int32_t dim, int32_t dim_pad, float *dst32,
                                    uint16_t *dst_hi, uint16_t *dst_lo, uint16_t *dst_bf16, int32_t *err, int err_bit,
-                                   cudaStream_t s, int64_t split = -1);
-
-// E4M3 copy of unit rows with a per-row scale (max|x| / 448).
-cudaError_t launch_quantize_fp8_rows(const float *src, int64_t rows, int32_t dim_pad, uint8_t *dst, float *scale,
-                                     cudaStream_t s);
+                                   cudaStream_t s, int64_t split = -1, uint8_t *dst_fp8 = nullptr,
+                                   float *scale = nullptr);
 
 // Pre-compute the per-view record of kViewStride floats from SoA views and
 // the objects' centres pos [3, n]: {ox, oy, oz, fx, fy, fz, rx, ry} (origin,

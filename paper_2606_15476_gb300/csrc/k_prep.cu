@@ -26,11 +26,18 @@ __device__ __forceinline__ uint16_t half_bits(__half h) { return *reinterpret_ca
 // above it the FP16 split only (a batch whose last rows run the FP32-accurate
 // similarity); split < 0: every requested copy of every row.  Rows from rows1
 // on come from src2.
+//
+// FP8: also the E4M3 copy of each row that gets the FP32 one, with the row's
+// scale max|x| / 448 (448: the largest finite E4M3 value).  A rounded division
+// is monotone, so the unit row's largest entry is the source's largest one over
+// the norm, and the copy needs no pass of its own over the written rows.
+template <bool FP8>
 __global__ void normalize_rows_kernel(const float *__restrict__ src, int64_t rows1, const float *__restrict__ src2,
                                       const int32_t *__restrict__ dst_rows, int64_t rows, int32_t dim, int32_t dim_pad,
                                       float *__restrict__ dst32, uint16_t *__restrict__ dst_hi,
                                       uint16_t *__restrict__ dst_lo, uint16_t *__restrict__ dst_bf16,
-                                      int64_t split, int32_t *err, int err_bit)
+                                      uint8_t *__restrict__ dst_fp8, float *__restrict__ scale, int64_t split,
+                                      int32_t *err, int err_bit)
 {
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -40,8 +47,8 @@ __global__ void normalize_rows_kernel(const float *__restrict__ src, int64_t row
     // (8 bytes for the 16-bit copies)
     auto al = [](const void *q, uintptr_t a) { return q == nullptr || (reinterpret_cast<uintptr_t>(q) & (a - 1)) == 0; };
     const bool vec = ((dim | dim_pad) & 3) == 0 && al(x, 16) && al(dst32, 16) && al(dst_hi, 8) && al(dst_lo, 8) &&
-                     al(dst_bf16, 8);
-    float ss = 0.f;
+                     al(dst_bf16, 8) && al(dst_fp8, 4);
+    float ss = 0.f, amax = 0.f;
     if (vec) {
         const float4 *x4 = reinterpret_cast<const float4 *>(x);
         const int n4 = dim >> 2;
@@ -57,11 +64,16 @@ __global__ void normalize_rows_kernel(const float *__restrict__ src, int64_t row
                 s1 = fmaf(v[u].y, v[u].y, s1);
                 s2 = fmaf(v[u].z, v[u].z, s2);
                 s3 = fmaf(v[u].w, v[u].w, s3);
+                if (FP8)
+                    amax = fmaxf(amax, fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w))));
             }
         }
         ss = (s0 + s1) + (s2 + s3);
     } else {
-        for (int k = lane; k < dim; k += 32) ss = fmaf(x[k], x[k], ss);
+        for (int k = lane; k < dim; k += 32) {
+            ss = fmaf(x[k], x[k], ss);
+            if (FP8) amax = fmaxf(amax, fabsf(x[k]));
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -71,8 +83,16 @@ __global__ void normalize_rows_kernel(const float *__restrict__ src, int64_t row
     const int64_t drow = dst_rows ? (int64_t)dst_rows[row] : row;
     const int64_t base = drow * (int64_t)dim_pad;
     if (split >= 0) {
-        if (drow >= split) dst32 = nullptr, dst_bf16 = nullptr;
+        if (drow >= split) dst32 = nullptr, dst_bf16 = nullptr, dst_fp8 = nullptr;
         else dst_hi = nullptr;
+    }
+    float sc = 1.f;
+    if (FP8 && dst_fp8) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+        amax = bad ? 0.f : amax / nrm;
+        sc = amax > 0.f ? amax / 448.f : 1.f;
+        if (lane == 0) scale[drow] = sc;
     }
     if (vec) {
         // dim_pad is a multiple of 4: groups of four entries, zero past dim
@@ -109,6 +129,12 @@ __global__ void normalize_rows_kernel(const float *__restrict__ src, int64_t row
                 reinterpret_cast<uint2 *>(dst_bf16 + base)[k] =
                     make_uint2((uint32_t)b[0] | (uint32_t)b[1] << 16, (uint32_t)b[2] | (uint32_t)b[3] << 16);
             }
+            if (FP8 && dst_fp8) {
+                uint32_t q = 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) q |= (uint32_t)__nv_fp8_e4m3(v[u] / sc).__x << (8 * u);
+                reinterpret_cast<uint32_t *>(dst_fp8 + base)[k] = q;
+            }
         }
         return;
     }
@@ -124,6 +150,7 @@ __global__ void normalize_rows_kernel(const float *__restrict__ src, int64_t row
             __nv_bfloat16 b = __float2bfloat16_rn(v);
             dst_bf16[base + k] = *reinterpret_cast<uint16_t *>(&b);
         }
+        if (FP8 && dst_fp8) dst_fp8[base + k] = __nv_fp8_e4m3(v / sc).__x;
     }
 }
 
@@ -165,62 +192,30 @@ __global__ void prepare_views_kernel(const float *__restrict__ v, const float *_
     o[8] = ze; o[9] = ue; o[10] = 0.f; o[11] = 0.f;
 }
 
-// One warp per unit row: scale = max|x| / 448 (the largest finite E4M3
-// value), q = E4M3(x / scale) with saturation.
-__global__ void quantize_fp8_rows_kernel(const float *__restrict__ src, int64_t rows, int32_t dim_pad,
-                                         uint8_t *__restrict__ dst, float *__restrict__ scale)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (row >= rows) return;
-    const float *x = src + row * (int64_t)dim_pad;
-    float amax = 0.f;
-    for (int k = lane; k < dim_pad; k += 32) amax = fmaxf(amax, fabsf(x[k]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    const float sc = amax > 0.f ? amax / 448.f : 1.f;
-    if (lane == 0) scale[row] = sc;
-    uint8_t *d = dst + row * (int64_t)dim_pad;
-    for (int k = lane; k < dim_pad; k += 32) {
-        const __nv_fp8_e4m3 v(x[k] / sc);
-        d[k] = v.__x;
-    }
-}
-
 }  // namespace
-
-cudaError_t launch_quantize_fp8_rows(const float *src, int64_t rows, int32_t dim_pad, uint8_t *dst, float *scale,
-                                     cudaStream_t s)
-{
-    if (rows <= 0) return cudaSuccess;
-    const int warps = 8;
-    quantize_fp8_rows_kernel<<<(unsigned)((rows + warps - 1) / warps), warps * 32, 0, s>>>(src, rows, dim_pad, dst,
-                                                                                             scale);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_normalize_rows2(const float *src, int64_t rows1, const float *src2, int64_t rows2,
                                    const int32_t *dst_rows, int32_t dim, int32_t dim_pad, float *dst32,
                                    uint16_t *dst_hi, uint16_t *dst_lo, uint16_t *dst_bf16, int32_t *err, int err_bit,
-                                   cudaStream_t s, int64_t split)
+                                   cudaStream_t s, int64_t split, uint8_t *dst_fp8, float *scale)
 {
     const int64_t rows = rows1 + rows2;
     if (rows <= 0) return cudaSuccess;
     const int warps = 8;
     const int64_t blocks = (rows + warps - 1) / warps;
-    normalize_rows_kernel<<<(unsigned)blocks, warps * 32, 0, s>>>(src, rows1, src2, dst_rows, rows, dim, dim_pad,
-                                                                   dst32, dst_hi, dst_lo, dst_bf16,
-                                                                   split, err, err_bit);
+    auto kern = dst_fp8 ? normalize_rows_kernel<true> : normalize_rows_kernel<false>;
+    kern<<<(unsigned)blocks, warps * 32, 0, s>>>(src, rows1, src2, dst_rows, rows, dim, dim_pad, dst32, dst_hi, dst_lo,
+                                                 dst_bf16, dst_fp8, scale, split, err, err_bit);
     return cudaGetLastError();
 }
 
 cudaError_t launch_normalize_rows(const float *src, const int32_t *dst_rows, int64_t rows,
                                   int32_t dim, int32_t dim_pad, float *dst32, uint16_t *dst_hi,
                                   uint16_t *dst_lo, uint16_t *dst_bf16, int32_t *err, int err_bit,
-                                  cudaStream_t s, int64_t split)
+                                  cudaStream_t s, int64_t split, uint8_t *dst_fp8, float *scale)
 {
     return launch_normalize_rows2(src, rows, nullptr, 0, dst_rows, dim, dim_pad, dst32, dst_hi, dst_lo, dst_bf16, err,
-                                  err_bit, s, split);
+                                  err_bit, s, split, dst_fp8, scale);
 }
 
 cudaError_t launch_prepare_views(const float *views_soa, const float *pos, int64_t n, int32_t n_views, float *out,
@@ -233,11 +228,12 @@ cudaError_t launch_prepare_views(const float *views_soa, const float *pos, int64
     return cudaGetLastError();
 }
 
-// Loads the normalisation kernel (modules and functions load lazily on first use).
+// Loads the normalisation kernels (modules and functions load lazily on first use).
 cudaError_t preload_prep()
 {
     cudaFuncAttributes a;
-    return cudaFuncGetAttributes(&a, normalize_rows_kernel);
+    const cudaError_t e = cudaFuncGetAttributes(&a, normalize_rows_kernel<false>);
+    return e != cudaSuccess ? e : cudaFuncGetAttributes(&a, normalize_rows_kernel<true>);
 }
 
 }  // namespace farm
