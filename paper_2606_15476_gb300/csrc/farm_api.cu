@@ -1023,7 +1023,7 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
     const int32_t keep_max = reduced ? std::max(cstride_t, cstride_l) : std::max(stride_t, stride_l);
     const int32_t fs = keep_max <= 128 ? 8 : (keep_max <= 256 ? 4 : 2);
     // A FP32 batch of at most kSimFewRows rows takes the few-row similarity
-    // (k_sim_few.cu) and selects from its stored rows: for so few rows the
+    // (k_sim_few.cu; sim_few_variant) and selects from its stored rows: for so few rows the
     // fused selection's two launches and its merge cost more than the stores.
     // So they do for a batch of fewer tiles (128 rows x 256 objects) than two
     // per SM, whose sample and other tiles each fill a part of one wave (64
@@ -1242,7 +1242,9 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
                    log2i((int64_t)(wn / (double)rows_total));
         auto it = c.tuned.find(tune_key);
         if (few) {
-            vlist = {farm::kSimFewVariant};
+            int64_t tiles128 = 0;
+            for (const auto &g : groups) tiles128 += farm::sim_cluster_tiles(g.nq + g.nc, c.scenes[g.sid].n, 1);
+            vlist = {farm::sim_few_variant(rows_total, tiles128, c.num_sms)};
         } else if (c.pinned_variant >= 0) {
             vlist = {c.pinned_variant};
         } else if (it != c.tuned.end()) {

@@ -310,17 +310,6 @@ constexpr int kSimVariants = 3;
 constexpr int kSimNarrowVariant = 3;
 constexpr int kSimFewVariant = 4;
 constexpr int kSimFewRows = 128;
-// A single problem of more than 96 of them takes the CTA pairs where the CTAs
-// of 128 objects fill less than a third of the SMs: there each CTA's own chain
-// of loads and MMAs is what takes the time, and it grows with the padded rows
-// (similarity and ranks of 128 rows, D = 1152: 2,000 objects 15.9 us with the
-// pairs, 16.6 so; 4,000: 16.5, 17.2; 8,000: 20.2, 19.3; 87 rows x 2,098
-// objects: 15.9, 15.8).
-constexpr int kSimFewRowsAlways = 96;
-inline bool sim_few_single(int64_t rows, int64_t n, int num_sms)
-{
-    return rows <= kSimFewRowsAlways || (rows <= kSimFewRows && (n + 127) / 128 * 3 >= num_sms);
-}
 constexpr int kSimPairVariant = 2;      // the single-problem launches use the CTA pairs
 inline int sim_variant_bn(int v) { return v == kSimNarrowVariant ? 64 : v == 1 || v == kSimFewVariant ? 128 : 256; }
 inline int sim_variant_cluster(int v) { return v == 2 ? 2 : 1; }
@@ -403,6 +392,37 @@ inline int64_t sim_cluster_tiles(int64_t rows, int64_t n, int variant, int mode 
     return (mt + cm - 1) / cm * col_tiles(n, (int)bn, mode, s);
 }
 
+// The FP32-accurate kernel for at most kSimFewRows rows, `tiles128` being their
+// 128 x 128 tiles.  Up to kSimFewAlways the few-row kernel; more rows are padded
+// to 128 there, and 128 x 128 tiles on at most half of the SMs are faster
+// (kernels alone, cold caches, 128 rows, D = 1152: 2,000 objects 27.6 us few-row,
+// 29.0 CTA pairs, 21.1 so; 8,000: 28.4, 30.1, 21.2; 64 rows x 2,000: 20.3, 28.1,
+// 20.4).  With more objects the few-row kernel, two CTAs to an SM, reads the
+// descriptors faster (128 rows x 20,000: 33.2 against 36.8).
+constexpr int kSimFewAlways = 64;
+inline int sim_few_variant(int64_t rows, int64_t tiles128, int num_sms)
+{
+    return rows > kSimFewAlways && tiles128 * 2 <= num_sms ? 1 : kSimFewVariant;
+}
+
+// The FP32-accurate variant of one problem of more rows: 128 x 128 tiles on at
+// most a quarter of the SMs, 128 x 256 ones where they save a fifth of the CTA pairs'
+// waves (a wave of them takes about a tenth longer), else the pairs.  Whole
+// calls, back to back: 200 rows x 2,000 objects 11.7 us with the pairs, 10.3
+// with 128 x 128 tiles (32 of them); but 250 x 4,864 (76) 13.0 and 13.6, 150 x
+// 9,728 (152) 15.6 and 21.0.  300 rows x
+// 20,000 objects 53.7 us with the pairs (3 waves), 46.7 with 128 x 256 tiles
+// (2); 384 x 38,000 94.3 (4), 83.4 (3).
+inline int sim_single_variant(int64_t rows, int64_t n, int num_sms)
+{
+    const int64_t tiles128 = sim_cluster_tiles(rows, n, 1), sms = num_sms > 2 ? num_sms : 2;
+    if (rows <= kSimFewRows) return sim_few_variant(rows, tiles128, num_sms);
+    if (tiles128 * 4 <= num_sms) return 1;
+    const int64_t waves = (sim_cluster_tiles(rows, n, 0) + sms - 1) / sms,
+                  pair_waves = (sim_cluster_tiles(rows, n, kSimPairVariant) + sms / 2 - 1) / (sms / 2);
+    return waves * 5 <= pair_waves * 4 ? 0 : kSimPairVariant;
+}
+
 // The fused rank selection's outputs of a kColRest launch, indexed by operand
 // row: each row's threshold (order-preserving key of its sample's R-th
 // value), candidate count and buffer of `cap` candidate words
@@ -449,7 +469,8 @@ cudaError_t launch_sim_few_grouped(const uint16_t *q_hi, const uint16_t *q_lo, i
 cudaError_t preload_sim_few();
 
 // One problem (rows x n, S leading dimension ld_s, group maxima at tops with
-// group_stride(n) floats per row, nullable) on the tensor cores, variant 2 (CTA pairs).
+// group_stride(n) floats per row, nullable) on the tensor cores, in the variant
+// sim_single_variant picks (2, the CTA pairs, with `emit` or a gate).
 // Three FP16 terms, hi*hi + 2^-11 (hi*lo + lo*hi), from the split the
 // normalisation writes.
 // With `emit` (more than kSimFewRows rows) nothing is stored: every entry

@@ -30,7 +30,9 @@ __device__ __forceinline__ uint16_t half_bits(__half h) { return *reinterpret_ca
 // FP8: also the E4M3 copy of each row that gets the FP32 one, with the row's
 // scale max|x| / 448 (448: the largest finite E4M3 value).  A rounded division
 // is monotone, so the unit row's largest entry is the source's largest one over
-// the norm, and the copy needs no pass of its own over the written rows.
+// the norm, and the copy needs no pass of its own over the written rows (36 us
+// for 20,000 rows of 1152; uploading such a scene and asking it 64 questions:
+// 206 us with that pass, 168 so).
 template <bool FP8>
 __global__ void normalize_rows_kernel(const float *__restrict__ src, int64_t rows1, const float *__restrict__ src2,
                                       const int32_t *__restrict__ dst_rows, int64_t rows, int32_t dim, int32_t dim_pad,

@@ -983,19 +983,19 @@ int32_t k_slices_of(int32_t dim_pad)
     return (dim_pad + Elem<MODE>::BK - 1) / Elem<MODE>::BK;
 }
 
-// One problem, tile configuration 2 (256 x 256 tiles on CTA pairs).
-template <int MODE>
+// One problem in the tile configuration of `V` (2: 256 x 256 tiles on CTA pairs).
+template <int MODE, int V = kSimPairVariant>
 cudaError_t launch_tc(const void *q0, const void *q1, const void *d0, const void *d1, float *S, int64_t rows,
                       int64_t n, int32_t dim_pad, int64_t ld_s, const float *scale_q, const float *scale_d,
                       float *tops, int num_sms, int32_t *err, cudaStream_t s, const FuseEmit *emit = nullptr,
                       const int32_t *gate = nullptr)
 {
-    constexpr int BN_ = 256, CM_ = 2;
-    static_assert(BN_ == 256 && CM_ == 2, "the tile count below is that of the pair variant");
+    constexpr int BN_ = V == 1 ? 128 : 256, CM_ = V == 2 ? 2 : 1;
+    constexpr bool PAIR_ = V == 2;
+    static_assert(V >= 0 && V < kSimVariants, "a tile variant");
     constexpr bool TWO = !Elem<MODE>::SPLIT;
     if (rows <= 0 || n <= 0) return cudaSuccess;
-    if (sim_variant_bn(kSimPairVariant) != BN_ || sim_variant_cluster(kSimPairVariant) != CM_)
-        return cudaErrorInvalidConfiguration;
+    if (sim_variant_bn(V) != BN_ || sim_variant_cluster(V) != CM_) return cudaErrorInvalidConfiguration;
     if (dim_pad % kDimAlign != 0 || rows > 0x7fffffffLL || n > 0x7fffffffLL || ld_s < n || ld_s > 0x7fffffffLL)
         return cudaErrorInvalidValue;
     if (!get_encoder()) return cudaErrorNotSupported;
@@ -1027,8 +1027,9 @@ cudaError_t launch_tc(const void *q0, const void *q1, const void *d0, const void
     single.col_mode = kColAll;
     single.col_stride = 0;
     single.n_store = (int32_t)n;
-    const int64_t tiles = sim_cluster_tiles(rows, n, kSimPairVariant);
-    if constexpr (MODE == kSimF16x3) {
+    const int64_t tiles = sim_cluster_tiles(rows, n, V);
+    if (emit && !(MODE == kSimF16x3 && PAIR_)) return cudaErrorInvalidValue;
+    if constexpr (MODE == kSimF16x3 && PAIR_) {
         if (emit) {
             if (!emit->tau_key || !emit->cnt || !emit->cand || emit->cap < 1) return cudaErrorInvalidValue;
             return launch_impl<MODE, BN_, CM_, false, true, true>(mq0, mq1, md0, md1, nullptr, 1, single, S, tops,
@@ -1038,8 +1039,8 @@ cudaError_t launch_tc(const void *q0, const void *q1, const void *d0, const void
     }
     FuseEmit none{};
     none.gate = gate;
-    return launch_impl<MODE, BN_, CM_, false, true>(mq0, mq1, md0, md1, nullptr, 1, single, S, tops,
-                                              k_slices_of<MODE>(dim_pad), tiles, scale_q, num_sms, err, s, none);
+    return launch_impl<MODE, BN_, CM_, false, PAIR_>(mq0, mq1, md0, md1, nullptr, 1, single, S, tops,
+                                                     k_slices_of<MODE>(dim_pad), tiles, scale_q, num_sms, err, s, none);
 }
 
 template <int MODE, int BN_, int CM_, bool PAIR = false>
@@ -1168,8 +1169,15 @@ cudaError_t launch_sim_tc_f16x3(const uint16_t *q_hi, const uint16_t *q_lo, cons
                                 const int32_t *gate)
 {
     if (rows <= kSimFewRows && (emit || gate)) return cudaErrorInvalidValue;
-    if (sim_few_single(rows, n, num_sms))
+    const int v = emit || gate ? kSimPairVariant : sim_single_variant(rows, n, num_sms);
+    if (v == kSimFewVariant)
         return launch_sim_few(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, tops, err, s);
+    if (v == 0)
+        return launch_tc<kSimF16x3, 0>(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, nullptr, nullptr, tops,
+                                       num_sms, err, s);
+    if (v == 1)
+        return launch_tc<kSimF16x3, 1>(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, nullptr, nullptr, tops,
+                                       num_sms, err, s);
     return launch_tc<kSimF16x3>(q_hi, q_lo, d_hi, d_lo, S, rows, n, dim_pad, ld_s, nullptr, nullptr, tops, num_sms,
                                 err, s, emit, gate);
 }
@@ -1194,7 +1202,9 @@ cudaError_t launch_sim_tc_fp8(const uint8_t *q, const float *scale_q, const uint
 cudaError_t preload_sim_tc_f16x3()
 {
     cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, sim_tc_kernel<kSimF16x3, 256, 2, false, true>);
+    cudaError_t e = cudaFuncGetAttributes(&a, sim_tc_kernel<kSimF16x3, 256, 2, false, true>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, sim_tc_kernel<kSimF16x3, 256, 1, false, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, sim_tc_kernel<kSimF16x3, 128, 1, false, false>);
     return e == cudaSuccess ? preload_sim_few() : e;
 }
 
