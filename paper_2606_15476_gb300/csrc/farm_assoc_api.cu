@@ -12,6 +12,14 @@ using farm::Ctx;
 
 namespace {
 
+// From this many cosines on a call keeps those reaching tau_f instead of storing
+// all.  Fewer (24 MB) stay in the L2, and the two launches that the lists need
+// cost more than they save: 307 detections x 589 entities 41.5 us with lists,
+// 34.8 stored; 1,000 x 4,000 41.6, 36.7.  At 8 million the two are even (4,000 x
+// 2,000 74.4, 72.0; 1,000 x 8,000 43.4, 44.3); 1,000 x 16,000 73.8, 83.1; 1,500
+// x 30,000 135, 176.
+constexpr int64_t kEmitCosines = int64_t(6) << 20;
+
 farm_status afail(Ctx &c, farm_status st, const std::string &msg)
 {
     c.err = msg;
@@ -82,10 +90,11 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
     float *h_emu = nullptr, *h_ecov = nullptr, *h_efeat = nullptr, *h_ew = nullptr, *h_dmu = nullptr,
           *h_dcov = nullptr, *h_dfeat = nullptr;
     int32_t *h_eact = nullptr;
-    // more detections than the few-row similarity takes: only the cosines
-    // reaching tau_f are kept, up to `cap` per detection (about as many as a
-    // fused selection's row; more of them: the stored rows)
-    const bool emitting = B > farm::kSimFewRows;
+    // more detections than the few-row similarity takes, and more cosines than
+    // kEmitCosines: only those reaching tau_f are kept, up to `cap` per
+    // detection (about as many as a fused selection's row; more of them: the
+    // stored rows)
+    const bool emitting = B > farm::kSimFewRows && (int64_t)B * N >= kEmitCosines;
     const int32_t cap = farm::fuse_merge_capacity(1);
     // the layout of the call's device memory: sized with a null base, then
     // carved from the context's grow-only buffer

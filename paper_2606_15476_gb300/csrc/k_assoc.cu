@@ -8,9 +8,9 @@
 //      H = sqrt(1 - BC),  ln BC = (ln det S_d + ln det S_e) / 4 - ln det S / 2
 //                                 - dmu' S^-1 dmu / 8,  S = (S_d + S_e) / 2,
 //    (1 - BC evaluated as -expm1(ln BC)); those with H <= h_max are sorted by
-//    (H, index) and the first max_m kept (one CTA per detection).  For more
-//    than kSimFewRows detections the similarity kernel keeps only the cosines
-//    reaching tau_f (the emitting form of the fused rank selection, its
+//    (H, index) and the first max_m kept (one CTA per detection).  For
+//    enough cosines, of more than kSimFewRows detections, the similarity kernel
+//    keeps only those reaching tau_f (the emitting form of the fused rank selection, its
 //    threshold tau_f for every row), so the detection-by-entity block is
 //    neither written nor read; a detection with more of them than its buffer
 //    holds is searched over its stored row, which is then computed;
