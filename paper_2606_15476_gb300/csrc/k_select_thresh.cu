@@ -251,7 +251,9 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     const int64_t n_groups = group_count(n, gshift);
     const int U = (int)min(n_groups, (int64_t)UNION_MAX);
     if (tid == 0) { s_cnt = 0; s_ng = 0; }
-    uint32_t T = 0u, top = 0xffffffffu;    // the candidates' keys lie in [T, top]
+    // the candidates' keys lie in [T, top] (of a row whose maxima are not all
+    // staged, once `top` has been raised to the candidates' below)
+    uint32_t T = 0u, top = 0xffffffffu;
 
     // For tau = key_value(T) and non-NaN x,
     // x >= tau holds exactly when order_key(x) >= T, so the passes below
@@ -324,6 +326,17 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     }
     __syncthreads();
     const int cnt = s_cnt;
+    if (U >= R && n_groups > U && cnt <= RANK_MAX) {
+        // the maxima were a prefix of the row's, and an entry past it may lie
+        // above them all: the upper end comes from the candidates themselves
+        uint32_t hi = 0u;
+        for (int c = tid; c < cnt; c += TT) hi = max(hi, (uint32_t)(cand[c] >> 32));
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if ((tid & 31) == 0) sm.s_mm[tid >> 5] = hi;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < TT / 32; ++w) top = max(top, sm.s_mm[w]);
+    }
     // (fewer than R candidates cannot happen with group maxima of this row;
     // the exact select then stands in rather than list unfilled entries)
     if (cnt >= R && cnt <= RANK_MAX) {
