@@ -171,11 +171,15 @@ cudaError_t ws_get(farm_ctx *ctx, Buf b, size_t bytes, void **out)
             ws.ptr[b] = nullptr;
             ws.bytes[b] = 0;
         }
+        ctx->c.ws_gen += 1;     // captured graphs that use the old buffer no longer match, whether or not the next is had
         size_t grow = bytes + bytes / 8;
         cudaError_t e = cudaMalloc(&ws.ptr[b], grow);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess) {
+            ws.ptr[b] = nullptr;
+            (void)cudaGetLastError();       // (reported here, not by the next launch)
+            return e;
+        }
         ws.bytes[b] = grow;
-        ctx->c.ws_gen += 1;     // captured graphs that use the old buffer no longer match
     }
     *out = ws.ptr[b];
     return cudaSuccess;
@@ -614,6 +618,12 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
     // a scene of the same shape is replaced in place: the copies and kernels
     // below follow the queued work that reads it on the same stream
     const bool reuse = s.present && s.n == n && s.dim == dim && s.n_views == n_views;
+    if (s.present) {
+        // from here on the old scene is gone, also when a call below fails:
+        // no recorded batch may be replayed over its arrays
+        c.scene_gen += 1;
+        ctx->replay.valid = false;
+    }
     if (reuse) {
         bool spaces = false;
         for (const auto &sp : s.spaces) spaces |= sp.hi != nullptr;
@@ -638,9 +648,13 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
     ns.dim_pad = (int32_t)round_up(dim, farm::kDimAlign);
     ns.n_views = n_views;
     const size_t nd = (size_t)n * ns.dim_pad;
+    float *tmp_desc = nullptr, *tmp_views = nullptr;
     auto bailmem = [&](cudaError_t e) {
-        if (reuse) cudaStreamSynchronize(c.stream);      // (queued work may still read it)
+        if (tmp_desc) cudaFreeAsync(tmp_desc, c.stream);
+        if (tmp_views) cudaFreeAsync(tmp_views, c.stream);
+        cudaStreamSynchronize(c.stream);                 // (queued work may still read the scene's arrays)
         free_scene(ns);
+        (void)cudaGetLastError();                        // (reported here, not by the next launch)
         return fail(ctx, e == cudaErrorMemoryAllocation ? FARM_ENOMEM : FARM_ECUDA,
                     std::string("scene upload: ") + cudaGetErrorString(e));
     };
@@ -660,9 +674,11 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
     }
     const cudaMemcpyKind kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const float *d_desc = desc;
-    float *tmp_desc = nullptr, *tmp_views = nullptr;
     if (!dev) {
-        if ((e = cudaMallocAsync(&tmp_desc, (size_t)n * dim * 4, c.stream)) != cudaSuccess) return bailmem(e);
+        if ((e = cudaMallocAsync(&tmp_desc, (size_t)n * dim * 4, c.stream)) != cudaSuccess) {
+            tmp_desc = nullptr;
+            return bailmem(e);
+        }
         if ((e = cudaMemcpyAsync(tmp_desc, desc, (size_t)n * dim * 4, kind, c.stream)) != cudaSuccess)
             return bailmem(e);
         d_desc = tmp_desc;
@@ -680,7 +696,10 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
         const float *d_views = views;
         if (!dev) {
             const size_t vb = (size_t)6 * n_views * n * 4;
-            if ((e = cudaMallocAsync(&tmp_views, vb, c.stream)) != cudaSuccess) return bailmem(e);
+            if ((e = cudaMallocAsync(&tmp_views, vb, c.stream)) != cudaSuccess) {
+                tmp_views = nullptr;
+                return bailmem(e);
+            }
             if ((e = cudaMemcpyAsync(tmp_views, views, vb, kind, c.stream)) != cudaSuccess) return bailmem(e);
             d_views = tmp_views;
         }
@@ -690,6 +709,7 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
     }
     if (tmp_desc) cudaFreeAsync(tmp_desc, c.stream);
     if (tmp_views) cudaFreeAsync(tmp_views, c.stream);
+    tmp_desc = tmp_views = nullptr;
     SceneDev sd{ns.pos, ns.views, ns.cls, ns.size, n, n_views, 0};
     if ((e = cudaMemcpyAsync(ctx->d_scenes + scene_id, &sd, sizeof(sd), cudaMemcpyHostToDevice, c.stream)) !=
         cudaSuccess)
