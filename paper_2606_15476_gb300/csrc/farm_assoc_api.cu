@@ -112,7 +112,9 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
         a.win = cv.take<unsigned long long>((size_t)T);
         a.mcnt = cv.take<int32_t>((size_t)T); a.off = cv.take<int32_t>((size_t)T);
         a.pos = cv.take<int32_t>((size_t)T); a.members = cv.take<int32_t>((size_t)T);
-        a.counters = cv.take<int32_t>(2);
+        a.counters = cv.take<int32_t>(farm::kAssocCounters);
+        a.items = cv.take<int2>((size_t)farm::assoc_items_of(T));
+        a.sums = cv.take<float>((size_t)farm::assoc_items_of(T) * (4 + F));
         if (emitting) {
             a.over = cv.take<int32_t>((size_t)B);
             a.emit.tau_key = cv.take<uint32_t>((size_t)B); a.emit.cnt = cv.take<int32_t>((size_t)B);
@@ -176,7 +178,7 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
     a.h_max = h_max;
     a.max_m = max_m;
     a.err = c.d_err;
-    c.launches += emitting ? 10 : 8;
+    c.launches += emitting ? 11 : 9;
     ACK(farm::launch_assoc_init(a, c.stream), "association kernels");
     if (emitting) {
         ACK(farm::launch_sim_tc_f16x3(dhi, dlo, ehi, elo, nullptr, B, N, F_pad, ld, nullptr, c.num_sms, c.d_err,

@@ -728,6 +728,10 @@ struct FuseArgs {
 cudaError_t launch_fuse(const FuseArgs &a, int part, cudaStream_t s);
 
 // Mapping-side association (k_assoc.cu): device arrays only.
+constexpr int kAssocItems = 2, kAssocCounters = 3;
+// The most work items that T slots can have: winners of at least 65 members, a
+// segment per 1,024 of them.
+inline int64_t assoc_items_of(int64_t T) { return T / 64 + T / 1024 + 1; }
 struct AssocArgs {
     int32_t N, B, F;                    // entities, detections, feature length
     const float *S;                     // [B, ld] detection-by-entity feature cosines
@@ -742,7 +746,10 @@ struct AssocArgs {
     int32_t *label;                     // [N + B] scratch: component labels
     unsigned long long *win;            // [N + B] scratch: winners
     int32_t *mcnt, *off, *pos, *members;    // [N + B] scratch: each winner's members
-    int32_t *counters;                  // [2] scratch: members' array in use; detections whose list overflowed
+    int32_t *counters;                  // [kAssocCounters] scratch: members' array in use; detections whose list
+                                        // overflowed; work items of the fusion
+    int2 *items;                        // [assoc_items_of(T)] scratch: those items, (winner, segment)
+    float *sums;                        // [items, 4 + F] scratch: their sums
     int32_t *over;                      // [B] scratch: those detections
     FuseEmit emit;                      // the emitting similarity's lists (cnt null: stored rows)
     int32_t *parent;                    // [N + B]

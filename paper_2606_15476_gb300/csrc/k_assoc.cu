@@ -168,7 +168,7 @@ assoc_init_kernel(int32_t T, int32_t B, float tau_f, int32_t *__restrict__ label
                   int32_t *__restrict__ cnt)
 {
     const int t = blockIdx.x * 256 + threadIdx.x;
-    if (t < 2) counters[t] = 0;
+    if (t < kAssocCounters) counters[t] = 0;
     if (t < T) {
         label[t] = t;
         win[t] = 0ull;
@@ -328,12 +328,25 @@ __global__ void assoc_parent_kernel(int32_t T, const int32_t *__restrict__ root,
     if (p != t) pos[t] = atomicAdd(&mcnt[p], 1);
 }
 
-// Each winner's stretch of the members' array (their order is free).
+constexpr int BIG_MEMBERS = 64;    // a winner of more is fused by whole blocks
+constexpr int SEG = 1024;          // members of it that a block sums at a time
+
+// Each winner's stretch of the members' array (their order is free), and the
+// segments of a winner of many members: (winner, segment) work items, as many
+// as bump[kAssocItems] counts in the end.  A winner's place among another's
+// members is unused: it counts the winner's finished segments.
 __global__ void assoc_offset_kernel(int32_t T, const int32_t *__restrict__ mcnt, int32_t *__restrict__ off,
-                                    int32_t *bump)
+                                    int32_t *__restrict__ pos, int32_t *bump, int2 *__restrict__ items)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < T && mcnt[t] > 0) off[t] = atomicAdd(bump, mcnt[t]);
+    if (t >= T) return;
+    const int m = mcnt[t];
+    if (m <= 0) return;
+    off[t] = atomicAdd(bump, m);
+    if (m <= BIG_MEMBERS) return;
+    const int segs = (m + SEG - 1) / SEG, at = atomicAdd(bump + kAssocItems, segs);
+    pos[t] = 0;
+    for (int k = 0; k < segs; ++k) items[at + k] = make_int2(t, k);
 }
 
 __global__ void assoc_members_kernel(int32_t T, const int32_t *__restrict__ parent, const int32_t *__restrict__ off,
@@ -358,23 +371,213 @@ struct Slots {
 };
 
 constexpr int FW = 8;              // slots (warps) per block of the fusion
-constexpr int BIG_MEMBERS = 64;    // a winner of more is fused by its whole block
-constexpr int FCHUNK = 512;        // features of a big winner at a time
+constexpr int FTH = FW * 32;
+constexpr int FU = 8;              // members whose features a lane has in flight
+constexpr int BIG_BLOCKS = 304;    // blocks that take the big winners' work items
 
-// out_w, out_mu, out_cov and out_feat of every slot: zeros for a merged one,
-// the slot's own values for a winner without members, sums over the members
-// (listed at members + off) otherwise.
-__global__ void __launch_bounds__(FW * 32)
+// The sum over the block's threads of N values each, to every thread.
+template <int N>
+__device__ __forceinline__ void block_sum(float (&v)[N], float (*part)[8], int lane, int warp)
+{
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    __syncthreads();                    // (part is free)
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < N; ++i) part[warp][i] = v[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        v[i] = 0.f;
+#pragma unroll
+        for (int w = 0; w < FW; ++w) v[i] += part[w][i];
+    }
+}
+
+// The members' weighted feature sums of a segment (ids and weights in shared
+// memory, n of them, the winner itself counted as one), V floats per lane and
+// load: put(j, x) for every feature j.  The lanes share out the columns of a
+// stretch of up to 32 loads and, when those are fewer than half a warp, several
+// members; eight members' loads are in flight per lane.
+template <int V, class Put>
+__device__ __forceinline__ void segment_features(const Slots &sl, const int32_t *ids, const float *ws, int n,
+                                                 float (*part)[V], int lane, int warp, Put put)
+{
+    const int cols = sl.F / V;
+    for (int c0 = 0; c0 < cols; c0 += 32) {
+        const int C = min(32, cols - c0), SUB = 32 / C, sub = lane / C, col = lane - sub * C;
+        const bool on = sub < SUB;
+        float acc[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[v] = 0.f;
+        for (int k0 = warp * SUB; k0 < n; k0 += FU * FW * SUB) {
+            float x[FU][V], w[FU];
+#pragma unroll
+            for (int u = 0; u < FU; ++u) {
+                const int k = k0 + u * FW * SUB + sub;
+                const bool in = on && k < n;
+                w[u] = in ? ws[k] : 0.f;
+                const float *f = in ? sl.feat(ids[k]) + (int64_t)(c0 + col) * V : nullptr;
+                if constexpr (V == 4) {
+                    const float4 y = in ? __ldg(reinterpret_cast<const float4 *>(f)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    x[u][0] = y.x; x[u][1] = y.y; x[u][2] = y.z; x[u][3] = y.w;
+                } else {
+                    x[u][0] = in ? __ldg(f) : 0.f;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < FU; ++u)
+#pragma unroll
+                for (int v = 0; v < V; ++v) acc[v] = fmaf(w[u], x[u][v], acc[v]);
+        }
+#pragma unroll
+        for (int v = 0; v < V; ++v) part[warp * 32 + lane][v] = acc[v];
+        __syncthreads();
+        if (threadIdx.x < C * V) {
+            const int c = threadIdx.x / V, v = threadIdx.x - c * V;
+            float x = 0.f;
+            for (int q = 0; q < FW; ++q)
+                for (int h = 0; h < SUB; ++h) x += part[q * 32 + h * C + c][v];
+            put((c0 + c) * V + v, x);
+        }
+        __syncthreads();
+    }
+}
+
+// One segment of a winner of many members: its sums of w, w (mu - c) (c the
+// winner's own mean) and w f go to the outputs when it is the winner's only
+// one, else to sums (4 + F floats per work item, the winner's from `first` on);
+// the block that finishes the winner's last segment adds them in order, and
+// sums the covariance about the fused mean over all members.
+__device__ __forceinline__ void fuse_big(const Slots &sl, int g, int seg, int item, const int32_t *__restrict__ mem,
+                                         int m, int32_t *done, float *sums, int vec, float *__restrict__ out_w,
+                                         float *__restrict__ out_mu, float *__restrict__ out_cov,
+                                         float *__restrict__ out_feat)
+{
+    __shared__ int32_t ids[SEG + 1];
+    __shared__ float ws[SEG + 1];
+    __shared__ __align__(16) float s_part[FTH][4];
+    __shared__ float s_red[FW][8];
+    __shared__ int s_last;
+    const int T = sl.N + sl.B, F = sl.F, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int segs = (m + SEG - 1) / SEG, first = item - seg;
+    const int k0 = seg * SEG, n0 = min(SEG, m - k0);
+    const float mg[3] = {sl.mu(g, 0), sl.mu(g, 1), sl.mu(g, 2)};
+    float a[4] = {0.f, 0.f, 0.f, 0.f};         // w (mu - c), w
+#pragma unroll
+    for (int u = 0; u < SEG / FTH; ++u) {
+        const int k = tid + u * FTH;
+        if (k >= n0) continue;
+        const int s = mem[k0 + k];
+        const float w = sl.w(s);
+        ids[k] = s;
+        ws[k] = w;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a[c] += w * (sl.mu(s, c) - mg[c]);
+        a[3] += w;
+    }
+    int n = n0;
+    if (seg == 0) {                            // the winner itself
+        if (tid == 0) {
+            ids[n0] = g;
+            ws[n0] = sl.w(g);
+            a[3] += ws[n0];
+        }
+        ++n;
+    }
+    block_sum<4>(a, s_red, lane, warp);        // (its barriers also cover ids and ws)
+    float *mine = sums + (int64_t)item * (4 + F);
+    const bool one = segs == 1;
+    {
+        const bool own = a[3] > 0.f;
+        float *of = one ? out_feat + (int64_t)g * F : mine + 4;
+        auto put = [&](int j, float x) { of[j] = one ? (own ? x / a[3] : 0.f) : x; };
+        if (vec) segment_features<4>(sl, ids, ws, n, s_part, lane, warp, put);
+        else segment_features<1>(sl, ids, ws, n, reinterpret_cast<float(*)[1]>(&s_part[0][0]), lane, warp, put);
+    }
+    if (!one) {
+        if (tid < 4) {
+            float v = a[0];                    // (no dynamic index into registers)
+#pragma unroll
+            for (int c = 1; c < 4; ++c) v = tid == c ? a[c] : v;
+            mine[tid] = v;
+        }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) s_last = atomicAdd(done, 1) == segs - 1;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        const float *all = sums + (int64_t)first * (4 + F);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) a[c] = 0.f;
+        for (int q = 0; q < segs; ++q)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) a[c] += __ldcg(all + (int64_t)q * (4 + F) + c);
+        for (int j = tid; j < F; j += FTH) {
+            float x = 0.f;
+#pragma unroll 4
+            for (int q = 0; q < segs; ++q) x += __ldcg(all + (int64_t)q * (4 + F) + 4 + j);
+            out_feat[(int64_t)g * F + j] = a[3] > 0.f ? x / a[3] : 0.f;
+        }
+    }
+    const float W = a[3];
+    const bool own = W > 0.f;
+    const float mean[3] = {mg[0] + a[0] / W, mg[1] + a[1] / W, mg[2] + a[2] / W};
+    const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
+    float cv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    auto add = [&](int s) {
+        const float w = sl.w(s), d[3] = {sl.mu(s, 0) - mean[0], sl.mu(s, 1) - mean[1], sl.mu(s, 2) - mean[2]};
+#pragma unroll
+        for (int c = 0; c < 6; ++c) cv[c] += w * (sl.cv(s, c) + d[ia[c]] * d[ib[c]]);
+    };
+    if (tid == 0) add(g);
+#pragma unroll 2
+    for (int k = tid; k < m; k += FTH) add(mem[k]);
+    block_sum<6>(cv, s_red, lane, warp);
+    if (tid == 0) {
+        out_w[g] = own ? W : 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) out_mu[(int64_t)c * T + g] = own ? mean[c] : 0.f;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) out_cov[(int64_t)c * T + g] = own ? cv[c] / W : 0.f;
+    }
+}
+
+// The work items of the winners of more than BIG_MEMBERS members.  Bound by the
+// gather of the members' rows: with one block per such winner and its members'
+// loads one after the other, 100,000 detections of 70 entities (F = 64) took
+// 1,734 us here and 300,000 of 40 11.4 ms; in segments with several loads in
+// flight per lane, 64 and 202.  Nothing to do: 2.5 us.
+__global__ void __launch_bounds__(FTH)
+assoc_fuse_big_kernel(Slots sl, const int32_t *__restrict__ mcnt, const int32_t *__restrict__ off,
+                      const int32_t *__restrict__ members, const int2 *__restrict__ items,
+                      const int32_t *__restrict__ n_items, int32_t *done, float *sums, float *__restrict__ out_w,
+                      float *__restrict__ out_mu, float *__restrict__ out_cov, float *__restrict__ out_feat, int vec)
+{
+    const int count = *n_items;
+    for (int k = blockIdx.x; k < count; k += gridDim.x) {
+        const int2 it = items[k];
+        fuse_big(sl, it.x, it.y, k, members + off[it.x], mcnt[it.x], done + it.x, sums, vec, out_w, out_mu, out_cov,
+                 out_feat);
+        __syncthreads();             // the next segment reuses the shared arrays
+    }
+}
+
+// out_w, out_mu, out_cov and out_feat of the other slots, a warp each: zeros for
+// a merged one, the slot's own values for a winner without members, sums over
+// the members (listed at members + off) otherwise.
+__global__ void __launch_bounds__(FTH)
 assoc_fuse_kernel(Slots sl, const int32_t *__restrict__ parent, const int32_t *__restrict__ mcnt,
                   const int32_t *__restrict__ off, const int32_t *__restrict__ members, float *__restrict__ out_w,
                   float *__restrict__ out_mu, float *__restrict__ out_cov, float *__restrict__ out_feat, int vec)
 {
-    __shared__ float s_part[FW][FCHUNK];
-    __shared__ float s_sum[FW][4], s_cov[FW][6], s_mean[4];
     const int T = sl.N + sl.B, F = sl.F;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-    const int t0 = blockIdx.x * FW, t = t0 + warp;
+    const int t = blockIdx.x * FW + warp;
     const unsigned FULL = 0xffffffffu;
     if (t < T) {
         // (the slot's first features are in flight while the rest is looked up)
@@ -452,80 +655,6 @@ assoc_fuse_kernel(Slots sl, const int32_t *__restrict__ parent, const int32_t *_
             }
         }
     }
-    // winners of many members: the block's warps take every FW-th of them
-    for (int q = 0; q < FW; ++q) {
-        const int g = t0 + q;
-        if (g >= T || parent[g] != g || mcnt[g] <= BIG_MEMBERS) continue;     // (uniform across the block)
-        const int m = mcnt[g];
-        const int32_t *mem = members + off[g];
-        float W = warp == 0 ? sl.w(g) : 0.f, dm = 0.f;
-        const float mt = lane < 3 ? sl.mu(g, lane) : 0.f;
-        for (int k = warp; k < m; k += FW) {
-            const int s = mem[k];
-            const float w = sl.w(s);
-            W += w;
-            if (lane < 3) dm += w * (sl.mu(s, lane) - mt);
-        }
-        if (lane < 3) s_sum[warp][lane] = dm;
-        if (lane == 3) s_sum[warp][3] = W;
-        __syncthreads();
-        if (warp == 0 && lane < 4) {
-            float x = 0.f;
-            for (int v = 0; v < FW; ++v) x += s_sum[v][lane];
-            s_mean[lane] = x;
-        }
-        __syncthreads();
-        W = s_mean[3];
-        const bool own = W > 0.f;
-        const int c = lane < 6 ? lane : 0, a = ia[c], b = ib[c];
-        const float ma = sl.mu(g, a) + s_mean[a] / W, mb = sl.mu(g, b) + s_mean[b] / W;
-        if (lane < 6) {
-            float acc = warp == 0 ? sl.w(g) * (sl.cv(g, c) + (sl.mu(g, a) - ma) * (sl.mu(g, b) - mb)) : 0.f;
-            for (int k = warp; k < m; k += FW) {
-                const int s = mem[k];
-                acc += sl.w(s) * (sl.cv(s, c) + (sl.mu(s, a) - ma) * (sl.mu(s, b) - mb));
-            }
-            s_cov[warp][c] = acc;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            if (lane == 0) out_w[g] = own ? W : 0.f;
-            if (lane < 3) out_mu[(int64_t)lane * T + g] = own ? mt + s_mean[lane] / W : 0.f;
-            if (lane < 6) {
-                float x = 0.f;
-                for (int v = 0; v < FW; ++v) x += s_cov[v][lane];
-                out_cov[(int64_t)lane * T + g] = own ? x / W : 0.f;
-            }
-        }
-        for (int f0 = 0; f0 < F; f0 += FCHUNK) {
-            const int fn = min(FCHUNK, F - f0);
-            float acc[FCHUNK / 32];
-#pragma unroll
-            for (int u = 0; u < FCHUNK / 32; ++u) {
-                const int j = lane + 32 * u;
-                acc[u] = warp == 0 && j < fn ? sl.w(g) * sl.feat(g)[f0 + j] : 0.f;
-            }
-            for (int k = warp; k < m; k += FW) {
-                const int s = mem[k];
-                const float w = sl.w(s);
-                const float *fs = sl.feat(s) + f0;
-#pragma unroll
-                for (int u = 0; u < FCHUNK / 32; ++u) {
-                    const int j = lane + 32 * u;
-                    if (j < fn) acc[u] = fmaf(w, __ldg(fs + j), acc[u]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < FCHUNK / 32; ++u) s_part[warp][lane + 32 * u] = acc[u];
-            __syncthreads();
-            for (int j = threadIdx.x; j < fn; j += FW * 32) {
-                float x = 0.f;
-                for (int v = 0; v < FW; ++v) x += s_part[v][j];
-                out_feat[(int64_t)g * F + f0 + j] = own ? x / W : 0.f;
-            }
-            __syncthreads();
-        }
-    }
 }
 
 }  // namespace
@@ -563,15 +692,18 @@ cudaError_t launch_assoc(const AssocArgs &a, cudaStream_t s)
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     assoc_parent_kernel<<<nb, 256, 0, s>>>(T, a.members, a.win, a.parent, a.mcnt, a.pos);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    assoc_offset_kernel<<<nb, 256, 0, s>>>(T, a.mcnt, a.off, a.counters);
+    assoc_offset_kernel<<<nb, 256, 0, s>>>(T, a.mcnt, a.off, a.pos, a.counters, a.items);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     assoc_members_kernel<<<nb, 256, 0, s>>>(T, a.parent, a.off, a.pos, a.members);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const Slots sl{N, B, a.F, a.ent_mu, a.ent_cov, a.ent_feat, a.ent_w, a.det_mu, a.det_cov, a.det_feat};
     const uintptr_t al = (uintptr_t)a.ent_feat | (uintptr_t)a.det_feat | (uintptr_t)a.out_feat;
     const int vec = a.F % 4 == 0 && (al & 15u) == 0 ? 1 : 0;
-    assoc_fuse_kernel<<<(unsigned)((T + FW - 1) / FW), FW * 32, 0, s>>>(sl, a.parent, a.mcnt, a.off, a.members, a.out_w,
-                                                                        a.out_mu, a.out_cov, a.out_feat, vec);
+    assoc_fuse_kernel<<<(unsigned)((T + FW - 1) / FW), FTH, 0, s>>>(sl, a.parent, a.mcnt, a.off, a.members, a.out_w,
+                                                                    a.out_mu, a.out_cov, a.out_feat, vec);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    assoc_fuse_big_kernel<<<BIG_BLOCKS, FTH, 0, s>>>(sl, a.mcnt, a.off, a.members, a.items, a.counters + kAssocItems,
+                                                     a.pos, a.sums, a.out_w, a.out_mu, a.out_cov, a.out_feat, vec);
     return cudaGetLastError();
 }
 
