@@ -231,14 +231,14 @@ assoc_search_kernel(const float *__restrict__ S, int64_t ld, int32_t N, int32_t 
 {
     __shared__ uint64_t cand[CAPA];
     __shared__ int32_t pre[CAPP];
-    __shared__ int s_cnt, s_np;
+    __shared__ int s_cnt, s_np[3];
     const int tid = threadIdx.x;
     const int count = over ? *n_over : B;
     for (int at = blockIdx.x; at < count; at += gridDim.x) {
         const int d = over ? over[at] : at;
         if (tid == 0) {
             s_cnt = 0;
-            s_np = 0;
+            s_np[0] = s_np[1] = s_np[2] = 0;
         }
         __syncthreads();
         float md[3], cd[6];
@@ -266,7 +266,10 @@ assoc_search_kernel(const float *__restrict__ S, int64_t ld, int32_t N, int32_t 
                 }
             }
         };
-        for (int g0 = 0; g0 < n4; g0 += TA * 4) {
+        // (a pass counts its entities past the `base` before it in a counter of its
+        // own: warps that are ahead fill the next pass's while others read this one's)
+        int base = 0, pass = 0;
+        for (int g0 = 0; g0 < n4; g0 += TA * 4, pass = pass == 2 ? 0 : pass + 1) {
             float4 v[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -279,18 +282,19 @@ assoc_search_kernel(const float *__restrict__ S, int64_t ld, int32_t N, int32_t 
                 const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    if (x[c] >= tau_f && e0 + c < N) pre[atomicAdd(&s_np, 1)] = e0 + c;
+                    if (x[c] >= tau_f && e0 + c < N) pre[base + atomicAdd(&s_np[pass], 1)] = e0 + c;
             }
             __syncthreads();
-            const int np = s_np;
-            if (np > CAPP - PER_PASS) {      // (uniform) at most PER_PASS more could come in the next pass
-                evaluate(np);
+            base += s_np[pass];
+            // (the previous pass's counter, read before this pass's barrier, is filled again in two passes)
+            if (tid == 0) s_np[pass == 0 ? 2 : pass - 1] = 0;
+            if (base > CAPP - PER_PASS) {    // (uniform) at most PER_PASS more could come in the next pass
+                evaluate(base);
                 __syncthreads();
-                if (tid == 0) s_np = 0;
-                __syncthreads();
+                base = 0;
             }
         }
-        evaluate(s_np);
+        evaluate(base);
         __syncthreads();
         finish_matches(cand, s_cnt, d, N, max_m, match_cnt, match_idx, match_h, label, err);
         __syncthreads();          // the next detection reuses the shared arrays
