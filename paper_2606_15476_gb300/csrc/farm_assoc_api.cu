@@ -13,11 +13,12 @@ using farm::Ctx;
 namespace {
 
 // From this many cosines on a call keeps those reaching tau_f instead of storing
-// all.  Fewer (24 MB) stay in the L2, and the two launches that the lists need
-// cost more than they save: 307 detections x 589 entities 41.5 us with lists,
-// 34.8 stored; 1,000 x 4,000 41.6, 36.7.  At 8 million the two are even (4,000 x
-// 2,000 74.4, 72.0; 1,000 x 8,000 43.4, 44.3); 1,000 x 16,000 73.8, 83.1; 1,500
-// x 30,000 135, 176.
+// all.  Fewer (24 MB) stay in the L2, and the launches that the lists need cost
+// more than they save: with F = 256, 307 detections x 589 entities 73 us with
+// lists, 59 stored; 1,000 x 4,000 79, 73.  At 6 to 8 million the two are even
+// (1,000 x 6,300 87.7, 85.1; 4,000 x 2,000 97.9, 100.3; 1,000 x 8,000 87.6,
+// 86.6); 1,000 x 16,000 107, 118; 16,000 x 1,000 152, 176; 1,500 x 30,000 163,
+// 214.
 constexpr int64_t kEmitCosines = int64_t(6) << 20;
 
 farm_status afail(Ctx &c, farm_status st, const std::string &msg)
@@ -92,10 +93,11 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
     int32_t *h_eact = nullptr;
     // more detections than the few-row similarity takes, and more cosines than
     // kEmitCosines: only those reaching tau_f are kept, up to `cap` per
-    // detection (about as many as a fused selection's row; more of them: the
-    // stored rows)
+    // detection; more of them: that detection's row is stored.  The lists lie in
+    // the place of the rows (at most as long), which are stored once the lists
+    // have been read.
     const bool emitting = B > farm::kSimFewRows && (int64_t)B * N >= kEmitCosines;
-    const int32_t cap = farm::fuse_merge_capacity(1);
+    const int32_t cap = (int32_t)std::min<int64_t>(farm::fuse_merge_capacity(1), ld / 2);
     // the layout of the call's device memory: sized with a null base, then
     // carved from the context's grow-only buffer
     auto layout = [&](Carve &cv) {
@@ -118,8 +120,10 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
         if (emitting) {
             a.over = cv.take<int32_t>((size_t)B);
             a.emit.tau_key = cv.take<uint32_t>((size_t)B); a.emit.cnt = cv.take<int32_t>((size_t)B);
-            a.emit.cand = cv.take<uint64_t>((size_t)B * cap);
+            a.emit.cand = reinterpret_cast<uint64_t *>(S);
             a.emit.cap = cap;
+            a.emit.gate = a.counters + farm::kAssocListRows;
+            a.chi = cv.take<uint16_t>((size_t)B * F_pad); a.clo = cv.take<uint16_t>((size_t)B * F_pad);
         }
         if (dev) {
             a.match_cnt = match_cnt; a.match_idx = match_idx; a.match_h = match_h; a.parent = parent;
@@ -178,6 +182,11 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
     a.h_max = h_max;
     a.max_m = max_m;
     a.err = c.d_err;
+    a.dhi = dhi;
+    a.dlo = dlo;
+    a.ehi = ehi;
+    a.F_pad = F_pad;
+    a.probe = c.d_probe;
     c.launches += emitting ? 11 : 9;
     ACK(farm::launch_assoc_init(a, c.stream), "association kernels");
     if (emitting) {
@@ -185,8 +194,9 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
                                       c.stream, &a.emit), "feature cosines");
         ACK(farm::launch_assoc_match(a, c.stream), "association kernels");
     }
-    ACK(farm::launch_sim_tc_f16x3(dhi, dlo, ehi, elo, S, B, N, F_pad, ld, nullptr, c.num_sms, c.d_err, c.stream,
-                                  nullptr, emitting ? a.counters + 1 : nullptr), "feature cosines");
+    ACK(farm::launch_sim_tc_f16x3(emitting ? a.chi : dhi, emitting ? a.clo : dlo, ehi, elo, S, B, N, F_pad, ld, nullptr,
+                                  c.num_sms, c.d_err, c.stream, nullptr, emitting ? a.counters + 1 : nullptr),
+        "feature cosines");
     ACK(farm::launch_assoc(a, c.stream), "association kernels");
     if (!dev) {
         const cudaMemcpyKind k = cudaMemcpyDeviceToHost;

@@ -160,6 +160,7 @@ struct Ctx {
     std::map<int64_t, int> tuned; // similarity class -> fastest tile variant (autotuner)
     int pinned_variant = -1;      // >= 0: every grouped similarity launch uses this variant
     int32_t *d_fallback = nullptr;  // rows the thresholded select handed to its exact fallback
+    int32_t *d_probe = nullptr;     // counts of a kernel that samples (0 between calls)
     int32_t *h_err = nullptr;     // pinned host mirror
     // batch state
     uint64_t batch_gen = 0;
@@ -427,7 +428,9 @@ inline int sim_single_variant(int64_t rows, int64_t n, int num_sms)
 // row: each row's threshold (order-preserving key of its sample's R-th
 // value), candidate count and buffer of `cap` candidate words
 // (key << 32 | (2^32 - 1 - object index)).
-// gate (nullable, any launch): the kernel returns at once when *gate is 0.
+// gate (nullable, launches of one problem): only the problem's first *gate rows
+// are computed (none: the kernel returns at once, an emitting one with every
+// row's count past any capacity).
 struct FuseEmit {
     uint32_t *tau_key;
     int32_t *cnt;
@@ -474,8 +477,8 @@ cudaError_t preload_sim_few();
 // Three FP16 terms, hi*hi + 2^-11 (hi*lo + lo*hi), from the split the
 // normalisation writes.
 // With `emit` (more than kSimFewRows rows) nothing is stored: every entry
-// reaching its row's threshold is appended to the row's buffer; with a gate the
-// launch does its work only when *gate is not 0.
+// reaching its row's threshold is appended to the row's buffer; with a gate
+// only the first *gate rows are computed.
 cudaError_t launch_sim_tc_f16x3(const uint16_t *q_hi, const uint16_t *q_lo, const uint16_t *d_hi,
                                 const uint16_t *d_lo, float *S, int64_t rows, int64_t n, int32_t dim_pad,
                                 int64_t ld_s, float *tops, int num_sms, int32_t *err, cudaStream_t s,
@@ -728,7 +731,7 @@ struct FuseArgs {
 cudaError_t launch_fuse(const FuseArgs &a, int part, cudaStream_t s);
 
 // Mapping-side association (k_assoc.cu): device arrays only.
-constexpr int kAssocItems = 2, kAssocCounters = 3;
+constexpr int kAssocItems = 2, kAssocTicket = 3, kAssocListRows = 4, kAssocCounters = 5;
 // The most work items that T slots can have: winners of at least 65 members, a
 // segment per 1,024 of them.
 inline int64_t assoc_items_of(int64_t T) { return T / 64 + T / 1024 + 1; }
@@ -746,19 +749,24 @@ struct AssocArgs {
     int32_t *label;                     // [N + B] scratch: component labels
     unsigned long long *win;            // [N + B] scratch: winners
     int32_t *mcnt, *off, *pos, *members;    // [N + B] scratch: each winner's members
-    int32_t *counters;                  // [kAssocCounters] scratch: members' array in use; detections whose list
-                                        // overflowed; work items of the fusion
+    int32_t *counters;                  // [kAssocCounters] scratch: members' array in use; detections to search
+                                        // over stored rows; work items of the fusion; such
+                                        // detections taken; rows to emit for (all or 0)
     int2 *items;                        // [assoc_items_of(T)] scratch: those items, (winner, segment)
     float *sums;                        // [items, 4 + F] scratch: their sums
     int32_t *over;                      // [B] scratch: those detections
-    FuseEmit emit;                      // the emitting similarity's lists (cnt null: stored rows)
+    const uint16_t *dhi, *dlo, *ehi;    // unit features in the FP16 split, F_pad per row
+    uint16_t *chi, *clo;                // [B, F_pad] scratch: the rows of those detections
+    int32_t F_pad;
+    int32_t *probe;                     // [1] 0 before and after (the context's)
+    FuseEmit emit;                      // the emitting similarity's lists (cnt null: stored rows; cand: in S's place)
     int32_t *parent;                    // [N + B]
     float *out_w, *out_mu, *out_cov, *out_feat;         // [T], [3, T], [6, T], [T, F]
     int32_t *err;
 };
-// In stream order: init; the similarity (emitting, then launch_assoc_match and
-// the storing form behind the gate counters + 1; or storing every row); the
-// rest.
+// In stream order: init; the similarity (emitting for counters[kAssocListRows]
+// rows, then launch_assoc_match and the storing form over the first counters[1]
+// rows of chi / clo; or storing every row); the rest.
 cudaError_t launch_assoc_init(const AssocArgs &a, cudaStream_t s);
 cudaError_t launch_assoc_match(const AssocArgs &a, cudaStream_t s);
 cudaError_t launch_assoc(const AssocArgs &a, cudaStream_t s);

@@ -12,8 +12,10 @@
 //    enough cosines, of more than kSimFewRows detections, the similarity kernel
 //    keeps only those reaching tau_f (the emitting form of the fused rank selection, its
 //    threshold tau_f for every row), so the detection-by-entity block is
-//    neither written nor read; a detection with more of them than its buffer
-//    holds is searched over its stored row, which is then computed;
+//    neither written nor read; the detections with more of them than their
+//    buffers hold are gathered, and those rows computed again, stored and
+//    searched (every row is, without lists, when a sample of the cosines says
+//    that most would overflow);
 //  * correspondence: the connected components of the graph joining each
 //    detection (node N + d) to its matches: a union-find over smallest nodes
 //    (roots hooked by compare-and-swap: every step moves a label to a smaller
@@ -34,6 +36,8 @@
 // (search 106 -> 25 us, components 57 -> the match kernel's tail, fusion and its
 // clearing 106 -> 39; the similarity 124 -> 111, 60% of the tensor rate: 17
 // tiles of eight K slices per CTA pair, each waiting for its fold).
+#include <cuda_fp16.h>
+
 #include "farm_internal.h"
 
 namespace farm {
@@ -160,43 +164,123 @@ __device__ __forceinline__ void finish_matches(uint64_t *cand, int cnt, int d, i
     }
 }
 
+constexpr int PROBE_BLOCKS = 64, PROBE_PAIRS = 2;      // of them, and cosines a warp samples
+
 // Before the search: labels, winners and member counts cleared; with the
-// emitting similarity, every detection's threshold and an empty buffer.
+// emitting similarity, every detection's threshold and an empty buffer, and
+// whether to emit at all.  A list that overflows costs a second product of its
+// row, and appending most of a row costs more than storing it, so 1,024 cosines
+// of detections and entities spread over both (the FP16 parts' leading ones) are
+// compared with tau_f, and with so many of them above it that the mean list would
+// fill more than 7/8 of a buffer every row is stored (the last of the sampling
+// warps decides).  4,096 x 20,000, F = 256: 3,000 of the entities alike 330 us
+// (323 with every row stored; 293 and 212 where all lists fit), classes of 2,222
+// 588 (563), all of one class 1,134 (1,111); without the sample, and a second
+// product of every row once a list overflows, 454, 1,070 and 2,490.
 __global__ void __launch_bounds__(256)
-assoc_init_kernel(int32_t T, int32_t B, float tau_f, int32_t *__restrict__ label, unsigned long long *__restrict__ win,
-                  int32_t *__restrict__ mcnt, int32_t *__restrict__ counters, uint32_t *__restrict__ tau_key,
-                  int32_t *__restrict__ cnt)
+assoc_init_kernel(int32_t T, int32_t N, int32_t B, float tau_f, int32_t *__restrict__ label,
+                  unsigned long long *__restrict__ win, int32_t *__restrict__ mcnt, int32_t *__restrict__ counters,
+                  uint32_t *__restrict__ tau_key, int32_t *__restrict__ cnt, int32_t cap,
+                  const uint16_t *__restrict__ dhi, const uint16_t *__restrict__ ehi, int32_t F_pad, int32_t *probe)
 {
-    const int t = blockIdx.x * 256 + threadIdx.x;
-    if (t < kAssocCounters) counters[t] = 0;
+    const int tid = threadIdx.x, t = blockIdx.x * 256 + tid;
+    if (t < kAssocListRows) counters[t] = 0;
     if (t < T) {
         label[t] = t;
         win[t] = 0ull;
         mcnt[t] = 0;
     }
-    if (tau_key && t < B) {
+    if (!tau_key) return;
+    if (t < B) {
         const uint32_t u = __float_as_uint(tau_f + 0.0f);      // the order key of the similarity kernels
         tau_key[t] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
         cnt[t] = 0;
+    }
+    const int blocks = min((int)gridDim.x, PROBE_BLOCKS);
+    if ((int)blockIdx.x >= blocks) return;
+    const int lane = tid & 31, pairs = blocks * 8 * PROBE_PAIRS, p0 = (blockIdx.x * 8 + (tid >> 5)) * PROBE_PAIRS;
+    const uint4 *x[PROBE_PAIRS], *y[PROBE_PAIRS];
+    float dot[PROBE_PAIRS];
+#pragma unroll
+    for (int k = 0; k < PROBE_PAIRS; ++k) {
+        const uint32_t p = (uint32_t)(p0 + k);
+        const int64_t d = (int64_t)p * B / pairs, e = (int64_t)(((uint64_t)(p * 2654435761u) * (uint32_t)N) >> 32);
+        x[k] = reinterpret_cast<const uint4 *>(dhi + d * F_pad);
+        y[k] = reinterpret_cast<const uint4 *>(ehi + e * F_pad);
+        dot[k] = 0.f;
+    }
+#pragma unroll 4
+    for (int j = lane; j < F_pad / 8; j += 32) {
+#pragma unroll
+        for (int k = 0; k < PROBE_PAIRS; ++k) {
+            const uint4 u = __ldg(x[k] + j), v = __ldg(y[k] + j);
+            const uint32_t ua[4] = {u.x, u.y, u.z, u.w}, va[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&ua[i]));
+                const float2 g = __half22float2(*reinterpret_cast<const __half2 *>(&va[i]));
+                dot[k] = fmaf(f.x, g.x, fmaf(f.y, g.y, dot[k]));
+            }
+        }
+    }
+    int hits = 0;
+#pragma unroll
+    for (int k = 0; k < PROBE_PAIRS; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dot[k] += __shfl_xor_sync(0xffffffffu, dot[k], o);
+        hits += dot[k] >= tau_f ? 1 : 0;
+    }
+    // (one word counts the warps and their hits)
+    if (lane == 0) {
+        const int old = atomicAdd(probe, (1 << 16) | hits);
+        if (old >> 16 == blocks * 8 - 1) {
+            const int64_t all = (old & 0xffff) + hits;
+            atomicExch(probe, 0);
+            counters[kAssocListRows] = all * N * 8 <= (int64_t)pairs * cap * 7 ? B : 0;
+        }
+    }
+}
+
+// The unit features' FP16 parts, and the place for those of listed detections.
+struct OverRows {
+    const uint16_t *dhi, *dlo;
+    uint16_t *chi, *clo;
+    int32_t F_pad;
+};
+
+// Row d's to row k, by the block (out of line: few detections take it).
+__device__ __noinline__ void copy_operands(const OverRows o, int d, int k)
+{
+    const int64_t from = (int64_t)d * o.F_pad, to = (int64_t)k * o.F_pad;
+    for (int j = 8 * threadIdx.x; j < o.F_pad; j += 8 * TA) {
+        *reinterpret_cast<uint4 *>(o.chi + to + j) = __ldg(reinterpret_cast<const uint4 *>(o.dhi + from + j));
+        *reinterpret_cast<uint4 *>(o.clo + to + j) = __ldg(reinterpret_cast<const uint4 *>(o.dlo + from + j));
     }
 }
 
 // One CTA per detection over the entities its cosine row reached tau_f for
 // (buffered by the similarity kernel, in any order); a detection whose buffer
-// overflowed is listed for assoc_search_kernel.
-__global__ void __launch_bounds__(TA)
+// overflowed (every one's, when nothing was emitted) is listed for
+// assoc_search_kernel, and its unit feature copied to the next row of those that
+// the storing similarity multiplies.
+__global__ void __launch_bounds__(TA, 12)
 assoc_match_kernel(FuseEmit emit, int32_t N, int32_t B, const float *__restrict__ ent_mu,
                    const float *__restrict__ ent_cov, const int32_t *__restrict__ ent_active,
                    const float *__restrict__ det_mu, const float *__restrict__ det_cov, float h_max, int32_t max_m,
                    int32_t *__restrict__ match_cnt, int32_t *__restrict__ match_idx, float *__restrict__ match_h,
-                   int32_t *label, int32_t *n_over, int32_t *__restrict__ over, int32_t *err)
+                   int32_t *label, int32_t *n_over, int32_t *__restrict__ over, const OverRows rows, int32_t *err)
 {
     __shared__ uint64_t cand[CAPA];
     __shared__ int s_cnt;
     const int d = blockIdx.x, tid = threadIdx.x;
     const int np = emit.cnt[d];
     if (np > emit.cap) {
-        if (tid == 0) over[atomicAdd(n_over, 1)] = d;
+        if (tid == 0) {
+            s_cnt = atomicAdd(n_over, 1);
+            over[s_cnt] = d;
+        }
+        __syncthreads();
+        copy_operands(rows, d, s_cnt);
         return;
     }
     if (tid == 0) s_cnt = 0;
@@ -220,27 +304,32 @@ assoc_match_kernel(FuseEmit emit, int32_t N, int32_t B, const float *__restrict_
 }
 
 // Detections over their stored cosine rows: all B of them, or (over non-null)
-// the *n_over listed ones.
+// the *n_over listed ones, the k-th of whose rows is S's k-th.
 __global__ void __launch_bounds__(TA)
 assoc_search_kernel(const float *__restrict__ S, int64_t ld, int32_t N, int32_t B, const float *__restrict__ ent_mu,
                     const float *__restrict__ ent_cov, const int32_t *__restrict__ ent_active,
                     const float *__restrict__ det_mu, const float *__restrict__ det_cov, float tau_f, float h_max,
                     int32_t max_m, int32_t *__restrict__ match_cnt, int32_t *__restrict__ match_idx,
                     float *__restrict__ match_h, int32_t *label, const int32_t *n_over,
-                    const int32_t *__restrict__ over, int32_t *err)
+                    const int32_t *__restrict__ over, int32_t *ticket, int32_t *err)
 {
     __shared__ uint64_t cand[CAPA];
     __shared__ int32_t pre[CAPP];
-    __shared__ int s_cnt, s_np[3];
+    __shared__ int s_cnt, s_np[3], s_at;
     const int tid = threadIdx.x;
+    // (one by one from `ticket` where the grid is smaller than their number may be)
     const int count = over ? *n_over : B;
-    for (int at = blockIdx.x; at < count; at += gridDim.x) {
-        const int d = over ? over[at] : at;
+    if (count == 0) return;
+    for (;;) {
         if (tid == 0) {
             s_cnt = 0;
             s_np[0] = s_np[1] = s_np[2] = 0;
+            s_at = over ? atomicAdd(ticket, 1) : (int)blockIdx.x;
         }
         __syncthreads();
+        const int at = s_at;
+        if (at >= count) return;
+        const int d = over ? over[at] : at;
         float md[3], cd[6];
 #pragma unroll
         for (int k = 0; k < 3; ++k) md[k] = det_mu[(int64_t)k * B + d];
@@ -253,7 +342,7 @@ assoc_search_kernel(const float *__restrict__ S, int64_t ld, int32_t N, int32_t 
         // together (one entity per thread), whenever the list could overflow in
         // the next pass and at the end: evaluated where they are found, they
         // would each run on one lane of a warp
-        const float *row = S + (int64_t)d * ld;
+        const float *row = S + (int64_t)at * ld;
         const float4 *row4 = reinterpret_cast<const float4 *>(row);
         const int n4 = (N + 3) >> 2;
         auto evaluate = [&](int np) {
@@ -297,6 +386,7 @@ assoc_search_kernel(const float *__restrict__ S, int64_t ld, int32_t N, int32_t 
         evaluate(base);
         __syncthreads();
         finish_matches(cand, s_cnt, d, N, max_m, match_cnt, match_idx, match_h, label, err);
+        if (!over) return;
         __syncthreads();          // the next detection reuses the shared arrays
     }
 }
@@ -666,8 +756,9 @@ assoc_fuse_kernel(Slots sl, const int32_t *__restrict__ parent, const int32_t *_
 cudaError_t launch_assoc_init(const AssocArgs &a, cudaStream_t s)
 {
     const int32_t T = a.N + a.B;
-    assoc_init_kernel<<<(unsigned)((T + 255) / 256), 256, 0, s>>>(T, a.B, a.tau_f, a.label, a.win, a.mcnt, a.counters,
-                                                                   a.emit.tau_key, a.emit.cnt);
+    assoc_init_kernel<<<(unsigned)((T + 255) / 256), 256, 0, s>>>(T, a.N, a.B, a.tau_f, a.label, a.win, a.mcnt, a.counters,
+                                                                   a.emit.tau_key, a.emit.cnt, a.emit.cap, a.dhi,
+                                                                   a.ehi, a.F_pad, a.probe);
     return cudaGetLastError();
 }
 
@@ -675,7 +766,8 @@ cudaError_t launch_assoc_match(const AssocArgs &a, cudaStream_t s)
 {
     assoc_match_kernel<<<(unsigned)a.B, TA, 0, s>>>(a.emit, a.N, a.B, a.ent_mu, a.ent_cov, a.ent_active, a.det_mu,
                                                     a.det_cov, a.h_max, a.max_m, a.match_cnt, a.match_idx, a.match_h,
-                                                    a.label, a.counters + 1, a.over, a.err);
+                                                    a.label, a.counters + 1, a.over,
+                                                    OverRows{a.dhi, a.dlo, a.chi, a.clo, a.F_pad}, a.err);
     return cudaGetLastError();
 }
 
@@ -686,10 +778,10 @@ cudaError_t launch_assoc(const AssocArgs &a, cudaStream_t s)
     cudaError_t e;
     // the stored rows: all of them, or those the emitted lists overflowed for
     const int32_t *over = a.emit.cnt ? a.over : nullptr;
-    const unsigned grid = over ? (unsigned)(B < 304 ? B : 304) : (unsigned)B;
+    const unsigned grid = (unsigned)(over && B > 1368 ? 1368 : B);     // (nine CTAs to an SM)
     assoc_search_kernel<<<grid, TA, 0, s>>>(a.S, a.ld, N, B, a.ent_mu, a.ent_cov, a.ent_active, a.det_mu, a.det_cov,
                                             a.tau_f, a.h_max, a.max_m, a.match_cnt, a.match_idx, a.match_h, a.label,
-                                            a.counters + 1, over, a.err);
+                                            a.counters + 1, over, a.counters + kAssocTicket, a.err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const unsigned nb = (unsigned)((T + 255) / 256);
     assoc_winner_kernel<<<nb, 256, 0, s>>>(N, T, a.ent_w, a.label, a.members, a.win);    // (roots: before the members)

@@ -368,7 +368,28 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
     uint64_t *emit_slots = reinterpret_cast<uint64_t *>(reinterpret_cast<uint8_t *>(tile_scales) + C::SCALE_BYTES);
     uint64_t *corr_free = acc_empty + 1;      // FOLD: the correction columns are free (tile accumulators: one)
 
-    if (emit.gate && *emit.gate == 0) return;      // (every thread of the launch alike)
+    // one problem behind a gate: its first *gate rows only (every thread of the launch alike)
+    if constexpr (!GROUPED) {
+        if (emit.gate) {
+            const int64_t rows = min(single.rows, *emit.gate);
+            if (rows <= 0) {
+                // (an emitting launch that does nothing leaves every list overflowed)
+                if constexpr (EMIT)
+                    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < single.rows;
+                         r += (int64_t)gridDim.x * blockDim.x)
+                        emit.cnt[r] = 0x7fffffff;
+                return;
+            }
+            const int64_t mt = (rows + BM - 1) / BM;
+            total = min(total, (int32_t)((mt + CM - 1) / CM * col_tiles(single.n, BN, kColAll, 0)));
+        }
+    }
+    auto piece_at = [&](int tile) {
+        GemmPiece p = piece_of<GROUPED>(tile, pieces, n_pieces, single);
+        if constexpr (!GROUPED)
+            if (emit.gate) p.rows = min(p.rows, *emit.gate);
+        return p;
+    };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const int cluster_id = blockIdx.x / CM, n_clusters = gridDim.x / CM;
@@ -407,7 +428,7 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
         if (lane == 0) {
             uint32_t it = 0;
             for (int tile = cluster_id; tile < total && !*abort_flag; tile += n_clusters) {
-                const GemmPiece pc = piece_of<GROUPED>(tile, pieces, n_pieces, single);
+                const GemmPiece pc = piece_at(tile);
                 int m0, n0, c0;
                 piece_tile<BN_, CM_>(pc, tile, rank, m0, n0, c0);
                 const int qa = (int)(pc.q_row0 + m0);     // A rows: the piece's rows in the operand arrays
@@ -598,7 +619,7 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
             GemmPiece pc;
             int m0 = 0, n0 = 0, c0 = 0;
             if constexpr (EMIT || !FOLD) {
-                pc = piece_of<GROUPED>(tile, pieces, n_pieces, single);
+                pc = piece_at(tile);
                 piece_tile<BN_, CM_>(pc, tile, rank, m0, n0, c0);
                 const int64_t tr = (int64_t)m0 + quad * 32 + lane;
                 if (EMIT && tr < pc.rows) tk = __ldg(emit.tau_key + pc.q_row0 + tr);
@@ -652,7 +673,7 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
                 }
             }
             if constexpr (FOLD) {
-                pc = piece_of<GROUPED>(tile, pieces, n_pieces, single);
+                pc = piece_at(tile);
                 piece_tile<BN_, CM_>(pc, tile, rank, m0, n0, c0);
             }
             const int64_t r = (int64_t)m0 + quad * 32 + lane;    // row within the piece
