@@ -92,21 +92,26 @@ __device__ __noinline__ float entity_distance(int e, int32_t N, const float *__r
     return hellinger_f(md, cd, me, ce);
 }
 
-// The union-find over node labels (label[x] <= x, a root labels itself).  Nodes
-// on a walk are pointed at their grandparents; labels are read past L1.
+// The union-find over node labels: label[x] <= x, and a root labels itself, so a
+// label other than the node's own is always of an ancestor with a smaller
+// number.  The walk to the root shortens its path as it goes, by halving
+// (Tarjan and van Leeuwen, J. ACM 31, 1984; used on GPUs as intermediate pointer
+// jumping by Jaiganesh and Burtscher, HPDC 2018): a node is given its
+// grandparent and the walk goes on there.  Walks run against one another and
+// against the hooking of roots: whatever label a plain store leaves in a node that
+// is no root is an ancestor's, and a root is changed by compare-and-swap only.
+// Labels are read past L1.
 __device__ __forceinline__ int find_root(int32_t *label, int x)
 {
-    volatile int32_t *l = label;
-    int cur = l[x];
-    if (cur != x) {
-        int prev = x, next;
-        while (cur > (next = l[cur])) {
-            l[prev] = next;
-            prev = cur;
-            cur = next;
-        }
+    volatile int32_t *const up = label;
+    for (;;) {
+        const int parent = up[x];
+        if (parent == x) return x;
+        const int grand = up[parent];
+        if (grand == parent) return parent;
+        up[x] = grand;
+        x = grand;
     }
-    return cur;
 }
 
 __device__ __forceinline__ void unite(int32_t *label, int u, int v)
