@@ -423,8 +423,8 @@ farm_status farm_similarity_variant(farm_ctx *ctx, int32_t scene_id, int64_t n_r
 
 /*
  * Frees an uploaded scene's device memory (after the context's queued work);
- * the scene id may then be uploaded again.  FARM_EINVAL for an id that holds
- * no scene.  Synchronises.
+ * the scene id may then be uploaded again.  Also frees what farm_mlp_train left
+ * with the context.  FARM_EINVAL for an id that holds no scene.  Synchronises.
  */
 farm_status farm_memory_release(farm_ctx *ctx, int32_t scene_id);
 
@@ -524,7 +524,10 @@ farm_status farm_rank_rows_noalloc(farm_ctx *ctx, int32_t scene_id, int64_t n_ro
  *   host, normalised on the GPU) with object pair_obj[i] of scene
  *   scene_ids[pair_scene[i]] (pair_scene may be NULL when n_scenes == 1).
  *   loss_out[epoch] (nullable) receives the mean batch loss.  Starts from the
- *   installed weights.  Synchronises.
+ *   installed weights.  Synchronises.  The call's working memory and its copy
+ *   of the inputs, where they take at most 512 MB each, stay with the context
+ *   for the next training call, until farm_memory_release or farm_destroy, or
+ *   until another allocation of the context would fail without them.
  * farm_mlp_embed: f of n_rows host rows x (normalised first) into host
  *   out [n_rows, out_dim], with FP32 CUDA-core kernels (FARM_PREC_FP32_SIMT)
  *   or the BF16 tensor-core inference path (FARM_PREC_BF16).

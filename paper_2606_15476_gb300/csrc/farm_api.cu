@@ -159,6 +159,39 @@ bool params_ok(const farm_params &p, std::string &why)
     return true;
 }
 
+// Frees what farm_mlp_train left with the context for its next call; false when
+// there is nothing, or a training call is using it.
+bool release_training(farm_ctx *ctx)
+{
+    farm::Ctx &c = ctx->c;
+    if (c.training || (!c.ws.ptr[farm::B_TRAIN] && !c.ws.ptr[farm::B_TRAIN_IN])) return false;
+    cudaStreamSynchronize(c.stream);
+    for (const Buf b : {farm::B_TRAIN, farm::B_TRAIN_IN}) {
+        cudaFree(c.ws.ptr[b]);
+        c.ws.ptr[b] = nullptr;
+        c.ws.bytes[b] = 0;
+    }
+    return true;
+}
+
+}  // namespace
+
+cudaError_t farm::dev_alloc_bytes(farm_ctx *ctx, void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        if (release_training(ctx)) e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        (void)cudaGetLastError();
+    }
+    return e;
+}
+
+namespace {
+
 cudaError_t ws_get(farm_ctx *ctx, Buf b, size_t bytes, void **out)
 {
     auto &ws = ctx->c.ws;
@@ -173,12 +206,8 @@ cudaError_t ws_get(farm_ctx *ctx, Buf b, size_t bytes, void **out)
         }
         ctx->c.ws_gen += 1;     // captured graphs that use the old buffer no longer match, whether or not the next is had
         size_t grow = bytes + bytes / 8;
-        cudaError_t e = cudaMalloc(&ws.ptr[b], grow);
-        if (e != cudaSuccess) {
-            ws.ptr[b] = nullptr;
-            (void)cudaGetLastError();       // (reported here, not by the next launch)
-            return e;
-        }
+        cudaError_t e = farm::dev_alloc_bytes(ctx, &ws.ptr[b], grow);
+        if (e != cudaSuccess) return e;
         ws.bytes[b] = grow;
     }
     *out = ws.ptr[b];
@@ -197,6 +226,21 @@ cudaError_t ws_get(farm_ctx *ctx, Buf b, size_t count, T **out)
     void *p = nullptr;
     cudaError_t e = ws_get(ctx, b, count * sizeof(T), &p);
     *out = static_cast<T *>(p);
+    return e;
+}
+
+// The same on the context's stream, for a call's own use.
+cudaError_t temp_alloc(farm_ctx *ctx, float **p, size_t bytes)
+{
+    cudaError_t e = cudaMallocAsync(p, bytes, ctx->c.stream);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        if (release_training(ctx)) e = cudaMallocAsync(p, bytes, ctx->c.stream);
+    }
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        (void)cudaGetLastError();
+    }
     return e;
 }
 
@@ -663,25 +707,22 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
     };
     cudaError_t e;
     if (!reuse) {
-        if ((e = cudaMalloc(&ns.desc32, nd * 4)) != cudaSuccess) return bailmem(e);
-        if ((e = cudaMalloc(&ns.desc_hi, nd * 2)) != cudaSuccess) return bailmem(e);
-        if ((e = cudaMalloc(&ns.desc_lo, nd * 2)) != cudaSuccess) return bailmem(e);
-        if ((e = cudaMalloc(&ns.desc_bf16, nd * 2)) != cudaSuccess) return bailmem(e);
-        if ((e = cudaMalloc(&ns.desc_fp8, nd)) != cudaSuccess) return bailmem(e);
-        if ((e = cudaMalloc(&ns.desc_scale, (size_t)n * 4)) != cudaSuccess) return bailmem(e);
-        if ((e = cudaMalloc(&ns.cls, (size_t)n * 4)) != cudaSuccess) return bailmem(e);
-        if ((e = cudaMalloc(&ns.pos, (size_t)n * 12)) != cudaSuccess) return bailmem(e);
-        if ((e = cudaMalloc(&ns.size, (size_t)n * 12)) != cudaSuccess) return bailmem(e);
-        if ((e = cudaMalloc(&ns.views, (size_t)n * std::max(n_views, 1) * farm::kViewStride * 4)) != cudaSuccess)
+        if ((e = farm::dev_alloc(ctx, &ns.desc32, nd * 4)) != cudaSuccess) return bailmem(e);
+        if ((e = farm::dev_alloc(ctx, &ns.desc_hi, nd * 2)) != cudaSuccess) return bailmem(e);
+        if ((e = farm::dev_alloc(ctx, &ns.desc_lo, nd * 2)) != cudaSuccess) return bailmem(e);
+        if ((e = farm::dev_alloc(ctx, &ns.desc_bf16, nd * 2)) != cudaSuccess) return bailmem(e);
+        if ((e = farm::dev_alloc(ctx, &ns.desc_fp8, nd)) != cudaSuccess) return bailmem(e);
+        if ((e = farm::dev_alloc(ctx, &ns.desc_scale, (size_t)n * 4)) != cudaSuccess) return bailmem(e);
+        if ((e = farm::dev_alloc(ctx, &ns.cls, (size_t)n * 4)) != cudaSuccess) return bailmem(e);
+        if ((e = farm::dev_alloc(ctx, &ns.pos, (size_t)n * 12)) != cudaSuccess) return bailmem(e);
+        if ((e = farm::dev_alloc(ctx, &ns.size, (size_t)n * 12)) != cudaSuccess) return bailmem(e);
+        if ((e = farm::dev_alloc(ctx, &ns.views, (size_t)n * std::max(n_views, 1) * farm::kViewStride * 4)) != cudaSuccess)
             return bailmem(e);
     }
     const cudaMemcpyKind kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const float *d_desc = desc;
     if (!dev) {
-        if ((e = cudaMallocAsync(&tmp_desc, (size_t)n * dim * 4, c.stream)) != cudaSuccess) {
-            tmp_desc = nullptr;
-            return bailmem(e);
-        }
+        if ((e = temp_alloc(ctx, &tmp_desc, (size_t)n * dim * 4)) != cudaSuccess) return bailmem(e);
         if ((e = cudaMemcpyAsync(tmp_desc, desc, (size_t)n * dim * 4, kind, c.stream)) != cudaSuccess)
             return bailmem(e);
         d_desc = tmp_desc;
@@ -699,10 +740,7 @@ farm_status farm_memory_upload(farm_ctx *ctx, int32_t scene_id, int64_t n, int32
         const float *d_views = views;
         if (!dev) {
             const size_t vb = (size_t)6 * n_views * n * 4;
-            if ((e = cudaMallocAsync(&tmp_views, vb, c.stream)) != cudaSuccess) {
-                tmp_views = nullptr;
-                return bailmem(e);
-            }
+            if ((e = temp_alloc(ctx, &tmp_views, vb)) != cudaSuccess) return bailmem(e);
             if ((e = cudaMemcpyAsync(tmp_views, views, vb, kind, c.stream)) != cudaSuccess) return bailmem(e);
             d_views = tmp_views;
         }
@@ -1677,12 +1715,12 @@ farm_status farm_memory_add_space(farm_ctx *ctx, int32_t scene_id, int32_t space
                     std::string("space upload: ") + cudaGetErrorString(e));
     };
     cudaError_t e;
-    if ((e = cudaMalloc(&ns.hi, nd * 2)) != cudaSuccess) return bail(e);
-    if ((e = cudaMalloc(&ns.lo, nd * 2)) != cudaSuccess) return bail(e);
+    if ((e = farm::dev_alloc(ctx, &ns.hi, nd * 2)) != cudaSuccess) return bail(e);
+    if ((e = farm::dev_alloc(ctx, &ns.lo, nd * 2)) != cudaSuccess) return bail(e);
     const float *d_desc = desc;
     float *tmp = nullptr;
     if (!dev) {
-        if ((e = cudaMallocAsync(&tmp, (size_t)n * dim * 4, c.stream)) != cudaSuccess) return bail(e);
+        if ((e = temp_alloc(ctx, &tmp, (size_t)n * dim * 4)) != cudaSuccess) return bail(e);
         if ((e = cudaMemcpyAsync(tmp, desc, (size_t)n * dim * 4, cudaMemcpyHostToDevice, c.stream)) != cudaSuccess)
             return bail(e);
         d_desc = tmp;
@@ -2043,6 +2081,7 @@ farm_status farm_memory_release(farm_ctx *ctx, int32_t scene_id)
     // queued work may still read the scene
     CK(cudaStreamSynchronize(c.stream));
     free_scene(c.scenes[scene_id]);
+    release_training(ctx);
     CK(cudaMemsetAsync(ctx->d_scenes + scene_id, 0, sizeof(SceneDev), c.stream));
     CK(cudaStreamSynchronize(c.stream));
     c.batch_valid = false;

@@ -160,6 +160,7 @@ struct Ctx {
     std::map<int64_t, int> tuned; // similarity class -> fastest tile variant (autotuner)
     int pinned_variant = -1;      // >= 0: every grouped similarity launch uses this variant
     int32_t *d_fallback = nullptr;  // rows the thresholded select handed to its exact fallback
+    bool training = false;          // a training call holds its buffers (B_TRAIN, B_TRAIN_IN)
     int32_t *d_probe = nullptr;     // counts of a kernel that samples (0 between calls)
     int32_t *h_err = nullptr;     // pinned host mirror
     // batch state
@@ -232,6 +233,19 @@ cudaError_t mlp_gelu_backward(const float *h, float *da, int64_t count, cudaStre
 cudaError_t mlp_colsum(const float *x, int64_t rows, int cols, float *out, bool accumulate, cudaStream_t s);
 cudaError_t mlp_adam(float *p, const float *g, float *m, float *v, int64_t count, float lr, int t, const MlpShape &shape,
                      cudaStream_t s);
+
+// Device memory; when there is none left, what the last training call left with
+// the context is freed and the allocation tried once more.  A failure is
+// reported here and not by a later launch.
+cudaError_t dev_alloc_bytes(farm_ctx *ctx, void **p, size_t bytes);
+template <class T>
+cudaError_t dev_alloc(farm_ctx *ctx, T **p, size_t bytes)
+{
+    void *v = nullptr;
+    const cudaError_t e = dev_alloc_bytes(ctx, &v, bytes);
+    *p = static_cast<T *>(v);
+    return e;
+}
 
 // Grow-only workspace buffer of the context (synchronises before a regrow).
 cudaError_t ws_alloc(farm_ctx *ctx, Buf b, size_t bytes, void **out);

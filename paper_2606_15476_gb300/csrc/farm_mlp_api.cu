@@ -62,7 +62,7 @@ struct TrainBufs {
     float *xq, *xd, *hq, *hd, *aq, *ad, *zq, *zd, *eq, *ed, *nq, *nd, *da, *grad, *m, *v, *loss, *y, *w;
 };
 
-cudaError_t train_alloc(TrainBufs &t, const Mlp &M, int64_t B, int64_t loss_slots)
+cudaError_t train_alloc(farm_ctx *ctx, TrainBufs &t, const Mlp &M, int64_t B, int64_t loss_slots)
 {
     const int64_t D = M.D, H = M.H, P = M.P, cnt = M.count();
     const int64_t sizes[] = {B * D, B * D, B * H, B * H, B * H, B * H, B * P, B * P, B * P, B * P,
@@ -72,7 +72,7 @@ cudaError_t train_alloc(TrainBufs &t, const Mlp &M, int64_t B, int64_t loss_slot
     auto rounded = [](int64_t n) { return (n + 63) / 64 * 64; };   // 256-byte aligned sub-arrays
     int64_t total = 0;
     for (int64_t n : sizes) total += rounded(n);
-    cudaError_t e = cudaMalloc(&t.base, (size_t)total * sizeof(float));
+    cudaError_t e = farm::dev_alloc(ctx, &t.base, (size_t)total * sizeof(float));
     if (e != cudaSuccess) return e;
     float *p = t.base;
     for (size_t i = 0; i < sizeof(sizes) / sizeof(sizes[0]); ++i) {
@@ -176,7 +176,9 @@ void gemm_shapes(const TcBufs &t, const Mlp &M, GemmShape (&g)[kGemmPieces])
 }
 
 // Buffers of a training call up to this size stay with the context for its next
-// one (allocating and freeing them takes longer than a few steps).
+// one (allocating and freeing them takes longer than a few steps); they are
+// given back by farm_memory_release, by farm_destroy, and to any allocation of
+// the context that would fail otherwise.
 constexpr int64_t kTrainKept = int64_t(512) << 20;
 
 // keep: the buffers may be the context's kept ones (t.base then stays null).
@@ -203,7 +205,7 @@ cudaError_t tc_alloc(farm_ctx *ctx, TcBufs &t, int64_t B, int64_t loss_slots, bo
     if (keep && total <= kTrainKept) {
         if ((e = farm::ws_alloc(ctx, farm::B_TRAIN, (size_t)total, &at)) != cudaSuccess) return e;
     } else {
-        if ((e = cudaMalloc(&t.base, (size_t)total)) != cudaSuccess) return e;
+        if ((e = farm::dev_alloc(ctx, &t.base, (size_t)total)) != cudaSuccess) return e;
         at = t.base;
     }
     char *p = static_cast<char *>(at);
@@ -336,7 +338,7 @@ cudaError_t farm::learned_refresh_scene(farm_ctx *ctx, int32_t scene_id)
     cudaError_t r;
     if (!s.comp) {
         if ((r = cudaStreamSynchronize(c.stream))) return r;
-        if ((r = cudaMalloc(&s.comp, (size_t)s.n * c.mlp.P * 2))) return r;
+        if ((r = farm::dev_alloc(ctx, &s.comp, (size_t)s.n * c.mlp.P * 2))) return r;
     }
     if ((r = learned_embed_rows(ctx, s.desc_bf16, s.n, s.comp))) return r;
     s.comp_version = c.mlp.version;
@@ -379,10 +381,10 @@ farm_status farm_mlp_set(farm_ctx *ctx, int32_t dim, int32_t hidden, int32_t out
         M.set = false;
     }
     if (!M.set) {
-        MCK(cudaMalloc(&M.params, (size_t)cnt * 4));
-        MCK(cudaMalloc(&M.w1b, (size_t)nm.H * nm.D_pad * 2));
-        MCK(cudaMalloc(&M.w2b, (size_t)nm.P * nm.H * 2));
-        MCK(cudaMalloc(&M.w2t, (size_t)nm.H * nm.P * 2));
+        MCK(farm::dev_alloc(ctx, &M.params, (size_t)cnt * 4));
+        MCK(farm::dev_alloc(ctx, &M.w1b, (size_t)nm.H * nm.D_pad * 2));
+        MCK(farm::dev_alloc(ctx, &M.w2b, (size_t)nm.P * nm.H * 2));
+        MCK(farm::dev_alloc(ctx, &M.w2t, (size_t)nm.H * nm.P * 2));
         M.D = nm.D; M.H = nm.H; M.P = nm.P; M.D_pad = nm.D_pad;
         // shape change: every scene cache is stale
         for (auto &s : c.scenes)
@@ -441,7 +443,7 @@ farm_status farm_mlp_loss_grad(farm_ctx *ctx, int64_t n_pairs, const float *xq, 
         e = tc_alloc(ctx, t, n_pairs, 1, false);
         if (e) return done(fail(c, e == cudaErrorMemoryAllocation ? FARM_ENOMEM : FARM_ECUDA,
                                 std::string("farm_mlp_loss_grad: ") + cudaGetErrorString(e)));
-        if (!e) e = cudaMalloc(&raw, 2 * xb);
+        if (!e) e = farm::dev_alloc(ctx, &raw, 2 * xb);
         if (!e) e = cudaMemcpyAsync(raw, xq, xb, cudaMemcpyHostToDevice, c.stream);
         if (!e) e = cudaMemcpyAsync(raw + (size_t)n_pairs * M.D, xd, xb, cudaMemcpyHostToDevice, c.stream);
         if (!e) e = cudaMemcpyAsync(t.y, y, (size_t)n_pairs * 4, cudaMemcpyHostToDevice, c.stream);
@@ -459,7 +461,7 @@ farm_status farm_mlp_loss_grad(farm_ctx *ctx, int64_t n_pairs, const float *xq, 
         return done(FARM_OK);
     }
     TrainBufs t;
-    MCK(train_alloc(t, M, n_pairs, 1));
+    MCK(train_alloc(ctx, t, M, n_pairs, 1));
     auto done = [&](farm_status st) { cudaFree(t.base); return st; };
     if (!e) e = cudaMemcpyAsync(t.xq, xq, xb, cudaMemcpyHostToDevice, c.stream);
     if (!e) e = cudaMemcpyAsync(t.xd, xd, xb, cudaMemcpyHostToDevice, c.stream);
@@ -516,6 +518,11 @@ farm_status farm_mlp_train(farm_ctx *ctx, int32_t n_scenes, const int32_t *scene
     const int64_t B = std::min<int64_t>(batch, n_pairs);
     const int64_t steps = (n_pairs + B - 1) / B;
     TcBufs t;
+    struct Busy {
+        bool &b;
+        explicit Busy(bool &x) : b(x) { b = true; }
+        ~Busy() { b = false; }
+    } busy(c.training);
     // the call's inputs: normalised rows (BF16 [n_rows, D_pad]), the rows as
     // given, the pairs' arrays as given, an epoch's order, the row tables
     uint16_t *qnb = nullptr;
@@ -541,7 +548,7 @@ farm_status farm_mlp_train(farm_ctx *ctx, int32_t n_scenes, const int32_t *scene
         for (size_t b : sizes) total += (b + 255) & ~size_t(255);
         void *at = nullptr;
         if ((int64_t)total <= kTrainKept) e = farm::ws_alloc(ctx, farm::B_TRAIN_IN, total, &at);
-        else if (!(e = cudaMalloc(&in_base, total))) at = in_base;
+        else if (!(e = farm::dev_alloc(ctx, &in_base, total))) at = in_base;
         if (e) return done(fail(c, e == cudaErrorMemoryAllocation ? FARM_ENOMEM : FARM_ECUDA,
                                 std::string("farm_mlp_train: ") + cudaGetErrorString(e)));
         uint8_t *p = static_cast<uint8_t *>(at);
@@ -629,14 +636,14 @@ farm_status farm_mlp_embed(farm_ctx *ctx, int64_t n_rows, const float *x, int32_
         cudaFree(raw); cudaFree(xn); cudaFree(h); cudaFree(a); cudaFree(z); cudaFree(e32); cudaFree(xb); cudaFree(eb);
         return st;
     };
-    cudaError_t e = cudaMalloc(&raw, (size_t)n_rows * M.D * 4);
+    cudaError_t e = farm::dev_alloc(ctx, &raw, (size_t)n_rows * M.D * 4);
     if (!e) e = cudaMemcpyAsync(raw, x, (size_t)n_rows * M.D * 4, cudaMemcpyHostToDevice, c.stream);
     if (precision == FARM_PREC_FP32_SIMT) {
-        if (!e) e = cudaMalloc(&xn, (size_t)n_rows * M.D * 4);
-        if (!e) e = cudaMalloc(&h, (size_t)n_rows * M.H * 4);
-        if (!e) e = cudaMalloc(&a, (size_t)n_rows * M.H * 4);
-        if (!e) e = cudaMalloc(&z, (size_t)n_rows * M.P * 4);
-        if (!e) e = cudaMalloc(&e32, (size_t)n_rows * M.P * 4);
+        if (!e) e = farm::dev_alloc(ctx, &xn, (size_t)n_rows * M.D * 4);
+        if (!e) e = farm::dev_alloc(ctx, &h, (size_t)n_rows * M.H * 4);
+        if (!e) e = farm::dev_alloc(ctx, &a, (size_t)n_rows * M.H * 4);
+        if (!e) e = farm::dev_alloc(ctx, &z, (size_t)n_rows * M.P * 4);
+        if (!e) e = farm::dev_alloc(ctx, &e32, (size_t)n_rows * M.P * 4);
         if (!e) e = farm::launch_normalize_rows(raw, nullptr, n_rows, M.D, M.D, xn, nullptr, nullptr, nullptr, c.d_err,
                                                 farm::kErrBadRow, c.stream);
         int64_t L = 1;
@@ -644,9 +651,9 @@ farm_status farm_mlp_embed(farm_ctx *ctx, int64_t n_rows, const float *x, int32_
         c.launches += L;
         if (!e) e = cudaMemcpyAsync(out, e32, (size_t)n_rows * M.P * 4, cudaMemcpyDeviceToHost, c.stream);
     } else {
-        if (!e) e = cudaMalloc(&xb, (size_t)n_rows * M.D_pad * 2);
-        if (!e) e = cudaMalloc(&eb, (size_t)n_rows * M.P * 2);
-        if (!e) e = cudaMalloc(&e32, (size_t)n_rows * M.P * 4);
+        if (!e) e = farm::dev_alloc(ctx, &xb, (size_t)n_rows * M.D_pad * 2);
+        if (!e) e = farm::dev_alloc(ctx, &eb, (size_t)n_rows * M.P * 2);
+        if (!e) e = farm::dev_alloc(ctx, &e32, (size_t)n_rows * M.P * 4);
         if (!e) e = farm::launch_normalize_rows(raw, nullptr, n_rows, M.D, M.D_pad, nullptr, nullptr, nullptr, xb,
                                                 c.d_err, farm::kErrBadRow, c.stream);
         c.launches += 1;
