@@ -239,6 +239,16 @@ __device__ __forceinline__ void tile_write_t(const uint16_t (*tile)[TSTRIDE], in
     *reinterpret_cast<uint4 *>(dst + (int64_t)(c0 + c) * ldd + r0 + k) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// The first row of a block's tile: the tiles of more rows than blockIdx.y may count
+// go on in blockIdx.z (a last plane's blocks past the rows have nothing to do).
+constexpr unsigned kGridY = 65535;
+__device__ __forceinline__ int64_t tile_row0() { return ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * TR; }
+dim3 tile_grid(int64_t cols, int64_t rows)
+{
+    const int64_t t = (rows + TR - 1) / TR;
+    return dim3((unsigned)(cols / TC), (unsigned)(t < kGridY ? t : kGridY), (unsigned)((t + kGridY - 1) / kGridY));
+}
+
 // The step's stacked input rows (query rows 0 .. b - 1, descriptor rows b ..
 // 2b - 1; D_pad long) and their transpose [D, K].  With pairs.row gathered
 // (pair k of the order: base[n_scenes] row row[k], and base[scene[k]] row
@@ -250,7 +260,8 @@ train_rows_kernel(TrainPairs pairs, int64_t off, int64_t b, int D, int D_pad, ui
     __shared__ __align__(4) uint16_t tile[TR][TSTRIDE];
     const int tid = threadIdx.x;
     const int c0 = blockIdx.x * TC;
-    const int64_t r0 = (int64_t)blockIdx.y * TR;
+    const int64_t r0 = tile_row0();
+    if (r0 >= K) return;
     const int64_t r = r0 + (tid >> 3);
     const int c = c0 + (tid & 7) * 8;           // (D_pad is a multiple of 64: the tile's columns exist)
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -283,7 +294,8 @@ gelu_bf16_kernel(const float *__restrict__ h, const float *__restrict__ b, int64
     __shared__ __align__(4) uint16_t tile[TR][TSTRIDE];
     const int tid = threadIdx.x;
     const int c0 = blockIdx.x * TC;
-    const int64_t r0 = (int64_t)blockIdx.y * TR;
+    const int64_t r0 = tile_row0();
+    if (r0 >= (aT ? K : rows)) return;
     const int64_t r = r0 + (tid >> 3);
     const int c = c0 + (tid & 7) * 8;
     uint16_t g[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -636,8 +648,7 @@ cudaError_t mlp_train_rows(const TrainPairs &pairs, int64_t off, int64_t b, int 
                            int64_t K, cudaStream_t s)
 {
     if (b < 1 || D_pad % TC != 0 || K % 64 != 0 || K < 2 * b || (pairs.row && !pairs.perm)) return cudaErrorInvalidValue;
-    dim3 grid((unsigned)(D_pad / TC), (unsigned)(K / TR));
-    train_rows_kernel<<<grid, 256, 0, s>>>(pairs, off, b, D, D_pad, x, xT, K);
+    train_rows_kernel<<<tile_grid(D_pad, K), 256, 0, s>>>(pairs, off, b, D, D_pad, x, xT, K);
     return cudaGetLastError();
 }
 
@@ -645,8 +656,7 @@ cudaError_t mlp_gelu_bf16(const float *h, const float *b, int64_t rows, int cols
                           cudaStream_t s)
 {
     if (rows < 1 || cols % TC != 0 || (aT && (K % 64 != 0 || K < rows))) return cudaErrorInvalidValue;
-    dim3 grid((unsigned)(cols / TC), (unsigned)(((aT ? K : rows) + TR - 1) / TR));
-    gelu_bf16_kernel<<<grid, 256, 0, s>>>(h, b, rows, cols, ab, aT, K);
+    gelu_bf16_kernel<<<tile_grid(cols, aT ? K : rows), 256, 0, s>>>(h, b, rows, cols, ab, aT, K);
     return cudaGetLastError();
 }
 
