@@ -802,7 +802,7 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
             const int64_t r_blk = (int64_t)m0 + quad * 32;       // first row of the warp's blocks
             const bool store = pc.s_off >= 0;     // s_off -1: the group maxima only (uniform across the warp)
             float *sblk = S + (store ? pc.s_off : 0) + r_blk * pc.ld;
-            const bool vec = (pc.ld % 4) == 0;
+            const bool vec = (pc.ld % 4) == 0 && (reinterpret_cast<uintptr_t>(S) & 15u) == 0;
             // stored columns c0 + ... are valid below ns_ exactly where their objects n0 + ... are below n
             const float sr = (MODE == kSimFp8 && live) ? scale_q[pc.q_row0 + r] : 1.f;
             // FP8 mode: the tile's column scales (zero past the row end), staged once
