@@ -390,8 +390,9 @@ farm_status farm_select_fallbacks(farm_ctx *ctx, int64_t *rows_out, int32_t rese
  * CTA; 2 = 256 x 256 tiles computed by a pair of CTAs with two-SM MMAs).
  * All compute each cosine with the same sequence of products, so they give
  * bitwise identical results.  A FARM_PREC_FP32 batch of at most 128 rows
- * (targets and constraints) takes a kernel for few rows with the same results
- * instead, unless a variant is pinned or FARM_FUSED given.  The first other
+ * (targets and constraints) and about 20 million cosines takes a kernel for few
+ * rows with the same results instead, unless a variant is pinned or FARM_FUSED
+ * given.  The first other
  * farm_query_batch of each class of batch (similarity mode, and the powers of two of its total rows and of its
  * mean objects per row) times every variant on its first similarity block and
  * keeps the fastest for the context.

@@ -1090,8 +1090,23 @@ farm_status farm_query_batch(farm_ctx *ctx, int64_t n_q, const int32_t *scene_of
     // per SM, whose sample and other tiles each fill a part of one wave (64
     // queries, 224 rows, 20,000 objects, cold caches: similarity and selection
     // 90 us stored, 99 us fused).
+    // (up to kFewCosines cosines: a CTA reads each stored row past the staged
+    // group maxima.  Calls of 9 / 36 / 126 rows, D = 64: 250,000 objects 113 /
+    // 144 / 229 us stored, 176 / 185 / 198 fused; 600,000 223 / 289 / 466, 259 /
+    // 277 / 289; 1,000,000 366 / 467 / 748, 354 / 374 / 396.  That reading costs the
+    // same however long the descriptors are, the fused launches do not: D = 512,
+    // 1,000,000 objects 590 / 653 / 979, 660 / 674 / 716.  Where the fused
+    // selection's threshold would let more of the sample through than it can
+    // refine (fuse_sound), its rows overflow to the exact fallback: 3,000,000
+    // objects 1.1 / 1.4 / 2.2 ms stored, 35 / 38 / 41 fused)
+    constexpr int64_t kFewCosines = int64_t(20) << 20, kFewShortObjects = int64_t(3) << 18;
+    int64_t cosines = 0;
+    for (const auto &g : groups) cosines += (g.nq + g.nc) * c.scenes[g.sid].n;
+    const bool fuse_sound = (int64_t)keep_max * (max_n / (32 * fs)) <= farm::kFuseTauKeys * farm::kFuseTauKeys;
     const bool few = precision == FARM_PREC_FP32 && c.pinned_variant < 0 && !(flags & FARM_FUSED) &&
-                     rows_total <= farm::kSimFewRows;
+                     rows_total <= farm::kSimFewRows &&
+                     ((cosines <= kFewCosines && (max_n <= kFewShortObjects || dim_pad >= 256)) || !fuse_sound ||
+                      !fusable);
     int64_t tiles_all = 0;
     for (const auto &g : groups) tiles_all += farm::sim_cluster_tiles(g.nq + g.nc, c.scenes[g.sid].n, 0);
     const bool fill = tiles_all >= 2 * (int64_t)c.num_sms;

@@ -616,6 +616,8 @@ cudaError_t launch_fuse_sample_tau(const float *S, const float *tops, const Piec
 // of its whole row (the similarity launch stored no values), at most gmax of
 // them per row (<= kMaximaTauKeys), and a zero count.
 constexpr int kMaximaTauKeys = 12288;
+// Group maxima, and then entries, of a sample that its rows' thresholds are found from.
+constexpr int64_t kFuseTauKeys = 1024;
 cudaError_t launch_fuse_maxima_tau(const float *tops, const Piece *pieces, int32_t n_pieces, int64_t total_rows,
                                    const FuseEmit &emit, int32_t gmax, cudaStream_t st);
 cudaError_t launch_fuse_final(const Piece *pieces, int32_t n_pieces, int64_t total_rows, int32_t *tsel_idx,

@@ -121,7 +121,7 @@ __device__ __forceinline__ RowList row_list(const Piece &pc, int64_t b, int32_t 
 // when the groups are fewer than the list length -- at most this many, a
 // prefix being still a subset of the row (small, so that many warps stay
 // resident to hide the loads' latency).
-constexpr int TAU_KEYS = 1024;
+constexpr int TAU_KEYS = (int)kFuseTauKeys;
 constexpr int TAU_WARPS = 4;
 // A lower bound of the R-th largest of n keys in shared memory (n >= R >= 1)
 // that at most a few more than R keys reach (value bins).  Never returns a key
