@@ -241,9 +241,9 @@ def cpu_baseline_mc(scene, spaces, qb, cq, k, n_sample, seed=0, budget_s=15.0):
 # (code_digest: the source without its comments):
 # (workload, precision, tile variant, fused) -> bytes
 SIM_TRAFFIC = {
-    ("site_n20k_d1152", "fp32", 2, True): (89.155584e6 + 123.307008e6) + (667.750144e6 + 20.646912e6),
+    ("site_n20k_d1152", "fp32", 2, True): (92.574208e6 + 117.734656e6) + (619.948288e6 + 18.919936e6),
 }
-SIM_TRAFFIC_SOURCE = "8b8390e1008ba89e"
+SIM_TRAFFIC_SOURCE = "b982ce61197be2e3"
 
 
 def code_digest(text):
