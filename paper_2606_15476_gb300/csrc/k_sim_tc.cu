@@ -330,7 +330,8 @@ __device__ __forceinline__ void store_rows_staged(float4 *blk, const float4 (&va
     __syncwarp();
 }
 
-template <int MODE, int BN_, int CM_, bool GROUPED, bool PAIR, bool EMIT = false, bool WIDE = false>
+template <int MODE, int BN_, int CM_, bool GROUPED, bool PAIR, bool EMIT = false, bool WIDE = false,
+          bool GATED = false>
 __global__ void __launch_bounds__((Cfg<MODE, BN_, CM_, PAIR, EMIT, WIDE>::THREADS), 1)
 sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant__ CUtensorMap map_q1,
               const __grid_constant__ CUtensorMap map_d0, const __grid_constant__ CUtensorMap map_d1,
@@ -368,26 +369,24 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
     uint64_t *emit_slots = reinterpret_cast<uint64_t *>(reinterpret_cast<uint8_t *>(tile_scales) + C::SCALE_BYTES);
     uint64_t *corr_free = acc_empty + 1;      // FOLD: the correction columns are free (tile accumulators: one)
 
-    // one problem behind a gate: its first *gate rows only (every thread of the launch alike)
-    if constexpr (!GROUPED) {
-        if (emit.gate) {
-            const int64_t rows = min(single.rows, *emit.gate);
-            if (rows <= 0) {
-                // (an emitting launch that does nothing leaves every list overflowed)
-                if constexpr (EMIT)
-                    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < single.rows;
-                         r += (int64_t)gridDim.x * blockDim.x)
-                        emit.cnt[r] = 0x7fffffff;
-                return;
-            }
-            const int64_t mt = (rows + BM - 1) / BM;
-            total = min(total, (int32_t)((mt + CM - 1) / CM * col_tiles(single.n, BN, kColAll, 0)));
+    // GATED: one problem behind a gate, its first *gate rows only (every thread of the launch alike)
+    if constexpr (GATED) {
+        static_assert(!GROUPED, "gated launches cover one problem");
+        const int64_t rows = min(single.rows, *emit.gate);
+        if (rows <= 0) {
+            // (an emitting launch that does nothing leaves every list overflowed)
+            if constexpr (EMIT)
+                for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < single.rows;
+                     r += (int64_t)gridDim.x * blockDim.x)
+                    emit.cnt[r] = 0x7fffffff;
+            return;
         }
+        const int64_t mt = (rows + BM - 1) / BM;
+        total = min(total, (int32_t)((mt + CM - 1) / CM * col_tiles(single.n, BN, kColAll, 0)));
     }
     auto piece_at = [&](int tile) {
         GemmPiece p = piece_of<GROUPED>(tile, pieces, n_pieces, single);
-        if constexpr (!GROUPED)
-            if (emit.gate) p.rows = min(p.rows, *emit.gate);
+        if constexpr (GATED) p.rows = min(p.rows, *emit.gate);
         return p;
     };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -802,7 +801,7 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
             const int64_t r_blk = (int64_t)m0 + quad * 32;       // first row of the warp's blocks
             const bool store = pc.s_off >= 0;     // s_off -1: the group maxima only (uniform across the warp)
             float *sblk = S + (store ? pc.s_off : 0) + r_blk * pc.ld;
-            const bool vec = (pc.ld % 4) == 0 && (reinterpret_cast<uintptr_t>(S) & 15u) == 0;
+            const bool vec = (((uint32_t)pc.ld << 2 | (uint32_t)reinterpret_cast<uintptr_t>(S)) & 15u) == 0;   // (S: multiples of 4 bytes)
             // stored columns c0 + ... are valid below ns_ exactly where their objects n0 + ... are below n
             const float sr = (MODE == kSimFp8 && live) ? scale_q[pc.q_row0 + r] : 1.f;
             // FP8 mode: the tile's column scales (zero past the row end), staged once
@@ -943,7 +942,8 @@ sim_tc_kernel(const __grid_constant__ CUtensorMap map_q0, const __grid_constant_
 // as can be resident at once (a GPC with an odd number of free SMs cannot
 // hold a whole cluster on its last SM); the count is cached per device and
 // kernel (concurrent first calls compute the same value).
-template <int MODE, int BN_, int CM_, bool GROUPED, bool PAIR = false, bool EMIT = false, bool WIDE = false>
+template <int MODE, int BN_, int CM_, bool GROUPED, bool PAIR = false, bool EMIT = false, bool WIDE = false,
+          bool GATED = false>
 cudaError_t launch_impl(const CUtensorMap &mq0, const CUtensorMap &mq1, const CUtensorMap &md0,
                         const CUtensorMap &md1, const GemmPiece *pieces, int32_t n_pieces, const GemmPiece &single,
                         float *S, float *tops, int32_t k_slices, int64_t total_tiles, const float *scale_q,
@@ -952,7 +952,7 @@ cudaError_t launch_impl(const CUtensorMap &mq0, const CUtensorMap &mq1, const CU
     using C = Cfg<MODE, BN_, CM_, PAIR, EMIT, WIDE>;
     if (total_tiles <= 0) return cudaSuccess;
     if (total_tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    auto kernel = sim_tc_kernel<MODE, BN_, CM_, GROUPED, PAIR, EMIT, WIDE>;
+    auto kernel = sim_tc_kernel<MODE, BN_, CM_, GROUPED, PAIR, EMIT, WIDE, GATED>;
     const int smem_bytes = C::SMEM_BYTES;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
     if (e != cudaSuccess) return e;
@@ -1049,19 +1049,25 @@ cudaError_t launch_tc(const void *q0, const void *q1, const void *d0, const void
     single.col_stride = 0;
     single.n_store = (int32_t)n;
     const int64_t tiles = sim_cluster_tiles(rows, n, V);
-    if (emit && !(MODE == kSimF16x3 && PAIR_)) return cudaErrorInvalidValue;
     if constexpr (MODE == kSimF16x3 && PAIR_) {
         if (emit) {
-            if (!emit->tau_key || !emit->cnt || !emit->cand || emit->cap < 1) return cudaErrorInvalidValue;
-            return launch_impl<MODE, BN_, CM_, false, true, true>(mq0, mq1, md0, md1, nullptr, 1, single, S, tops,
-                                                                  k_slices_of<MODE>(dim_pad), tiles, scale_q, num_sms,
-                                                                  err, s, *emit);
+            if (!emit->tau_key || !emit->cnt || !emit->cand || emit->cap < 1 || !emit->gate)
+                return cudaErrorInvalidValue;
+            return launch_impl<MODE, BN_, CM_, false, true, true, false, true>(
+                mq0, mq1, md0, md1, nullptr, 1, single, S, tops, k_slices_of<MODE>(dim_pad), tiles, scale_q, num_sms,
+                err, s, *emit);
+        }
+        if (gate) {
+            FuseEmit only{};
+            only.gate = gate;
+            return launch_impl<MODE, BN_, CM_, false, true, false, false, true>(
+                mq0, mq1, md0, md1, nullptr, 1, single, S, tops, k_slices_of<MODE>(dim_pad), tiles, scale_q, num_sms,
+                err, s, only);
         }
     }
-    FuseEmit none{};
-    none.gate = gate;
+    if (emit || gate) return cudaErrorInvalidValue;
     return launch_impl<MODE, BN_, CM_, false, PAIR_>(mq0, mq1, md0, md1, nullptr, 1, single, S, tops,
-                                                     k_slices_of<MODE>(dim_pad), tiles, scale_q, num_sms, err, s, none);
+                                                     k_slices_of<MODE>(dim_pad), tiles, scale_q, num_sms, err, s);
 }
 
 template <int MODE, int BN_, int CM_, bool PAIR = false>
