@@ -14,11 +14,11 @@ namespace {
 
 // From this many cosines on a call keeps those reaching tau_f instead of storing
 // all.  Fewer (24 MB) stay in the L2, and the launches that the lists need cost
-// more than they save: with F = 256, 307 detections x 589 entities 73 us with
-// lists, 59 stored; 1,000 x 4,000 79, 73.  At 6 to 8 million the two are even
-// (1,000 x 6,300 87.7, 85.1; 4,000 x 2,000 97.9, 100.3; 1,000 x 8,000 87.6,
-// 86.6); 1,000 x 16,000 107, 118; 16,000 x 1,000 152, 176; 1,500 x 30,000 163,
-// 214.
+// more than they save: with F = 256, 307 detections x 589 entities 69 us with
+// lists, 56 stored; 1,000 x 4,000 74.6, 68.8.  At 6 to 8 million the two are even
+// (1,000 x 6,300 83.5, 80.7; 4,000 x 2,000 93.5, 95.9; 1,000 x 8,000 83.6,
+// 81.1); 1,000 x 16,000 106, 116; 16,000 x 1,000 148, 173; 1,500 x 30,000 160,
+// 210.
 constexpr int64_t kEmitCosines = int64_t(6) << 20;
 
 farm_status afail(Ctx &c, farm_status st, const std::string &msg)
@@ -187,7 +187,7 @@ extern "C" farm_status farm_associate(farm_ctx *ctx, int64_t n_ent, const float 
     a.ehi = ehi;
     a.F_pad = F_pad;
     a.probe = c.d_probe;
-    c.launches += emitting ? 11 : 9;
+    c.launches += emitting ? 10 : 8;
     ACK(farm::launch_assoc_init(a, c.stream), "association kernels");
     if (emitting) {
         ACK(farm::launch_sim_tc_f16x3(dhi, dlo, ehi, elo, nullptr, B, N, F_pad, ld, nullptr, c.num_sms, c.d_err,

@@ -651,7 +651,8 @@ cudaError_t launch_copy_lists(const Piece *pieces, int32_t n_pieces, int64_t row
                               const float *bsel_tv, int32_t cstride_t, const int32_t *bsel_l, int32_t cstride_l,
                               int32_t *tsel_idx, float *tsel_cos, int32_t stride_t, int32_t *lsel_idx,
                               int32_t stride_l, cudaStream_t s);
-// Grouped FP32 rescore (one block per launch row): the keep_t / keep_l
+// Grouped FP32 rescore (a block per four rows of one class in launches of at
+// least 2,048 rows of at most 2,048 floats, else one per row): the fkeep_t / fkeep_l
 // candidates of bsel_* (strides cstride_t / cstride_l; descending by their
 // reduced-precision values bsel_tv / bsel_lv, nullable) are re-scored with
 // exact FP32 dot products of the unit rows Q32 and the descriptors d32, and

@@ -23,18 +23,19 @@
 //    soon as they are found; the winner of a component is its entity of
 //    largest weight (lower index on ties), a component without an entity is a
 //    lone detection that starts a new entity;
-//  * fusion: a warp per slot; a winner sums w (mu - c) and w f over the slots
+//  * fusion: a warp per slot (blocks for the winners of more than BIG_MEMBERS
+//    members, a segment of them at a time); a winner sums w (mu - c) and w f over the slots
 //    merged into it (listed per winner; c the winner's own mean: a shift that
 //    keeps FP32 digits at site coordinates), then w (S + (mu - mu_g)(mu -
 //    mu_g)') -- the sufficient-statistics merge M1 = w mu, M2 = w (S + mu mu')
 //    in a form free of the cancellation of M2 / w - mu mu'.  The members'
 //    order (and the last bits) may vary from run to run.
 //
-// 4,096 detections x 20,000 entities, F = 256: 183 us a call against 300 when
+// 4,096 detections x 20,000 entities, F = 256: 173 us a call against 300 when
 // the similarity stored the 328 MB block and a scan read it back, the
 // components took one CTA's rounds and the fusion four passes of atomics
 // (search 106 -> 25 us, components 57 -> the match kernel's tail, fusion and its
-// clearing 106 -> 39; the similarity 124 -> 111, 60% of the tensor rate: 17
+// clearing 106 -> 42; the similarity 124 -> 111, 60% of the tensor rate: 17
 // tiles of eight K slices per CTA pair, each waiting for its fold).
 #include <cuda_fp16.h>
 
@@ -178,9 +179,9 @@ constexpr int PROBE_BLOCKS = 64, PROBE_PAIRS = 2;      // of them, and cosines a
 // of detections and entities spread over both (the FP16 parts' leading ones) are
 // compared with tau_f, and with so many of them above it that the mean list would
 // fill more than 7/8 of a buffer every row is stored (the last of the sampling
-// warps decides).  4,096 x 20,000, F = 256: 3,000 of the entities alike 330 us
-// (323 with every row stored; 293 and 212 where all lists fit), classes of 2,222
-// 588 (563), all of one class 1,134 (1,111); without the sample, and a second
+// warps decides).  4,096 x 20,000, F = 256: 3,000 of the entities alike 324 us
+// (320 with every row stored; where all lists fit 209 and 288), classes of 2,222
+// 580 (559), all of one class 1,134 (1,101); without the sample, and a second
 // product of every row once a list overflows, 454, 1,070 and 2,490.
 __global__ void __launch_bounds__(256)
 assoc_init_kernel(int32_t T, int32_t N, int32_t B, float tau_f, int32_t *__restrict__ label,
@@ -209,7 +210,8 @@ assoc_init_kernel(int32_t T, int32_t N, int32_t B, float tau_f, int32_t *__restr
 #pragma unroll
     for (int k = 0; k < PROBE_PAIRS; ++k) {
         const uint32_t p = (uint32_t)(p0 + k);
-        const int64_t d = (int64_t)p * B / pairs, e = (int64_t)(((uint64_t)(p * 2654435761u) * (uint32_t)N) >> 32);
+        // (multiplicative hashing, two constants: places spread evenly over each)
+        const int64_t d = __umulhi(p * 2246822519u, (uint32_t)B), e = __umulhi(p * 2654435761u, (uint32_t)N);
         x[k] = reinterpret_cast<const uint4 *>(dhi + d * F_pad);
         y[k] = reinterpret_cast<const uint4 *>(ehi + e * F_pad);
         dot[k] = 0.f;
@@ -471,7 +473,7 @@ struct Slots {
 
 constexpr int FW = 8;              // slots (warps) per block of the fusion
 constexpr int FTH = FW * 32;
-constexpr int FU = 8;              // members whose features a lane has in flight
+constexpr int FU = 3;              // members whose features a lane has in flight
 constexpr int BIG_BLOCKS = 304;    // blocks that take the big winners' work items
 
 // The sum over the block's threads of N values each, to every thread.
@@ -645,38 +647,35 @@ __device__ __forceinline__ void fuse_big(const Slots &sl, int g, int seg, int it
     }
 }
 
-// The work items of the winners of more than BIG_MEMBERS members.  Bound by the
+// out_w, out_mu, out_cov and out_feat of every slot, a warp each: zeros for a
+// merged one, the slot's own values for a winner without members, sums over the
+// members (listed at members + off) otherwise.  The first BIG_BLOCKS blocks take
+// the work items of the winners of more than BIG_MEMBERS members.  Bound by the
 // gather of the members' rows: with one block per such winner and its members'
 // loads one after the other, 100,000 detections of 70 entities (F = 64) took
 // 1,734 us here and 300,000 of 40 11.4 ms; in segments with several loads in
-// flight per lane, 64 and 202.  Nothing to do: 2.5 us.
-__global__ void __launch_bounds__(FTH)
-assoc_fuse_big_kernel(Slots sl, const int32_t *__restrict__ mcnt, const int32_t *__restrict__ off,
-                      const int32_t *__restrict__ members, const int2 *__restrict__ items,
-                      const int32_t *__restrict__ n_items, int32_t *done, float *sums, float *__restrict__ out_w,
-                      float *__restrict__ out_mu, float *__restrict__ out_cov, float *__restrict__ out_feat, int vec)
-{
-    const int count = *n_items;
-    for (int k = blockIdx.x; k < count; k += gridDim.x) {
-        const int2 it = items[k];
-        fuse_big(sl, it.x, it.y, k, members + off[it.x], mcnt[it.x], done + it.x, sums, vec, out_w, out_mu, out_cov,
-                 out_feat);
-        __syncthreads();             // the next segment reuses the shared arrays
-    }
-}
-
-// out_w, out_mu, out_cov and out_feat of the other slots, a warp each: zeros for
-// a merged one, the slot's own values for a winner without members, sums over
-// the members (listed at members + off) otherwise.
-__global__ void __launch_bounds__(FTH)
+// flight per lane 51 and 159.  (64 registers: a kernel of its own for them, with more
+// loads in flight, costs every call a launch that mostly finds nothing, 3 us.)
+__global__ void __launch_bounds__(FTH, 4)
 assoc_fuse_kernel(Slots sl, const int32_t *__restrict__ parent, const int32_t *__restrict__ mcnt,
-                  const int32_t *__restrict__ off, const int32_t *__restrict__ members, float *__restrict__ out_w,
+                  const int32_t *__restrict__ off, const int32_t *__restrict__ members, const int2 *__restrict__ items,
+                  const int32_t *__restrict__ n_items, int32_t *done, float *sums, float *__restrict__ out_w,
                   float *__restrict__ out_mu, float *__restrict__ out_cov, float *__restrict__ out_feat, int vec)
 {
+    if (blockIdx.x < BIG_BLOCKS) {
+        const int count = *n_items;
+        for (int k = blockIdx.x; k < count; k += BIG_BLOCKS) {
+            const int2 it = items[k];
+            fuse_big(sl, it.x, it.y, k, members + off[it.x], mcnt[it.x], done + it.x, sums, vec, out_w, out_mu,
+                     out_cov, out_feat);
+            __syncthreads();             // the next segment reuses the shared arrays
+        }
+        return;
+    }
     const int T = sl.N + sl.B, F = sl.F;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-    const int t = blockIdx.x * FW + warp;
+    const int t = (blockIdx.x - BIG_BLOCKS) * FW + warp;
     const unsigned FULL = 0xffffffffu;
     if (t < T) {
         // (the slot's first features are in flight while the rest is looked up)
@@ -800,11 +799,9 @@ cudaError_t launch_assoc(const AssocArgs &a, cudaStream_t s)
     const Slots sl{N, B, a.F, a.ent_mu, a.ent_cov, a.ent_feat, a.ent_w, a.det_mu, a.det_cov, a.det_feat};
     const uintptr_t al = (uintptr_t)a.ent_feat | (uintptr_t)a.det_feat | (uintptr_t)a.out_feat;
     const int vec = a.F % 4 == 0 && (al & 15u) == 0 ? 1 : 0;
-    assoc_fuse_kernel<<<(unsigned)((T + FW - 1) / FW), FTH, 0, s>>>(sl, a.parent, a.mcnt, a.off, a.members, a.out_w,
-                                                                    a.out_mu, a.out_cov, a.out_feat, vec);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    assoc_fuse_big_kernel<<<BIG_BLOCKS, FTH, 0, s>>>(sl, a.mcnt, a.off, a.members, a.items, a.counters + kAssocItems,
-                                                     a.pos, a.sums, a.out_w, a.out_mu, a.out_cov, a.out_feat, vec);
+    assoc_fuse_kernel<<<(unsigned)((T + FW - 1) / FW + BIG_BLOCKS), FTH, 0, s>>>(
+        sl, a.parent, a.mcnt, a.off, a.members, a.items, a.counters + kAssocItems, a.pos, a.sums, a.out_w, a.out_mu,
+        a.out_cov, a.out_feat, vec);
     return cudaGetLastError();
 }
 
