@@ -554,7 +554,6 @@ farm_status farm_destroy(farm_ctx *ctx)
     for (int b = 0; b < farm::B_COUNT; ++b) cudaFree(c.ws.ptr[b]);
     cudaFree(c.d_err);
     cudaFree(c.d_fallback);
-    cudaFree(c.d_probe);
     cudaFree(ctx->d_scenes);
     cudaFree(c.mlp.params);
     cudaFree(c.mlp.w1b);
@@ -611,10 +610,9 @@ farm_status farm_create(farm_ctx **out, int device, void *cuda_stream, const far
     }
     if (cudaMalloc(&c.d_err, sizeof(int32_t)) != cudaSuccess) return bail(FARM_ENOMEM);
     if (cudaMemset(c.d_err, 0, sizeof(int32_t)) != cudaSuccess) return bail(FARM_ECUDA);
-    if (cudaMalloc(&c.d_fallback, sizeof(int32_t)) != cudaSuccess) return bail(FARM_ENOMEM);
-    if (cudaMemset(c.d_fallback, 0, sizeof(int32_t)) != cudaSuccess) return bail(FARM_ECUDA);
-    if (cudaMalloc(&c.d_probe, sizeof(int32_t)) != cudaSuccess) return bail(FARM_ENOMEM);
-    if (cudaMemset(c.d_probe, 0, sizeof(int32_t)) != cudaSuccess) return bail(FARM_ECUDA);
+    if (cudaMalloc(&c.d_fallback, 2 * sizeof(int32_t)) != cudaSuccess) return bail(FARM_ENOMEM);
+    if (cudaMemset(c.d_fallback, 0, 2 * sizeof(int32_t)) != cudaSuccess) return bail(FARM_ECUDA);
+    c.d_probe = c.d_fallback + 1;
     if (cudaHostAlloc(&c.h_err, sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess) return bail(FARM_ENOMEM);
     if (cudaMalloc(&ctx->d_scenes, kMaxScenes * sizeof(SceneDev)) != cudaSuccess) return bail(FARM_ENOMEM);
     if (cudaMemset(ctx->d_scenes, 0, kMaxScenes * sizeof(SceneDev)) != cudaSuccess) return bail(FARM_ECUDA);

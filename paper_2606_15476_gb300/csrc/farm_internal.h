@@ -161,7 +161,7 @@ struct Ctx {
     int pinned_variant = -1;      // >= 0: every grouped similarity launch uses this variant
     int32_t *d_fallback = nullptr;  // rows the thresholded select handed to its exact fallback
     bool training = false;          // a training call holds its buffers (B_TRAIN, B_TRAIN_IN)
-    int32_t *d_probe = nullptr;     // counts of a kernel that samples (0 between calls)
+    int32_t *d_probe = nullptr;     // counts of a kernel that samples (0 between calls), behind d_fallback
     int32_t *h_err = nullptr;     // pinned host mirror
     // batch state
     uint64_t batch_gen = 0;

@@ -204,6 +204,22 @@ __device__ __forceinline__ void rank_words(const uint64_t *cand, int cnt, int R,
     }
 }
 
+// The largest key of the candidates that may be ranked by bins, at least `top`:
+// of a row whose group maxima are staged as a prefix, an entry past it may lie
+// above them all.  (Out of line: only rows of more than UNION_MAX groups take it.)
+__device__ __noinline__ uint32_t largest_key(const uint64_t *cand, const int *s_cnt, uint32_t *s_mm, uint32_t top)
+{
+    __syncthreads();                 // the candidates are listed
+    const int tid = threadIdx.x, cnt = min(*s_cnt, RANK_MAX);
+    uint32_t hi = 0u;
+    for (int c = tid; c < cnt; c += TT) hi = max(hi, (uint32_t)(cand[c] >> 32));
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((tid & 31) == 0) s_mm[tid >> 5] = hi;
+    __syncthreads();
+    for (int w = 0; w < TT / 32; ++w) top = max(top, s_mm[w]);
+    return top;
+}
+
 // Shared memory of one CTA of the block-level select.
 struct ThreshSmem {
     uint32_t *ukeys;        // staged group maxima or a short row (dynamic)
@@ -251,9 +267,7 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     const int64_t n_groups = group_count(n, gshift);
     const int U = (int)min(n_groups, (int64_t)UNION_MAX);
     if (tid == 0) { s_cnt = 0; s_ng = 0; }
-    // the candidates' keys lie in [T, top] (of a row whose maxima are not all
-    // staged, once `top` has been raised to the candidates' below)
-    uint32_t T = 0u, top = 0xffffffffu;
+    uint32_t T = 0u, top = 0xffffffffu;    // the candidates' keys lie in [T, top]
 
     // For tau = key_value(T) and non-NaN x,
     // x >= tau holds exactly when order_key(x) >= T, so the passes below
@@ -307,6 +321,7 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
         } else {
             stream_tail(row, 0, n, tau, cand, &s_cnt);
         }
+        if (n_groups > U) top = largest_key(cand, &s_cnt, sm.s_mm, top);
     } else if (n <= kSelectSortAll) {
         // a short row: every entry staged, its R-th largest key found in shared memory
         for (int j = tid; j < n; j += TT) ukeys[j] = order_key(__ldcs(row + j));
@@ -326,17 +341,6 @@ __device__ __forceinline__ void thresh_row(const float *__restrict__ S, const fl
     }
     __syncthreads();
     const int cnt = s_cnt;
-    if (U >= R && n_groups > U && cnt <= RANK_MAX) {
-        // the maxima were a prefix of the row's, and an entry past it may lie
-        // above them all: the upper end comes from the candidates themselves
-        uint32_t hi = 0u;
-        for (int c = tid; c < cnt; c += TT) hi = max(hi, (uint32_t)(cand[c] >> 32));
-        hi = __reduce_max_sync(0xffffffffu, hi);
-        if ((tid & 31) == 0) sm.s_mm[tid >> 5] = hi;
-        __syncthreads();
-#pragma unroll
-        for (int w = 0; w < TT / 32; ++w) top = max(top, sm.s_mm[w]);
-    }
     // (fewer than R candidates cannot happen with group maxima of this row;
     // the exact select then stands in rather than list unfilled entries)
     if (cnt >= R && cnt <= RANK_MAX) {
