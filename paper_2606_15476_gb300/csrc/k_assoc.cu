@@ -31,7 +31,7 @@
 //    in a form free of the cancellation of M2 / w - mu mu'.  The members'
 //    order (and the last bits) may vary from run to run.
 //
-// 4,096 detections x 20,000 entities, F = 256: 173 us a call against 300 when
+// 4,096 detections x 20,000 entities, F = 256: 176 us a call against 300 when
 // the similarity stored the 328 MB block and a scan read it back, the
 // components took one CTA's rounds and the fusion four passes of atomics
 // (search 106 -> 25 us, components 57 -> the match kernel's tail, fusion and its
