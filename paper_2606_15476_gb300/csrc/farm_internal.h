@@ -490,7 +490,7 @@ cudaError_t preload_sim_few();
 // sim_single_variant picks (2, the CTA pairs, with `emit` or a gate).
 // Three FP16 terms, hi*hi + 2^-11 (hi*lo + lo*hi), from the split the
 // normalisation writes.
-// With `emit` (more than kSimFewRows rows) nothing is stored: every entry
+// With `emit` (more than kSimFewRows rows; its own gate set) nothing is stored: every entry
 // reaching its row's threshold is appended to the row's buffer; with a gate
 // only the first *gate rows are computed.
 cudaError_t launch_sim_tc_f16x3(const uint16_t *q_hi, const uint16_t *q_lo, const uint16_t *d_hi,
